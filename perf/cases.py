@@ -107,19 +107,35 @@ def draw(rng):
     return c
 
 
+def _tensors(case, seed):
+    """The tensors of the sequence(s): seeded draws on the GPU."""
+    c = case
+    kw = dict(seed=seed, B=c["B"], T=c["T"], H=c["H"], W=c["W"], cube=(c["ct"], c["ch"], c["cw"]), n_text=c["n_text"],
+              Hq=c["Hq"], Hkv=c["Hkv"], D=c["D"], top_p=c["p"], offset_std=c["sigma"], device="cuda")
+    if c["static_half"]:
+        return inputs.make_heterogeneous("case", with_q=c["kind"] != "decode", **kw)
+    return inputs.make_prefill("case", with_q=c["kind"] != "decode", n_prefix=c["n_prefix"],
+                               q_offset_std=1.0 if c["cohesive"] else 0.0,
+                               q_noise_std=0.25 if c["cohesive"] else 1.0, **kw)
+
+
+def _new_tokens(case, seed):
+    """A decode step's new token of every conversation, and how much text each of them holds."""
+    c = case
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed + 7)
+    new = lambda heads: torch.randn(c["B"], 1, heads, c["D"], generator=g, device="cuda").to(torch.bfloat16)  # noqa: E731
+    q, k, v = new(c["Hq"]), new(c["Hkv"]), new(c["Hkv"])
+    held = torch.randint(c["n_text"] // 2, c["n_text"] + 1, (c["B"],), generator=g, device="cuda")
+    return q, k, v, held.to(torch.int32)
+
+
 def prepare(case, seed):
     """The engine with its caches and workspace, the call's tensors, and an output buffer."""
     c = case
     cube = (c["ct"], c["ch"], c["cw"])
-    kw = dict(seed=seed, B=c["B"], T=c["T"], H=c["H"], W=c["W"], cube=cube, n_text=c["n_text"], Hq=c["Hq"],
-              Hkv=c["Hkv"], D=c["D"], top_p=c["p"], offset_std=c["sigma"], device="cuda")
     decode, chunk = c["kind"] == "decode", c["kind"] == "chunk"
-    if c["static_half"]:
-        wl = inputs.make_heterogeneous("case", with_q=not decode, **kw)
-    else:
-        wl = inputs.make_prefill("case", with_q=not decode, n_prefix=c["n_prefix"],
-                                 q_offset_std=1.0 if c["cohesive"] else 0.0,
-                                 q_noise_std=0.25 if c["cohesive"] else 1.0, **kw)
+    wl = _tensors(c, seed)
     eng = binding.AdaSAttn(cube=cube, n_q_heads=c["Hq"], n_kv_heads=c["Hkv"], head_dim=c["D"], top_p=c["p"],
                            top_k=c["top_k"])
     if decode:
@@ -127,13 +143,8 @@ def prepare(case, seed):
     eng.partition(c["B"], c["T"], c["H"], c["W"], c["n_text"] + c["n_prefix"] + (16 if decode else 0))
     state = {"case": c, "eng": eng}
     if decode:
-        g = torch.Generator(device="cuda")
-        g.manual_seed(seed + 7)
-        new = lambda heads: torch.randn(c["B"], 1, heads, c["D"], generator=g, device="cuda").to(torch.bfloat16)  # noqa: E731
-        state.update(q=new(c["Hq"]), k=new(c["Hkv"]), v=new(c["Hkv"]))
         # the conversations of a batch hold texts of different lengths
-        held = torch.randint(c["n_text"] // 2, c["n_text"] + 1, (c["B"],), generator=g, device="cuda")
-        state["text_len"] = held.to(torch.int32)
+        state["q"], state["k"], state["v"], state["text_len"] = _new_tokens(c, seed)
         eng.forward(None, wl.k, wl.v, c["n_text"])
     elif chunk:
         tok, t0, t1 = c["H"] * c["W"], c["frame_begin"], c["frame_begin"] + c["frame_count"]
@@ -225,3 +236,99 @@ def tolerance(case):
     rounded once.  The selection is exact up to ties (rows whose boundary lies within 1e-6 of the mass); no bit
     differed between the two paths."""
     return {"rel": 1.2e-2, "max": 0.4, "differ": 1e-5}
+
+
+# What `exact` takes on in about ten seconds: (query row, key) pairs of all heads.
+_MAX_EXACT_PAIRS = 28 * 70000 ** 2
+
+
+def _cube_order(case):
+    """For every raster video token its cube, and the tokens in cube order."""
+    c = case
+    t, y, x = torch.meshgrid(torch.arange(c["T"]), torch.arange(c["H"]), torch.arange(c["W"]), indexing="ij")
+    nH, nW = -(-c["H"] // c["ch"]), -(-c["W"] // c["cw"])
+    cube = ((t // c["ct"] * nH + y // c["ch"]) * nW + x // c["cw"]).reshape(-1)
+    rank = (((t % c["ct"]) * c["ch"] + y % c["ch"]) * c["cw"] + x % c["cw"]).reshape(-1)
+    order = torch.argsort(cube * (c["ct"] * c["ch"] * c["cw"]) + rank)
+    return cube.cuda(), order.cuda()
+
+
+def _kept_cubes(case, scores, candidates):
+    """Eq. 2 for rows of scores: the shortest prefix of the descending order whose mass reaches p (Top-K: the K first)
+    of the first `candidates[row]` cubes."""
+    c = case
+    N = scores.shape[-1]
+    cand = torch.arange(N, device=scores.device) < candidates[:, None]
+    if c["top_k"] == 0 and c["p"] >= 1.0:
+        return cand
+    prob = torch.nan_to_num(torch.softmax(scores.masked_fill(~cand, -math.inf), dim=-1), nan=0.0)
+    prob = torch.where(cand, prob, -1.0)                       # what is no candidate comes last
+    prob, at = torch.sort(prob, dim=-1, descending=True, stable=True)
+    if c["top_k"]:
+        first = (torch.arange(N, device=scores.device) < c["top_k"]).expand_as(prob)
+    else:
+        live = prob.clamp(min=0.0)
+        first = torch.cumsum(live, dim=-1) - live < float(torch.tensor(c["p"], dtype=torch.float32))
+    return torch.zeros_like(cand).scatter_(-1, at, first) & cand
+
+
+def _attend(q, k, v, keep, column, causal_from):
+    """Softmax attention of rows q [R, D] over keys [M, D]: key m is seen if keep[row, column[m]] and m <= causal_from + row."""
+    s = q @ k.T / math.sqrt(q.shape[-1])
+    seen = keep[:, column]
+    if causal_from is not None:
+        R, M = s.shape
+        seen &= torch.arange(M, device=q.device) <= causal_from + torch.arange(R, device=q.device)[:, None]
+    return torch.softmax(s.masked_fill_(~seen, -math.inf), dim=-1) @ v
+
+
+def exact(case, seed):
+    """Eqs. 1-3 in 64 bits with plain torch, in the layout of `run`.  The caches of keys and values are copies."""
+    c = case
+    Hq, Hkv, D, B = c["Hq"], c["Hkv"], c["D"], c["B"]
+    G, vid, n_pre = Hq // Hkv, c["T"] * c["H"] * c["W"], c["n_prefix"]
+    decode, chunk = c["kind"] == "decode", c["kind"] == "chunk"
+    if not decode and B * Hq * vid ** 2 > _MAX_EXACT_PAIRS:
+        return None
+    wl = _tensors(c, seed)
+    cube, order = _cube_order(c)
+    N = int(cube.max()) + 1
+    tok = c["H"] * c["W"]
+    begin = c["frame_begin"] * tok if chunk else 0             # the call's tokens, in sequence order
+    seen_video = (c["frame_begin"] + c["frame_count"]) * tok if chunk else vid
+    end = wl.k.shape[1] if seen_video == vid else seen_video
+    # rows and keys in the order [prefix][video by cube][text], where everything a token sees comes before it
+    seq = torch.cat([torch.arange(n_pre, device="cuda"), order + n_pre, torch.arange(n_pre + vid, wl.k.shape[1], device="cuda")])
+    column = torch.cat([torch.full((n_pre,), N, device="cuda"), cube[order], torch.full((wl.k.shape[1] - n_pre - vid,), N, device="cuda")])
+    seq, column = seq[:end], column[:end]
+    candidates = torch.where(column < N, column, N)            # preceding cubes; all cubes for the text,
+    candidates[:n_pre] = 0                                     # none for the prefix
+    held = torch.zeros(N, dtype=torch.float64, device="cuda").index_add_(0, cube, torch.ones(vid, dtype=torch.float64, device="cuda"))
+    means = torch.zeros(B, Hkv, N, D, dtype=torch.float64, device="cuda")
+    if decode:
+        q_new, k_new, v_new, text_len = _new_tokens(c, seed)
+    out = torch.zeros(B, 1 if decode else end - begin, Hq, D, dtype=torch.float64, device="cuda")
+    rows_at_once = max(64, (1 << 26) // end)
+    for b in range(B):
+        for kv in range(Hkv):
+            k, v = wl.k[b, seq, kv].double(), wl.v[b, seq, kv].double()
+            n_vid = min(seen_video, vid)
+            mean = means[b, kv].index_add_(0, column[n_pre:n_pre + n_vid], k[n_pre:n_pre + n_vid])
+            mean /= held[:, None]
+            for h in range(kv * G, kv * G + G):
+                if decode:
+                    n = n_pre + vid + int(text_len[b])
+                    q = q_new[b, :, h].double()
+                    keep = _kept_cubes(c, q @ mean.T / math.sqrt(D), torch.tensor([N], device="cuda"))
+                    keep = torch.cat([keep, torch.ones_like(keep[:, :1])], dim=1)
+                    ks, vs = torch.cat([k[:n], k_new[b, :, kv].double()]), torch.cat([v[:n], v_new[b, :, kv].double()])
+                    out[b, :, h] = _attend(q, ks, vs, keep, torch.cat([column[:n], column.new_tensor([N])]), None)
+                    continue
+                for r0 in range(begin, end, rows_at_once):
+                    r1 = min(r0 + rows_at_once, end)
+                    q = wl.q[b, seq[r0:r1], h].double()
+                    keep = _kept_cubes(c, q @ mean.T / math.sqrt(D), candidates[r0:r1])
+                    keep = torch.cat([keep, torch.ones_like(keep[:, :1])], dim=1)          # text and prefix
+                    keep.scatter_(1, column[r0:r1, None], True)                            # the own cube
+                    out[b, seq[r0:r1] - begin, h] = _attend(q, k[:r1], v[:r1], keep, column[:r1], r0)
+    return {"out": out, "k_cube": None, "v_cube": None, "cube_keys": means}
