@@ -19,7 +19,7 @@
 #include "decode_splitkv.cuh"
 #ifdef ADASPARK_WITH_TCGEN05
 #include "attn_prefill_tc.cuh"
-#include "score_select_fused.cuh"
+#include "select_nucleus.cuh"
 #include "attn_gather.cuh"
 #endif
 
@@ -32,9 +32,10 @@ struct adaspark_attn {
     int C, N, S_v, S_cap;
     adaspark_attn_layout_t layout;
     // workspace carving (byte offsets)
-    size_t fw_status_off, fw_headmax_off, fw_valid_off, fw_gcol_off, fw_mask_off, fw_union_off, fw_fallback_off, fw_scratch_off,
-        fw_kplanes_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
+    size_t fw_status_off, fw_headmax_off, fw_valid_off, fw_gcol_off, fw_mask_off, fw_union_off, fw_fallback_off,
+        fw_kplanes_off, fw_rowrange_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
         fw_gpartml_off, fw_total;
+    int score_items;            // query tiles per launch of the score / selection pair
     // query-gather path of the prefill: capacity in (row, key block) entries, decision threshold, byte budget
     uint32_t gather_cap;
     int gather_windows;
@@ -54,7 +55,7 @@ struct adaspark_attn {
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kExactCtas = 296;   // CTAs of the fp64 selection kernel (its scratch rows are sized for them)
+constexpr int kExactCtas = 592;   // CTAs of the fp64 selection kernel: four per SM
 // query-gather path: pairs of query tiles take it when their rows' (row, key block) entries are at most this
 // many per key block of the pair's union (measured break-even on a B200, see the attention profile), and the
 // partial results of all such pairs must fit this many bytes of workspace
@@ -62,6 +63,12 @@ constexpr float kGatherDefaultPairsPerBlock = 30.f;
 constexpr uint64_t kGatherDefaultBudget = 24ull << 30;
 constexpr uint64_t kGatherEntriesPerRow = 128;
 constexpr size_t kGatherWindowBytes = 40u << 20;
+// Scores of the query tiles of one launch (int32, all columns; about half of it is touched over a causal sequence):
+// in whole waves of one tile per SM, as many as fit this budget.  Fewer, longer launches beat a buffer that stays in
+// the L2: 64 MB / 160 MB / 640 MB give 0.53 / 0.52 / 0.46 ms at 16384 tokens and 6.84 / 6.87 / 5.65 ms at 65536 (28
+// heads, 64-token cubes).
+constexpr size_t kScoreBytes = 640u << 20;
+constexpr int kScoreWave = 148;
 size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 
 adaspark_status_t fail(adaspark_attn* h, adaspark_status_t st, const char* fmt, ...) {
@@ -214,10 +221,10 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     L.cube_keys_bytes = (int64_t)((size_t)batch * Hkv * N * D * 4);
 
     // forward workspace: header | head exponents | per-tile mask matrix | per-tile union words | rows left to
-    // the fp64 selection kernel | its score scratch | key digit planes (tcgen05 path)
+    // the fp64 selection kernel | key digit planes (tcgen05 path)
     size_t off = 0;
     h->fw_status_off = off; off = align_up(off + 256);
-    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 2);   // key exponents, then largest |k|^2
+    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 3);   // mean-key exponents, largest |k|^2, largest |mean key|^2
     h->fw_valid_off = off; off = align_up(off + (size_t)(S_cap / kBlockTok) * 2 * 4);   // which slots of a block hold a token
     const size_t n_cols = (size_t)(S_v + kBlockTok - 1) / kBlockTok;                     // key blocks that hold video
     // query-gather path: the rows are cut into windows whose slice of Q (all heads) is about a third of the L2
@@ -231,10 +238,18 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     h->fw_mask_off = off; off = align_up(off + (size_t)batch * Hq * n_tiles_cap * n_words * kTileRows * 4);
     h->fw_union_off = off; off = align_up(off + (size_t)batch * Hq * n_tiles_cap * n_words * 4);
     h->fw_fallback_off = off; off = align_up(off + (size_t)batch * Hq * n_tiles_cap * kTileRows * 4);
-    h->fw_scratch_off = off; off = align_up(off + (size_t)kExactCtas * kExactWarps * N_ld * 8);
     // digit planes (4 x int8 [B*Hkv*N_ld, 128]) of the mean keys; 128 rows of slack so that the last TMA box
     // stays inside the allocation
     h->fw_kplanes_off = off; off = align_up(off + ((size_t)4 * batch * Hkv * N_ld + 128) * 128);
+    // scores and score ranges of one launch of the score / selection pair
+    {
+        const size_t tile_bytes = (size_t)kTileRows * N_ld * 4, n_items = (size_t)batch * Hq * n_tiles_cap;
+        size_t waves = kScoreBytes / (tile_bytes * kScoreWave);
+        if (waves < 1) waves = 1;
+        h->score_items = (int)(waves * kScoreWave < n_items ? waves * kScoreWave : n_items);
+        h->fw_rowrange_off = off; off = align_up(off + (size_t)h->score_items * kTileRows * kRangeParts * sizeof(float2));
+        h->fw_scores_off = off; off = align_up(off + (size_t)h->score_items * tile_bytes);
+    }
     // query-gather path: per pair (mode, entries, offset) | per row (entries, first partial) | per row (m, l) of the
     // local range | per key block offsets + work items | entries | partial outputs | partial (m, l)
     {
@@ -385,14 +400,13 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             h->sm_count = sms;
         }
         int32_t* fallback_rows = (int32_t*)(ws + h->fw_fallback_off);
-        double* scratch = (double*)(ws + h->fw_scratch_off);
         const bool all = g.top_k <= 0 && !(g.top_p < 1.0);
         auto launch_exact = [&](const int32_t* rows, const uint32_t* n_list, long long n_ids) {
             if (D == 128)
-                select_exact_kernel<128><<<kExactCtas, kExactWarps * 32, 0, st>>>(g, qb, cube_keys, rows, n_list, n_ids, scratch,
+                select_exact_kernel<128><<<kExactCtas, kExactWarps * 32, g.N_ld * 8, st>>>(g, qb, cube_keys, rows, n_list, n_ids,
                                                                                    tile_mask, tile_union, sel_bitmap, sel_count);
             else
-                select_exact_kernel<64><<<kExactCtas, kExactWarps * 32, 0, st>>>(g, qb, cube_keys, rows, n_list, n_ids, scratch,
+                select_exact_kernel<64><<<kExactCtas, kExactWarps * 32, g.N_ld * 8, st>>>(g, qb, cube_keys, rows, n_list, n_ids,
                                                                                   tile_mask, tile_union, sel_bitmap, sel_count);
             return launch_ok(h, "select_exact_kernel");
         };
@@ -403,30 +417,60 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
 #ifdef ADASPARK_WITH_TCGEN05
         else if (h->prefill_kernel == 1) {
             uint32_t* head_max = (uint32_t*)(ws + h->fw_headmax_off);
+            uint32_t* head_norm2 = head_max + 2 * g.B * g.Hkv;
             unsigned char* kplanes = (unsigned char*)(ws + h->fw_kplanes_off);
+            auto* row_range = (float2*)(ws + h->fw_rowrange_off);
+            float* scores = (float*)(ws + h->fw_scores_off);
             const int n_rows = g.B * g.Hkv * g.N_ld;
-            key_exponent_kernel<<<dim3(g.B * g.Hkv, 8), 256, 0, st>>>(g, cube_keys, head_max);
+            key_exponent_kernel<<<dim3(g.B * g.Hkv, 8), 256, 0, st>>>(g, cube_keys, head_max, head_norm2);
             if (!launch_ok(h, "key_exponent_kernel")) return ADASPARK_ERR_CUDA;
             slice_keys_kernel<<<(n_rows + 3) / 4, 128, 0, st>>>(g, cube_keys, head_max, kplanes);
             if (!launch_ok(h, "slice_keys_kernel")) return ADASPARK_ERR_CUDA;
-            CUtensorMap tmKs;
-            if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols))
+            CUtensorMap tmKs, tmS;
+            if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
+                !encode_f32_2d(&tmS, scores, (uint64_t)h->score_items * kTileRows, g.N_ld, 32))
                 return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
-            const int n_items = g.B * g.Hq * (g.n_tiles - g.tile_begin);
-            const int grid = n_items < h->sm_count ? n_items : h->sm_count;
+            const int n_hb = g.B * g.Hq, n_items = n_hb * (g.n_tiles - g.tile_begin);
             const bool by_count = g.top_k > 0;
-#define ADASPARK_LAUNCH_FUSED(DD, BC)                                                                                  \
+            for (int item0 = 0; item0 < n_items; item0 += h->score_items) {
+                const int n_here = n_items - item0 < h->score_items ? n_items - item0 : h->score_items;
+                const int grid = n_here < h->sm_count ? n_here : h->sm_count;
+                int n_max = 0;                       // largest candidate count of the launch
+                for (int lvl = item0 / n_hb; lvl <= (item0 + n_here - 1) / n_hb; ++lvl) {
+                    const int m = tile_max_candidates(g, g.n_tiles - 1 - lvl);
+                    n_max = m > n_max ? m : n_max;
+                }
+#define ADASPARK_LAUNCH_SCORE(DD)                                                                                      \
     do {                                                                                                               \
-        const size_t smem = sizeof(FusedSmem<DD>) + 1024;                                                              \
-        if (!set_smem(h, score_select_fused_kernel<DD, BC>, smem, "score_select_fused_kernel")) return ADASPARK_ERR_CUDA; \
-        score_select_fused_kernel<DD, BC><<<grid, kFusedThreads, smem, st>>>(                                           \
-            g, n_items, qb, tmKs, head_max, tile_mask, tile_union, sel_bitmap, sel_count, fallback_rows,         \
-            &hdr->fallback_rows, &hdr->status);                                                                        \
+        const size_t smem = sizeof(ScoreSmem<DD>) + 1024;                                                              \
+        if (!set_smem(h, score_tc_kernel<DD>, smem, "score_tc_kernel")) return ADASPARK_ERR_CUDA;                      \
+        score_tc_kernel<DD><<<grid, kScoreThreads, smem, st>>>(g, item0, n_here, qb, tmKs, tmS, head_max, head_norm2,  \
+                                                               row_range, tile_union, &hdr->status);                   \
     } while (0)
-            if (D == 128) { if (by_count) ADASPARK_LAUNCH_FUSED(128, true); else ADASPARK_LAUNCH_FUSED(128, false); }
-            else { if (by_count) ADASPARK_LAUNCH_FUSED(64, true); else ADASPARK_LAUNCH_FUSED(64, false); }
-#undef ADASPARK_LAUNCH_FUSED
-            if (!launch_ok(h, "score_select_fused_kernel")) return ADASPARK_ERR_CUDA;
+                if (D == 128) ADASPARK_LAUNCH_SCORE(128); else ADASPARK_LAUNCH_SCORE(64);
+#undef ADASPARK_LAUNCH_SCORE
+                if (!launch_ok(h, "score_tc_kernel")) return ADASPARK_ERR_CUDA;
+#define ADASPARK_LAUNCH_SELECT(GG, KK, RES, BC)                                                                       \
+    do {                                                                                                               \
+        const size_t smem = select_smem_bytes(sizeof(SelectWarpSmem<GG>), g.n_words);                                  \
+        if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, BC>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
+        select_nucleus_kernel<GG, KK, RES, BC><<<2 * n_here, kSelectThreads, smem, st>>>(                              \
+            g, item0, scores, (const float4*)row_range, tile_mask, tile_union, sel_bitmap, sel_count, fallback_rows,   \
+            &hdr->fallback_rows);                                                                                      \
+    } while (0)
+#define ADASPARK_LAUNCH_SELECT_K(GG, KK, RES)                                                                         \
+    do {                                                                                                               \
+        if (by_count) ADASPARK_LAUNCH_SELECT(GG, KK, RES, true); else ADASPARK_LAUNCH_SELECT(GG, KK, RES, false);      \
+    } while (0)
+                if (n_max <= 256) ADASPARK_LAUNCH_SELECT_K(8, 32, 4);
+                else if (n_max <= 512) ADASPARK_LAUNCH_SELECT_K(16, 32, 4);
+                else if (n_max <= 1024) ADASPARK_LAUNCH_SELECT_K(32, 32, 4);
+                else if (n_max <= 2048) ADASPARK_LAUNCH_SELECT_K(32, 64, 2);
+                else ADASPARK_LAUNCH_SELECT_K(32, 128, 1);
+#undef ADASPARK_LAUNCH_SELECT_K
+#undef ADASPARK_LAUNCH_SELECT
+                if (!launch_ok(h, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA;
+            }
             // the rows it left over (normally none): list length is read on the device
             if (!launch_exact(fallback_rows, &hdr->fallback_rows, 0)) return ADASPARK_ERR_CUDA;
         }

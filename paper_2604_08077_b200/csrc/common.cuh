@@ -103,17 +103,17 @@ __device__ __forceinline__ size_t io_row(const Geom& g, int b, int pos) {
 
 // Number of candidate cubes of the row at `pos`: preceding cubes for video, none for the prefix, all cubes
 // for the text after the video.
-__device__ __forceinline__ int n_candidates(const Geom& g, int pos) {
+__host__ __device__ __forceinline__ int n_candidates(const Geom& g, int pos) {
     return pos < g.S_v ? (pos >> g.c_shift) : (pos < g.S_v + g.n_prefix ? 0 : g.N);
 }
 
 // Largest candidate count among the rows of query tile `tile` (candidate counts grow along the video, drop
 // to zero on the text prefix and are N on the text after it).
-__device__ __forceinline__ int tile_max_candidates(const Geom& g, int tile) {
-    const int first = tile * kTileRows, last = min(first + kTileRows, g.S) - 1;
-    int m = n_candidates(g, last);
-    if (first < g.S_v && last >= g.S_v) m = max(m, n_candidates(g, g.S_v - 1));
-    return m;
+__host__ __device__ __forceinline__ int tile_max_candidates(const Geom& g, int tile) {
+    const int first = tile * kTileRows, last = (first + kTileRows < g.S ? first + kTileRows : g.S) - 1;
+    const int m = n_candidates(g, last);
+    const int m_video = first < g.S_v && last >= g.S_v ? n_candidates(g, g.S_v - 1) : 0;
+    return m > m_video ? m : m_video;
 }
 
 // First 64-key block of the local range of the 256-row pair of query tiles that starts at pair_pos0: the block
@@ -232,7 +232,12 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
 // byte offset of 16-byte chunk `chunk` of 128-byte row `row` under the 128-byte swizzle
 __device__ __forceinline__ int sw128(int row, int chunk) { return row * 128 + ((chunk ^ (row & 7)) << 4); }
 
-// ---- sm_100 three-input float maximum ------------------------------------------
+// ---- sm_100 three-input float maximum and minimum --------------------------------
+__device__ __forceinline__ float fmin3(float a, float b, float c) {
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));

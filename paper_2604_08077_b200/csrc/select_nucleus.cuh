@@ -1,0 +1,408 @@
+// K3b: nucleus selection (Eq. 2) from the scores of score_tc.cuh, G lanes of a warp per query row.
+//
+// Scores s_j are in log2 units; the order is descending score, then ascending cube index, the mass of a cube is
+// 2^(s_j - max).  A row's scores stay in registers (kK per lane) and are swept twice:
+//   sweep 1  masses are added to the row's total Z and, quantised, to a histogram over the distance from the maximum
+//            in shared memory (16 G buckets; the last takes everything beyond): the bucket in which the cumulative
+//            mass crosses p Z is found from it
+//   sweep 2  cubes before that bucket are selected (one bit each, collected from the sign of a subtraction) and their
+//            exact mass is summed; the few cubes inside it (widened by kGuard at both ends) are listed, and each
+//            learns the cumulative mass up to it: it is selected if the mass before it has not reached p Z
+// A bucket with more than kSelectCand cubes is split by further histograms over its cubes alone (rare, slow path).
+// Top-K (kByCount): the same with every mass = 1 and a target of min(top_k, candidates).
+//
+// Everything here is fp32, so a row is decided here only if its boundary is clear of what fp32 can be off by, and
+// handed to the fp64 kernel (list in the workspace) otherwise: a cumulative mass within eps of p Z, or a last selected
+// and a first rejected cube whose scores differ by less than kGapEps.  eps: an error e of the masses, of whatever sign,
+// moves a cumulative share by at most 2 p (1 - p) e <= e / 2; ex2.approx is off by up to 2^-22, a score by 2^-24 of its
+// size and its distance from the maximum by 2^-25 of its size (both times ln 2; the cubes that carry mass lie within
+// about 8 units of the maximum and no further from 0 than it), and the sums of Z and of the base by about 1e-7
+// together: (2.4e-7 + 4.1e-8 (|max| + (8 + |max|) / 2)) / 2 + 1e-7 < 4e-7 + 3.2e-8 |max|.  On the benchmark inputs that
+// is one row in 10^4 to 10^3.  So are the rows the score kernel
+// marked, and rows with more equal scores at the boundary than the list holds.
+//
+// What bounds it: instruction issue, about 18 instructions per cube and lane and 300 per warp.  Sharing a warp among
+// 32 / G rows spreads the second figure over several rows; the per-cube work is spread over the pipes (the bits come
+// from funnel shifts of signs, clamps from saturating multiply-adds, the exponential from the MUFU unit), because the
+// integer / comparison pipe issues at half the rate of the fp32 pipe.
+#pragma once
+#include "score_tc.cuh"
+
+namespace adaspark {
+
+constexpr int kSelectThreads = 256;
+constexpr int kSelectRows = 8;           // consecutive rows of a warp: its mask words fill 32-byte sectors
+constexpr int kSelectWarps = kSelectThreads / 32;
+constexpr int kSelectCand = 32;          // cubes of the crossing bucket a row may list
+constexpr int kMaxHistLevels = 8;        // histograms of a row before it is handed to the fp64 kernel
+constexpr float kMassEps = 4e-7f, kMassEpsTop = 3.2e-8f;   // of Z: the first plus |max| times the second
+constexpr float kGapEps = 2.4e-7f;       // of the larger of |s| and 1/4 (2^-22: twice the error of two scores)
+constexpr float kGuard = 1e-3f;          // of a bucket
+constexpr float kBucketsPerUnit = 8.f;   // first histogram, per log2 unit: at least so many (more if the row's range is small)
+
+// Lanes per row and scores per lane by candidate count: 16 G buckets of 1/8 (1/16, 1/32) log2 unit hold at most about
+// 6 (normal scores of deviation 1.5) of 256 (512, 1024) cubes.
+// Shared memory of one warp; its mask words [n_words][8 rows] follow those of all warps.
+template <int G>
+struct SelectWarpSmem {
+    uint32_t hist[512];                                   // [bucket][row of the warp]
+    float4 cand[32 / G][kSelectCand];                     // score, mass, cube
+    int32_t count[32 / G];
+    int32_t pad[4 - (32 / G) % 4];
+};
+__host__ __device__ inline size_t select_smem_bytes(size_t warp_bytes, int n_words) {
+    return kSelectWarps * (warp_bytes + (size_t)n_words * kSelectRows * 4);
+}
+
+__device__ __forceinline__ float sat_fma(float a, float b, float c) {     // min(max(a b + c, 0), 1)
+    return __saturatef(fmaf(a, b, c));
+}
+
+// One warp per 8 rows of a tile, warps work on their own: 2 CTAs per item of the launch.  scores / row_range: what score_tc_kernel left for the items [item0, ..).
+// tile_mask as mask_index() describes; tile_union (cleared) receives the OR of each word over the tile's rows;
+// fallback_rows[0 .. *fallback_count) receives ((b*Hq+h)*n_tiles_cap + tile)*128 + r of the rows left to the fp64
+// kernel.  G * kK >= the launch's largest candidate count; kBits: G * kK masses of at most 2^kBits fit 32 bits.
+template <int G, int kK, int kResident, bool kByCount>
+__global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kernel(
+    Geom g, int item0, const float* __restrict__ scores, const float4* __restrict__ row_range,
+    uint32_t* __restrict__ tile_mask, uint32_t* __restrict__ tile_union, uint32_t* __restrict__ sel_bitmap,
+    int32_t* __restrict__ sel_count, int32_t* __restrict__ fallback_rows, uint32_t* __restrict__ fallback_count) {
+    extern __shared__ __align__(16) unsigned char select_raw[];
+    constexpr int R = 32 / G, kBuckets = 16 * G, kSteps = kK / 4;          // rows per warp; steps of 4 columns per lane
+    constexpr int kMasks = (kK + 31) / 32;                                 // bit words per lane
+    constexpr int kBits = kByCount ? 0 : (G * kK <= 256 ? 22 : G * kK <= 1024 ? 21 : G * kK <= 2048 ? 20 : 19);
+    constexpr float kUnit = (float)(1 << kBits);
+    constexpr uint32_t kFull = 0xffffffffu;
+    constexpr float kMagic = 8388608.f;                                    // 2^23: low mantissa bits = the integer part
+    constexpr uint32_t kMagicBits = 0x4B000000u;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int s = lane & (G - 1), row_w = lane / G;                        // lane inside the row's group, row of the warp
+    const int item = blockIdx.x >> 1, row0 = ((blockIdx.x & 1) * kSelectWarps + warp) * kSelectRows;   // first row of the warp
+    const ScoreItem w = score_item(g, item0 + item);
+    const size_t gt_cap = (size_t)(w.b * g.Hq + w.h) * g.n_tiles_cap + w.tile;
+    const int n_words_live = min(2 * w.n_ct, g.n_words);                   // words that can hold a candidate
+    SelectWarpSmem<G>& sm = reinterpret_cast<SelectWarpSmem<G>*>(select_raw)[warp];
+    uint32_t* words = reinterpret_cast<uint32_t*>(select_raw + kSelectWarps * sizeof(SelectWarpSmem<G>)) + (size_t)warp * g.n_words * kSelectRows;
+    uint32_t* hist = sm.hist;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = lane; i < n_words_live * kSelectRows; i += 32) words[i] = 0u;
+    __syncwarp();
+
+    auto group_sum = [&](float x) -> float {
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+        return x;
+    };
+    auto group_any = [&](bool p) -> bool {
+        const uint32_t m = __ballot_sync(kFull, p);
+        return ((G == 32 ? m : (m >> (row_w * G)) & ((1u << (G & 31)) - 1u))) != 0u;
+    };
+#pragma unroll 1
+    for (int pass = 0; pass < kSelectRows / R; ++pass) {
+        const int rl = pass * R + row_w, r = row0 + rl;
+        const int pos = w.tile * kTileRows + r;
+        const int n = slot_live(g, pos) ? n_candidates(g, pos) : 0;
+        const int n_most = __reduce_max_sync(kFull, n), n_least = __reduce_min_sync(kFull, n);
+        if (n_most == 0) continue;
+        const size_t srow = (size_t)item * kTileRows + r;
+        // the rows of the next pass on their way into the L1 (one 128-byte line per lane and 32 scores per lane)
+        if (pass + 1 < kSelectRows / R) {
+#pragma unroll
+            for (int u = 0; u < kMasks; ++u)
+                if (s * 32 + u * 32 * G < n_most)
+                    asm volatile("prefetch.global.L1 [%0];\n" ::"l"(scores + ((size_t)item * kTileRows + r + R) * g.N_ld + s * 32 + u * 32 * G));
+        }
+        // ---- the row's scores (column 4 G c + 4 s + i in v[4 c + i]), largest and smallest
+        const float* src = scores + srow * g.N_ld + 4 * s;
+        float v[kK];
+#pragma unroll
+        for (int c = 0; c < kSteps; ++c) {
+            float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            if (c * 4 * G < n_most) {
+                const int col = c * 4 * G + 4 * s;
+                if (col < n) x = __ldg(reinterpret_cast<const float4*>(src + c * 4 * G));
+                if ((c + 1) * 4 * G > n_least) {                           // the end of a row's candidates
+                    if (col + 1 >= n) x.y = -INFINITY;
+                    if (col + 2 >= n) x.z = -INFINITY;
+                    if (col + 3 >= n) x.w = -INFINITY;
+                }
+            }
+            v[4 * c] = x.x; v[4 * c + 1] = x.y; v[4 * c + 2] = x.z; v[4 * c + 3] = x.w;
+        }
+        float top = 0.f, low = 0.f;
+        if (n > 0) {
+            const float4 ra = row_range[2 * srow], rb = row_range[2 * srow + 1];
+            top = fmaxf(fmaxf(ra.x, ra.z), fmaxf(rb.x, rb.z));
+            low = fminf(fminf(ra.y, ra.w), fminf(rb.y, rb.w));
+        }
+        bool give_up = n > 0 && !(top > -INFINITY && low > -INFINITY);     // marked by the score kernel
+        if (give_up) top = low = 0.f;
+        // mass of a score at the distance d = s - max from the maximum; distances are taken the maximum; distances are taken from the maximum first, where they are exact
+        auto mass = [&](float d) -> float { return kByCount ? (d > -INFINITY ? 1.f : 0.f) : fast_exp2(d); };
+
+        // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, bucket = round(u)
+        const float per_unit = fminf(fmaxf(kBucketsPerUnit * (G / 8), (float)(kBuckets - 1) / (top - low)), 1e18f);
+        float a_mul = -per_unit, a_add = 0.f;                              // u = d * a_mul + a_add
+        float z = 0.f;
+        uint32_t* my_hist = hist + row_w;
+        const float u_mul = a_mul * (1.f / (kBuckets - 1));
+        const uint32_t hist_addr = smem_u32(my_hist) - kMagicBits * (4u * R);   // plus 4 R times the bits of 2^23 + bucket
+#pragma unroll
+        for (int c = 0; c < kSteps; ++c) {
+            if (c * 4 * G < n_most) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float d = v[4 * c + i] - top;
+                    v[4 * c + i] = d;
+                    const float m = mass(d);
+                    z += m;
+                    const uint32_t b = __float_as_uint(fmaf(__saturatef(d * u_mul), (float)(kBuckets - 1), kMagic));
+                    const uint32_t q = __float_as_uint(fmaf(m, kUnit, kMagic)) - kMagicBits;
+                    asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(hist_addr + b * (4u * R)), "r"(q) : "memory");
+                }
+            }
+        }
+        z = group_sum(z);
+        const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * g.top_p);
+        const float eps = kByCount ? 0.f : z * fmaf(fabsf(top), kMassEpsTop, kMassEps);
+        float base = 0.f;                                                  // mass selected so far
+        uint32_t before[kMasks], inside[kMasks];                           // per lane: bit e = its e-th score
+#pragma unroll
+        for (int k = 0; k < kMasks; ++k) { before[k] = 0u; inside[k] = 0u; }
+        bool unsure = false;
+        bool active = n > 0 && !give_up;                                   // the row still narrows its interval
+        int n_cand = 0;
+#pragma unroll 1
+        for (int level = 0;; ++level) {
+            __syncwarp();
+            // ---- the bucket in which the cumulative (quantised) mass crosses the target: first the lane whose 16
+            // buckets hold it, then the bucket (read in an order of its own by each lane: no bank is met twice)
+            uint32_t sum = 0u;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) sum += my_hist[(s * 16 + (u ^ (s & 15))) * R];
+            uint32_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < G; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, o, G);
+                if (s >= o) incl += t;
+            }
+            const uint32_t thr = max((uint32_t)fmaxf((target - base) * kUnit, 0.f), 1u);
+            uint32_t over = __ballot_sync(kFull, incl >= thr);
+            if (G < 32) over = (over >> (row_w * G)) & ((1u << (G & 31)) - 1u);
+            const int own = over ? __ffs(over) - 1 : G - 1;
+            const uint32_t cum = __shfl_sync(kFull, incl - sum, own, G);
+            constexpr int kPer = 16 / (G < 16 ? G : 16);                   // buckets per lane in the second step
+            uint32_t part[kPer], psum = 0u;
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                part[u] = s * kPer < 16 ? my_hist[(own * 16 + (s & 15) * kPer + u) * R] : 0u;
+                psum += part[u];
+            }
+            uint32_t pincl = psum;
+#pragma unroll
+            for (int o = 1; o < (G < 16 ? G : 16); o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, pincl, o, G);
+                if (s >= o) pincl += t;
+            }
+            over = __ballot_sync(kFull, s * kPer < 16 && cum + pincl >= thr);
+            if (G < 32) over = (over >> (row_w * G)) & ((1u << (G & 31)) - 1u);
+            const int own2 = over ? __ffs(over) - 1 : (G < 16 ? G : 16) - 1;
+            int cb = s * kPer;
+            if (kPer == 2 && cum + (pincl - psum) + part[0] < thr) ++cb;
+            cb = __shfl_sync(kFull, cb, own2, G) + own * 16;
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
+            // ---- sweep 2: before / inside the bucket [cb - 1/2, cb + 1/2], widened by the guard
+            const float lo_u = (float)cb - (0.5f + kGuard);
+            const float hi_u = cb == kBuckets - 1 ? 3e38f : (float)cb + (0.5f + kGuard);
+            float add = 0.f;
+            n_cand = 0;
+            if (level == 0) {
+#pragma unroll
+                for (int c = kSteps - 1; c >= 0; --c) {
+                    if (c * 4 * G < n_most) {
+#pragma unroll
+                        for (int i = 3; i >= 0; --i) {
+                            const float d = v[4 * c + i];
+                            const int k = (4 * c + i) >> 5;
+                            const float ua = fmaf(d, a_mul, -lo_u);
+                            before[k] = __funnelshift_l(__float_as_uint(ua), before[k], 1);
+                            inside[k] = __funnelshift_l(__float_as_uint(fmaf(d, a_mul, -hi_u)), inside[k], 1);
+                            add = fmaf(mass(d), __saturatef(ua * -1099511627776.f), add);   // times 2^40: 1 before, 0 else
+                        }
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kMasks; ++k) inside[k] &= ~before[k];
+            } else {
+                for (int k = 0; k < kMasks; ++k) {
+                    uint32_t bits = active ? inside[k] : 0u;
+                    while (bits) {
+                        const int e = __ffs(bits) - 1;
+                        bits &= bits - 1u;
+                        const float d = __ldg(src + (((k * 32 + e) >> 2) * 4 * G + (e & 3))) - top;
+                        const float u = fmaf(d, a_mul, a_add);
+                        if (u < lo_u) { before[k] |= 1u << e; inside[k] &= ~(1u << e); add += mass(d); }
+                        else if (!(u < hi_u)) inside[k] &= ~(1u << e);
+                    }
+                }
+                __syncwarp();
+            }
+#pragma unroll
+            for (int k = 0; k < kMasks; ++k) n_cand += __popc(inside[k]);
+            add = group_sum(add);
+            n_cand = (int)(group_sum((float)n_cand) + 0.5f);
+            if (active) base += add;
+            if (n_cand <= kSelectCand) active = false;
+            if (active && level + 1 == kMaxHistLevels) { give_up = true; active = false; }
+            if (!__any_sync(kFull, active)) break;
+            // ---- rare: split the bucket of the rows that hold too many cubes in it
+            const float width = cb == kBuckets - 1 ? fmaxf(fmaf(low - top, a_mul, a_add) - lo_u, 1.f) : 1.f + 2.f * kGuard;
+            const float fine = (float)(kBuckets - 1) / width;
+            if (active) {
+                a_add = (a_add - lo_u) * fine;
+                a_mul = a_mul * fine;
+                if (!(fabsf(a_mul) < 1e30f)) { give_up = true; active = false; }
+            }
+            for (int k = 0; k < kMasks; ++k) {
+                uint32_t bits = active ? inside[k] : 0u;
+                while (bits) {
+                    const int e = __ffs(bits) - 1;
+                    bits &= bits - 1u;
+                    const float d = __ldg(src + (((k * 32 + e) >> 2) * 4 * G + (e & 3))) - top;
+                    const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), a_add * (1.f / (kBuckets - 1)));
+                    const uint32_t b = __float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)) - kMagicBits;
+                    atomicAdd(&my_hist[b * R], __float_as_uint(fmaf(mass(d), kUnit, kMagic)) - kMagicBits);
+                }
+            }
+            __syncwarp();
+        }
+        // ---- list the cubes inside the bucket
+        const bool decide = n > 0 && !give_up;
+        const int n_list = decide ? n_cand : 0;
+        const int n_list_most = __reduce_max_sync(kFull, n_list);
+        if (s == 0) sm.count[row_w] = 0;
+        for (int i = n_list + s; i < n_list_most; i += G) sm.cand[row_w][i] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kMasks; ++k) {
+            uint32_t bits = decide ? inside[k] : 0u;
+            int slot = bits ? atomicAdd(&sm.count[row_w], __popc(bits)) : 0;
+            while (bits) {
+                const int e = __ffs(bits) - 1;
+                bits &= bits - 1u;
+                const int j = ((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3);
+                const float x = __ldg(scores + srow * g.N_ld + j);
+                sm.cand[row_w][slot++] = make_float4(x, mass(x - top), __int_as_float(j), 0.f);
+            }
+        }
+        __syncwarp();
+        // ---- the words of what lies before the bucket: lane s holds nibble s & 7 of words (s >> 3) + c G / 8
+#pragma unroll
+        for (int k = 0; k < kMasks; ++k) {
+            uint32_t t = decide ? before[k] : 0u;                          // nibble c: columns of step 8 k + c
+            // transpose the 8 x 8 nibbles of 8 neighbouring lanes: lane c then holds word c
+            uint32_t o = __shfl_xor_sync(kFull, t, 4);
+            t = (s & 4) ? ((t & 0xffff0000u) | (o >> 16)) : ((t & 0x0000ffffu) | (o << 16));
+            o = __shfl_xor_sync(kFull, t, 2);
+            t = (s & 2) ? ((t & 0xff00ff00u) | ((o >> 8) & 0x00ff00ffu)) : ((t & 0x00ff00ffu) | ((o << 8) & 0xff00ff00u));
+            o = __shfl_xor_sync(kFull, t, 1);
+            t = (s & 1) ? ((t & 0xf0f0f0f0u) | ((o >> 4) & 0x0f0f0f0fu)) : ((t & 0x0f0f0f0fu) | ((o << 4) & 0xf0f0f0f0u));
+            const int wd = (8 * k + (s & 7)) * (G / 8) + (s >> 3);
+            if (wd < n_words_live && n > 0) words[wd * kSelectRows + rl] = t;
+        }
+        __syncwarp();
+        // ---- each listed cube: the mass up to and including it
+        float last = INFINITY, next = -INFINITY;                           // lowest selected, highest rejected score of my cubes
+        bool reached = false;
+        for (int i0 = 0; i0 < n_list_most; i0 += G) {
+            const int i = i0 + s;
+            const bool mine = i < n_list;
+            const float4 me = sm.cand[row_w][min(i, n_list_most - 1)];
+            const int ji = __float_as_int(me.z);
+            float acc = base;                                              // and the listed cubes before mine
+            for (int k = 0; k < n_list_most; ++k) {
+                const float4 ck = sm.cand[row_w][k];
+                if (ck.x > me.x || (ck.x == me.x && __float_as_int(ck.z) < ji)) acc += ck.y;
+            }
+            if (mine) {
+                if (acc < target) {
+                    atomicOr(&words[(ji >> 5) * kSelectRows + rl], 1u << (ji & 31));
+                    last = fminf(last, me.x);
+                } else {
+                    next = fmaxf(next, me.x);
+                }
+                reached = reached || acc + me.y >= target;
+                if (!kByCount) unsure = unsure || fabsf(acc - target) <= eps || fabsf(acc + me.y - target) <= eps;
+            }
+        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) {
+            last = fminf(last, __shfl_xor_sync(kFull, last, o));
+            next = fmaxf(next, __shfl_xor_sync(kFull, next, o));
+        }
+        unsure = unsure || last - next <= kGapEps * fmaxf(fabsf(last), 0.25f);   // infinite unless both exist
+        const bool any_unsure = group_any(unsure), any_reached = group_any(reached);   // both by all lanes
+        unsure = any_unsure || !any_reached || !(base < target);
+        if (n > 0 && (give_up || unsure)) {
+            for (int wd = s; wd < n_words_live; wd += G) words[wd * kSelectRows + rl] = 0u;
+            if (s == 0) fallback_rows[atomicAdd(fallback_count, 1u)] = (int32_t)(gt_cap * kTileRows + r);
+        }
+        __syncwarp();
+    }
+    // ---- mask words (32-byte sectors of 8 rows), union words, the caller's copies
+    for (int i = lane; i < g.n_words * 2; i += 32) {
+        const int wd = i >> 1, c4 = i & 1;
+        const uint4 val = wd < n_words_live ? *reinterpret_cast<const uint4*>(&words[wd * kSelectRows + c4 * 4]) : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(tile_mask + (gt_cap * g.n_words + wd) * kTileRows + row0 + c4 * 4) = val;
+    }
+    for (int wd = lane; wd < n_words_live; wd += 32) {
+        const uint4 x = *reinterpret_cast<const uint4*>(&words[wd * kSelectRows]), y = *reinterpret_cast<const uint4*>(&words[wd * kSelectRows + 4]);
+        const uint32_t u = (x.x | x.y | x.z | x.w) | (y.x | y.y | y.z | y.w);
+        if (u) atomicOr(tile_union + gt_cap * g.n_words + wd, u);
+    }
+    if (sel_bitmap != nullptr || sel_count != nullptr) {
+        for (int rl = 0; rl < kSelectRows; ++rl) {
+            const int pos = w.tile * kTileRows + row0 + rl;
+            if (!slot_live(g, pos)) continue;
+            const size_t raster_row = (size_t)(w.b * g.Hq + w.h) * g.S_io + (pos_to_io(g, pos) - g.pos_begin);
+            int cnt = 0;
+            for (int wd = lane; wd < g.n_words; wd += 32) {
+                const uint32_t word = wd < n_words_live ? words[wd * kSelectRows + rl] : 0u;
+                cnt += __popc(word);
+                if (sel_bitmap) sel_bitmap[raster_row * g.n_words + wd] = word;
+            }
+            cnt = __reduce_add_sync(kFull, cnt);
+            if (sel_count && lane == 0) sel_count[raster_row] = cnt;
+        }
+    }
+}
+
+// p >= 1 without Top-K: every candidate cube is selected (Eq. 2 with p = 1).  grid (tiles of the call, Hq, B),
+// 128 threads = rows of the tile.
+__global__ void __launch_bounds__(128) select_all_kernel(Geom g, uint32_t* __restrict__ tile_mask,
+                                                         uint32_t* __restrict__ tile_union, uint32_t* __restrict__ sel_bitmap,
+                                                         int32_t* __restrict__ sel_count) {
+    const int tile = blockIdx.x + g.tile_begin, h = blockIdx.y, b = blockIdx.z, r = threadIdx.x;
+    const int pos = tile * kTileRows + r;
+    const bool live = slot_live(g, pos);
+    const int n = live ? n_candidates(g, pos) : 0;
+    const size_t gt_cap = (size_t)(b * g.Hq + h) * g.n_tiles_cap + tile;
+    const size_t raster_row = live ? (size_t)(b * g.Hq + h) * g.S_io + (pos_to_io(g, pos) - g.pos_begin) : 0;
+    const int n_max = tile_max_candidates(g, tile);
+    for (int w = 0; w < g.n_words; ++w) {
+        const int rem = n - w * 32;
+        const uint32_t word = rem >= 32 ? 0xffffffffu : (rem > 0 ? (1u << rem) - 1u : 0u);
+        tile_mask[(gt_cap * g.n_words + w) * kTileRows + r] = word;
+        if (sel_bitmap && live) sel_bitmap[raster_row * g.n_words + w] = word;
+        if (r == 0) {
+            const int remx = n_max - w * 32;
+            tile_union[gt_cap * g.n_words + w] = remx >= 32 ? 0xffffffffu : (remx > 0 ? (1u << remx) - 1u : 0u);
+        }
+    }
+    if (sel_count && live) sel_count[raster_row] = n;
+}
+
+}  // namespace adaspark

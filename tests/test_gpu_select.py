@@ -1,0 +1,62 @@
+"""Selection from the tensor-core scores: bit by bit the selection of the fp64 kernel.
+
+Rows whose boundary is nearer than fp32 can tell are handed to the fp64 kernel, all others are decided from fp32
+scores, so no bit may differ.  The candidate counts are those at which the kernel changes its shape (lanes per row,
+scores per lane, mask words) and their neighbours."""
+from __future__ import annotations
+
+import pytest
+import torch
+
+from paper_2604_08077_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _selection(wl, kernel, k=None):
+    eng = binding.AdaSAttn(cube=wl.cube, n_q_heads=wl.Hq, n_kv_heads=wl.Hkv, head_dim=wl.D, top_p=wl.top_p, top_k=wl.top_k)
+    binding.adaspark_attn_set_prefill_kernel(eng.handle, kernel)
+    eng.set_gather(0.0, 0)
+    eng.partition(wl.B, wl.T, wl.H, wl.W, wl.n_text + wl.n_prefix)
+    k = wl.k if k is None else k
+    _, bitmap, count = eng.forward(wl.q.cuda(), k.cuda(), wl.v.cuda(), wl.n_text, want_selection=True, n_prefix=wl.n_prefix)
+    torch.cuda.synchronize()
+    hdr = eng.header()
+    assert hdr.status == 0
+    return bitmap, count, hdr
+
+
+def _equal(wl, k=None):
+    got, want = _selection(wl, 1, k), _selection(wl, 0, k)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    return got[2]
+
+
+@pytest.mark.parametrize("n_cubes", [1, 2, 31, 33, 64, 65, 255, 257, 511, 513, 1023, 1025, 2047, 2049, 4096])
+@pytest.mark.parametrize("rule", ["p", "k"])
+def test_candidate_counts_around_every_shape(n_cubes, rule):
+    # text rows have all the cubes as candidates, the video rows every smaller count
+    wl = inputs.make_prefill("counts", seed=900 + n_cubes, B=1, T=n_cubes, H=4, W=4, cube=(1, 4, 4), n_text=129, Hq=2,
+                             Hkv=1, D=64 if n_cubes % 2 else 128, top_p=0.9, offset_std=1.5)
+    if rule == "k":
+        wl.top_k = min(24, max(1, n_cubes // 3))
+    _equal(wl)
+
+
+@pytest.mark.parametrize("top_p", [1e-6, 0.3, 0.999])
+@pytest.mark.parametrize("offset_std", [0.0, 0.05, 4.0])
+def test_flat_and_sharp_scores(top_p, offset_std):
+    wl = inputs.make_prefill("flat", seed=77, B=2, T=24, H=8, W=12, cube=(2, 4, 4), n_text=40, n_prefix=5, Hq=6, Hkv=2,
+                             D=64, top_p=top_p, offset_std=offset_std)
+    _equal(wl)
+
+
+@pytest.mark.parametrize("copies", [2, 8, 40])
+def test_equal_scores(copies):
+    """Groups of identical cubes: the boundary falls among equal scores (more of them than the list holds, too)."""
+    wl = inputs.make_prefill("ties", seed=78, B=1, T=80, H=8, W=8, cube=(2, 4, 4), n_text=33, Hq=4, Hkv=2, D=128,
+                             top_p=0.8, offset_std=1.0)
+    k = wl.k.clone()
+    frames = k[:, :wl.S_v].view(1, 40, 2, 64, 2, 128)
+    frames.copy_(frames[:, ::copies].repeat_interleave(copies, 1)[:, :40])
+    assert _equal(wl, k).fallback_rows > 0
