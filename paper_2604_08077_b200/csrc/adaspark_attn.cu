@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <utility>
 
 #include "common.cuh"
 #include "relayout_pool.cuh"
@@ -143,6 +144,24 @@ bool launch_ok(adaspark_attn* h, const char* what) {
     }
     h->launches++;
     return true;
+}
+
+// Launches a kernel that may start while the kernel before it in the stream still runs; it waits for that one's
+// results itself (wait_for_previous_kernel).
+template <typename... KArgs, typename... Args>
+void launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);   // an error is picked up by launch_ok
 }
 
 template <typename K>
@@ -694,7 +713,6 @@ adaspark_status_t adaspark_attn_decode(adaspark_attn_t* h, const void* q_new, co
     char* ws = (char*)workspace;
     auto* hdr = (adaspark_attn_workspace_header_t*)(ws + h->dc_status_off);
     int32_t* status = &hdr->status;
-    cudaMemsetAsync(hdr, 0, 256, st);
     mark(h, 0, st);
     uint32_t* dec_bitmap = (uint32_t*)(ws + h->dc_bitmap_off);
     int32_t* items = (int32_t*)(ws + h->dc_items_off);
@@ -707,13 +725,12 @@ adaspark_status_t adaspark_attn_decode(adaspark_attn_t* h, const void* q_new, co
     mark(h, 1, st);
     {
         size_t smem = decode_select_smem_bytes(g.N_ld, g.G, g.n_words);
-        auto* blocks = (unsigned long long*)&hdr->decode_kv_blocks;
         if (D == 128) {
             if (!set_smem(h, decode_select_plan_kernel<128>, smem, "decode_select_plan_kernel")) return ADASPARK_ERR_CUDA;
-            decode_select_plan_kernel<128><<<dim3(g.Hkv, g.B), 256, smem, st>>>(g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, blocks, status);
+            decode_select_plan_kernel<128><<<dim3(kPlanCtas, g.Hkv, g.B), kPlanWarps * 32, smem, st>>>(g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, (uint32_t*)hdr);
         } else {
             if (!set_smem(h, decode_select_plan_kernel<64>, smem, "decode_select_plan_kernel")) return ADASPARK_ERR_CUDA;
-            decode_select_plan_kernel<64><<<dim3(g.Hkv, g.B), 256, smem, st>>>(g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, blocks, status);
+            decode_select_plan_kernel<64><<<dim3(kPlanCtas, g.Hkv, g.B), kPlanWarps * 32, smem, st>>>(g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, (uint32_t*)hdr);
         }
         if (!launch_ok(h, "decode_select_plan_kernel")) return ADASPARK_ERR_CUDA;
     }
@@ -727,16 +744,20 @@ adaspark_status_t adaspark_attn_decode(adaspark_attn_t* h, const void* q_new, co
         if (D == 128) {
             size_t smem = sizeof(DecodeSmem<128>) + 1024;
             if (!set_smem(h, decode_splitkv_kernel<128>, smem, "decode_splitkv_kernel")) return ADASPARK_ERR_CUDA;
-            decode_splitkv_kernel<128><<<grid, kDecodeThreads, smem, st>>>(g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
+            launch_overlapped(decode_splitkv_kernel<128>, grid, dim3(kDecodeThreads), smem, st, g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
         } else {
             size_t smem = sizeof(DecodeSmem<64>) + 1024;
             if (!set_smem(h, decode_splitkv_kernel<64>, smem, "decode_splitkv_kernel")) return ADASPARK_ERR_CUDA;
-            decode_splitkv_kernel<64><<<grid, kDecodeThreads, smem, st>>>(g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
+            launch_overlapped(decode_splitkv_kernel<64>, grid, dim3(kDecodeThreads), smem, st, g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
         }
         if (!launch_ok(h, "decode_splitkv_kernel")) return ADASPARK_ERR_CUDA;
     }
     mark(h, 3, st);
-    decode_combine_kernel<<<dim3(g.Hq, g.B), D, 0, st>>>(g, h->dc_splits, partial, (__nv_bfloat16*)out);
+    {
+        auto* blocks = (unsigned long long*)&hdr->decode_kv_blocks;
+        if (D == 128) launch_overlapped(decode_combine_kernel<128>, dim3(g.Hq, g.B), dim3(512), 0, st, g, h->dc_splits, (const float*)partial, text_len, (const int32_t*)n_items, blocks, status, (__nv_bfloat16*)out);
+        else launch_overlapped(decode_combine_kernel<64>, dim3(g.Hq, g.B), dim3(512), 0, st, g, h->dc_splits, (const float*)partial, text_len, (const int32_t*)n_items, blocks, status, (__nv_bfloat16*)out);
+    }
     if (!launch_ok(h, "decode_combine_kernel")) return ADASPARK_ERR_CUDA;
     mark(h, 4, st);
     return ADASPARK_OK;

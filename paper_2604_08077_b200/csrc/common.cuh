@@ -140,6 +140,13 @@ __device__ __forceinline__ bool key_allowed(const Geom& g, int pr, int pk, uint3
     return (word >> ((pk >> g.c_shift) & 31)) & 1u;                                // selected cube
 }
 
+// Programmatic dependent launch.  launch_dependents: the next kernel of the stream, if it was launched to overlap, may
+// start once every CTA of this one has come here (or ended); wait_for_previous_kernel: everything the kernels before
+// have written is visible from here on.  Whatever a kernel reads or writes that an earlier kernel of the same call
+// touches comes after its wait.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

@@ -29,13 +29,14 @@ struct DecodeSmem {
 };
 
 
+// (What the kernel before writes is passed without __restrict__: loads of read-only data may be moved above the wait.)
 // grid (n_splits, Hkv, B).  partial[((b*Hkv+gk)*n_splits + split)*G + row] = {m, l, o[D]}
 // (base-2 running max, sum, unnormalised output).
 template <int D>
 __global__ void __launch_bounds__(kDecodeThreads) decode_splitkv_kernel(
     Geom g, int n_splits, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-    const __nv_bfloat16* __restrict__ q_new, const uint32_t* __restrict__ dec_bitmap,
-    const int32_t* __restrict__ text_len, const int32_t* __restrict__ items, const int32_t* __restrict__ n_items,
+    const __nv_bfloat16* __restrict__ q_new, const uint32_t* dec_bitmap,
+    const int32_t* __restrict__ text_len, const int32_t* items, const int32_t* n_items,
     float* __restrict__ partial, int32_t* __restrict__ status) {
     extern __shared__ unsigned char dec_smem_raw[];
     DecodeSmem<D>& sm = *reinterpret_cast<DecodeSmem<D>*>((reinterpret_cast<uintptr_t>(dec_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -45,11 +46,13 @@ __global__ void __launch_bounds__(kDecodeThreads) decode_splitkv_kernel(
 
     const int split = blockIdx.x, gk = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n_it = n_items[b * g.Hkv + gk];
-    const int per = (n_it + n_splits - 1) / n_splits;
-    const int it0 = min(split * per, n_it), it1 = min(it0 + per, n_it);
     const int32_t* my_items = items + (size_t)(b * g.Hkv + gk) * g.n_kv_blocks_cap;
 
+    launch_dependents();
+    if (warp == 4 && lane == 0) {
+        tc::prefetch_tensormap(&tmK);
+        tc::prefetch_tensormap(&tmV);
+    }
     if (tid == 0) {
         for (int s = 0; s < kDecodeStages; ++s) {
             tc::mbar_init(&sm.full[s], 1);
@@ -60,6 +63,10 @@ __global__ void __launch_bounds__(kDecodeThreads) decode_splitkv_kernel(
     }
     __syncthreads();
     volatile int* abort_flag = &sm.abort_flag;
+    wait_for_previous_kernel();                       // the block lists and the appended token are there
+    const int n_it = n_items[b * g.Hkv + gk];
+    const int per = (n_it + n_splits - 1) / n_splits;
+    const int it0 = min(split * per, n_it), it1 = min(it0 + per, n_it);
 
     float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;
     float o[kDTiles][4];
@@ -69,8 +76,6 @@ __global__ void __launch_bounds__(kDecodeThreads) decode_splitkv_kernel(
 
     if (warp == 4) {
         if (lane == 0) {
-            tc::prefetch_tensormap(&tmK);
-            tc::prefetch_tensormap(&tmV);
             const int kv_row0 = (b * g.Hkv + gk) * g.S_cap;
             const int v_row0 = (b * g.Hkv + gk) * g.n_kv_blocks_cap * D;
             for (int it = it0; it < it1; ++it) {
