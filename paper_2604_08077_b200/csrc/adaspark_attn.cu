@@ -164,6 +164,24 @@ void launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);   // an error is picked up by launch_ok
 }
 
+#ifdef ADASPARK_WITH_TCGEN05
+// Could the query-gather path save what it costs, whatever the rows select?  Its estimate (gather_scan_kernel) for a
+// pair of query tiles is kGatherBreakEven x U - P entries' worth of time, U = key blocks of the pair's union, all
+// before its local range, and P >= U its entries.  When even the largest possible sum over all pairs is below the least
+// worthwhile gain, the six kernels of the path (20 us, most of it launches) would find nothing to do and are left out:
+// up to 6976 (pair, block) products, a causal sequence of about 2800 tokens with 28 heads.  (A threshold above the break-even
+// estimate forces the path and is not judged.)
+bool gather_can_pay(const Geom& g, float pairs_per_block) {
+    if (pairs_per_block > (float)kGatherBreakEven) return true;
+    long long blocks = 0;
+    for (int pair = g.pos_begin / kPairRows; pair < (g.S + kPairRows - 1) / kPairRows; ++pair) {
+        blocks += (long long)g.Hq * g.B * pair_first_local_blk(g, pair * kPairRows);
+        if (blocks * (kGatherBreakEven - 1) >= kGatherMinGain) return true;
+    }
+    return false;
+}
+#endif
+
 template <typename K>
 bool set_smem(adaspark_attn* h, K kernel, size_t bytes, const char* what) {
     if (bytes <= 48 * 1024) return true;
@@ -441,9 +459,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             auto* row_range = (float2*)(ws + h->fw_rowrange_off);
             float* scores = (float*)(ws + h->fw_scores_off);
             const int n_rows = g.B * g.Hkv * g.N_ld;
-            key_exponent_kernel<<<dim3(g.B * g.Hkv, 8), 256, 0, st>>>(g, cube_keys, head_max, head_norm2);
-            if (!launch_ok(h, "key_exponent_kernel")) return ADASPARK_ERR_CUDA;
-            slice_keys_kernel<<<(n_rows + 3) / 4, 128, 0, st>>>(g, cube_keys, head_max, kplanes);
+            slice_keys_kernel<<<dim3(kSliceCtas, g.B * g.Hkv), 256, 0, st>>>(g, cube_keys, head_max, head_norm2, kplanes);
             if (!launch_ok(h, "slice_keys_kernel")) return ADASPARK_ERR_CUDA;
             CUtensorMap tmKs, tmS;
             if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
@@ -523,7 +539,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         const uint32_t* slot_valid_c = (const uint32_t*)(ws + h->fw_valid_off);
         // query-gather path for pairs of query tiles with sparse selections (off for p >= 1: nothing is skipped)
         const bool all_sel = g.top_k <= 0 && !(g.top_p < 1.0);
-        const bool gather = h->prefill_kernel == 1 && !all_sel && h->gather_cap > 0 && h->gather_pairs_per_block > 0.f;
+        const bool gather = h->prefill_kernel == 1 && !all_sel && h->gather_cap > 0 && h->gather_pairs_per_block > 0.f &&
+                            gather_can_pay(g, h->gather_pairs_per_block);
         GatherWs gw;
         std::memset(&gw, 0, sizeof(gw));
         if (gather) {

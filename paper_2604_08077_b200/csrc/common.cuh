@@ -119,7 +119,7 @@ __host__ __device__ __forceinline__ int tile_max_candidates(const Geom& g, int t
 // First 64-key block of the local range of the 256-row pair of query tiles that starts at pair_pos0: the block
 // that holds the first slot of the own cube of the pair's first row (video) or the first text slot.  Cubes
 // that end before this block are attended only if selected; from this block on the per-key rule applies.
-__device__ __forceinline__ int pair_first_local_blk(const Geom& g, int pair_pos0) {
+__host__ __device__ __forceinline__ int pair_first_local_blk(const Geom& g, int pair_pos0) {
     const int local_start = pair_pos0 < g.S_v ? ((pair_pos0 >> g.c_shift) << g.c_shift) : g.S_v;
     return local_start / kBlockTok;
 }
@@ -149,6 +149,17 @@ __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("gridd
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+// ---- thread-block clusters
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+// address of this CTA's shared variable in the CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t cluster_address(const void* p, int rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
 }
 
 __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gmem_src) {

@@ -43,16 +43,6 @@ __host__ __device__ inline size_t decode_select_smem_bytes(int N_ld, int G, int 
     return (size_t)decode_head_slots(G) * ((size_t)N_ld + kSelHistWords + kDecodeCandCap) * 8 + (size_t)n_words * 4;
 }
 
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-// address of this CTA's shared variable in the CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t cluster_address(const void* p, int rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-    return a;
-}
-
 // grid (8, Hkv, B) in clusters of 8, 128 threads.
 // items[(b*Hkv+gk) * n_kv_blocks_cap + i] = index of the i-th block to visit.  header: 256 bytes, set to zero.
 template <int D>

@@ -74,19 +74,29 @@ __device__ __forceinline__ uint32_t gather_byte(uint32_t w0, uint32_t w1, uint32
     return __byte_perm(lo, hi, 0x5410);
 }
 
-// Largest |mean key element| of every (batch, kv head), as float bits (non-negative floats order like
-// their bit patterns): head_max_bits[b*Hkv + gk], and the largest squared norm of a mean key:
-// head_norm2_bits[b*Hkv + gk]; both zeroed by the caller.  grid (B*Hkv, 8); D / 4 consecutive lanes hold one key.
-__global__ void __launch_bounds__(256) key_exponent_kernel(Geom g, const float* __restrict__ cube_keys,
-                                                           uint32_t* __restrict__ head_max_bits,
-                                                           uint32_t* __restrict__ head_norm2_bits) {
-    const int bh = blockIdx.x;
-    const size_t n4 = (size_t)g.N_live * g.D / 4;             // the cubes present so far
+__device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exponent_from_field((int)((max_bits >> 23) & 0xffu)); }
+
+// Digit planes of the mean keys: planes[p][(b*Hkv+gk)*N_ld + cube][128 bytes] (int8, zero beyond D), all cubes of a
+// (batch, kv head) in the fixed point of that head's exponent; rows >= N inside the padded leading dimension are
+// zero-filled.  A cluster of 8 CTAs per (batch, kv head) first finds the largest |element| and the largest squared norm
+// of the head's mean keys (exchanged through distributed shared memory, float bits: non-negative floats order like
+// their bit patterns), leaves them in head_max_bits / head_norm2_bits, and then slices.  grid (8, B*Hkv), 256 threads,
+// D / 4 consecutive lanes hold one key.  (One kernel for both: two cost a launch more, 3 us of a short call.)
+constexpr int kSliceCtas = 8;
+__global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_keys_kernel(
+    Geom g, const float* __restrict__ cube_keys, uint32_t* __restrict__ head_max_bits, uint32_t* __restrict__ head_norm2_bits,
+    unsigned char* __restrict__ planes) {
+    __shared__ uint32_t head[2];
+    const int rank = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31;
+    if (threadIdx.x < 2) head[threadIdx.x] = 0u;
+    cluster_sync();                                           // every CTA of the cluster runs: its memory may be written
     const float4* src = reinterpret_cast<const float4*>(cube_keys + (size_t)bh * g.N * g.D);
+    const int n4 = g.N_live * (g.D / 4);                      // the cubes present so far
     uint32_t mx = 0;
     float mx2 = 0.f;
-    for (size_t i0 = (size_t)blockIdx.y * 256; i0 < n4; i0 += (size_t)gridDim.y * 256) {   // whole warps stay together
-        const size_t i = i0 + threadIdx.x;
+#pragma unroll 4
+    for (int i0 = rank * 256; i0 < n4; i0 += kSliceCtas * 256) {   // whole warps stay together
+        const int i = i0 + threadIdx.x;
         const float4 x = i < n4 ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         mx = max(max(mx, __float_as_uint(fabsf(x.x))), max(__float_as_uint(fabsf(x.y)),
                  max(__float_as_uint(fabsf(x.z)), __float_as_uint(fabsf(x.w)))));
@@ -96,36 +106,28 @@ __global__ void __launch_bounds__(256) key_exponent_kernel(Geom g, const float* 
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     const uint32_t m2 = __reduce_max_sync(0xffffffffu, __float_as_uint(mx2));
-    if ((threadIdx.x & 31) == 0 && mx) {
-        atomicMax(head_max_bits + bh, mx);
-        atomicMax(head_norm2_bits + bh, m2);
+    if (lane < kSliceCtas) {
+        const uint32_t dst = cluster_address(head, lane);
+        asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(dst), "r"(mx) : "memory");
+        asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(dst + 4u), "r"(m2) : "memory");
     }
-}
-__device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exponent_from_field((int)((max_bits >> 23) & 0xffu)); }
-
-// Digit planes of the mean keys: planes[p][(b*Hkv+gk)*N_ld + cube][128 bytes] (int8, zero beyond D), all
-// cubes of a (batch, kv head) in the fixed point of that head's exponent.  One warp per cube row, four
-// elements per lane; rows >= N inside the padded leading dimension are zero-filled.
-__global__ void __launch_bounds__(128) slice_keys_kernel(Geom g, const float* __restrict__ cube_keys,
-                                                         const uint32_t* __restrict__ head_max_bits,
-                                                         unsigned char* __restrict__ planes) {
-    const int lane = threadIdx.x & 31;
-    const int row = blockIdx.x * 4 + (threadIdx.x >> 5);              // (b*Hkv+gk)*N_ld + cube
-    const int n_rows = g.B * g.Hkv * g.N_ld;
-    if (row >= n_rows) return;
-    const int bh = row / g.N_ld, cube = row - bh * g.N_ld;
-    const size_t plane_stride = (size_t)n_rows * kDigitRowBytes;
-    const bool live = cube < g.N_live && lane * 4 < g.D;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (live) x = *reinterpret_cast<const float4*>(cube_keys + ((size_t)bh * g.N + cube) * g.D + lane * 4);
-    const float mult = digit_scale(head_exponent(head_max_bits[bh]));
-    const uint32_t w0 = packed_digits(x.x, mult), w1 = packed_digits(x.y, mult);
-    const uint32_t w2 = packed_digits(x.z, mult), w3 = packed_digits(x.w, mult);
-    unsigned char* dst = planes + (size_t)row * kDigitRowBytes + lane * 4;
-    *reinterpret_cast<uint32_t*>(dst) = gather_byte<3>(w0, w1, w2, w3);
-    *reinterpret_cast<uint32_t*>(dst + plane_stride) = gather_byte<2>(w0, w1, w2, w3);
-    *reinterpret_cast<uint32_t*>(dst + 2 * plane_stride) = gather_byte<1>(w0, w1, w2, w3);
-    *reinterpret_cast<uint32_t*>(dst + 3 * plane_stride) = gather_byte<0>(w0, w1, w2, w3);
+    cluster_sync();
+    const uint32_t max_bits = head[0];
+    if (rank == 0 && threadIdx.x == 0) { head_max_bits[bh] = max_bits; head_norm2_bits[bh] = head[1]; }
+    const float mult = digit_scale(head_exponent(max_bits));
+    const size_t plane_stride = (size_t)g.B * g.Hkv * g.N_ld * kDigitRowBytes;
+#pragma unroll 2
+    for (int cube = rank * 8 + (threadIdx.x >> 5); cube < g.N_ld; cube += kSliceCtas * 8) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (cube < g.N_live && lane * 4 < g.D) x = src[(size_t)cube * (g.D / 4) + lane];
+        const uint32_t w0 = packed_digits(x.x, mult), w1 = packed_digits(x.y, mult);
+        const uint32_t w2 = packed_digits(x.z, mult), w3 = packed_digits(x.w, mult);
+        unsigned char* dst = planes + ((size_t)bh * g.N_ld + cube) * kDigitRowBytes + lane * 4;
+        *reinterpret_cast<uint32_t*>(dst) = gather_byte<3>(w0, w1, w2, w3);
+        *reinterpret_cast<uint32_t*>(dst + plane_stride) = gather_byte<2>(w0, w1, w2, w3);
+        *reinterpret_cast<uint32_t*>(dst + 2 * plane_stride) = gather_byte<1>(w0, w1, w2, w3);
+        *reinterpret_cast<uint32_t*>(dst + 3 * plane_stride) = gather_byte<0>(w0, w1, w2, w3);
+    }
 }
 
 template <int D>
