@@ -165,6 +165,11 @@ void launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 #ifdef ADASPARK_WITH_TCGEN05
+// Kernel shape for up to n candidates a row: lanes per row x scores per lane = 8 x 8, 8 x 16, 8 x 32, 16 x 32, 32 x 32,
+// 32 x 64, 32 x 128.  A shape costs by the scores it has room for as much as by those it holds (registers, and with them
+// warps on an SM): 8 x 32 for 64 candidates took 0.29 instead of 0.23 ms (16384 tokens, 28 heads, 64 cubes).
+int select_shape(int n) { return n <= 64 ? 0 : n <= 128 ? 1 : n <= 256 ? 2 : n <= 512 ? 3 : n <= 1024 ? 4 : n <= 2048 ? 5 : 6; }
+
 // Could the query-gather path save what it costs, whatever the rows select?  Its estimate (gather_scan_kernel) for a
 // pair of query tiles is kGatherBreakEven x U - P entries' worth of time, U = key blocks of the pair's union, all
 // before its local range, and P >= U its entries.  When even the largest possible sum over all pairs is below the least
@@ -261,7 +266,7 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // the fp64 selection kernel | key digit planes (tcgen05 path)
     size_t off = 0;
     h->fw_status_off = off; off = align_up(off + 256);
-    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 3);   // mean-key exponents, largest |k|^2, largest |mean key|^2
+    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 3);   // mean-key exponents, largest |k|^2, largest |mean key|
     h->fw_valid_off = off; off = align_up(off + (size_t)(S_cap / kBlockTok) * 2 * 4);   // which slots of a block hold a token
     const size_t n_cols = (size_t)(S_v + kBlockTok - 1) / kBlockTok;                     // key blocks that hold video
     // query-gather path: the rows are cut into windows whose slice of Q (all heads) is about a third of the L2
@@ -454,12 +459,12 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
 #ifdef ADASPARK_WITH_TCGEN05
         else if (h->prefill_kernel == 1) {
             uint32_t* head_max = (uint32_t*)(ws + h->fw_headmax_off);
-            uint32_t* head_norm2 = head_max + 2 * g.B * g.Hkv;
+            float* head_norm = (float*)(head_max + 2 * g.B * g.Hkv);
             unsigned char* kplanes = (unsigned char*)(ws + h->fw_kplanes_off);
             auto* row_range = (float2*)(ws + h->fw_rowrange_off);
             float* scores = (float*)(ws + h->fw_scores_off);
             const int n_rows = g.B * g.Hkv * g.N_ld;
-            slice_keys_kernel<<<dim3(kSliceCtas, g.B * g.Hkv), 256, 0, st>>>(g, cube_keys, head_max, head_norm2, kplanes);
+            slice_keys_kernel<<<dim3(kSliceCtas, g.B * g.Hkv), 256, 0, st>>>(g, cube_keys, head_max, head_norm, kplanes);
             if (!launch_ok(h, "slice_keys_kernel")) return ADASPARK_ERR_CUDA;
             CUtensorMap tmKs, tmS;
             if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
@@ -470,16 +475,11 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             for (int item0 = 0; item0 < n_items; item0 += h->score_items) {
                 const int n_here = n_items - item0 < h->score_items ? n_items - item0 : h->score_items;
                 const int grid = n_here < h->sm_count ? n_here : h->sm_count;
-                int n_max = 0;                       // largest candidate count of the launch
-                for (int lvl = item0 / n_hb; lvl <= (item0 + n_here - 1) / n_hb; ++lvl) {
-                    const int m = tile_max_candidates(g, g.n_tiles - 1 - lvl);
-                    n_max = m > n_max ? m : n_max;
-                }
 #define ADASPARK_LAUNCH_SCORE(DD)                                                                                      \
     do {                                                                                                               \
         const size_t smem = sizeof(ScoreSmem<DD>) + 1024;                                                              \
         if (!set_smem(h, score_tc_kernel<DD>, smem, "score_tc_kernel")) return ADASPARK_ERR_CUDA;                      \
-        score_tc_kernel<DD><<<grid, kScoreThreads, smem, st>>>(g, item0, n_here, qb, tmKs, tmS, head_max, head_norm2,  \
+        score_tc_kernel<DD><<<grid, kScoreThreads, smem, st>>>(g, item0, n_here, qb, tmKs, tmS, head_max, head_norm,   \
                                                                row_range, tile_union, &hdr->status);                   \
     } while (0)
                 if (D == 128) ADASPARK_LAUNCH_SCORE(128); else ADASPARK_LAUNCH_SCORE(64);
@@ -487,24 +487,40 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
                 if (!launch_ok(h, "score_tc_kernel")) return ADASPARK_ERR_CUDA;
 #define ADASPARK_LAUNCH_SELECT(GG, KK, RES, BC)                                                                       \
     do {                                                                                                               \
-        const size_t smem = select_smem_bytes(sizeof(SelectWarpSmem<GG>), g.n_words);                                  \
+        const size_t smem = select_smem_bytes(sizeof(SelectWarpSmem<GG, KK>), g.n_words);                              \
         if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, BC>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
-        select_nucleus_kernel<GG, KK, RES, BC><<<2 * n_here, kSelectThreads, smem, st>>>(                              \
-            g, item0, scores, (const float4*)row_range, tile_mask, tile_union, sel_bitmap, sel_count, fallback_rows,   \
+        select_nucleus_kernel<GG, KK, RES, BC><<<2 * (next - first), kSelectThreads, smem, st>>>(                      \
+            g, item0, first, scores, (const float4*)row_range, tile_mask, tile_union, sel_bitmap, sel_count, fallback_rows,   \
             &hdr->fallback_rows);                                                                                      \
     } while (0)
 #define ADASPARK_LAUNCH_SELECT_K(GG, KK, RES)                                                                         \
     do {                                                                                                               \
         if (by_count) ADASPARK_LAUNCH_SELECT(GG, KK, RES, true); else ADASPARK_LAUNCH_SELECT(GG, KK, RES, false);      \
     } while (0)
-                if (n_max <= 256) ADASPARK_LAUNCH_SELECT_K(8, 32, 4);
-                else if (n_max <= 512) ADASPARK_LAUNCH_SELECT_K(16, 32, 4);
-                else if (n_max <= 1024) ADASPARK_LAUNCH_SELECT_K(32, 32, 4);
-                else if (n_max <= 2048) ADASPARK_LAUNCH_SELECT_K(32, 64, 2);
-                else ADASPARK_LAUNCH_SELECT_K(32, 128, 1);
+                // Candidate counts fall with the items (late tiles come first): runs of items of one kernel shape, a run
+                // of less than eight tiles per SM joins its neighbour (another launch would cost what it saves).
+                for (int first = 0, next; first < n_here; first = next) {
+                    const int shape = select_shape(tile_max_candidates(g, g.n_tiles - 1 - (item0 + first) / n_hb));
+                    int largest = shape;
+                    for (next = first; next < n_here; next = ((item0 + next) / n_hb + 1) * n_hb - item0) {
+                        const int here = select_shape(tile_max_candidates(g, g.n_tiles - 1 - (item0 + next) / n_hb));
+                        if (here != shape && next - first >= 8 * kScoreWave && n_here - next >= 8 * kScoreWave) break;
+                        largest = here > largest ? here : largest;
+                    }
+                    next = next < n_here ? next : n_here;
+                    switch (largest) {
+                        case 0: ADASPARK_LAUNCH_SELECT_K(8, 8, 5); break;
+                        case 1: ADASPARK_LAUNCH_SELECT_K(8, 16, 4); break;
+                        case 2: ADASPARK_LAUNCH_SELECT_K(8, 32, 3); break;
+                        case 3: ADASPARK_LAUNCH_SELECT_K(16, 32, 3); break;
+                        case 4: ADASPARK_LAUNCH_SELECT_K(32, 32, 3); break;
+                        case 5: ADASPARK_LAUNCH_SELECT_K(32, 64, 2); break;
+                        default: ADASPARK_LAUNCH_SELECT_K(32, 128, 1);
+                    }
+                    if (!launch_ok(h, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA;
+                }
 #undef ADASPARK_LAUNCH_SELECT_K
 #undef ADASPARK_LAUNCH_SELECT
-                if (!launch_ok(h, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA;
             }
             // the rows it left over (normally none): list length is read on the device
             if (!launch_exact(fallback_rows, &hdr->fallback_rows, 0)) return ADASPARK_ERR_CUDA;

@@ -247,6 +247,12 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
     return d;
 }
 
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {   // subnormal results are kept
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // byte offset of 16-byte chunk `chunk` of 128-byte row `row` under the 128-byte swizzle
 __device__ __forceinline__ int sw128(int row, int chunk) { return row * 128 + ((chunk ^ (row & 7)) << 4); }
 

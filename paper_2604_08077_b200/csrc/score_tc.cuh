@@ -52,12 +52,12 @@ constexpr int kDigitRowBytes = 128;      // bytes per row of a digit plane
 constexpr double kMaxScorePerUnit = 0.125 / 268435456.0;
 constexpr int kMaxRowShift = 16;         // |V| < D * 2^36 = 2^43 by construction, so a shift of 12 always suffices
 
-// The four signed base-256 digits of v = round(x * 2^(29 - e)) (|v| < 2^30), packed in one word:
+// The four signed base-256 digits of v = round(y), y = x * 2^(29 - e) (|v| < 2^30), packed in one word:
 // byte 3 = d0 (most significant) ... byte 0 = d3.  Adding 0x80 to every byte position turns the
 // balanced digits into the plain unsigned bytes of v + 0x80808080, so two integer operations give
 // all four.
-__device__ __forceinline__ uint32_t packed_digits(float x, float mult) {
-    const uint32_t u = (uint32_t)__float2int_rn(x * mult) + 0x80808080u;
+__device__ __forceinline__ uint32_t packed_digits(float y) {
+    const uint32_t u = (uint32_t)__float2int_rn(y) + 0x80808080u;
     return u ^ 0x80808080u;
 }
 __device__ __forceinline__ float digit_scale(int e) {             // 2^(29 - e), exact for e >= -97
@@ -66,25 +66,28 @@ __device__ __forceinline__ float digit_scale(int e) {             // 2^(29 - e),
 __device__ __forceinline__ int row_exponent_from_field(int biased) {   // 8-bit exponent field of the row maximum
     return biased == 0 ? 0 : max(biased - 127, -90);               // rows smaller than 2^-90 keep fewer digits
 }
-// Byte k of four packed words -> one word (element i in byte i): digit plane 3 - k of four elements.
-template <int k>
-__device__ __forceinline__ uint32_t gather_byte(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3) {
-    const uint32_t lo = __byte_perm(w0, w1, (uint32_t)k | ((uint32_t)(4 + k) << 4));
-    const uint32_t hi = __byte_perm(w2, w3, (uint32_t)k | ((uint32_t)(4 + k) << 4));
-    return __byte_perm(lo, hi, 0x5410);
+// The digits of four elements by plane: plane[p] holds digit p (p = 0 most significant) of element i in byte i, a
+// transposition of the 4 x 4 bytes.
+__device__ __forceinline__ void digit_planes(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t (&plane)[4]) {
+    const uint32_t a = __byte_perm(w0, w1, 0x5140), b = __byte_perm(w2, w3, 0x5140);
+    const uint32_t c = __byte_perm(w0, w1, 0x7362), d = __byte_perm(w2, w3, 0x7362);
+    plane[3] = __byte_perm(a, b, 0x5410);
+    plane[2] = __byte_perm(a, b, 0x7632);
+    plane[1] = __byte_perm(c, d, 0x5410);
+    plane[0] = __byte_perm(c, d, 0x7632);
 }
-
 __device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exponent_from_field((int)((max_bits >> 23) & 0xffu)); }
 
 // Digit planes of the mean keys: planes[p][(b*Hkv+gk)*N_ld + cube][128 bytes] (int8, zero beyond D), all cubes of a
 // (batch, kv head) in the fixed point of that head's exponent; rows >= N inside the padded leading dimension are
-// zero-filled.  A cluster of 8 CTAs per (batch, kv head) first finds the largest |element| and the largest squared norm
-// of the head's mean keys (exchanged through distributed shared memory, float bits: non-negative floats order like
-// their bit patterns), leaves them in head_max_bits / head_norm2_bits, and then slices.  grid (8, B*Hkv), 256 threads,
-// D / 4 consecutive lanes hold one key.  (One kernel for both: two cost a launch more, 3 us of a short call.)
+// zero-filled.  A cluster of 8 CTAs per (batch, kv head) first finds the largest |element| of the head's mean keys
+// (exchanged through distributed shared memory, float bits: non-negative floats order like their bit patterns), then
+// slices, and leaves the largest |element| in head_max_bits and the largest norm of a mean key times 2^(29 - E_K) in
+// head_norm (of the scaled values: no size of input over- or underflows the squares).  grid (8, B*Hkv), 256 threads.
+// (One kernel for all: two cost a launch more, 3 us of a short call.)
 constexpr int kSliceCtas = 8;
 __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_keys_kernel(
-    Geom g, const float* __restrict__ cube_keys, uint32_t* __restrict__ head_max_bits, uint32_t* __restrict__ head_norm2_bits,
+    Geom g, const float* __restrict__ cube_keys, uint32_t* __restrict__ head_max_bits, float* __restrict__ head_norm,
     unsigned char* __restrict__ planes) {
     __shared__ uint32_t head[2];
     const int rank = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31;
@@ -93,41 +96,37 @@ __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_
     const float4* src = reinterpret_cast<const float4*>(cube_keys + (size_t)bh * g.N * g.D);
     const int n4 = g.N_live * (g.D / 4);                      // the cubes present so far
     uint32_t mx = 0;
-    float mx2 = 0.f;
 #pragma unroll 4
-    for (int i0 = rank * 256; i0 < n4; i0 += kSliceCtas * 256) {   // whole warps stay together
-        const int i = i0 + threadIdx.x;
-        const float4 x = i < n4 ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = rank * 256 + threadIdx.x; i < n4; i += kSliceCtas * 256) {
+        const float4 x = src[i];
         mx = max(max(mx, __float_as_uint(fabsf(x.x))), max(__float_as_uint(fabsf(x.y)),
                  max(__float_as_uint(fabsf(x.z)), __float_as_uint(fabsf(x.w)))));
-        float n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
-        for (int o = g.D / 8; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-        mx2 = fmaxf(mx2, n2);
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
-    const uint32_t m2 = __reduce_max_sync(0xffffffffu, __float_as_uint(mx2));
-    if (lane < kSliceCtas) {
-        const uint32_t dst = cluster_address(head, lane);
-        asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(dst), "r"(mx) : "memory");
-        asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(dst + 4u), "r"(m2) : "memory");
-    }
+    if (lane < kSliceCtas) asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(cluster_address(head, lane)), "r"(mx) : "memory");
     cluster_sync();
     const uint32_t max_bits = head[0];
-    if (rank == 0 && threadIdx.x == 0) { head_max_bits[bh] = max_bits; head_norm2_bits[bh] = head[1]; }
     const float mult = digit_scale(head_exponent(max_bits));
     const size_t plane_stride = (size_t)g.B * g.Hkv * g.N_ld * kDigitRowBytes;
+    float norm2 = 0.f;
 #pragma unroll 2
     for (int cube = rank * 8 + (threadIdx.x >> 5); cube < g.N_ld; cube += kSliceCtas * 8) {
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (cube < g.N_live && lane * 4 < g.D) x = src[(size_t)cube * (g.D / 4) + lane];
-        const uint32_t w0 = packed_digits(x.x, mult), w1 = packed_digits(x.y, mult);
-        const uint32_t w2 = packed_digits(x.z, mult), w3 = packed_digits(x.w, mult);
+        x.x *= mult; x.y *= mult; x.z *= mult; x.w *= mult;
+        float n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        norm2 = fmaxf(norm2, n2);
+        uint32_t plane[4];
+        digit_planes(packed_digits(x.x), packed_digits(x.y), packed_digits(x.z), packed_digits(x.w), plane);
         unsigned char* dst = planes + ((size_t)bh * g.N_ld + cube) * kDigitRowBytes + lane * 4;
-        *reinterpret_cast<uint32_t*>(dst) = gather_byte<3>(w0, w1, w2, w3);
-        *reinterpret_cast<uint32_t*>(dst + plane_stride) = gather_byte<2>(w0, w1, w2, w3);
-        *reinterpret_cast<uint32_t*>(dst + 2 * plane_stride) = gather_byte<1>(w0, w1, w2, w3);
-        *reinterpret_cast<uint32_t*>(dst + 3 * plane_stride) = gather_byte<0>(w0, w1, w2, w3);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) *reinterpret_cast<uint32_t*>(dst + p * plane_stride) = plane[p];
     }
+    if (lane == 0) asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(cluster_address(head + 1, 0)), "r"(__float_as_uint(norm2)) : "memory");
+    cluster_sync();
+    if (rank == 0 && threadIdx.x == 0) { head_max_bits[bh] = max_bits; head_norm[bh] = sqrtf(__uint_as_float(head[1])); }
 }
 
 template <int D>
@@ -166,7 +165,7 @@ template <int D>
 __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
     Geom g, int item0, int n_items, const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap tmK,
     const __grid_constant__ CUtensorMap tmS, const uint32_t* __restrict__ head_max_bits,
-    const uint32_t* __restrict__ head_norm2_bits, float2* __restrict__ row_range, uint32_t* __restrict__ tile_union,
+    const float* __restrict__ head_norm, float2* __restrict__ row_range, uint32_t* __restrict__ tile_union,
     int32_t* __restrict__ status) {
     extern __shared__ unsigned char score_raw[];
     ScoreSmem<D>& sm = *reinterpret_cast<ScoreSmem<D>*>((reinterpret_cast<uintptr_t>(score_raw) + 1023) & ~(uintptr_t)1023);
@@ -284,60 +283,50 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
 #pragma unroll
                 for (int c = 0; c < D / 16; ++c) v[c] = make_uint4(0u, 0u, 0u, 0u);
             }
-            uint32_t mxbits = 0;
-            float q2 = 0.f;
+            uint32_t mx2 = 0;                                     // largest magnitudes of the even and the odd elements
 #pragma unroll
-            for (int c = 0; c < D / 16; ++c) {
-                const uint32_t wd[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    mxbits = max(mxbits, max(wd[i] & 0x7fffu, (wd[i] >> 16) & 0x7fffu));
-                    const float lo = __uint_as_float(wd[i] << 16), hi = __uint_as_float(wd[i] & 0xffff0000u);
-                    q2 = fmaf(lo, lo, fmaf(hi, hi, q2));
-                }
-            }
+            for (int c = 0; c < D / 16; ++c)
+                mx2 = __vmaxu2(__vmaxu2(__vmaxu2(mx2, v[c].x & 0x7fff7fffu), v[c].y & 0x7fff7fffu),
+                               __vmaxu2(v[c].z & 0x7fff7fffu, v[c].w & 0x7fff7fffu));
+            uint32_t mxbits = max(mx2 & 0xffffu, mx2 >> 16);
             mxbits = max(mxbits, __shfl_xor_sync(0xffffffffu, mxbits, 1));
-            q2 += __shfl_xor_sync(0xffffffffu, q2, 1);
             const int e_q = row_exponent_from_field((int)(mxbits >> 7));
             const float mult = digit_scale(e_q);
-            // ---- the row's constants
-            const int bh = w.b * g.Hkv + w.gk;
-            const int e_sum = e_q + head_exponent(__ldg(head_max_bits + bh));
-            const double f = __hiloint2double((1023 + e_sum - 34) << 20, 0) * g.scale_d;       // score per unit of V
-            // |V| <= |q| max|k| 2^(34 - e_sum); 1 % covers the rounding of the norms, 2^26 the digits' own rounding
-            const double vmax = sqrt((double)q2 * (double)__uint_as_float(__ldg(head_norm2_bits + bh))) * 1.01 *
-                                    __hiloint2double((1023 + 34 - e_sum) << 20, 0) + 67108864.0;
-            int sh = max(((__double2hiint(vmax) >> 20) & 0x7ff) - 1023 + 1 - 31, 0);           // vmax < 2^(31 + sh)
-            const bool give_up = !(f <= kMaxScorePerUnit) || sh > kMaxRowShift;                // also non-finite rows
-            sh = min(sh, kMaxRowShift);
-            const double per_w = f * __hiloint2double((1023 + sh) << 20, 0) * 1.4426950408889634;
             // the tile before the last is done with this buffer: its MMAs with the planes, its epilogue with the constants
             if (n_done >= 2 && !(ok = tc::mbar_wait(&sm.qd_free[qb], ((n_done >> 1) - 1) & 1, abort_flag))) break;
-            if (part == 0) {
-                sm.row_shift[qb][r] = (uint8_t)sh;
-                sm.row_scale[qb][r] = give_up ? __int_as_float(0x7fffffff) : (float)per_w;
-            }
             unsigned char* dst = &sm.qd[qb][0][0][0];
+            float q2 = 0.f;                                       // |q|^2 2^(2 (29 - e_q))
 #pragma unroll
             for (int c = 0; c < D / 16; ++c) {                    // 8 elements = half a 16-byte chunk of every plane
                 const uint32_t wd[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
-                uint32_t pw[4][2];                                // [plane][4 elements per word]
+                uint32_t pw[2][4];                                // [4 elements][plane]
 #pragma unroll
                 for (int q2w = 0; q2w < 2; ++q2w) {
                     const uint32_t wa = wd[2 * q2w], wb = wd[2 * q2w + 1];
-                    const uint32_t w0 = packed_digits(__uint_as_float(wa << 16), mult);
-                    const uint32_t w1 = packed_digits(__uint_as_float(wa & 0xffff0000u), mult);
-                    const uint32_t w2 = packed_digits(__uint_as_float(wb << 16), mult);
-                    const uint32_t w3 = packed_digits(__uint_as_float(wb & 0xffff0000u), mult);
-                    pw[0][q2w] = gather_byte<3>(w0, w1, w2, w3);
-                    pw[1][q2w] = gather_byte<2>(w0, w1, w2, w3);
-                    pw[2][q2w] = gather_byte<1>(w0, w1, w2, w3);
-                    pw[3][q2w] = gather_byte<0>(w0, w1, w2, w3);
+                    const float y0 = __uint_as_float(wa << 16) * mult, y1 = __uint_as_float(wa & 0xffff0000u) * mult;
+                    const float y2 = __uint_as_float(wb << 16) * mult, y3 = __uint_as_float(wb & 0xffff0000u) * mult;
+                    q2 = fmaf(y0, y0, fmaf(y1, y1, fmaf(y2, y2, fmaf(y3, y3, q2))));
+                    digit_planes(packed_digits(y0), packed_digits(y1), packed_digits(y2), packed_digits(y3), pw[q2w]);
                 }
                 const int off = sw128(r, c) + 8 * part;           // elements 16 c + 8 part .. +7 of the plane row
 #pragma unroll
                 for (int pl = 0; pl < 4; ++pl)
-                    *reinterpret_cast<uint2*>(dst + (size_t)pl * sizeof(sm.qd[0][0]) + off) = make_uint2(pw[pl][0], pw[pl][1]);
+                    *reinterpret_cast<uint2*>(dst + (size_t)pl * sizeof(sm.qd[0][0]) + off) = make_uint2(pw[0][pl], pw[1][pl]);
+            }
+            // ---- the row's constants
+            q2 += __shfl_xor_sync(0xffffffffu, q2, 1);
+            if (part == 0) {
+                const int bh = w.b * g.Hkv + w.gk;
+                const int e_sum = e_q + head_exponent(__ldg(head_max_bits + bh));
+                const double f = __hiloint2double((1023 + e_sum - 34) << 20, 0) * g.scale_d;   // score per unit of V
+                // |V| <= |q| max|k| 2^(34 - e_sum), 1 % covers the rounding of the norms, 2^26 the digits' own rounding
+                const float vmax = sqrtf(q2) * __ldg(head_norm + bh) * (1.01f / 16777216.f) + 67108864.f;
+                int sh = max((int)(__float_as_uint(vmax) >> 23) - 127 + 1 - 31, 0);            // vmax < 2^(31 + sh)
+                const bool give_up = !(f <= kMaxScorePerUnit) || sh > kMaxRowShift;            // also non-finite rows
+                sh = min(sh, kMaxRowShift);
+                sm.row_shift[qb][r] = (uint8_t)sh;
+                sm.row_scale[qb][r] = give_up ? __int_as_float(0x7fffffff)
+                                              : (float)(f * __hiloint2double((1023 + sh) << 20, 0) * 1.4426950408889634);
             }
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // digit planes visible to the tensor core
             __syncwarp();

@@ -3,7 +3,7 @@
 // Scores s_j are in log2 units; the order is descending score, then ascending cube index, the mass of a cube is
 // 2^(s_j - max).  A row's scores stay in registers (kK per lane) and are swept twice:
 //   sweep 1  masses are added to the row's total Z and, quantised, to a histogram over the distance from the maximum
-//            in shared memory (16 G buckets; the last takes everything beyond): the bucket in which the cumulative
+//            in shared memory (16 G buckets from the largest score to the smallest): the bucket in which the cumulative
 //            mass crosses p Z is found from it
 //   sweep 2  cubes before that bucket are selected (one bit each, collected from the sign of a subtraction) and their
 //            exact mass is summed; the few cubes inside it (widened by kGuard at both ends) are listed, and each
@@ -38,13 +38,14 @@ constexpr int kMaxHistLevels = 8;        // histograms of a row before it is han
 constexpr float kMassEps = 4e-7f, kMassEpsTop = 3.2e-8f;   // of Z: the first plus |max| times the second
 constexpr float kGapEps = 2.4e-7f;       // of the larger of |s| and 1/4 (2^-22: twice the error of two scores)
 constexpr float kGuard = 1e-3f;          // of a bucket
-constexpr float kBucketsPerUnit = 8.f;   // first histogram, per log2 unit: at least so many (more if the row's range is small)
 
-// Lanes per row and scores per lane by candidate count: 16 G buckets of 1/8 (1/16, 1/32) log2 unit hold at most about
-// 6 (normal scores of deviation 1.5) of 256 (512, 1024) cubes.
+// Lanes per row grow with the candidate count, and the buckets with the lanes: a bucket holds at most about 5 of 256
+// cubes (G = 8), 512 (16) or 1024 (32) with normally distributed scores.
 // Shared memory of one warp; its mask words [n_words][8 rows] follow those of all warps.
-template <int G>
+template <int G, int kK>
 struct SelectWarpSmem {
+    float rows[32 / G][G * kK];                           // scores of the rows of a pass
+    float4 range[32 / G][2];                              // partial ranges of the rows of a pass
     uint32_t hist[512];                                   // [bucket][row of the warp]
     float4 cand[32 / G][kSelectCand];                     // score, mass, cube
     int32_t count[32 / G];
@@ -58,13 +59,13 @@ __device__ __forceinline__ float sat_fma(float a, float b, float c) {     // min
     return __saturatef(fmaf(a, b, c));
 }
 
-// One warp per 8 rows of a tile, warps work on their own: 2 CTAs per item of the launch.  scores / row_range: what score_tc_kernel left for the items [item0, ..).
+// One warp per 8 rows of a tile, warps work on their own: 2 CTAs per item, items [first, ..) of those that the scores were computed for.  scores / row_range: what score_tc_kernel left for the items [item0, ..).
 // tile_mask as mask_index() describes; tile_union (cleared) receives the OR of each word over the tile's rows;
 // fallback_rows[0 .. *fallback_count) receives ((b*Hq+h)*n_tiles_cap + tile)*128 + r of the rows left to the fp64
-// kernel.  G * kK >= the launch's largest candidate count; kBits: G * kK masses of at most 2^kBits fit 32 bits.
+// kernel.  G * kK >= the largest candidate count of these items; kBits: G * kK masses of at most 2^kBits fit 32 bits.
 template <int G, int kK, int kResident, bool kByCount>
 __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kernel(
-    Geom g, int item0, const float* __restrict__ scores, const float4* __restrict__ row_range,
+    Geom g, int item0, int first, const float* __restrict__ scores, const float4* __restrict__ row_range,
     uint32_t* __restrict__ tile_mask, uint32_t* __restrict__ tile_union, uint32_t* __restrict__ sel_bitmap,
     int32_t* __restrict__ sel_count, int32_t* __restrict__ fallback_rows, uint32_t* __restrict__ fallback_count) {
     extern __shared__ __align__(16) unsigned char select_raw[];
@@ -77,12 +78,12 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
     constexpr uint32_t kMagicBits = 0x4B000000u;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s = lane & (G - 1), row_w = lane / G;                        // lane inside the row's group, row of the warp
-    const int item = blockIdx.x >> 1, row0 = ((blockIdx.x & 1) * kSelectWarps + warp) * kSelectRows;   // first row of the warp
+    const int item = first + (blockIdx.x >> 1), row0 = ((blockIdx.x & 1) * kSelectWarps + warp) * kSelectRows;   // first row of the warp
     const ScoreItem w = score_item(g, item0 + item);
     const size_t gt_cap = (size_t)(w.b * g.Hq + w.h) * g.n_tiles_cap + w.tile;
     const int n_words_live = min(2 * w.n_ct, g.n_words);                   // words that can hold a candidate
-    SelectWarpSmem<G>& sm = reinterpret_cast<SelectWarpSmem<G>*>(select_raw)[warp];
-    uint32_t* words = reinterpret_cast<uint32_t*>(select_raw + kSelectWarps * sizeof(SelectWarpSmem<G>)) + (size_t)warp * g.n_words * kSelectRows;
+    SelectWarpSmem<G, kK>& sm = reinterpret_cast<SelectWarpSmem<G, kK>*>(select_raw)[warp];
+    uint32_t* words = reinterpret_cast<uint32_t*>(select_raw + kSelectWarps * sizeof(SelectWarpSmem<G, kK>)) + (size_t)warp * g.n_words * kSelectRows;
     uint32_t* hist = sm.hist;
 #pragma unroll
     for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
@@ -98,30 +99,45 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         const uint32_t m = __ballot_sync(kFull, p);
         return ((G == 32 ? m : (m >> (row_w * G)) & ((1u << (G & 31)) - 1u))) != 0u;
     };
+    // The scores of a pass come through shared memory, requested while the pass before is still being decided (a warp
+    // that loaded them when it needed them spent half of its time waiting, with 32 warps on the SM).
+    auto candidates = [&](int pass) -> int {
+        const int pos = w.tile * kTileRows + row0 + pass * R + row_w;
+        return slot_live(g, pos) ? n_candidates(g, pos) : 0;
+    };
+    auto request = [&](int pass, int n) {
+        const size_t srow = (size_t)item * kTileRows + row0 + pass * R + row_w;
+        const float* src = scores + srow * g.N_ld + 4 * s;
+        float* dst = &sm.rows[row_w][4 * s];
+#pragma unroll
+        for (int c = 0; c < kSteps; ++c)
+            if (c * 4 * G + 4 * s < n) cp_async_16(dst + c * 4 * G, src + c * 4 * G);
+        if (s < 2 && n > 0) cp_async_16(&sm.range[row_w][s], row_range + 2 * srow + s);
+        cp_async_commit();
+    };
+    int n_next = candidates(0);
+    request(0, n_next);
 #pragma unroll 1
     for (int pass = 0; pass < kSelectRows / R; ++pass) {
         const int rl = pass * R + row_w, r = row0 + rl;
-        const int pos = w.tile * kTileRows + r;
-        const int n = slot_live(g, pos) ? n_candidates(g, pos) : 0;
+        const int n = n_next;
         const int n_most = __reduce_max_sync(kFull, n), n_least = __reduce_min_sync(kFull, n);
-        if (n_most == 0) continue;
-        const size_t srow = (size_t)item * kTileRows + r;
-        // the rows of the next pass on their way into the L1 (one 128-byte line per lane and 32 scores per lane)
-        if (pass + 1 < kSelectRows / R) {
-#pragma unroll
-            for (int u = 0; u < kMasks; ++u)
-                if (s * 32 + u * 32 * G < n_most)
-                    asm volatile("prefetch.global.L1 [%0];\n" ::"l"(scores + ((size_t)item * kTileRows + r + R) * g.N_ld + s * 32 + u * 32 * G));
+        cp_async_wait<0>();
+        __syncwarp();
+        n_next = pass + 1 < kSelectRows / R ? candidates(pass + 1) : 0;
+        if (n_most == 0) {
+            request(pass + 1, n_next);
+            continue;
         }
         // ---- the row's scores (column 4 G c + 4 s + i in v[4 c + i]), largest and smallest
-        const float* src = scores + srow * g.N_ld + 4 * s;
+        const float* row_scores = sm.rows[row_w];
         float v[kK];
 #pragma unroll
         for (int c = 0; c < kSteps; ++c) {
             float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
             if (c * 4 * G < n_most) {
                 const int col = c * 4 * G + 4 * s;
-                if (col < n) x = __ldg(reinterpret_cast<const float4*>(src + c * 4 * G));
+                if (col < n) x = *reinterpret_cast<const float4*>(row_scores + col);
                 if ((c + 1) * 4 * G > n_least) {                           // the end of a row's candidates
                     if (col + 1 >= n) x.y = -INFINITY;
                     if (col + 2 >= n) x.z = -INFINITY;
@@ -132,36 +148,73 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         }
         float top = 0.f, low = 0.f;
         if (n > 0) {
-            const float4 ra = row_range[2 * srow], rb = row_range[2 * srow + 1];
+            const float4 ra = sm.range[row_w][0], rb = sm.range[row_w][1];
             top = fmaxf(fmaxf(ra.x, ra.z), fmaxf(rb.x, rb.z));
             low = fminf(fminf(ra.y, ra.w), fminf(rb.y, rb.w));
         }
         bool give_up = n > 0 && !(top > -INFINITY && low > -INFINITY);     // marked by the score kernel
-        if (give_up) top = low = 0.f;
-        // mass of a score at the distance d = s - max from the maximum; distances are taken the maximum; distances are taken from the maximum first, where they are exact
+        if (give_up) {
+            top = low = 0.f;
+#pragma unroll
+            for (int e = 0; e < kK; ++e) v[e] = -INFINITY;
+        }
+        const int n_whole = __any_sync(kFull, give_up) ? 0 : n_least;      // columns below are scores in every row of the warp
+        // mass of a score at d = s - max
         auto mass = [&](float d) -> float { return kByCount ? (d > -INFINITY ? 1.f : 0.f) : fast_exp2(d); };
 
-        // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, bucket = round(u)
-        const float per_unit = fminf(fmaxf(kBucketsPerUnit * (G / 8), (float)(kBuckets - 1) / (top - low)), 1e18f);
+        // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, bucket = round(u): the buckets span the row
+        const float per_unit = fminf((float)(kBuckets - 1) / (top - low), 1e18f);
         float a_mul = -per_unit, a_add = 0.f;                              // u = d * a_mul + a_add
         float z = 0.f;
         uint32_t* my_hist = hist + row_w;
-        const float u_mul = a_mul * (1.f / (kBuckets - 1));
         const uint32_t hist_addr = smem_u32(my_hist) - kMagicBits * (4u * R);   // plus 4 R times the bits of 2^23 + bucket
+        const float q_unit = __int_as_float(1 << kBits);                   // 2^(kBits - 149): m times it is a subnormal whose bits are m 2^kBits, rounded
+        auto add_to_bucket = [&](uint32_t bucket_bits, uint32_t q) {
+            asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(hist_addr + bucket_bits * (4u * R)), "r"(q) : "memory");
+        };
+        {
+            unsigned long long z2 = 0ull;
+            const unsigned long long neg_top2 = pack_f32x2(-top, -top), a_mul2 = pack_f32x2(a_mul, a_mul);
+            const unsigned long long magic2 = pack_f32x2(kMagic, kMagic), q_unit2 = pack_f32x2(q_unit, q_unit);
 #pragma unroll
-        for (int c = 0; c < kSteps; ++c) {
-            if (c * 4 * G < n_most) {
+            for (int c = 0; c < kSteps; ++c) {
+                if ((c + 1) * 4 * G <= n_whole) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float d = v[4 * c + i] - top;
-                    v[4 * c + i] = d;
-                    const float m = mass(d);
-                    z += m;
-                    const uint32_t b = __float_as_uint(fmaf(__saturatef(d * u_mul), (float)(kBuckets - 1), kMagic));
-                    const uint32_t q = __float_as_uint(fmaf(m, kUnit, kMagic)) - kMagicBits;
-                    asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(hist_addr + b * (4u * R)), "r"(q) : "memory");
+                    for (int i = 0; i < 4; i += 2) {
+                        const unsigned long long d2 = add_f32x2(pack_f32x2(v[4 * c + i], v[4 * c + i + 1]), neg_top2);
+                        float d0, d1, b0, b1;
+                        unpack_f32x2(d2, d0, d1);
+                        v[4 * c + i] = d0;
+                        v[4 * c + i + 1] = d1;
+                        unpack_f32x2(fma_f32x2(d2, a_mul2, magic2), b0, b1);
+                        if (kByCount) {
+                            z += 2.f;
+                            add_to_bucket(__float_as_uint(b0), 1u);
+                            add_to_bucket(__float_as_uint(b1), 1u);
+                        } else {
+                            const unsigned long long m2 = pack_f32x2(mass(d0), mass(d1));
+                            z2 = add_f32x2(z2, m2);
+                            float q0, q1;
+                            unpack_f32x2(mul_f32x2(m2, q_unit2), q0, q1);
+                            add_to_bucket(__float_as_uint(b0), __float_as_uint(q0));
+                            add_to_bucket(__float_as_uint(b1), __float_as_uint(q1));
+                        }
+                    }
+                } else if (c * 4 * G < n_most) {                           // some columns hold no candidate (-inf: no mass)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float d = v[4 * c + i] - top;
+                        v[4 * c + i] = d;
+                        const float m = mass(d);
+                        z += m;
+                        const float u01 = __saturatef(d * (a_mul * (1.f / (kBuckets - 1))));
+                        add_to_bucket(__float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)), __float_as_uint(m * q_unit));
+                    }
                 }
             }
+            float z0, z1;
+            unpack_f32x2(z2, z0, z1);
+            z += z0 + z1;
         }
         z = group_sum(z);
         const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * g.top_p);
@@ -216,24 +269,37 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
             // ---- sweep 2: before / inside the bucket [cb - 1/2, cb + 1/2], widened by the guard
             const float lo_u = (float)cb - (0.5f + kGuard);
-            const float hi_u = cb == kBuckets - 1 ? 3e38f : (float)cb + (0.5f + kGuard);
+            const float hi_u = (float)cb + (0.5f + kGuard);
             float add = 0.f;
             n_cand = 0;
             if (level == 0) {
+                const unsigned long long a_mul2 = pack_f32x2(a_mul, a_mul), lo2 = pack_f32x2(-lo_u, -lo_u);
+                const unsigned long long width2 = pack_f32x2(lo_u - hi_u, lo_u - hi_u);
+                unsigned long long add2 = 0ull;
 #pragma unroll
                 for (int c = kSteps - 1; c >= 0; --c) {
                     if (c * 4 * G < n_most) {
 #pragma unroll
-                        for (int i = 3; i >= 0; --i) {
-                            const float d = v[4 * c + i];
+                        for (int i = 2; i >= 0; i -= 2) {
+                            const float d0 = v[4 * c + i], d1 = v[4 * c + i + 1];
                             const int k = (4 * c + i) >> 5;
-                            const float ua = fmaf(d, a_mul, -lo_u);
-                            before[k] = __funnelshift_l(__float_as_uint(ua), before[k], 1);
-                            inside[k] = __funnelshift_l(__float_as_uint(fmaf(d, a_mul, -hi_u)), inside[k], 1);
-                            add = fmaf(mass(d), __saturatef(ua * -1099511627776.f), add);   // times 2^40: 1 before, 0 else
+                            const unsigned long long u2 = fma_f32x2(pack_f32x2(d0, d1), a_mul2, lo2);
+                            float ua0, ua1, ub0, ub1;
+                            unpack_f32x2(u2, ua0, ua1);
+                            unpack_f32x2(add_f32x2(u2, width2), ub0, ub1);
+                            before[k] = __funnelshift_l(__float_as_uint(ua1), before[k], 1);
+                            before[k] = __funnelshift_l(__float_as_uint(ua0), before[k], 1);
+                            inside[k] = __funnelshift_l(__float_as_uint(ub1), inside[k], 1);
+                            inside[k] = __funnelshift_l(__float_as_uint(ub0), inside[k], 1);
+                            // the mass of what lies before: times 2^40 and clamped, the distance is 1 before and 0 else
+                            add2 = fma_f32x2(pack_f32x2(mass(d0), mass(d1)),
+                                             pack_f32x2(__saturatef(ua0 * -1099511627776.f), __saturatef(ua1 * -1099511627776.f)), add2);
                         }
                     }
                 }
+                float add0, add1;
+                unpack_f32x2(add2, add0, add1);
+                add = add0 + add1;
 #pragma unroll
                 for (int k = 0; k < kMasks; ++k) inside[k] &= ~before[k];
             } else {
@@ -242,7 +308,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                     while (bits) {
                         const int e = __ffs(bits) - 1;
                         bits &= bits - 1u;
-                        const float d = __ldg(src + (((k * 32 + e) >> 2) * 4 * G + (e & 3))) - top;
+                        const float d = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)] - top;
                         const float u = fmaf(d, a_mul, a_add);
                         if (u < lo_u) { before[k] |= 1u << e; inside[k] &= ~(1u << e); add += mass(d); }
                         else if (!(u < hi_u)) inside[k] &= ~(1u << e);
@@ -259,8 +325,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             if (active && level + 1 == kMaxHistLevels) { give_up = true; active = false; }
             if (!__any_sync(kFull, active)) break;
             // ---- rare: split the bucket of the rows that hold too many cubes in it
-            const float width = cb == kBuckets - 1 ? fmaxf(fmaf(low - top, a_mul, a_add) - lo_u, 1.f) : 1.f + 2.f * kGuard;
-            const float fine = (float)(kBuckets - 1) / width;
+            constexpr float fine = (float)(kBuckets - 1) / (1.f + 2.f * kGuard);
             if (active) {
                 a_add = (a_add - lo_u) * fine;
                 a_mul = a_mul * fine;
@@ -271,10 +336,10 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                 while (bits) {
                     const int e = __ffs(bits) - 1;
                     bits &= bits - 1u;
-                    const float d = __ldg(src + (((k * 32 + e) >> 2) * 4 * G + (e & 3))) - top;
+                    const float d = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)] - top;
                     const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), a_add * (1.f / (kBuckets - 1)));
                     const uint32_t b = __float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)) - kMagicBits;
-                    atomicAdd(&my_hist[b * R], __float_as_uint(fmaf(mass(d), kUnit, kMagic)) - kMagicBits);
+                    atomicAdd(&my_hist[b * R], __float_as_uint(mass(d) * q_unit));
                 }
             }
             __syncwarp();
@@ -294,11 +359,12 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                 const int e = __ffs(bits) - 1;
                 bits &= bits - 1u;
                 const int j = ((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3);
-                const float x = __ldg(scores + srow * g.N_ld + j);
+                const float x = row_scores[j];
                 sm.cand[row_w][slot++] = make_float4(x, mass(x - top), __int_as_float(j), 0.f);
             }
         }
         __syncwarp();
+        request(pass + 1, n_next);                                         // the rows' scores are no longer read
         // ---- the words of what lies before the bucket: lane s holds nibble s & 7 of words (s >> 3) + c G / 8
 #pragma unroll
         for (int k = 0; k < kMasks; ++k) {
@@ -353,15 +419,14 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         __syncwarp();
     }
     // ---- mask words (32-byte sectors of 8 rows), union words, the caller's copies
-    for (int i = lane; i < g.n_words * 2; i += 32) {
-        const int wd = i >> 1, c4 = i & 1;
+    for (int i0 = 0; i0 < g.n_words * 2; i0 += 32) {
+        const int wd = (i0 + lane) >> 1, c4 = lane & 1;
         const uint4 val = wd < n_words_live ? *reinterpret_cast<const uint4*>(&words[wd * kSelectRows + c4 * 4]) : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(tile_mask + (gt_cap * g.n_words + wd) * kTileRows + row0 + c4 * 4) = val;
-    }
-    for (int wd = lane; wd < n_words_live; wd += 32) {
-        const uint4 x = *reinterpret_cast<const uint4*>(&words[wd * kSelectRows]), y = *reinterpret_cast<const uint4*>(&words[wd * kSelectRows + 4]);
-        const uint32_t u = (x.x | x.y | x.z | x.w) | (y.x | y.y | y.z | y.w);
-        if (u) atomicOr(tile_union + gt_cap * g.n_words + wd, u);
+        if (wd < g.n_words)
+            *reinterpret_cast<uint4*>(tile_mask + (gt_cap * g.n_words + wd) * kTileRows + row0 + c4 * 4) = val;
+        uint32_t u = (val.x | val.y) | (val.z | val.w);                    // OR over the two lanes of the word
+        u |= __shfl_xor_sync(kFull, u, 1);
+        if (c4 == 0 && u) atomicOr(tile_union + gt_cap * g.n_words + wd, u);
     }
     if (sel_bitmap != nullptr || sel_count != nullptr) {
         for (int rl = 0; rl < kSelectRows; ++rl) {

@@ -13,8 +13,9 @@ from paper_2604_08077_b200 import binding, inputs
 pytestmark = pytest.mark.gpu
 
 
-def _selection(wl, kernel, k=None):
-    eng = binding.AdaSAttn(cube=wl.cube, n_q_heads=wl.Hq, n_kv_heads=wl.Hkv, head_dim=wl.D, top_p=wl.top_p, top_k=wl.top_k)
+def _selection(wl, kernel, k=None, softmax_scale=0.0):
+    eng = binding.AdaSAttn(cube=wl.cube, n_q_heads=wl.Hq, n_kv_heads=wl.Hkv, head_dim=wl.D, top_p=wl.top_p, top_k=wl.top_k,
+                           softmax_scale=softmax_scale)
     binding.adaspark_attn_set_prefill_kernel(eng.handle, kernel)
     eng.set_gather(0.0, 0)
     eng.partition(wl.B, wl.T, wl.H, wl.W, wl.n_text + wl.n_prefix)
@@ -26,8 +27,8 @@ def _selection(wl, kernel, k=None):
     return bitmap, count, hdr
 
 
-def _equal(wl, k=None):
-    got, want = _selection(wl, 1, k), _selection(wl, 0, k)
+def _equal(wl, k=None, softmax_scale=0.0):
+    got, want = _selection(wl, 1, k, softmax_scale), _selection(wl, 0, k, softmax_scale)
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     return got[2]
 
@@ -60,3 +61,13 @@ def test_equal_scores(copies):
     frames = k[:, :wl.S_v].view(1, 40, 2, 64, 2, 128)
     frames.copy_(frames[:, ::copies].repeat_interleave(copies, 1)[:, :40])
     assert _equal(wl, k).fallback_rows > 0
+
+
+@pytest.mark.parametrize("scale_k", [2.0 ** -70, 2.0 ** -20, 2.0 ** 40])
+def test_sizes_whose_squares_leave_fp32(scale_k):
+    """Mean keys far from 1 with a logit scale that makes up for it: same sets, and no row needs the fp64 kernel for it."""
+    wl = inputs.make_prefill("sizes", seed=79, B=1, T=16, H=8, W=8, cube=(4, 4, 4), n_text=21, Hq=4, Hkv=2, D=128, top_p=0.9,
+                             offset_std=1.5)
+    k = (wl.k.float() * scale_k).to(torch.bfloat16)
+    hdr = _equal(wl, k, softmax_scale=128 ** -0.5 / scale_k)
+    assert hdr.fallback_rows < 0.01 * wl.S * wl.Hq
