@@ -146,10 +146,14 @@ bool launch_ok(adaspark_attn* h, const char* what) {
     return true;
 }
 
-// Launches a kernel that may start while the kernel before it in the stream still runs; it waits for that one's
-// results itself (wait_for_previous_kernel).
+// Launches a kernel that waits for the results of the one before it itself (wait_for_previous_kernel).  overlap: it may
+// be put on the SMs while that one still runs.  That hides the launch and the set-up, but the CTAs that wait take their
+// places SM by SM as these become free: a grid of several waves ends up unevenly spread, and a kernel that lives off its
+// L1 gets what the previous one's shared memory left.  Measured against plain launches: 544 tokens 55.5 -> 45.8 us; but
+// 65536 tokens with every launch overlapped 4.39 -> 4.66 ms in the selection stage (the selection kernel) and 4.42 -> 4.69
+// ms in the attention stage of sparse selections (the merge kernel).
 template <typename... KArgs, typename... Args>
-void launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+void launch_kernel(bool overlap, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = grid;
@@ -160,8 +164,19 @@ void launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = overlap ? 1 : 0;
     (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);   // an error is picked up by launch_ok
+}
+
+template <typename K>
+bool set_smem(adaspark_attn* h, K kernel, size_t bytes, const char* what) {
+    if (bytes <= 48 * 1024) return true;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) {
+        fail(h, ADASPARK_ERR_CUDA, "%s: cudaFuncSetAttribute(%zu): %s", what, bytes, cudaGetErrorString(e));
+        return false;
+    }
+    return true;
 }
 
 #ifdef ADASPARK_WITH_TCGEN05
@@ -186,17 +201,6 @@ bool gather_can_pay(const Geom& g, float pairs_per_block) {
     return false;
 }
 #endif
-
-template <typename K>
-bool set_smem(adaspark_attn* h, K kernel, size_t bytes, const char* what) {
-    if (bytes <= 48 * 1024) return true;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) {
-        fail(h, ADASPARK_ERR_CUDA, "%s: cudaFuncSetAttribute(%zu): %s", what, bytes, cudaGetErrorString(e));
-        return false;
-    }
-    return true;
-}
 
 }  // namespace
 
@@ -421,7 +425,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         if (!launch_ok(h, "relayout_pool_kernel")) return ADASPARK_ERR_CUDA;
         const int cube_begin = g.pos_begin >> g.c_shift;
         if (g.C > kBlockTok && g.N_live > cube_begin) {
-            pool_large_cubes_kernel<<<dim3(g.N_live - cube_begin, g.Hkv, g.B), D, 0, st>>>(g, kc, cube_keys);
+            launch_kernel(true, pool_large_cubes_kernel, dim3(g.N_live - cube_begin, g.Hkv, g.B), dim3(D), 0, st, g, kc, cube_keys);
             if (!launch_ok(h, "pool_large_cubes_kernel")) return ADASPARK_ERR_CUDA;
         }
     }
@@ -443,17 +447,18 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         }
         int32_t* fallback_rows = (int32_t*)(ws + h->fw_fallback_off);
         const bool all = g.top_k <= 0 && !(g.top_p < 1.0);
+        const bool small = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 3 * kScoreWave / 2;   // the selection kernel fits the chip at once
         auto launch_exact = [&](const int32_t* rows, const uint32_t* n_list, long long n_ids) {
             if (D == 128)
-                select_exact_kernel<128><<<kExactCtas, kExactWarps * 32, g.N_ld * 8, st>>>(g, qb, cube_keys, rows, n_list, n_ids,
+                launch_kernel(small, select_exact_kernel<128>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
                                                                                    tile_mask, tile_union, sel_bitmap, sel_count);
             else
-                select_exact_kernel<64><<<kExactCtas, kExactWarps * 32, g.N_ld * 8, st>>>(g, qb, cube_keys, rows, n_list, n_ids,
+                launch_kernel(small, select_exact_kernel<64>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
                                                                                   tile_mask, tile_union, sel_bitmap, sel_count);
             return launch_ok(h, "select_exact_kernel");
         };
         if (all) {
-            select_all_kernel<<<dim3(g.n_tiles - g.tile_begin, g.Hq, g.B), kTileRows, 0, st>>>(g, tile_mask, tile_union, sel_bitmap, sel_count);
+            launch_kernel(true, select_all_kernel, dim3(g.n_tiles - g.tile_begin, g.Hq, g.B), dim3(kTileRows), 0, st, g, tile_mask, tile_union, sel_bitmap, sel_count);
             if (!launch_ok(h, "select_all_kernel")) return ADASPARK_ERR_CUDA;
         }
 #ifdef ADASPARK_WITH_TCGEN05
@@ -464,7 +469,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             auto* row_range = (float2*)(ws + h->fw_rowrange_off);
             float* scores = (float*)(ws + h->fw_scores_off);
             const int n_rows = g.B * g.Hkv * g.N_ld;
-            slice_keys_kernel<<<dim3(kSliceCtas, g.B * g.Hkv), 256, 0, st>>>(g, cube_keys, head_max, head_norm, kplanes);
+            launch_kernel(true, slice_keys_kernel, dim3(kSliceCtas, g.B * g.Hkv), dim3(256), 0, st, g, cube_keys, head_max, head_norm, kplanes);
             if (!launch_ok(h, "slice_keys_kernel")) return ADASPARK_ERR_CUDA;
             CUtensorMap tmKs, tmS;
             if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
@@ -479,8 +484,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
     do {                                                                                                               \
         const size_t smem = sizeof(ScoreSmem<DD>) + 1024;                                                              \
         if (!set_smem(h, score_tc_kernel<DD>, smem, "score_tc_kernel")) return ADASPARK_ERR_CUDA;                      \
-        score_tc_kernel<DD><<<grid, kScoreThreads, smem, st>>>(g, item0, n_here, qb, tmKs, tmS, head_max, head_norm,   \
-                                                               row_range, tile_union, &hdr->status);                   \
+        launch_kernel(true, score_tc_kernel<DD>, dim3(grid), dim3(kScoreThreads), smem, st, g, item0, n_here, qb, tmKs, \
+                      tmS, head_max, head_norm, row_range, tile_union, &hdr->status);                                  \
     } while (0)
                 if (D == 128) ADASPARK_LAUNCH_SCORE(128); else ADASPARK_LAUNCH_SCORE(64);
 #undef ADASPARK_LAUNCH_SCORE
@@ -489,9 +494,9 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
     do {                                                                                                               \
         const size_t smem = select_smem_bytes(sizeof(SelectWarpSmem<GG, KK>), g.n_words);                              \
         if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, BC>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
-        select_nucleus_kernel<GG, KK, RES, BC><<<2 * (next - first), kSelectThreads, smem, st>>>(                      \
-            g, item0, first, scores, (const float4*)row_range, tile_mask, tile_union, sel_bitmap, sel_count, fallback_rows,   \
-            &hdr->fallback_rows);                                                                                      \
+        launch_kernel(small, select_nucleus_kernel<GG, KK, RES, BC>, dim3(2 * (next - first)), dim3(kSelectThreads),   \
+                      smem, st, g, item0, first, (const float*)scores, (const float4*)row_range, tile_mask, tile_union, \
+                      sel_bitmap, sel_count, fallback_rows, &hdr->fallback_rows);                                      \
     } while (0)
 #define ADASPARK_LAUNCH_SELECT_K(GG, KK, RES)                                                                         \
     do {                                                                                                               \
@@ -591,12 +596,12 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             gw.pairs_per_window = (n_pairs_win + h->gather_windows - 1) / h->gather_windows;
             gw.n_pairs_cap = (int)n_pairs_cap;
             gw.pairs_per_block = h->gather_pairs_per_block;
-            gather_count_kernel<<<grid, 256, 0, st>>>(g, gw, tile_mask, tile_union);
+            launch_kernel(true, gather_count_kernel, dim3(grid), dim3(256), 0, st, g, gw, tile_mask, tile_union);
             if (!launch_ok(h, "gather_count_kernel")) return ADASPARK_ERR_CUDA;
-            gather_scan_kernel<<<1, 1024, 0, st>>>(g, gw);
+            launch_kernel(true, gather_scan_kernel, dim3(1), dim3(1024), 0, st, g, gw);
             if (!launch_ok(h, "gather_scan_kernel")) return ADASPARK_ERR_CUDA;
             const int icta = (int)((n_col_all + 7) / 8);
-            gather_items_kernel<<<icta < 4 * h->sm_count ? icta : 4 * h->sm_count, 256, 0, st>>>(g, gw);
+            launch_kernel(true, gather_items_kernel, dim3(icta < 4 * h->sm_count ? icta : 4 * h->sm_count), dim3(256), 0, st, g, gw);
             if (!launch_ok(h, "gather_items_kernel")) return ADASPARK_ERR_CUDA;
         }
         const uint32_t* pair_mode_c = gather ? gw.pair_mode : nullptr;
@@ -605,20 +610,20 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         if (D == 128) {
             size_t smem = sizeof(TcAttnSmem<128>) + 1024;
             if (!set_smem(h, attn_prefill_tc_kernel<128>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
-            attn_prefill_tc_kernel<128><<<grid, kTcThreads, smem, st>>>(g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
+            launch_kernel(true, attn_prefill_tc_kernel<128>, dim3(grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
                                                                         gw.n_pairs_cap, gw.ml_local, key_norm2_c, (__nv_bfloat16*)out,
                                                                         (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);
         } else {
             size_t smem = sizeof(TcAttnSmem<64>) + 1024;
             if (!set_smem(h, attn_prefill_tc_kernel<64>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
-            attn_prefill_tc_kernel<64><<<grid, kTcThreads, smem, st>>>(g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
+            launch_kernel(true, attn_prefill_tc_kernel<64>, dim3(grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
                                                                        gw.n_pairs_cap, gw.ml_local, key_norm2_c, (__nv_bfloat16*)out,
                                                                        (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);
         }
         if (!launch_ok(h, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
         mark(h, 6, st);
         if (gather) {
-            gather_fill_kernel<<<grid, 256, 0, st>>>(g, gw, tile_mask);
+            launch_kernel(true, gather_fill_kernel, dim3(grid), dim3(256), 0, st, g, gw, tile_mask);
             if (!launch_ok(h, "gather_fill_kernel")) return ADASPARK_ERR_CUDA;
             CUtensorMap tmKg;      // one key block per load: box of 64 d x 64 keys (tmK's) serves as it is
             tmKg = tmK;
@@ -627,19 +632,19 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             if (D == 128) {
                 const size_t smem = sizeof(GatherSmem<128>) + 1024;
                 if (!set_smem(h, attn_gather_kernel<128>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                attn_gather_kernel<128><<<ggrid, kGatherThreads, smem, st>>>(g, gw, tmKg, tmV, qb, slot_valid_c,
+                launch_kernel(true, attn_gather_kernel<128>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmKg, tmV, qb, slot_valid_c,
                                                                             (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
                 if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
                 const long long ctas = (n_rows + 15) / 16;
-                gather_merge_kernel<128><<<(unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count), 256, 0, st>>>(g, gw, (__nv_bfloat16*)out);
+                launch_kernel(false, gather_merge_kernel<128>, dim3((unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count)), dim3(256), 0, st, g, gw, (__nv_bfloat16*)out);
             } else {
                 const size_t smem = sizeof(GatherSmem<64>) + 1024;
                 if (!set_smem(h, attn_gather_kernel<64>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                attn_gather_kernel<64><<<ggrid, kGatherThreads, smem, st>>>(g, gw, tmKg, tmV, qb, slot_valid_c,
+                launch_kernel(true, attn_gather_kernel<64>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmKg, tmV, qb, slot_valid_c,
                                                                            (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
                 if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
                 const long long ctas = (n_rows + 31) / 32;
-                gather_merge_kernel<64><<<(unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count), 256, 0, st>>>(g, gw, (__nv_bfloat16*)out);
+                launch_kernel(false, gather_merge_kernel<64>, dim3((unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count)), dim3(256), 0, st, g, gw, (__nv_bfloat16*)out);
             }
             if (!launch_ok(h, "gather_merge_kernel")) return ADASPARK_ERR_CUDA;
         }
@@ -777,19 +782,19 @@ adaspark_status_t adaspark_attn_decode(adaspark_attn_t* h, const void* q_new, co
         if (D == 128) {
             size_t smem = sizeof(DecodeSmem<128>) + 1024;
             if (!set_smem(h, decode_splitkv_kernel<128>, smem, "decode_splitkv_kernel")) return ADASPARK_ERR_CUDA;
-            launch_overlapped(decode_splitkv_kernel<128>, grid, dim3(kDecodeThreads), smem, st, g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
+            launch_kernel(true, decode_splitkv_kernel<128>, grid, dim3(kDecodeThreads), smem, st, g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
         } else {
             size_t smem = sizeof(DecodeSmem<64>) + 1024;
             if (!set_smem(h, decode_splitkv_kernel<64>, smem, "decode_splitkv_kernel")) return ADASPARK_ERR_CUDA;
-            launch_overlapped(decode_splitkv_kernel<64>, grid, dim3(kDecodeThreads), smem, st, g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
+            launch_kernel(true, decode_splitkv_kernel<64>, grid, dim3(kDecodeThreads), smem, st, g, h->dc_splits, tmK, tmV, qn, dec_bitmap, text_len, items, n_items, partial, status);
         }
         if (!launch_ok(h, "decode_splitkv_kernel")) return ADASPARK_ERR_CUDA;
     }
     mark(h, 3, st);
     {
         auto* blocks = (unsigned long long*)&hdr->decode_kv_blocks;
-        if (D == 128) launch_overlapped(decode_combine_kernel<128>, dim3(g.Hq, g.B), dim3(512), 0, st, g, h->dc_splits, (const float*)partial, text_len, (const int32_t*)n_items, blocks, status, (__nv_bfloat16*)out);
-        else launch_overlapped(decode_combine_kernel<64>, dim3(g.Hq, g.B), dim3(512), 0, st, g, h->dc_splits, (const float*)partial, text_len, (const int32_t*)n_items, blocks, status, (__nv_bfloat16*)out);
+        if (D == 128) launch_kernel(true, decode_combine_kernel<128>, dim3(g.Hq, g.B), dim3(512), 0, st, g, h->dc_splits, (const float*)partial, text_len, (const int32_t*)n_items, blocks, status, (__nv_bfloat16*)out);
+        else launch_kernel(true, decode_combine_kernel<64>, dim3(g.Hq, g.B), dim3(512), 0, st, g, h->dc_splits, (const float*)partial, text_len, (const int32_t*)n_items, blocks, status, (__nv_bfloat16*)out);
     }
     if (!launch_ok(h, "decode_combine_kernel")) return ADASPARK_ERR_CUDA;
     mark(h, 4, st);

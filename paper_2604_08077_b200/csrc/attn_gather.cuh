@@ -139,7 +139,7 @@ __device__ __forceinline__ uint32_t row_entries(const Geom& g, const PairItem& i
     uint32_t cnt = 0;
 #pragma unroll 4
     for (int w = 0; w < it.n_w; ++w) {
-        uint32_t word = __ldg(my + (size_t)w * kTileRows);
+        uint32_t word = *(my + (size_t)w * kTileRows);
         if (w == it.n_w - 1) word &= it.last_keep;
         cnt += (uint32_t)__popc(fold_to_blocks(word, g.c_shift)) << bshift;
     }
@@ -148,8 +148,10 @@ __device__ __forceinline__ uint32_t row_entries(const Geom& g, const PairItem& i
 
 // ------------------------------------------------------------------------------------------------ count
 // One CTA per pair of query tiles and head.
-__global__ void __launch_bounds__(256) gather_count_kernel(Geom g, GatherWs ws, const uint32_t* __restrict__ tile_mask,
-                                                           const uint32_t* __restrict__ tile_union) {
+__global__ void __launch_bounds__(256) gather_count_kernel(Geom g, GatherWs ws, const uint32_t* tile_mask,
+                                                           const uint32_t* tile_union) {
+    launch_dependents();
+    wait_for_previous_kernel();
     __shared__ uint32_t red[2][8];
     __shared__ uint32_t s_mode;
     const PairItem it = pair_item(g, blockIdx.x);
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(256) gather_count_kernel(Geom g, GatherWs ws, 
     for (int w = tid; w < it.n_w; w += 256) {
         uint32_t u = 0;
         for (int t = 0; t < 2; ++t)
-            if (it.pair * 2 + t < g.n_tiles) u |= __ldg(tile_union + (bh * g.n_tiles_cap + it.pair * 2 + t) * g.n_words + w);
+            if (it.pair * 2 + t < g.n_tiles) u |= *(tile_union + (bh * g.n_tiles_cap + it.pair * 2 + t) * g.n_words + w);
         if (w == it.n_w - 1) u &= it.last_keep;
         ub += (uint32_t)__popc(fold_to_blocks(u, g.c_shift)) << bshift;
     }
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(256) gather_count_kernel(Geom g, GatherWs ws, 
     for (int w0 = 0; w0 < it.n_w; w0 += 4) {
         uint32_t wd[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) wd[k] = w0 + k < it.n_w ? __ldg(my + (size_t)(w0 + k) * kTileRows) : 0u;
+        for (int k = 0; k < 4; ++k) wd[k] = w0 + k < it.n_w ? *(my + (size_t)(w0 + k) * kTileRows) : 0u;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             if (w0 + k >= it.n_w) break;
@@ -242,6 +244,8 @@ __device__ __forceinline__ uint32_t cta_exclusive_scan_1024(uint32_t v, uint32_t
 }
 
 __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) {
+    launch_dependents();
+    wait_for_previous_kernel();
     __shared__ uint32_t warp_sums[32];
     __shared__ uint32_t total_s, total_s2;
     const int tid = threadIdx.x;
@@ -373,6 +377,8 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
 
 // Work items of every key block: chunks of up to 128 entries of its list.  One warp per block.
 __global__ void __launch_bounds__(256) gather_items_kernel(Geom g, GatherWs ws) {
+    launch_dependents();
+    wait_for_previous_kernel();
     if (ws.ctrl[0] == 0u) return;
     const int n_cols_all = ws.n_lists * ws.n_cols;
     const int lane = threadIdx.x & 31;
@@ -384,7 +390,9 @@ __global__ void __launch_bounds__(256) gather_items_kernel(Geom g, GatherWs ws) 
 }
 
 // ------------------------------------------------------------------------------------------------ fill
-__global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, const uint32_t* __restrict__ tile_mask) {
+__global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, const uint32_t* tile_mask) {
+    launch_dependents();
+    wait_for_previous_kernel();
     __shared__ uint32_t warp_tot[8];
     const PairItem it = pair_item(g, blockIdx.x);
     const size_t bh = (size_t)(it.b * g.Hq + it.h);
@@ -426,7 +434,7 @@ __global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, c
     for (int w0 = 0; w0 < it.n_w; w0 += 4) {
         uint32_t wd[4], fw[4], tw[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) wd[k] = w0 + k < it.n_w ? __ldg(my + (size_t)(w0 + k) * kTileRows) : 0u;
+        for (int k = 0; k < 4; ++k) wd[k] = w0 + k < it.n_w ? *(my + (size_t)(w0 + k) * kTileRows) : 0u;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             if (w0 + k == it.n_w - 1) wd[k] &= it.last_keep;
@@ -503,9 +511,10 @@ struct GatherSmem {
 template <int D>
 __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
     Geom g, GatherWs ws, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-    const __nv_bfloat16* __restrict__ q, const uint32_t* __restrict__ slot_valid,
-    unsigned long long* __restrict__ executed_blocks, int32_t* __restrict__ status) {
+    const __nv_bfloat16* __restrict__ q, const uint32_t* slot_valid, unsigned long long* executed_blocks, int32_t* status) {
     extern __shared__ unsigned char gather_smem_raw[];
+    launch_dependents();
+    wait_for_previous_kernel();
     GatherSmem<D>& sm = *reinterpret_cast<GatherSmem<D>*>((reinterpret_cast<uintptr_t>(gather_smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int kPanels = D / 64, kQKSteps = D / 16;
     constexpr uint32_t kIdescS = tc::make_idesc_bf16(128, 64);   // S: 128 gathered rows x 64 keys
@@ -554,7 +563,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
     volatile int* abort_flag = &sm.abort_flag;
     // item i of this CTA: (column = ((window x batch) x kv head) * n_cols + key block, first entry, entries, -)
     auto item_at = [&](int i) -> uint4 {
-        return __ldg(ws.items + ((size_t)(i / kGatherRun) * gridDim.x + blockIdx.x) * kGatherRun + (i % kGatherRun));
+        return *(ws.items + ((size_t)(i / kGatherRun) * gridDim.x + blockIdx.x) * kGatherRun + (i % kGatherRun));
     };
 
     if (warp < 8) {
@@ -564,7 +573,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
         const float scale_log2 = g.scale_log2;
         uint4 d_cur = c < my_items ? item_at(c) : make_uint4(0u, 0u, 0u, 0u);
         uint32_t ent = 0u;
-        if (c < my_items && row < (int)d_cur.z) ent = __ldg(ws.entries + d_cur.y + row);
+        if (c < my_items && row < (int)d_cur.z) ent = *(ws.entries + d_cur.y + row);
         for (int i = c, j = 0; i < my_items; i += 2, ++j) {
             // the next item of this warpgroup: descriptor and entry are requested now, used after the epilogue
             uint4 d_nxt = make_uint4(0u, 0u, 0u, 0u);
@@ -585,8 +594,8 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
                 }
                 if (g.ragged) {
                     const int blk = (int)(d_cur.x % (uint32_t)ws.n_cols);
-                    m0 &= __ldg(slot_valid + 2 * blk);
-                    m1 &= __ldg(slot_valid + 2 * blk + 1);
+                    m0 &= *(slot_valid + 2 * blk);
+                    m1 &= *(slot_valid + 2 * blk + 1);
                 }
             }
             if (!tc::mbar_wait(&sm.s_full[c], j & 1, abort_flag)) break;
@@ -653,7 +662,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
             tc::tc_fence_before_sync();
             tc::mbar_arrive(&sm.p_full[c]);
             uint32_t e_nxt = 0u;
-            if (i + 2 < my_items && row < (int)d_nxt.z) e_nxt = __ldg(ws.entries + d_nxt.y + row);
+            if (i + 2 < my_items && row < (int)d_nxt.z) e_nxt = *(ws.entries + d_nxt.y + row);
             // ---- epilogue: normalised partial output, (reference, sum)
             if (!tc::mbar_wait(&sm.o_full[c], j & 1, abort_flag)) break;
             tc::tc_fence_after_sync();
@@ -714,7 +723,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
         // right before its copy left this warpgroup waiting on L2 latency once per pass
         uint32_t e_cur[kPasses], e_nxt[kPasses];
 #pragma unroll
-        for (int ps = 0; ps < kPasses; ++ps) e_cur[ps] = (ps * kRowsPerPass + rsub < (int)d_cur.z) ? __ldg(ws.entries + d_cur.y + ps * kRowsPerPass + rsub) : 0u;
+        for (int ps = 0; ps < kPasses; ++ps) e_cur[ps] = (ps * kRowsPerPass + rsub < (int)d_cur.z) ? *(ws.entries + d_cur.y + ps * kRowsPerPass + rsub) : 0u;
         bool ok = true;
         for (int i = 0; i < my_items; ++i) {
             const int st = i % kGatherStages;
@@ -722,7 +731,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
             if (i + 1 < my_items) d_nxt = item_at(i + 1);
             const int n = (int)d_cur.z;
 #pragma unroll
-            for (int ps = 0; ps < kPasses; ++ps) e_nxt[ps] = (ps * kRowsPerPass + rsub < (int)d_nxt.z) ? __ldg(ws.entries + d_nxt.y + ps * kRowsPerPass + rsub) : 0u;
+            for (int ps = 0; ps < kPasses; ++ps) e_nxt[ps] = (ps * kRowsPerPass + rsub < (int)d_nxt.z) ? *(ws.entries + d_nxt.y + ps * kRowsPerPass + rsub) : 0u;
             if (!(ok = tc::mbar_wait(&sm.q_empty[st], ((i / kGatherStages) & 1) ^ 1, abort_flag))) break;
             const int bg = (int)(d_cur.x / (uint32_t)ws.n_cols) % (g.B * g.Hkv);
             const int b = bg / g.Hkv, gk = bg - b * g.Hkv;
@@ -835,21 +844,23 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
 // D/8 threads per row, 16 bytes (8 elements) of the row each.  The partials are folded in one pass with a
 // running reference exponent (their loads do not depend on it, so several are in flight per thread).
 template <int D>
-__global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, __nv_bfloat16* __restrict__ out) {
+__global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, __nv_bfloat16* out) {
+    launch_dependents();
+    wait_for_previous_kernel();
     if (ws.ctrl[0] == 0u) return;
     constexpr int kLanes = D / 8, kRowsPerCta = 256 / kLanes;
     const int sub = threadIdx.x % kLanes;
     const long long n_rows = (long long)ws.ctrl[2] * kPairRows;    // the rows of the pairs on this path
     for (long long idx = (long long)blockIdx.x * kRowsPerCta + threadIdx.x / kLanes; idx < n_rows; idx += (long long)gridDim.x * kRowsPerCta) {
-        const uint32_t slot = __ldg(ws.pair_list + (idx >> 8));
+        const uint32_t slot = *(ws.pair_list + (idx >> 8));
         const int bh = (int)(slot / (uint32_t)ws.n_pairs_cap);
         const int pos = (int)(slot - (uint32_t)bh * (uint32_t)ws.n_pairs_cap) * kPairRows + (int)(idx & 255);
         if (pos >= g.S) continue;
         const size_t row = (size_t)bh * g.S_cap + pos;
         // everything that does not depend on the row's count is requested first (one round of memory latency)
-        const uint32_t cnt = __ldg(ws.row_cnt + row);              // 0: a pair on the union path, or a slot without token
-        const uint32_t ptr = __ldg(ws.row_ptr + row);
-        const float2 loc = __ldg(ws.ml_local + row);
+        const uint32_t cnt = *(ws.row_cnt + row);              // 0: a pair on the union path, or a slot without token
+        const uint32_t ptr = *(ws.row_ptr + row);
+        const float2 loc = *(ws.ml_local + row);
         if (cnt == 0u) continue;
         const int b = bh / g.Hq, h = bh - b * g.Hq;
         uint4* dst = reinterpret_cast<uint4*>(out + (io_row(g, b, pos) * g.Hq + h) * D) + sub;
@@ -871,7 +882,7 @@ __global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, 
             float2 ml[4];
             uint4 v[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) e[k] = i0 + k < cnt ? __ldg(ws.row_slots + ptr + i0 + k) : 0xffffffffu;
+            for (int k = 0; k < 4; ++k) e[k] = i0 + k < cnt ? *(ws.row_slots + ptr + i0 + k) : 0xffffffffu;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 ml[k] = make_float2(0.f, 0.f);

@@ -67,10 +67,9 @@ struct BlockIter {
 template <int D>
 __global__ void __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
     Geom g, const __grid_constant__ CUtensorMap tmQ, const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap tmK,
-    const __grid_constant__ CUtensorMap tmV, const uint32_t* __restrict__ tile_mask,
-    const uint32_t* __restrict__ tile_union, const uint32_t* __restrict__ slot_valid, const uint32_t* __restrict__ pair_mode,
-    int n_pairs_cap, float2* __restrict__ ml_local, const uint32_t* __restrict__ key_norm2_bits, __nv_bfloat16* __restrict__ out,
-    unsigned long long* __restrict__ executed_blocks, uint32_t* __restrict__ max_tile_blocks, int32_t* __restrict__ status) {
+    const __grid_constant__ CUtensorMap tmV, const uint32_t* tile_mask, const uint32_t* tile_union, const uint32_t* slot_valid,
+    const uint32_t* pair_mode, int n_pairs_cap, float2* ml_local, const uint32_t* key_norm2_bits, __nv_bfloat16* out,
+    unsigned long long* executed_blocks, uint32_t* max_tile_blocks, int32_t* status) {
     extern __shared__ unsigned char tc_smem_raw[];
     TcAttnSmem<D>& sm = *reinterpret_cast<TcAttnSmem<D>*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int kPanels = D / 64;
@@ -95,9 +94,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
     const int n_blk_own = (pair_end + kBlockTok - 1) / kBlockTok;
     const int n_blk = sees_prefix ? max(n_blk_own, prefix_blk1) : n_blk_own;
     const int first_local_blk = pair_first_local_blk(g, pair_pos0);
-    // A pair whose selected cubes go through the query-gather kernels (attn_gather.cuh) visits only its local
-    // range and the text prefix here and leaves (reference exponent, sum) of every row for the merge.
-    const bool gathered = pair_mode != nullptr && __ldg(pair_mode + (size_t)(b * g.Hq + h) * n_pairs_cap + pair) != 0u;
 
     // ---------------------------------------------------------------- set-up
     if (tid == 0) {
@@ -115,6 +111,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
         sm.abort_flag = 0;
         tc::fence_barrier_init();
     }
+    launch_dependents();
+    wait_for_previous_kernel();
+    // A pair whose selected cubes go through the query-gather kernels (attn_gather.cuh) visits only its local
+    // range and the text prefix here and leaves (reference exponent, sum) of every row for the merge.
+    const bool gathered = pair_mode != nullptr && pair_mode[(size_t)(b * g.Hq + h) * n_pairs_cap + pair] != 0u;
     if (warp == 8) {
         tc::tmem_alloc<512>(&sm.tmem_base);
         if (lane == 0) {
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const int tile = pair * 2 + t;
-            if (tile < g.n_tiles) u |= __ldg(tile_union + ((size_t)(b * g.Hq + h) * g.n_tiles_cap + tile) * g.n_words + w);
+            if (tile < g.n_tiles) u |= tile_union[((size_t)(b * g.Hq + h) * g.n_tiles_cap + tile) * g.n_words + w];
         }
         sm.union_words[w] = u;
     }
@@ -374,7 +375,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
                         q2 = fmaf(lo, lo, fmaf(hi, hi, q2));
                     }
                 }
-                const float k2 = __uint_as_float(__ldg(key_norm2_bits + b * g.Hkv + gk));
+                const float k2 = __uint_as_float(key_norm2_bits[b * g.Hkv + gk]);
                 bound = sqrtf(q2 * k2) * scale_log2 * 1.01f + 0.01f;     // 1 % for the rounding of the norms and of s
             }
             fixed_ref = __all_sync(0xffffffffu, bound <= kFixedRefMax);
@@ -428,8 +429,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
                     m1 = gm[2] | (gm[3] << 16);
                 }
                 if (g.ragged && pk0 < g.S_v && !(hf == 1 && !has_b)) {   // empty slots of boundary cubes are never attended
-                    m0 &= __ldg(slot_valid + 2 * kb);
-                    m1 &= __ldg(slot_valid + 2 * kb + 1);
+                    m0 &= slot_valid[2 * kb];
+                    m1 &= slot_valid[2 * kb + 1];
                 }
                 amask[hf * 2] = m0;
                 amask[hf * 2 + 1] = m1;

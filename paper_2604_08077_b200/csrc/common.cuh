@@ -143,7 +143,8 @@ __device__ __forceinline__ bool key_allowed(const Geom& g, int pr, int pk, uint3
 // Programmatic dependent launch.  launch_dependents: the next kernel of the stream, if it was launched to overlap, may
 // start once every CTA of this one has come here (or ended); wait_for_previous_kernel: everything the kernels before
 // have written is visible from here on.  Whatever a kernel reads or writes that an earlier kernel of the same call
-// touches comes after its wait.
+// touches comes after its wait.  (Such data is not passed as const __restrict__ nor read with __ldg: the compiler may
+// move loads of read-only data above the wait.)
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 

@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
                                                             float* __restrict__ cube_keys,
                                                             uint32_t* __restrict__ slot_valid,
                                                             uint32_t* __restrict__ key_norm2_bits) {
+    launch_dependents();
     constexpr int kChunks = D / 8;    // 16-byte chunks per row
     constexpr int kVPitch = D + 2;    // padded pitch (elements) of the V staging tile
     __shared__ __align__(16) __nv_bfloat16 Ks[kBlockTok][D];
@@ -111,8 +112,9 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
 
 // Mean keys for cubes of more than 64 tokens: one CTA per (cube, kv head, batch), D threads,
 // reading the cube-major keys just written by relayout_pool_kernel.
-__global__ void pool_large_cubes_kernel(Geom g, const __nv_bfloat16* __restrict__ k_cube,
-                                        float* __restrict__ cube_keys) {
+__global__ void pool_large_cubes_kernel(Geom g, const __nv_bfloat16* k_cube, float* cube_keys) {
+    launch_dependents();
+    wait_for_previous_kernel();
     const int cube = blockIdx.x + (g.pos_begin >> g.c_shift), gk = blockIdx.y, b = blockIdx.z, d = threadIdx.x;
     if (d >= g.D) return;
     const __nv_bfloat16* src = k_cube + ((size_t)(b * g.Hkv + gk) * g.S_cap + (size_t)cube * g.C) * g.D + d;

@@ -87,12 +87,13 @@ __device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exp
 // (One kernel for all: two cost a launch more, 3 us of a short call.)
 constexpr int kSliceCtas = 8;
 __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_keys_kernel(
-    Geom g, const float* __restrict__ cube_keys, uint32_t* __restrict__ head_max_bits, float* __restrict__ head_norm,
-    unsigned char* __restrict__ planes) {
+    Geom g, const float* cube_keys, uint32_t* head_max_bits, float* head_norm, unsigned char* planes) {
     __shared__ uint32_t head[2];
+    launch_dependents();
     const int rank = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31;
     if (threadIdx.x < 2) head[threadIdx.x] = 0u;
     cluster_sync();                                           // every CTA of the cluster runs: its memory may be written
+    wait_for_previous_kernel();
     const float4* src = reinterpret_cast<const float4*>(cube_keys + (size_t)bh * g.N * g.D);
     const int n4 = g.N_live * (g.D / 4);                      // the cubes present so far
     uint32_t mx = 0;
@@ -164,9 +165,8 @@ __device__ __forceinline__ ScoreItem score_item(const Geom& g, int it) {
 template <int D>
 __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
     Geom g, int item0, int n_items, const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap tmK,
-    const __grid_constant__ CUtensorMap tmS, const uint32_t* __restrict__ head_max_bits,
-    const float* __restrict__ head_norm, float2* __restrict__ row_range, uint32_t* __restrict__ tile_union,
-    int32_t* __restrict__ status) {
+    const __grid_constant__ CUtensorMap tmS, const uint32_t* head_max_bits, const float* head_norm,
+    float2* row_range, uint32_t* tile_union, int32_t* status) {
     extern __shared__ unsigned char score_raw[];
     ScoreSmem<D>& sm = *reinterpret_cast<ScoreSmem<D>*>((reinterpret_cast<uintptr_t>(score_raw) + 1023) & ~(uintptr_t)1023);
     constexpr uint32_t kIdesc = tc::make_idesc_s8(128, kScoreTcCols);
@@ -185,6 +185,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
         sm.abort_flag = 0;
         tc::fence_barrier_init();
     }
+    launch_dependents();
+    wait_for_previous_kernel();
     if (warp == kProducerWarp) {
         tc::tmem_alloc<512>(&sm.tmem_base);
         if (lane == 0) {
@@ -317,10 +319,10 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
             q2 += __shfl_xor_sync(0xffffffffu, q2, 1);
             if (part == 0) {
                 const int bh = w.b * g.Hkv + w.gk;
-                const int e_sum = e_q + head_exponent(__ldg(head_max_bits + bh));
+                const int e_sum = e_q + head_exponent(head_max_bits[bh]);
                 const double f = __hiloint2double((1023 + e_sum - 34) << 20, 0) * g.scale_d;   // score per unit of V
                 // |V| <= |q| max|k| 2^(34 - e_sum), 1 % covers the rounding of the norms, 2^26 the digits' own rounding
-                const float vmax = sqrtf(q2) * __ldg(head_norm + bh) * (1.01f / 16777216.f) + 67108864.f;
+                const float vmax = sqrtf(q2) * head_norm[bh] * (1.01f / 16777216.f) + 67108864.f;
                 int sh = max((int)(__float_as_uint(vmax) >> 23) - 127 + 1 - 31, 0);            // vmax < 2^(31 + sh)
                 const bool give_up = !(f <= kMaxScorePerUnit) || sh > kMaxRowShift;            // also non-finite rows
                 sh = min(sh, kMaxRowShift);

@@ -24,13 +24,14 @@ constexpr int kExactCandCap = 256;
 // dynamic shared memory: N_ld doubles.
 template <int D>
 __global__ void __launch_bounds__(kExactWarps * 32) select_exact_kernel(
-    Geom g, const __nv_bfloat16* __restrict__ q, const float* __restrict__ cube_keys, const int32_t* __restrict__ rows,
-    const uint32_t* __restrict__ n_list, long long n_ids, uint32_t* __restrict__ tile_mask,
-    uint32_t* __restrict__ tile_union, uint32_t* __restrict__ sel_bitmap, int32_t* __restrict__ sel_count) {
+    Geom g, const __nv_bfloat16* __restrict__ q, const float* cube_keys, const int32_t* rows, const uint32_t* n_list,
+    long long n_ids, uint32_t* tile_mask, uint32_t* tile_union, uint32_t* sel_bitmap, int32_t* sel_count) {
     extern __shared__ __align__(16) double exact_scores[];
     __shared__ __align__(16) unsigned long long hist[kSelHistWords + kExactCandCap];
     __shared__ unsigned long long boundary;
     __shared__ int row_total;
+    launch_dependents();
+    wait_for_previous_kernel();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane & 3;
     const long long total = rows ? (long long)*n_list : n_ids;
     unsigned long long* keys = reinterpret_cast<unsigned long long*>(exact_scores);
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(kExactWarps * 32) select_exact_kernel(
                 const float* kr = kbase + (size_t)min(j, n - 1) * D;
                 float4 kv[D / 16];
 #pragma unroll
-                for (int i = 0; i < D / 16; ++i) kv[i] = __ldg(reinterpret_cast<const float4*>(kr + 16 * i));
+                for (int i = 0; i < D / 16; ++i) kv[i] = *reinterpret_cast<const float4*>(kr + 16 * i);
                 double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
 #pragma unroll
                 for (int i = 0; i < D / 16; ++i) {

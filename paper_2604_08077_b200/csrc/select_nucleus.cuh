@@ -65,9 +65,8 @@ __device__ __forceinline__ float sat_fma(float a, float b, float c) {     // min
 // kernel.  G * kK >= the largest candidate count of these items; kBits: G * kK masses of at most 2^kBits fit 32 bits.
 template <int G, int kK, int kResident, bool kByCount>
 __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kernel(
-    Geom g, int item0, int first, const float* __restrict__ scores, const float4* __restrict__ row_range,
-    uint32_t* __restrict__ tile_mask, uint32_t* __restrict__ tile_union, uint32_t* __restrict__ sel_bitmap,
-    int32_t* __restrict__ sel_count, int32_t* __restrict__ fallback_rows, uint32_t* __restrict__ fallback_count) {
+    Geom g, int item0, int first, const float* scores, const float4* row_range, uint32_t* tile_mask, uint32_t* tile_union,
+    uint32_t* sel_bitmap, int32_t* sel_count, int32_t* fallback_rows, uint32_t* fallback_count) {
     extern __shared__ __align__(16) unsigned char select_raw[];
     constexpr int R = 32 / G, kBuckets = 16 * G, kSteps = kK / 4;          // rows per warp; steps of 4 columns per lane
     constexpr int kMasks = (kK + 31) / 32;                                 // bit words per lane
@@ -89,6 +88,8 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
     for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
     for (int i = lane; i < n_words_live * kSelectRows; i += 32) words[i] = 0u;
     __syncwarp();
+    launch_dependents();
+    wait_for_previous_kernel();
 
     auto group_sum = [&](float x) -> float {
 #pragma unroll
@@ -447,9 +448,10 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
 
 // p >= 1 without Top-K: every candidate cube is selected (Eq. 2 with p = 1).  grid (tiles of the call, Hq, B),
 // 128 threads = rows of the tile.
-__global__ void __launch_bounds__(128) select_all_kernel(Geom g, uint32_t* __restrict__ tile_mask,
-                                                         uint32_t* __restrict__ tile_union, uint32_t* __restrict__ sel_bitmap,
-                                                         int32_t* __restrict__ sel_count) {
+__global__ void __launch_bounds__(128) select_all_kernel(Geom g, uint32_t* tile_mask, uint32_t* tile_union,
+                                                         uint32_t* sel_bitmap, int32_t* sel_count) {
+    launch_dependents();
+    wait_for_previous_kernel();
     const int tile = blockIdx.x + g.tile_begin, h = blockIdx.y, b = blockIdx.z, r = threadIdx.x;
     const int pos = tile * kTileRows + r;
     const bool live = slot_live(g, pos);
