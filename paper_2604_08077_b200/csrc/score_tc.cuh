@@ -76,6 +76,13 @@ __device__ __forceinline__ void digit_planes(uint32_t w0, uint32_t w1, uint32_t 
     plane[1] = __byte_perm(c, d, 0x5410);
     plane[0] = __byte_perm(c, d, 0x7632);
 }
+// V >> sh = S_0 2^(24-sh) + S_1 2^(16-sh) + ((S_2 2^8 + S_3) >> sh) for sh <= 16; m0 = 2^(24-sh), m1 = 2^(16-sh).  The sum
+// fits 32 bits, its terms need not (S_0 and S_1 may cancel), so they are added as unsigned words, which wrap.
+// |S_2 2^8 + S_3| < 2^31.
+__host__ __device__ __forceinline__ int32_t shifted_levels(int32_t s0, int32_t s1, int32_t s2, int32_t s3, uint32_t m0, uint32_t m1, int sh) {
+    const int32_t low = s2 * 256 + s3;
+    return (int32_t)((uint32_t)s0 * m0 + ((uint32_t)s1 * m1 + (uint32_t)(low >> sh)));
+}
 __device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exponent_from_field((int)((max_bits >> 23) & 0xffu)); }
 
 // Digit planes of the mean keys: planes[p][(b*Hkv+gk)*N_ld + cube][128 bytes] (int8, zero beyond D), all cubes of a
@@ -355,8 +362,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
             const float per_w = sm.row_scale[qb][quarter * 32 + lane];
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&sm.qd_free[qb]);
-            // V >> sh = S_0 2^(24-sh) + S_1 2^(16-sh) + ((S_2 2^8 + S_3) >> sh): sh <= 16, the result fits 32 bits
-            const int m1 = 1 << (16 - sh), m0 = m1 << 8;
+            const uint32_t m1 = 1u << (16 - sh), m0 = m1 << 8;
             float top = -INFINITY, low = INFINITY;
             for (int ct = 0; ok && ct < w.n_ct; ++ct, ++c) {
                 const int s = c & 1;
@@ -385,8 +391,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
 #pragma unroll
                             for (int i = 0; i < 4; ++i) {
                                 const int e = 4 * c4 + i;
-                                const int lw = (int)lv[2][e] * 256 + (int)lv[3][e];
-                                sv[i] = (float)((int)lv[0][e] * m0 + ((int)lv[1][e] * m1 + (lw >> sh))) * per_w;
+                                sv[i] = (float)shifted_levels((int)lv[0][e], (int)lv[1][e], (int)lv[2][e], (int)lv[3][e], m0, m1, sh) * per_w;
                             }
                             *reinterpret_cast<float4*>(stage + (((hf * 2 + c4) ^ swz) << 4)) = make_float4(sv[0], sv[1], sv[2], sv[3]);
                             if (whole) {
