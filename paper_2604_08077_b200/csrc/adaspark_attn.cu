@@ -34,9 +34,9 @@ struct adaspark_attn {
     adaspark_attn_layout_t layout;
     // workspace carving (byte offsets)
     size_t fw_status_off, fw_headmax_off, fw_valid_off, fw_gcol_off, fw_mask_off, fw_union_off, fw_fallback_off,
-        fw_kplanes_off, fw_rowrange_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
-        fw_gpartml_off, fw_total;
-    int score_items;            // query tiles per launch of the score / selection pair
+        fw_kplanes_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
+        fw_gpartml_off, fw_min, fw_total;      // fw_min: the smallest workspace a forward takes, fw_total: the one it is best given
+    int score_items;            // query tiles per launch of the score / selection pair, at most
     // query-gather path of the prefill: capacity in (row, key block) entries, decision threshold, byte budget
     uint32_t gather_cap;
     int gather_windows;
@@ -64,13 +64,16 @@ constexpr float kGatherDefaultPairsPerBlock = 30.f;
 constexpr uint64_t kGatherDefaultBudget = 24ull << 30;
 constexpr uint64_t kGatherEntriesPerRow = 128;
 constexpr size_t kGatherWindowBytes = 40u << 20;
-// Scores of the query tiles of one launch (int32, all columns; about half of it is touched over a causal sequence):
-// in whole waves of one tile per SM, as many as fit this budget.  Fewer, longer launches beat a buffer that stays in
-// the L2: 64 MB / 160 MB / 640 MB give 0.53 / 0.52 / 0.46 ms at 16384 tokens and 6.84 / 6.87 / 5.65 ms at 65536 (28
-// heads, 64-token cubes).
+// Scores of the query tiles of one launch (fp32, all columns; about half of it is touched over a causal sequence):
+// in whole waves of one tile per SM, as many as fit this budget.  They lie where the query-gather path keeps its lists and
+// partial results: the selection is over when those are begun.  A workspace that holds fewer tiles' scores is taken as it
+// is, down to kScoreItemsMin tiles (less than the 9472 N_ld bytes that the fp64 kernel's score rows once took).
 constexpr size_t kScoreBytes = 640u << 20;
 constexpr int kScoreWave = 148;
+constexpr int kScoreItemsMin = 8;
 size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
+// one query tile's scores and score ranges (a multiple of kAlign)
+size_t score_item_bytes(size_t N_ld) { return (size_t)kTileRows * (N_ld * 4 + kRangeParts * sizeof(float2)); }
 
 adaspark_status_t fail(adaspark_attn* h, adaspark_status_t st, const char* fmt, ...) {
     if (h) {
@@ -267,7 +270,8 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     L.cube_keys_bytes = (int64_t)((size_t)batch * Hkv * N * D * 4);
 
     // forward workspace: header | head exponents | per-tile mask matrix | per-tile union words | rows left to
-    // the fp64 selection kernel | key digit planes (tcgen05 path)
+    // the fp64 selection kernel | key digit planes (tcgen05 path) | scores of one launch, then, in the same place, the
+    // buffers of the query-gather path
     size_t off = 0;
     h->fw_status_off = off; off = align_up(off + 256);
     h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 3);   // mean-key exponents, largest |k|^2, largest |mean key|
@@ -287,17 +291,19 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // digit planes (4 x int8 [B*Hkv*N_ld, 128]) of the mean keys; 128 rows of slack so that the last TMA box
     // stays inside the allocation
     h->fw_kplanes_off = off; off = align_up(off + ((size_t)4 * batch * Hkv * N_ld + 128) * 128);
-    // scores and score ranges of one launch of the score / selection pair
-    {
-        const size_t tile_bytes = (size_t)kTileRows * N_ld * 4, n_items = (size_t)batch * Hq * n_tiles_cap;
-        size_t waves = kScoreBytes / (tile_bytes * kScoreWave);
+    // score ranges and scores of one launch of the score / selection pair (p >= 1 scores nothing)
+    h->fw_scores_off = off;
+    size_t scores_end = off, scores_end_min = off;
+    if (c.top_k > 0 || c.top_p < 1.f) {
+        const size_t n_items = (size_t)batch * Hq * n_tiles_cap;
+        size_t waves = kScoreBytes / ((size_t)kTileRows * N_ld * 4 * kScoreWave);
         if (waves < 1) waves = 1;
         h->score_items = (int)(waves * kScoreWave < n_items ? waves * kScoreWave : n_items);
-        h->fw_rowrange_off = off; off = align_up(off + (size_t)h->score_items * kTileRows * kRangeParts * sizeof(float2));
-        h->fw_scores_off = off; off = align_up(off + (size_t)h->score_items * tile_bytes);
+        scores_end += (size_t)h->score_items * score_item_bytes(N_ld);
+        scores_end_min += (n_items < kScoreItemsMin ? n_items : kScoreItemsMin) * score_item_bytes(N_ld);
     }
-    // query-gather path: per pair (mode, entries, offset) | per row (entries, first partial) | per row (m, l) of the
-    // local range | per key block offsets + work items | entries | partial outputs | partial (m, l)
+    // query-gather path, in the place of the scores: per pair (mode, entries, offset) | per row (entries, first partial) |
+    // per row (m, l) of the local range | per key block offsets + work items | entries | partial outputs | partial (m, l)
     {
         const size_t rows_cap = (size_t)batch * Hq * S_cap, n_pairs_cap = ((size_t)S_cap + 255) / 256;
         const uint64_t per_entry = 2ull * D + 16ull + 8ull;      // partial output + (m, l) + entry
@@ -317,8 +323,9 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
         h->fw_gparto_off = off; off = align_up(off + (size_t)cap * D * 2);
         h->fw_gpartml_off = off; off = align_up(off + (size_t)cap * 8);
     }
-    h->fw_total = off;
-    L.forward_workspace_bytes = (int64_t)off;
+    h->fw_min = off > scores_end_min ? off : scores_end_min;
+    h->fw_total = off > scores_end ? off : scores_end;
+    L.forward_workspace_bytes = (int64_t)h->fw_total;
 
     // decode workspace: status | bitmaps | block lists | counts | split partials
     // split count: at least ~2 waves of CTAs over the 148 SMs, and among those the count that
@@ -394,7 +401,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
     const bool cache_only = (q == nullptr);
     if (!cache_only) {
         if (!workspace) return fail(h, ADASPARK_ERR_INVALID_ARG, "%s: NULL workspace", who);
-        if (workspace_bytes < h->fw_total) return fail(h, ADASPARK_ERR_WORKSPACE_TOO_SMALL, "%s: workspace %zu < %zu bytes", who, workspace_bytes, h->fw_total);
+        if (workspace_bytes < h->fw_min) return fail(h, ADASPARK_ERR_WORKSPACE_TOO_SMALL, "%s: workspace %zu < %zu bytes", who, workspace_bytes, h->fw_min);
         if ((uintptr_t)workspace % kAlign) return fail(h, ADASPARK_ERR_INVALID_ARG, "%s: workspace not 256-byte aligned", who);
     }
     cudaError_t ce = cudaSetDevice(h->cfg.device);
@@ -466,19 +473,21 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             uint32_t* head_max = (uint32_t*)(ws + h->fw_headmax_off);
             float* head_norm = (float*)(head_max + 2 * g.B * g.Hkv);
             unsigned char* kplanes = (unsigned char*)(ws + h->fw_kplanes_off);
-            auto* row_range = (float2*)(ws + h->fw_rowrange_off);
-            float* scores = (float*)(ws + h->fw_scores_off);
+            const size_t room = (workspace_bytes - h->fw_scores_off) / score_item_bytes(g.N_ld);
+            const int score_items = room < (size_t)h->score_items ? (int)room : h->score_items;
+            auto* row_range = (float2*)(ws + h->fw_scores_off);
+            float* scores = (float*)(row_range + (size_t)score_items * kTileRows * kRangeParts);
             const int n_rows = g.B * g.Hkv * g.N_ld;
             launch_kernel(true, slice_keys_kernel, dim3(kSliceCtas, g.B * g.Hkv), dim3(256), 0, st, g, cube_keys, head_max, head_norm, kplanes);
             if (!launch_ok(h, "slice_keys_kernel")) return ADASPARK_ERR_CUDA;
             CUtensorMap tmKs, tmS;
             if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
-                !encode_f32_2d(&tmS, scores, (uint64_t)h->score_items * kTileRows, g.N_ld, 32))
+                !encode_f32_2d(&tmS, scores, (uint64_t)score_items * kTileRows, g.N_ld, 32))
                 return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
             const int n_hb = g.B * g.Hq, n_items = n_hb * (g.n_tiles - g.tile_begin);
             const bool by_count = g.top_k > 0;
-            for (int item0 = 0; item0 < n_items; item0 += h->score_items) {
-                const int n_here = n_items - item0 < h->score_items ? n_items - item0 : h->score_items;
+            for (int item0 = 0; item0 < n_items; item0 += score_items) {
+                const int n_here = n_items - item0 < score_items ? n_items - item0 : score_items;
                 const int grid = n_here < h->sm_count ? n_here : h->sm_count;
 #define ADASPARK_LAUNCH_SCORE(DD)                                                                                      \
     do {                                                                                                               \
