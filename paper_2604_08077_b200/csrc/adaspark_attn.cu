@@ -34,7 +34,7 @@ struct adaspark_attn {
     adaspark_attn_layout_t layout;
     // workspace carving (byte offsets)
     size_t fw_status_off, fw_headmax_off, fw_valid_off, fw_gcol_off, fw_mask_off, fw_union_off, fw_fallback_off,
-        fw_kplanes_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
+        fw_kplanes_off, fw_keyhash_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
         fw_gpartml_off, fw_min, fw_total;      // fw_min: the smallest workspace a forward takes, fw_total: the one it is best given
     int score_items;            // query tiles per launch of the score / selection pair, at most
     // query-gather path of the prefill: capacity in (row, key block) entries, decision threshold, byte budget
@@ -291,7 +291,9 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // digit planes (4 x int8 [B*Hkv*N_ld, 128]) of the mean keys; 128 rows of slack so that the last TMA box
     // stays inside the allocation
     h->fw_kplanes_off = off; off = align_up(off + ((size_t)4 * batch * Hkv * N_ld + 128) * 128);
-    // score ranges and scores of one launch of the score / selection pair (p >= 1 scores nothing)
+    // a hash of every mean key; score ranges and scores of one launch of the score / selection pair (p >= 1 scores nothing)
+    h->fw_keyhash_off = off;
+    if (c.top_k > 0 || c.top_p < 1.f) off = align_up(off + (size_t)batch * Hkv * N_ld * 8);
     h->fw_scores_off = off;
     size_t scores_end = off, scores_end_min = off;
     if (c.top_k > 0 || c.top_p < 1.f) {
@@ -477,8 +479,9 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             const int score_items = room < (size_t)h->score_items ? (int)room : h->score_items;
             auto* row_range = (float2*)(ws + h->fw_scores_off);
             float* scores = (float*)(row_range + (size_t)score_items * kTileRows * kRangeParts);
+            auto* key_hash = (unsigned long long*)(ws + h->fw_keyhash_off);
             const int n_rows = g.B * g.Hkv * g.N_ld;
-            launch_kernel(true, slice_keys_kernel, dim3(kSliceCtas, g.B * g.Hkv), dim3(256), 0, st, g, cube_keys, head_max, head_norm, kplanes);
+            launch_kernel(true, slice_keys_kernel, dim3(kSliceCtas, g.B * g.Hkv), dim3(256), 0, st, g, cube_keys, head_max, head_norm, kplanes, key_hash);
             if (!launch_ok(h, "slice_keys_kernel")) return ADASPARK_ERR_CUDA;
             CUtensorMap tmKs, tmS;
             if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
@@ -505,7 +508,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, BC>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
         launch_kernel(small, select_nucleus_kernel<GG, KK, RES, BC>, dim3(2 * (next - first)), dim3(kSelectThreads),   \
                       smem, st, g, item0, first, (const float*)scores, (const float4*)row_range, tile_mask, tile_union, \
-                      sel_bitmap, sel_count, fallback_rows, &hdr->fallback_rows);                                      \
+                      (const unsigned long long*)key_hash, sel_bitmap, sel_count, fallback_rows, &hdr->fallback_rows);                                      \
     } while (0)
 #define ADASPARK_LAUNCH_SELECT_K(GG, KK, RES)                                                                         \
     do {                                                                                                               \

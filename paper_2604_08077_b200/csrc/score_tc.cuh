@@ -92,9 +92,17 @@ __device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exp
 // slices, and leaves the largest |element| in head_max_bits and the largest norm of a mean key times 2^(29 - E_K) in
 // head_norm (of the scaled values: no size of input over- or underflows the squares).  grid (8, B*Hkv), 256 threads.
 // (One kernel for all: two cost a launch more, 3 us of a short call.)
+// key_hash[(b*Hkv+gk)*N_ld + cube]: 64 bits of the mean key's own bits.  Equal keys have equal words; that two different
+// keys share one is left to chance (2^-64), and asked only of keys whose scores are too near to tell apart.
 constexpr int kSliceCtas = 8;
+__device__ __forceinline__ unsigned long long hash_multiplier(uint32_t i) {      // an odd word per element (splitmix64)
+    unsigned long long z = (i + 1) * 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return (z ^ (z >> 31)) | 1ull;
+}
 __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_keys_kernel(
-    Geom g, const float* cube_keys, uint32_t* head_max_bits, float* head_norm, unsigned char* planes) {
+    Geom g, const float* cube_keys, uint32_t* head_max_bits, float* head_norm, unsigned char* planes, unsigned long long* key_hash) {
     __shared__ uint32_t head[2];
     launch_dependents();
     const int rank = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31;
@@ -116,16 +124,22 @@ __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_
     const uint32_t max_bits = head[0];
     const float mult = digit_scale(head_exponent(max_bits));
     const size_t plane_stride = (size_t)g.B * g.Hkv * g.N_ld * kDigitRowBytes;
+    const unsigned long long hm[4] = {hash_multiplier(lane * 4), hash_multiplier(lane * 4 + 1), hash_multiplier(lane * 4 + 2), hash_multiplier(lane * 4 + 3)};
     float norm2 = 0.f;
 #pragma unroll 2
     for (int cube = rank * 8 + (threadIdx.x >> 5); cube < g.N_ld; cube += kSliceCtas * 8) {
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (cube < g.N_live && lane * 4 < g.D) x = src[(size_t)cube * (g.D / 4) + lane];
+        unsigned long long hash = __float_as_uint(x.x) * hm[0] + __float_as_uint(x.y) * hm[1] + __float_as_uint(x.z) * hm[2] + __float_as_uint(x.w) * hm[3];
         x.x *= mult; x.y *= mult; x.z *= mult; x.w *= mult;
         float n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        for (int o = 16; o > 0; o >>= 1) {
+            n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+            hash += __shfl_xor_sync(0xffffffffu, hash, o);
+        }
         norm2 = fmaxf(norm2, n2);
+        if (lane == 0) key_hash[(size_t)bh * g.N_ld + cube] = hash;
         uint32_t plane[4];
         digit_planes(packed_digits(x.x), packed_digits(x.y), packed_digits(x.z), packed_digits(x.w), plane);
         unsigned char* dst = planes + ((size_t)bh * g.N_ld + cube) * kDigitRowBytes + lane * 4;

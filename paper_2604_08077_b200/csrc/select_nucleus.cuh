@@ -13,7 +13,7 @@
 //
 // Everything here is fp32, so a row is decided here only if its boundary is clear of what fp32 can be off by, and
 // handed to the fp64 kernel (list in the workspace) otherwise: a cumulative mass within eps of p Z, or a last selected
-// and a first rejected cube whose scores differ by less than kGapEps.  eps: an error e of the masses, of whatever sign,
+// and a first rejected cube whose scores differ by less than kGapEps and which are not copies of one cube.  eps: an error e of the masses, of whatever sign,
 // moves a cumulative share by at most 2 p (1 - p) e <= e / 2; ex2.approx is off by up to 2^-22, a score by 2^-24 of its
 // size and its distance from the maximum by 2^-25 of its size (both times ln 2; the cubes that carry mass lie within
 // about 8 units of the maximum and no further from 0 than it), and the sums of Z and of the base by about 1e-7
@@ -69,7 +69,7 @@ __device__ __forceinline__ float sat_fma(float a, float b, float c) {     // min
 template <int G, int kK, int kResident, bool kByCount>
 __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kernel(
     Geom g, int item0, int first, const float* scores, const float4* row_range, uint32_t* tile_mask, uint32_t* tile_union,
-    uint32_t* sel_bitmap, int32_t* sel_count, int32_t* fallback_rows, uint32_t* fallback_count) {
+    const unsigned long long* key_hash, uint32_t* sel_bitmap, int32_t* sel_count, int32_t* fallback_rows, uint32_t* fallback_count) {
     extern __shared__ __align__(16) unsigned char select_raw[];
     constexpr int R = 32 / G, kBuckets = 16 * G, kSteps = kK / 4;          // rows per warp; steps of 4 columns per lane
     constexpr int kMasks = (kK + 31) / 32;                                 // bit words per lane
@@ -413,7 +413,30 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             last = fminf(last, __shfl_xor_sync(kFull, last, o));
             next = fmaxf(next, __shfl_xor_sync(kFull, next, o));
         }
-        unsure = unsure || last - next <= kGapEps * fmaxf(fabsf(last), 0.25f);   // infinite unless both exist
+        const float gap = kGapEps * fmaxf(fabsf(last), 0.25f);
+        bool tied = last < INFINITY && last - next <= gap;                 // (a row without a listed cube that is selected is unsure)
+        if (__any_sync(kFull, tied)) {
+            // The boundary runs through cubes whose order these scores cannot tell.  If they are copies of one cube (frames
+            // that repeat: the mean keys are equal bit by bit) their scores are equal in fp64 too and the index orders them.
+            // (All such rows went to the fp64 kernel: every frame twice, 65536 tokens, 57.8 instead of 4.3 ms of selection.)
+            const unsigned long long* hash = key_hash + (size_t)(w.b * g.Hkv + w.gk) * g.N_ld;
+            unsigned long long h_min = ~0ull, h_max = 0ull;
+            for (int i = s; i < n_list; i += G) {
+                const float4 me = sm.cand[row_w][i];
+                if (last - me.x <= gap && me.x - next <= gap) {
+                    const unsigned long long hj = hash[__float_as_int(me.z)];
+                    h_min = min(h_min, hj);
+                    h_max = max(h_max, hj);
+                }
+            }
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) {
+                h_min = min(h_min, __shfl_xor_sync(kFull, h_min, o));
+                h_max = max(h_max, __shfl_xor_sync(kFull, h_max, o));
+            }
+            tied = tied && h_min != h_max;
+        }
+        unsure = unsure || tied || !(last < INFINITY);
         const bool any_unsure = group_any(unsure), any_reached = group_any(reached);   // both by all lanes
         unsure = any_unsure || !any_reached || !(base < target);
         if (n > 0 && (give_up || unsure)) {

@@ -52,15 +52,34 @@ def test_flat_and_sharp_scores(top_p, offset_std):
     _equal(wl)
 
 
+@pytest.mark.parametrize("rule", ["p", "k"])
 @pytest.mark.parametrize("copies", [2, 8, 40])
-def test_equal_scores(copies):
-    """Groups of identical cubes: the boundary falls among equal scores (more of them than the list holds, too)."""
+def test_equal_scores(copies, rule):
+    """Groups of identical cubes: the boundary falls among equal scores, which the cube index orders.  Only with more of
+    them than the list holds do the rows need the fp64 kernel."""
     wl = inputs.make_prefill("ties", seed=78, B=1, T=80, H=8, W=8, cube=(2, 4, 4), n_text=33, Hq=4, Hkv=2, D=128,
+                             top_p=0.8, offset_std=1.0)
+    if rule == "k":
+        wl.top_k = 13
+    k = wl.k.clone()
+    frames = k[:, :wl.S_v].view(1, 40, 2, 64, 2, 128)
+    frames.copy_(frames[:, ::copies].repeat_interleave(copies, 1)[:, :40])
+    rows = _equal(wl, k).fallback_rows
+    assert rows > 0 if copies > 32 else rows < 0.002 * wl.S * wl.Hq
+
+
+@pytest.mark.parametrize("copies", [2, 8])
+def test_equal_scores_of_different_cubes(copies):
+    """Cubes whose mean keys differ in an element that the queries leave out: their scores are equal too, their keys are not,
+    and the fp64 kernel decides."""
+    wl = inputs.make_prefill("ties", seed=81, B=1, T=80, H=8, W=8, cube=(2, 4, 4), n_text=33, Hq=4, Hkv=2, D=128,
                              top_p=0.8, offset_std=1.0)
     k = wl.k.clone()
     frames = k[:, :wl.S_v].view(1, 40, 2, 64, 2, 128)
     frames.copy_(frames[:, ::copies].repeat_interleave(copies, 1)[:, :40])
-    assert _equal(wl, k).fallback_rows > 0
+    frames[..., 5] = torch.arange(40).view(1, 40, 1, 1, 1).to(torch.bfloat16) / 16
+    wl.q[..., 5] = 0.0
+    assert _equal(wl, k).fallback_rows > 0.1 * wl.S * wl.Hq
 
 
 @pytest.mark.parametrize("scale_k", [2.0 ** -70, 2.0 ** -20, 2.0 ** 40])
