@@ -2,20 +2,22 @@
 //
 // The selection must follow an fp64 evaluation of Eqs. 1-2 (rows may differ only inside a 1e-6 probability
 // margin), so plain bf16/fp32 tensor-core arithmetic is not accurate enough.  Every query row q and every mean
-// key k are written in fixed point,
+// key k, less the head's first mean key k_0, are written in fixed point,
 //     x = 2^(e - 29) * (d0*2^24 + d1*2^16 + d2*2^8 + d3),   digits d_i signed bytes in [-128, 127],
-// with e the exponent of the largest element of the query row (e_q) or of all mean keys of the
-// (batch, kv head) (E_K).  tcgen05.mma of kind::i8 multiplies the digit planes with exact int32
+// with e the exponent of the largest element of the query row (e_q) or of all differences k_j - k_0 of the
+// (batch, kv head) (E_K).  What all keys of a head share (a bias) moves all scores of a row alike and has no part in its
+// selection, but would cost the fp32 scores their low bits.  Cube 0 is a candidate of every row that has one: no score is
+// larger than the row's spread.  tcgen05.mma of kind::i8 multiplies the digit planes with exact int32
 // accumulation,  S_L = sum_{a+b=L} Q_a . K_b  (10 digit pairs, levels L = 0..3, four TMEM
 // accumulators), and
-//     q . k_j = 2^(e_q + E_K - 34) * V_j,      V_j = S_0*2^24 + S_1*2^16 + S_2*2^8 + S_3   (an int64),
+//     q . (k_j - k_0) = 2^(e_q + E_K - 34) * V_j,      V_j = S_0*2^24 + S_1*2^16 + S_2*2^8 + S_3   (an int64),
 // up to the dropped levels >= 4 and the rounding of elements far below the row maximum.  Because the
 // key exponent is shared by the whole head, all scores of a row are the SAME positive factor
 // f = 2^(e_q + E_K - 34) * scale times an integer.
 //
 // What leaves the kernel per (row, cube) is the score in log2 units as fp32, s_j = W_j * (f 2^sh log2 e) with
-// W_j = V_j >> sh an int32: sh is the row's own shift, the smallest for which |q| max|k| (Cauchy-Schwarz over the mean
-// keys of the head) proves that no score overflows (on the benchmark inputs sh = 8: one unit of W is 1e-8 in the
+// W_j = V_j >> sh an int32: sh is the row's own shift, the smallest for which |q| max|k_j - k_0| (Cauchy-Schwarz over the
+// head) proves that no score overflows (on the benchmark inputs sh = 8: one unit of W is 1e-8 in the
 // scaled logit, below the 2e-8 that the dropped levels leave), and the largest and smallest score of every row.  The
 // selection kernel (select_nucleus.cuh) reads them from an L2-sized scratch buffer and decides every row whose
 // boundary is clearer than fp32 can be wrong; a launch covers as many query tiles as the buffer holds, and the two
@@ -52,12 +54,12 @@ constexpr int kDigitRowBytes = 128;      // bytes per row of a digit plane
 constexpr double kMaxScorePerUnit = 0.125 / 268435456.0;
 constexpr int kMaxRowShift = 16;         // |V| < D * 2^36 = 2^43 by construction, so a shift of 12 always suffices
 
-// The four signed base-256 digits of v = round(y), y = x * 2^(29 - e) (|v| < 2^30), packed in one word:
+// The four signed base-256 digits of v = round(x * 2^(29 - e)) (|v| <= 2^30), packed in one word:
 // byte 3 = d0 (most significant) ... byte 0 = d3.  Adding 0x80 to every byte position turns the
 // balanced digits into the plain unsigned bytes of v + 0x80808080, so two integer operations give
 // all four.
-__device__ __forceinline__ uint32_t packed_digits(float y) {
-    const uint32_t u = (uint32_t)__float2int_rn(y) + 0x80808080u;
+__device__ __forceinline__ uint32_t packed_digits(int v) {
+    const uint32_t u = (uint32_t)v + 0x80808080u;
     return u ^ 0x80808080u;
 }
 __device__ __forceinline__ float digit_scale(int e) {             // 2^(29 - e), exact for e >= -97
@@ -85,12 +87,11 @@ __host__ __device__ __forceinline__ int32_t shifted_levels(int32_t s0, int32_t s
 }
 __device__ __forceinline__ int head_exponent(uint32_t max_bits) { return row_exponent_from_field((int)((max_bits >> 23) & 0xffu)); }
 
-// Digit planes of the mean keys: planes[p][(b*Hkv+gk)*N_ld + cube][128 bytes] (int8, zero beyond D), all cubes of a
-// (batch, kv head) in the fixed point of that head's exponent; rows >= N inside the padded leading dimension are
-// zero-filled.  A cluster of 8 CTAs per (batch, kv head) first finds the largest |element| of the head's mean keys
-// (exchanged through distributed shared memory, float bits: non-negative floats order like their bit patterns), then
-// slices, and leaves the largest |element| in head_max_bits and the largest norm of a mean key times 2^(29 - E_K) in
-// head_norm (of the scaled values: no size of input over- or underflows the squares).  grid (8, B*Hkv), 256 threads.
+// Digit planes of the mean keys less the head's first: planes[p][(b*Hkv+gk)*N_ld + cube][128 bytes] (int8, zero beyond D),
+// all cubes of a (batch, kv head) in the fixed point of that head's exponent; rows >= N inside the padded leading
+// dimension are zero-filled.  A cluster of 8 CTAs per (batch, kv head) first finds the largest |element| (exchanged through distributed shared memory, float bits: non-negative floats order like their bit patterns), then
+// slices (the differences in fp64, rounded once to the fixed point), and leaves the largest |element| in head_max_bits and the
+// largest norm times 2^(29 - E_K) in head_norm (of the scaled values: no size of input over- or underflows the squares).  grid (8, B*Hkv), 256 threads.
 // (One kernel for all: two cost a launch more, 3 us of a short call.)
 // key_hash[(b*Hkv+gk)*N_ld + cube]: 64 bits of the mean key's own bits.  Equal keys have equal words; that two different
 // keys share one is left to chance (2^-64), and asked only of keys whose scores are too near to tell apart.
@@ -112,27 +113,29 @@ __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_
     const float4* src = reinterpret_cast<const float4*>(cube_keys + (size_t)bh * g.N * g.D);
     const int n4 = g.N_live * (g.D / 4);                      // the cubes present so far
     uint32_t mx = 0;
+    const float4 a = src[threadIdx.x & (g.D / 4 - 1)];        // of cube 0, the thread's elements in both loops (D / 4 divides 256)
 #pragma unroll 4
     for (int i = rank * 256 + threadIdx.x; i < n4; i += kSliceCtas * 256) {
         const float4 x = src[i];
-        mx = max(max(mx, __float_as_uint(fabsf(x.x))), max(__float_as_uint(fabsf(x.y)),
-                 max(__float_as_uint(fabsf(x.z)), __float_as_uint(fabsf(x.w)))));
+        mx = max(max(mx, __float_as_uint(fabsf(x.x - a.x))), max(__float_as_uint(fabsf(x.y - a.y)),
+                 max(__float_as_uint(fabsf(x.z - a.z)), __float_as_uint(fabsf(x.w - a.w)))));
     }
     mx = __reduce_max_sync(0xffffffffu, mx);
     if (lane < kSliceCtas) asm volatile("red.shared::cluster.max.u32 [%0], %1;\n" ::"r"(cluster_address(head, lane)), "r"(mx) : "memory");
     cluster_sync();
     const uint32_t max_bits = head[0];
-    const float mult = digit_scale(head_exponent(max_bits));
+    const double mult = (double)digit_scale(head_exponent(max_bits));
     const size_t plane_stride = (size_t)g.B * g.Hkv * g.N_ld * kDigitRowBytes;
     const unsigned long long hm[4] = {hash_multiplier(lane * 4), hash_multiplier(lane * 4 + 1), hash_multiplier(lane * 4 + 2), hash_multiplier(lane * 4 + 3)};
     float norm2 = 0.f;
 #pragma unroll 2
     for (int cube = rank * 8 + (threadIdx.x >> 5); cube < g.N_ld; cube += kSliceCtas * 8) {
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 x = a;
         if (cube < g.N_live && lane * 4 < g.D) x = src[(size_t)cube * (g.D / 4) + lane];
         unsigned long long hash = __float_as_uint(x.x) * hm[0] + __float_as_uint(x.y) * hm[1] + __float_as_uint(x.z) * hm[2] + __float_as_uint(x.w) * hm[3];
-        x.x *= mult; x.y *= mult; x.z *= mult; x.w *= mult;
-        float n2 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
+        const double y0 = ((double)x.x - (double)a.x) * mult, y1 = ((double)x.y - (double)a.y) * mult;
+        const double y2 = ((double)x.z - (double)a.z) * mult, y3 = ((double)x.w - (double)a.w) * mult;
+        float n2 = fmaf((float)y0, (float)y0, fmaf((float)y1, (float)y1, fmaf((float)y2, (float)y2, (float)y3 * (float)y3)));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             n2 += __shfl_xor_sync(0xffffffffu, n2, o);
@@ -141,7 +144,8 @@ __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_
         norm2 = fmaxf(norm2, n2);
         if (lane == 0) key_hash[(size_t)bh * g.N_ld + cube] = hash;
         uint32_t plane[4];
-        digit_planes(packed_digits(x.x), packed_digits(x.y), packed_digits(x.z), packed_digits(x.w), plane);
+        digit_planes(packed_digits(__double2int_rn(y0)), packed_digits(__double2int_rn(y1)), packed_digits(__double2int_rn(y2)),
+                     packed_digits(__double2int_rn(y3)), plane);
         unsigned char* dst = planes + ((size_t)bh * g.N_ld + cube) * kDigitRowBytes + lane * 4;
 #pragma unroll
         for (int p = 0; p < 4; ++p) *reinterpret_cast<uint32_t*>(dst + p * plane_stride) = plane[p];
@@ -329,7 +333,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
                     const float y0 = __uint_as_float(wa << 16) * mult, y1 = __uint_as_float(wa & 0xffff0000u) * mult;
                     const float y2 = __uint_as_float(wb << 16) * mult, y3 = __uint_as_float(wb & 0xffff0000u) * mult;
                     q2 = fmaf(y0, y0, fmaf(y1, y1, fmaf(y2, y2, fmaf(y3, y3, q2))));
-                    digit_planes(packed_digits(y0), packed_digits(y1), packed_digits(y2), packed_digits(y3), pw[q2w]);
+                    digit_planes(packed_digits(__float2int_rn(y0)), packed_digits(__float2int_rn(y1)), packed_digits(__float2int_rn(y2)),
+                                 packed_digits(__float2int_rn(y3)), pw[q2w]);
                 }
                 const int off = sw128(r, c) + 8 * part;           // elements 16 c + 8 part .. +7 of the plane row
 #pragma unroll
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
                 const int bh = w.b * g.Hkv + w.gk;
                 const int e_sum = e_q + head_exponent(head_max_bits[bh]);
                 const double f = __hiloint2double((1023 + e_sum - 34) << 20, 0) * g.scale_d;   // score per unit of V
-                // |V| <= |q| max|k| 2^(34 - e_sum), 1 % covers the rounding of the norms, 2^26 the digits' own rounding
+                // |V| <= |q| max|k_j - k_0| 2^(34 - e_sum), 1 % covers the rounding of the norms, 2^26 the digits' own rounding
                 const float vmax = sqrtf(q2) * head_norm[bh] * (1.01f / 16777216.f) + 67108864.f;
                 int sh = max((int)(__float_as_uint(vmax) >> 23) - 127 + 1 - 31, 0);            // vmax < 2^(31 + sh)
                 const bool give_up = !(f <= kMaxScorePerUnit) || sh > kMaxRowShift;            // also non-finite rows

@@ -90,3 +90,30 @@ def test_sizes_whose_squares_leave_fp32(scale_k):
     k = (wl.k.float() * scale_k).to(torch.bfloat16)
     hdr = _equal(wl, k, softmax_scale=128 ** -0.5 / scale_k)
     assert hdr.fallback_rows < 0.01 * wl.S * wl.Hq
+
+
+@pytest.mark.parametrize("shared", [(9.0, 3.0), (20.0, 0.0)])
+def test_a_bias_that_all_keys_share(shared):
+    """A vector added to all keys of a head moves a row's scores by a common offset (up to 300 here): same sets, and no more
+    rows than without it are too near to call."""
+    wl = inputs.make_prefill("bias", seed=82, B=1, T=64, H=8, W=8, cube=(1, 4, 4), n_text=31, Hq=4, Hkv=2, D=128, top_p=0.99,
+                             offset_std=1.5)
+    plain = _equal(wl).fallback_rows
+    sign = torch.randint(0, 2, (128,), generator=torch.Generator().manual_seed(1)) * 2.0 - 1.0
+    k = (wl.k.float() + shared[0] * sign).to(torch.bfloat16)
+    wl.q = (wl.q.float() + shared[1] * sign).to(torch.bfloat16)
+    assert _equal(wl, k).fallback_rows <= 2 * plain + 0.001 * wl.S * wl.Hq
+
+
+@pytest.mark.parametrize("first", [0.0, 8.0])
+@pytest.mark.parametrize("outlier", [0.0, 30.0])
+def test_first_cube_and_one_other_far_from_the_rest(first, outlier):
+    """Scores are taken relative to cube 0, in the fixed point of the head's largest element: a first cube and one in the
+    middle that are far larger than all others cost resolution, not correctness."""
+    wl = inputs.make_prefill("far", seed=83, B=1, T=40, H=8, W=8, cube=(1, 4, 4), n_text=31, Hq=4, Hkv=2, D=64, top_p=0.9,
+                             offset_std=1.0)
+    k = wl.k.float()
+    frames = k[:, :wl.S_v].view(1, 40, 2, 4, 2, 4, 2, 64)
+    frames[:, 0, 0, :, 0] += first
+    frames[:, 17, 1, :, 0] -= outlier
+    _equal(wl, k.to(torch.bfloat16))
