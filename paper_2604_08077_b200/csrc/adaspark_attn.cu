@@ -72,8 +72,8 @@ constexpr size_t kScoreBytes = 640u << 20;
 constexpr int kScoreWave = 148;
 constexpr int kScoreItemsMin = 8;
 size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
-// one query tile's scores and score ranges (a multiple of kAlign)
-size_t score_item_bytes(size_t N_ld) { return (size_t)kTileRows * (N_ld * 4 + kRangeParts * sizeof(float2)); }
+// one query tile's scores, score ranges and error bounds (a multiple of kAlign)
+size_t score_item_bytes(size_t N_ld) { return (size_t)kTileRows * (N_ld * 4 + kRangeParts * sizeof(float2) + sizeof(float)); }
 
 adaspark_status_t fail(adaspark_attn* h, adaspark_status_t st, const char* fmt, ...) {
     if (h) {
@@ -478,7 +478,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             const size_t room = (workspace_bytes - h->fw_scores_off) / score_item_bytes(g.N_ld);
             const int score_items = room < (size_t)h->score_items ? (int)room : h->score_items;
             auto* row_range = (float2*)(ws + h->fw_scores_off);
-            float* scores = (float*)(row_range + (size_t)score_items * kTileRows * kRangeParts);
+            float* row_err = (float*)(row_range + (size_t)score_items * kTileRows * kRangeParts);
+            float* scores = row_err + (size_t)score_items * kTileRows;
             auto* key_hash = (unsigned long long*)(ws + h->fw_keyhash_off);
             const int n_rows = g.B * g.Hkv * g.N_ld;
             launch_kernel(true, slice_keys_kernel, dim3(kSliceCtas, g.B * g.Hkv), dim3(256), 0, st, g, cube_keys, head_max, head_norm, kplanes, key_hash);
@@ -497,22 +498,26 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         const size_t smem = sizeof(ScoreSmem<DD>) + 1024;                                                              \
         if (!set_smem(h, score_tc_kernel<DD>, smem, "score_tc_kernel")) return ADASPARK_ERR_CUDA;                      \
         launch_kernel(true, score_tc_kernel<DD>, dim3(grid), dim3(kScoreThreads), smem, st, g, item0, n_here, qb, tmKs, \
-                      tmS, head_max, head_norm, row_range, tile_union, &hdr->status);                                  \
+                      tmS, head_max, head_norm, row_range, row_err, tile_union, &hdr->status);                         \
     } while (0)
                 if (D == 128) ADASPARK_LAUNCH_SCORE(128); else ADASPARK_LAUNCH_SCORE(64);
 #undef ADASPARK_LAUNCH_SCORE
                 if (!launch_ok(h, "score_tc_kernel")) return ADASPARK_ERR_CUDA;
-#define ADASPARK_LAUNCH_SELECT(GG, KK, RES, BC)                                                                       \
+#define ADASPARK_LAUNCH_SELECT(GG, KK, RES, RULE)                                                                     \
     do {                                                                                                               \
         const size_t smem = select_smem_bytes(sizeof(SelectWarpSmem<GG, KK>), g.n_words);                              \
-        if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, BC>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
-        launch_kernel(small, select_nucleus_kernel<GG, KK, RES, BC>, dim3(2 * (next - first)), dim3(kSelectThreads),   \
-                      smem, st, g, item0, first, (const float*)scores, (const float4*)row_range, tile_mask, tile_union, \
-                      (const unsigned long long*)key_hash, sel_bitmap, sel_count, fallback_rows, &hdr->fallback_rows);                                      \
+        if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, RULE>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
+        launch_kernel(small, select_nucleus_kernel<GG, KK, RES, RULE>, dim3(2 * (next - first)), dim3(kSelectThreads), \
+                      smem, st, g, select_target(RULE, g.top_p, GG * KK, GG * KK <= 256 ? 22 : GG * KK <= 1024 ? 21 : GG * KK <= 2048 ? 20 : 19), \
+                      item0, first, (const float*)scores, (const float4*)row_range, (const float*)row_err, tile_mask,  \
+                      tile_union, (const unsigned long long*)key_hash, sel_bitmap, sel_count, fallback_rows,           \
+                      &hdr->fallback_rows);                                                                            \
     } while (0)
 #define ADASPARK_LAUNCH_SELECT_K(GG, KK, RES)                                                                         \
     do {                                                                                                               \
-        if (by_count) ADASPARK_LAUNCH_SELECT(GG, KK, RES, true); else ADASPARK_LAUNCH_SELECT(GG, KK, RES, false);      \
+        if (by_count) ADASPARK_LAUNCH_SELECT(GG, KK, RES, kCount);                                                     \
+        else if (g.top_p < 0.5) ADASPARK_LAUNCH_SELECT(GG, KK, RES, kHead);                                            \
+        else ADASPARK_LAUNCH_SELECT(GG, KK, RES, kTail);                                                               \
     } while (0)
                 // Candidate counts fall with the items (late tiles come first): runs of items of one kernel shape, a run
                 // of less than eight tiles per SM joins its neighbour (another launch would cost what it saves).

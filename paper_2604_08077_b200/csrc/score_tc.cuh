@@ -48,10 +48,16 @@ constexpr int kEpilogueWarps = 16;
 constexpr int kRangeParts = 4;          // partial score ranges per row: one per column group of the epilogue
 constexpr int kScoreTcCols = 64;         // cubes per column tile
 constexpr int kDigitRowBytes = 128;      // bytes per row of a digit plane
-// Largest score per unit of V (f) that is decided from these scores: 2^(6 - 34) / sqrt(64), i.e. exponents up to
-// e_q + E_K = 6 at the default scale of head_dim 64 (the fixed-point error grows with f; the benchmark
-// inputs reach e_q + E_K = 5 at head_dim 128)
-constexpr double kMaxScorePerUnit = 0.125 / 268435456.0;
+// Largest score per unit of V (f) that is decided from these scores: 2^(7 - 34) / sqrt(64), i.e. exponents up to
+// e_q + E_K = 7 at the default scale of head_dim 64: with twice the largest mean key as the largest difference, mean keys up
+// to the size that was decided when the scores were not relative to k_0.  (The fixed-point error grows with f, and with it
+// the share of rows that are too near to call.)
+constexpr double kMaxScorePerUnit = 0.125 / 134217728.0;
+// Units of V that the digits leave open in a score's distance from another's: the dropped levels and the rounding of the
+// elements.  Against 64-bit products, over normal, uniform, heavy-tailed and constant queries and keys, each 512 rows x 512
+// keys: rms 180 (D = 64) and 255 (D = 128), at most 1021 and 2065.
+template <int D>
+constexpr float kFixedErr = 16.f * D;
 constexpr int kMaxRowShift = 16;         // |V| < D * 2^36 = 2^43 by construction, so a shift of 12 always suffices
 
 // The four signed base-256 digits of v = round(x * 2^(29 - e)) (|v| <= 2^30), packed in one word:
@@ -108,6 +114,7 @@ __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_
     launch_dependents();
     const int rank = blockIdx.x, bh = blockIdx.y, lane = threadIdx.x & 31;
     if (threadIdx.x < 2) head[threadIdx.x] = 0u;
+    const unsigned long long hm[4] = {hash_multiplier(lane * 4), hash_multiplier(lane * 4 + 1), hash_multiplier(lane * 4 + 2), hash_multiplier(lane * 4 + 3)};
     cluster_sync();                                           // every CTA of the cluster runs: its memory may be written
     wait_for_previous_kernel();
     const float4* src = reinterpret_cast<const float4*>(cube_keys + (size_t)bh * g.N * g.D);
@@ -126,7 +133,6 @@ __global__ void __cluster_dims__(kSliceCtas, 1, 1) __launch_bounds__(256) slice_
     const uint32_t max_bits = head[0];
     const double mult = (double)digit_scale(head_exponent(max_bits));
     const size_t plane_stride = (size_t)g.B * g.Hkv * g.N_ld * kDigitRowBytes;
-    const unsigned long long hm[4] = {hash_multiplier(lane * 4), hash_multiplier(lane * 4 + 1), hash_multiplier(lane * 4 + 2), hash_multiplier(lane * 4 + 3)};
     float norm2 = 0.f;
 #pragma unroll 2
     for (int cube = rank * 8 + (threadIdx.x >> 5); cube < g.N_ld; cube += kSliceCtas * 8) {
@@ -185,13 +191,13 @@ __device__ __forceinline__ ScoreItem score_item(const Geom& g, int it) {
 // Scores of the items [item0, item0 + n_items): row r of item item0 + i goes to row 128 * i + r of the scratch
 // matrix that tmS describes (fp32 [rows][N_ld]; columns beyond the tile's last candidate are not written), the
 // largest and smallest score of its candidates to row_range[4 * (128 * i + r) + part], part = which 16 of every 64
-// columns.  q: the call's queries [B, S_io, Hq, D].  tile_union words of the items are
+// columns, and what the fixed point leaves open in its scores to row_err[128 * i + r].  q: the call's queries [B, S_io, Hq, D].  tile_union words of the items are
 // set to zero for the selection kernel.
 template <int D>
 __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
     Geom g, int item0, int n_items, const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap tmK,
     const __grid_constant__ CUtensorMap tmS, const uint32_t* head_max_bits, const float* head_norm,
-    float2* row_range, uint32_t* tile_union, int32_t* status) {
+    float2* row_range, float* row_err, uint32_t* tile_union, int32_t* status) {
     extern __shared__ unsigned char score_raw[];
     ScoreSmem<D>& sm = *reinterpret_cast<ScoreSmem<D>*>((reinterpret_cast<uintptr_t>(score_raw) + 1023) & ~(uintptr_t)1023);
     constexpr uint32_t kIdesc = tc::make_idesc_s8(128, kScoreTcCols);
@@ -352,6 +358,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
                 int sh = max((int)(__float_as_uint(vmax) >> 23) - 127 + 1 - 31, 0);            // vmax < 2^(31 + sh)
                 const bool give_up = !(f <= kMaxScorePerUnit) || sh > kMaxRowShift;            // also non-finite rows
                 sh = min(sh, kMaxRowShift);
+                row_err[(size_t)it * kTileRows + r] = (float)(f * 1.4426950408889634) * (kFixedErr<D> + (float)(1 << sh));   // and one unit of W
                 sm.row_shift[qb][r] = (uint8_t)sh;
                 sm.row_scale[qb][r] = give_up ? __int_as_float(0x7fffffff)
                                               : (float)(f * __hiloint2double((1023 + sh) << 20, 0) * 1.4426950408889634);

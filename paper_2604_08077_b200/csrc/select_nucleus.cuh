@@ -9,17 +9,25 @@
 //            exact mass is summed; the few cubes inside it (widened by kGuard at both ends) are listed, and each
 //            learns the cumulative mass up to it: it is selected if the mass before it has not reached p Z
 // A bucket with more than kSelectCand cubes is split by further histograms over its cubes alone (rare, slow path).
-// Top-K (kByCount): the same with every mass = 1 and a target of min(top_k, candidates).
+// Top-K (kCount): the same with every mass = 1 and a target of min(top_k, candidates).
+//
+// From p = 1/2 on everything runs from the other end (kTail): the order is ascending, the target (1 - p) Z, "before" is what
+// is rejected, and a cube is rejected if the mass up to and including it does not exceed the target.  Masses, sums and their
+// errors are then those of the 1 - p that is left out.
 //
 // Everything here is fp32, so a row is decided here only if its boundary is clear of what fp32 can be off by, and
-// handed to the fp64 kernel (list in the workspace) otherwise: a cumulative mass within eps of p Z, or a last selected
-// and a first rejected cube whose scores differ by less than kGapEps and which are not copies of one cube.  eps: an error e of the masses, of whatever sign,
-// moves a cumulative share by at most 2 p (1 - p) e <= e / 2; ex2.approx is off by up to 2^-22, a score by 2^-24 of its
-// size and its distance from the maximum by 2^-25 of its size (both times ln 2; the cubes that carry mass lie within
-// about 8 units of the maximum and no further from 0 than it), and the sums of Z and of the base by about 1e-7
-// together: (2.4e-7 + 4.1e-8 (|max| + (8 + |max|) / 2)) / 2 + 1e-7 < 4e-7 + 3.2e-8 |max|.  On the benchmark inputs that
-// is one row in 10^4 to 10^3.  So are the rows the score kernel marked, and rows with more equal scores at the boundary
-// than the list holds.
+// handed to the fp64 kernel (list in the workspace) otherwise:
+//   - a cumulative mass within eps of the target.  With R the row's spread, S its largest |score| (relative to cube 0's: at
+//     most R) and rho what the fixed point leaves open in a score, one unit of W included (row_err), a score's distance from
+//     the maximum is off by rho + 2 (R + S) 2^-24 (R: the roundings of the factor of W and of the difference, S: of W and of the
+//     product) and a mass by e = ln 2 times that plus 2^-22 (ex2.approx).  Masses off by e, of whatever signs, move a share q by at most
+//     2 q (1 - q) e; a sum in which no term passes through more than a additions is off by a 2^-24.  With q the smaller of p and
+//     1 - p:  eps = q Z (2 (1 - q) e + (additions of Z, of the base and of the list + 2) 2^-24).
+//   - a last selected cube and a first rejected one, or the edge of the list, that lie less than 2 rho + 4 |s| 2^-24 apart and
+//     are not copies of one cube.
+// That is one row in 10^4 to 10^3 on the benchmark inputs, and no more with p nearer to 1 (sums up to p Z and an eps in
+// proportion to Z left 0.7 / 2.1 / 5.5 % undecided at p = 0.99 / 0.999 / 0.9999, 65536 tokens).  With them go the rows the score
+// kernel marked, and rows with more equal scores at the boundary than the list holds.
 //
 // What bounds it: instruction issue at few candidates (about 12 instructions per cube and lane and 800 per pass of 32 / G
 // rows, issue slots 60 to 65 % used), the stream of scores from memory at many (4 bytes per pair).  Sharing a warp among
@@ -29,6 +37,9 @@
 // Measured, scoring and selection together, 28 heads, against one kernel that recomputed the scores in every pass: 0.78 ->
 // 0.345 ms at 16384 tokens and 256 cubes, 13.6 -> 4.4 at 65536 and 1024, 59.5 -> 24.3 at 131072 and 2048.
 #pragma once
+#include <cmath>
+#include <cstring>
+
 #include "score_tc.cuh"
 
 namespace adaspark {
@@ -38,9 +49,39 @@ constexpr int kSelectRows = 8;           // consecutive rows of a warp: its mask
 constexpr int kSelectWarps = kSelectThreads / 32;
 constexpr int kSelectCand = 32;          // cubes of the crossing bucket a row may list
 constexpr int kMaxHistLevels = 8;        // histograms of a row before it is handed to the fp64 kernel
-constexpr float kMassEps = 4e-7f, kMassEpsTop = 3.2e-8f;   // of Z: the first plus |max| times the second
-constexpr float kGapEps = 2.4e-7f;       // of the larger of |s| and 1/4 (2^-22: twice the error of two scores)
+constexpr float kUlp = 5.9604645e-8f;    // 2^-24: the largest relative error of a rounding
 constexpr float kGuard = 1e-3f;          // of a bucket
+constexpr int kSumSteps = 8;             // steps of a lane (2 additions each) whose masses are summed before they join the rest
+enum SelectRule { kHead, kTail, kCount };                 // Top-p from the front and from the other end, Top-K
+
+// What a row is decided by (the same for all rows of a launch).
+struct SelectTarget {
+    double share;      // the target, of Z
+    float eps_mass;    // 1.01 x 2 q (1 - q): eps per Z and error of a mass
+    float eps_add;     // 1.01 q 2^-24: and per addition
+    float unit;        // masses are counted in 1 / unit
+    float q_unit;      // 2^-149 unit: a mass times it has the bits of mass x unit, rounded, up to 2^24 (a subnormal or the first binade)
+};
+// capacity: the scores that the kernel's shape holds.  2^head_bits: all of them, of mass 1, fit 32 bits.  From the tail the
+// sums need to fit up to the target only (what comes after it may wrap), and with p near 1 the masses that matter are small:
+// the target, at most q x capacity, stays below 2^31 units and, where single masses pass 2^24 units, below those.  A mass of
+// more than 2^24 units is counted as less, but as more than the target.  A histogram that misleads costs a row its decision,
+// no more.
+inline SelectTarget select_target(SelectRule rule, double top_p, int capacity, int head_bits) {
+    SelectTarget t;
+    t.share = rule == kCount ? 0.0 : rule == kTail ? 1.0 - top_p : top_p;
+    int bits = rule == kCount ? 0 : head_bits;
+    if (rule == kTail) {
+        const int il = std::ilogb(t.share * capacity), linear = 30 - il < 24 ? 30 - il : 24;
+        bits = 23 - il > linear ? 23 - il : linear;
+    }
+    t.eps_mass = (float)(2.02 * t.share * (1.0 - t.share));
+    t.eps_add = (float)(1.01 * t.share) * kUlp;
+    t.unit = std::ldexp(1.f, bits);
+    const uint32_t q_bits = bits < 23 ? 1u << bits : (uint32_t)(bits - 22) << 23;      // (by its bits: the host may flush subnormals)
+    std::memcpy(&t.q_unit, &q_bits, 4);
+    return t;
+}
 
 // Lanes per row grow with the candidate count, and the buckets with the lanes: a bucket holds at most about 5 of 256
 // cubes (G = 8), 512 (16) or 1024 (32) with normally distributed scores.
@@ -51,8 +92,8 @@ struct SelectWarpSmem {
     float4 range[32 / G][2];                              // partial ranges of the rows of a pass
     uint32_t hist[512];                                   // [bucket][row of the warp]
     float4 cand[32 / G][kSelectCand];                     // score, mass, cube
+    float err[2][32 / G];                                 // row_err of this pass and of the next
     int32_t count[32 / G];
-    int32_t pad[4 - (32 / G) % 4];
 };
 __host__ __device__ inline size_t select_smem_bytes(size_t warp_bytes, int n_words) {
     return kSelectWarps * (warp_bytes + (size_t)n_words * kSelectRows * 4);
@@ -62,19 +103,21 @@ __device__ __forceinline__ float sat_fma(float a, float b, float c) {     // min
     return __saturatef(fmaf(a, b, c));
 }
 
-// One warp per 8 rows of a tile, warps work on their own: 2 CTAs per item, items [first, ..) of those that the scores were computed for.  scores / row_range: what score_tc_kernel left for the items [item0, ..).
+// One warp per 8 rows of a tile, warps work on their own: 2 CTAs per item, items [first, ..) of those that the scores were
+// computed for.  scores / row_range / row_err: what score_tc_kernel left for the items [item0, ..).
 // tile_mask as mask_index() describes; tile_union (cleared) receives the OR of each word over the tile's rows;
 // fallback_rows[0 .. *fallback_count) receives ((b*Hq+h)*n_tiles_cap + tile)*128 + r of the rows left to the fp64
-// kernel.  G * kK >= the largest candidate count of these items; kBits: G * kK masses of at most 2^kBits fit 32 bits.
-template <int G, int kK, int kResident, bool kByCount>
+// kernel.  G * kK >= the largest candidate count of these items.
+template <int G, int kK, int kResident, SelectRule kRule>
 __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kernel(
-    Geom g, int item0, int first, const float* scores, const float4* row_range, uint32_t* tile_mask, uint32_t* tile_union,
+    Geom g, SelectTarget rule, int item0, int first, const float* scores, const float4* row_range, const float* row_err, uint32_t* tile_mask, uint32_t* tile_union,
     const unsigned long long* key_hash, uint32_t* sel_bitmap, int32_t* sel_count, int32_t* fallback_rows, uint32_t* fallback_count) {
     extern __shared__ __align__(16) unsigned char select_raw[];
     constexpr int R = 32 / G, kBuckets = 16 * G, kSteps = kK / 4;          // rows per warp; steps of 4 columns per lane
     constexpr int kMasks = (kK + 31) / 32;                                 // bit words per lane
-    constexpr int kBits = kByCount ? 0 : (G * kK <= 256 ? 22 : G * kK <= 1024 ? 21 : G * kK <= 2048 ? 20 : 19);
-    constexpr float kUnit = (float)(1 << kBits);
+    constexpr bool kByCount = kRule == kCount, tail = kRule == kTail;
+    constexpr int kBlocks = (kSteps + kSumSteps - 1) / kSumSteps;
+    constexpr int kAdds = kK / 2 / kBlocks + kBlocks + (G == 8 ? 3 : G == 16 ? 4 : 5);    // a mass passes through, in a row's sum
     constexpr uint32_t kFull = 0xffffffffu;
     constexpr float kMagic = 8388608.f;                                    // 2^23: low mantissa bits = the integer part
     constexpr uint32_t kMagicBits = 0x4B000000u;
@@ -94,6 +137,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
     launch_dependents();
     wait_for_previous_kernel();
 
+    constexpr float a_add0 = tail ? (float)(kBuckets - 1) : 0.f;
     auto group_sum = [&](float x) -> float {
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
@@ -117,6 +161,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         for (int c = 0; c < kSteps; ++c)
             if (c * 4 * G + 4 * s < n) cp_async_16(dst + c * 4 * G, src + c * 4 * G);
         if (s < 2 && n > 0) cp_async_16(&sm.range[row_w][s], row_range + 2 * srow + s);
+        if (s == 2 && n > 0) cp_async_4(&sm.err[pass & 1][row_w], row_err + srow);
         cp_async_commit();
     };
     int n_next = candidates(0);
@@ -166,20 +211,20 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         // mass of a score at d = s - max
         auto mass = [&](float d) -> float { return kByCount ? (d > -INFINITY ? 1.f : 0.f) : fast_exp2(d); };
 
-        // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, bucket = round(u): the buckets span the row
+        // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, or from the other end, bucket = round(u): the
+        // buckets span the row
         const float per_unit = fminf((float)(kBuckets - 1) / (top - low), 1e18f);
-        float a_mul = -per_unit, a_add = 0.f;                              // u = d * a_mul + a_add
+        float a_mul = tail ? per_unit : -per_unit, a_add = a_add0;         // u = d * a_mul + a_add
         float z = 0.f;
         uint32_t* my_hist = hist + row_w;
         const uint32_t hist_addr = smem_u32(my_hist) - kMagicBits * (4u * R);   // plus 4 R times the bits of 2^23 + bucket
-        const float q_unit = __int_as_float(1 << kBits);                   // 2^(kBits - 149): m times it is a subnormal whose bits are m 2^kBits, rounded
         auto add_to_bucket = [&](uint32_t bucket_bits, uint32_t q) {
             asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(hist_addr + bucket_bits * (4u * R)), "r"(q) : "memory");
         };
         {
-            unsigned long long z2 = 0ull;
+            unsigned long long z2 = 0ull, zs2 = 0ull;                      // of all steps, of the last few
             const unsigned long long neg_top2 = pack_f32x2(-top, -top), a_mul2 = pack_f32x2(a_mul, a_mul);
-            const unsigned long long magic2 = pack_f32x2(kMagic, kMagic), q_unit2 = pack_f32x2(q_unit, q_unit);
+            const unsigned long long magic2 = pack_f32x2(kMagic + a_add0, kMagic + a_add0), q_unit2 = pack_f32x2(rule.q_unit, rule.q_unit);
 #pragma unroll
             for (int c = 0; c < kSteps; ++c) {
                 if ((c + 1) * 4 * G <= n_whole) {
@@ -197,7 +242,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                             add_to_bucket(__float_as_uint(b1), 1u);
                         } else {
                             const unsigned long long m2 = pack_f32x2(mass(d0), mass(d1));
-                            z2 = add_f32x2(z2, m2);
+                            zs2 = add_f32x2(zs2, m2);
                             float q0, q1;
                             unpack_f32x2(mul_f32x2(m2, q_unit2), q0, q1);
                             add_to_bucket(__float_as_uint(b0), __float_as_uint(q0));
@@ -206,14 +251,22 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                     }
                 } else if (c * 4 * G < n_most) {                           // some columns hold no candidate (-inf: no mass)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float d = v[4 * c + i] - top;
-                        v[4 * c + i] = d;
-                        const float m = mass(d);
-                        z += m;
-                        const float u01 = __saturatef(d * (a_mul * (1.f / (kBuckets - 1))));
-                        add_to_bucket(__float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)), __float_as_uint(m * q_unit));
+                    for (int i = 0; i < 4; i += 2) {
+                        float m[2];
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            const float d = v[4 * c + i + k] - top;
+                            v[4 * c + i + k] = d;
+                            m[k] = mass(d);
+                            const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), tail ? 1.f : 0.f);
+                            add_to_bucket(__float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)), __float_as_uint(m[k] * rule.q_unit));
+                        }
+                        zs2 = add_f32x2(zs2, pack_f32x2(m[0], m[1]));
                     }
+                }
+                if (c % kSumSteps == kSumSteps - 1 || c == kSteps - 1) {
+                    z2 = c < kSumSteps ? zs2 : add_f32x2(z2, zs2);
+                    zs2 = 0ull;
                 }
             }
             float z0, z1;
@@ -221,9 +274,10 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             z += z0 + z1;
         }
         z = group_sum(z);
-        const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * g.top_p);
-        const float eps = kByCount ? 0.f : z * fmaf(fabsf(top), kMassEpsTop, kMassEps);
-        float base = 0.f;                                                  // mass selected so far
+        const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * rule.share);
+        float base = 0.f;                                                  // mass before the bucket
+        float to_edge = 0.f;                                               // u less this: where the list ends on the rejected side
+        int adds = 2 * kAdds + 2;
         uint32_t before[kMasks], inside[kMasks];                           // per lane: bit e = its e-th score
 #pragma unroll
         for (int k = 0; k < kMasks; ++k) { before[k] = 0u; inside[k] = 0u; }
@@ -244,7 +298,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                 const uint32_t t = __shfl_up_sync(kFull, incl, o, G);
                 if (s >= o) incl += t;
             }
-            const uint32_t thr = max((uint32_t)fmaxf((target - base) * kUnit, 0.f), 1u);
+            const uint32_t thr = max((uint32_t)fmaxf((target - base) * rule.unit, 0.f), 1u);
             uint32_t over = __ballot_sync(kFull, incl >= thr);
             if (G < 32) over = (over >> (row_w * G)) & ((1u << (G & 31)) - 1u);
             const int own = over ? __ffs(over) - 1 : G - 1;
@@ -277,9 +331,9 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             float add = 0.f;
             n_cand = 0;
             if (level == 0) {
-                const unsigned long long a_mul2 = pack_f32x2(a_mul, a_mul), lo2 = pack_f32x2(-lo_u, -lo_u);
+                const unsigned long long a_mul2 = pack_f32x2(a_mul, a_mul), lo2 = pack_f32x2(a_add0 - lo_u, a_add0 - lo_u);
                 const unsigned long long width2 = pack_f32x2(lo_u - hi_u, lo_u - hi_u);
-                unsigned long long add2 = 0ull;
+                unsigned long long add2 = 0ull, adds2 = 0ull;              // of all steps, of the last few
 #pragma unroll
                 for (int c = kSteps - 1; c >= 0; --c) {
                     if (c * 4 * G < n_most) {
@@ -295,10 +349,14 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                             before[k] = __funnelshift_l(__float_as_uint(ua0), before[k], 1);
                             inside[k] = __funnelshift_l(__float_as_uint(ub1), inside[k], 1);
                             inside[k] = __funnelshift_l(__float_as_uint(ub0), inside[k], 1);
-                            // the mass of what lies before: times 2^40 and clamped, the distance is 1 before and 0 else
-                            add2 = fma_f32x2(pack_f32x2(mass(d0), mass(d1)),
-                                             pack_f32x2(__saturatef(ua0 * -1099511627776.f), __saturatef(ua1 * -1099511627776.f)), add2);
+                            // the mass of what lies before: times 2^100 and clamped, the distance is 1 before and 0 else
+                            adds2 = fma_f32x2(pack_f32x2(mass(d0), mass(d1)),
+                                              pack_f32x2(__saturatef(ua0 * -1.2676506e30f), __saturatef(ua1 * -1.2676506e30f)), adds2);
                         }
+                    }
+                    if (c % kSumSteps == 0) {
+                        add2 = c + kSumSteps >= kSteps ? adds2 : add_f32x2(add2, adds2);
+                        adds2 = 0ull;
                     }
                 }
                 float add0, add1;
@@ -323,8 +381,17 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
 #pragma unroll
             for (int k = 0; k < kMasks; ++k) n_cand += __popc(inside[k]);
             add = group_sum(add);
-            n_cand = (int)(group_sum((float)n_cand) + 0.5f);
-            if (active) base += add;
+            if (G == 32) {
+                n_cand = __reduce_add_sync(kFull, n_cand);
+            } else {
+#pragma unroll
+                for (int o = G / 2; o > 0; o >>= 1) n_cand += __shfl_xor_sync(kFull, n_cand, o);
+            }
+            if (active) {
+                base += add;
+                to_edge = a_add - (tail ? lo_u : hi_u);
+                adds += level > 0 ? kK + 1 : 0;
+            }
             if (n_cand <= kSelectCand) active = false;
             if (active && level + 1 == kMaxHistLevels) { give_up = true; active = false; }
             if (!__any_sync(kFull, active)) break;
@@ -343,7 +410,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
                     const float d = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)] - top;
                     const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), a_add * (1.f / (kBuckets - 1)));
                     const uint32_t b = __float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)) - kMagicBits;
-                    atomicAdd(&my_hist[b * R], __float_as_uint(mass(d) * q_unit));
+                    atomicAdd(&my_hist[b * R], __float_as_uint(mass(d) * rule.q_unit));
                 }
             }
             __syncwarp();
@@ -369,10 +436,11 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         }
         __syncwarp();
         request(pass + 1, n_next);                                         // the rows' scores are no longer read
-        // ---- the words of what lies before the bucket: lane s holds nibble s & 7 of words (s >> 3) + c G / 8
+        // ---- the words of what lies before the bucket, or else of what is neither before nor inside it: lane s holds nibble
+        // s & 7 of words (s >> 3) + c G / 8
 #pragma unroll
         for (int k = 0; k < kMasks; ++k) {
-            uint32_t t = decide ? before[k] : 0u;                          // nibble c: columns of step 8 k + c
+            uint32_t t = tail ? before[k] | inside[k] : before[k];         // nibble c: columns of step 8 k + c
             // transpose the 8 x 8 nibbles of 8 neighbouring lanes: lane c then holds word c
             uint32_t o = __shfl_xor_sync(kFull, t, 4);
             t = (s & 4) ? ((t & 0xffff0000u) | (o >> 16)) : ((t & 0x0000ffffu) | (o << 16));
@@ -381,10 +449,16 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             o = __shfl_xor_sync(kFull, t, 1);
             t = (s & 1) ? ((t & 0xf0f0f0f0u) | ((o >> 4) & 0x0f0f0f0fu)) : ((t & 0x0f0f0f0fu) | ((o << 4) & 0xf0f0f0f0u));
             const int wd = (8 * k + (s & 7)) * (G / 8) + (s >> 3);
-            if (wd < n_words_live && n > 0) words[wd * kSelectRows + rl] = t;
+            if (tail) {
+                t = ~t & __funnelshift_lc(0xffffffffu, 0u, max(n - wd * 32, 0));   // of the row's candidates in the word
+            }
+            if (wd < n_words_live && decide) words[wd * kSelectRows + rl] = t;
         }
         __syncwarp();
-        // ---- each listed cube: the mass up to and including it
+        // ---- each listed cube: the mass before it and with it
+        const float err = n > 0 ? sm.err[pass & 1][row_w] : 0.f;
+        const float mass_err = fmaf(0.6931472f, fmaf(2.f * kUlp, (top - low) + fmaxf(top, -low), err), 4.f * kUlp);
+        const float eps = kByCount ? 0.f : z * fmaf(rule.eps_mass, mass_err, rule.eps_add * (float)(adds + n_list));
         float last = INFINITY, next = -INFINITY;                           // lowest selected, highest rejected score of my cubes
         bool reached = false;
         for (int i0 = 0; i0 < n_list_most; i0 += G) {
@@ -395,16 +469,18 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             float acc = base;                                              // and the listed cubes before mine
             for (int k = 0; k < n_list_most; ++k) {
                 const float4 ck = sm.cand[row_w][k];
-                if (ck.x > me.x || (ck.x == me.x && __float_as_int(ck.z) < ji)) acc += ck.y;
+                const bool earlier = tail ? ck.x < me.x || (ck.x == me.x && __float_as_int(ck.z) > ji)
+                                          : ck.x > me.x || (ck.x == me.x && __float_as_int(ck.z) < ji);
+                if (earlier) acc += ck.y;
             }
             if (mine) {
-                if (acc < target) {
+                if (tail ? acc + me.y > target : acc < target) {
                     atomicOr(&words[(ji >> 5) * kSelectRows + rl], 1u << (ji & 31));
                     last = fminf(last, me.x);
                 } else {
                     next = fmaxf(next, me.x);
                 }
-                reached = reached || acc + me.y >= target;
+                reached = reached || (tail ? acc + me.y > target : acc + me.y >= target);
                 if (!kByCount) unsure = unsure || fabsf(acc - target) <= eps || fabsf(acc + me.y - target) <= eps;
             }
         }
@@ -413,7 +489,9 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             last = fminf(last, __shfl_xor_sync(kFull, last, o));
             next = fmaxf(next, __shfl_xor_sync(kFull, next, o));
         }
-        const float gap = kGapEps * fmaxf(fabsf(last), 0.25f);
+        const float gap = fmaf(4.f * kUlp, fabsf(last), 2.f * err);
+        // an unlisted cube lies beyond the edge (u is off by a small part of the guard)
+        unsure = unsure || (n_list < n && fabsf(fmaf(last - top, a_mul, to_edge)) <= fmaf(gap, fabsf(a_mul), 0.5f * kGuard));
         bool tied = last < INFINITY && last - next <= gap;                 // (a row without a listed cube that is selected is unsure)
         if (__any_sync(kFull, tied)) {
             // The boundary runs through cubes whose order these scores cannot tell.  If they are copies of one cube (frames
@@ -438,7 +516,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         }
         unsure = unsure || tied || !(last < INFINITY);
         const bool any_unsure = group_any(unsure), any_reached = group_any(reached);   // both by all lanes
-        unsure = any_unsure || !any_reached || !(base < target);
+        unsure = any_unsure || !any_reached || !(tail ? base <= target : base < target);
         if (n > 0 && (give_up || unsure)) {
             for (int wd = s; wd < n_words_live; wd += G) words[wd * kSelectRows + rl] = 0u;
             if (s == 0) fallback_rows[atomicAdd(fallback_count, 1u)] = (int32_t)(gt_cap * kTileRows + r);

@@ -117,3 +117,22 @@ def test_first_cube_and_one_other_far_from_the_rest(first, outlier):
     frames[:, 0, 0, :, 0] += first
     frames[:, 17, 1, :, 0] -= outlier
     _equal(wl, k.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("top_p", [0.5, 0.99, 0.999, 0.9999, 0.99999, 0.9999999])
+@pytest.mark.parametrize("n_cubes,offset_std", [(250, 1.5), (1000, 1.5), (1000, 0.3), (700, 3.0)])
+def test_p_near_one(top_p, n_cubes, offset_std):
+    """What is left out is 1 - p: the nearer p to 1, the smaller the sums that decide and their errors, so no more rows than
+    at other p are too near to call (mass within eps of the target, eps = 5e-6 (1 - p) Z here, at boundary cubes that hold
+    about 1 % of the rest)."""
+    wl = inputs.make_prefill("rest", seed=84, B=1, T=n_cubes, H=4, W=4, cube=(1, 4, 4), n_text=200, Hq=2, Hkv=1, D=128, top_p=top_p,
+                             offset_std=offset_std)
+    assert _equal(wl).fallback_rows < 0.005 * wl.S * wl.Hq
+
+
+@pytest.mark.parametrize("top_p", [0.3, 0.9])
+def test_many_masses_that_are_nearly_equal(top_p):
+    """4000 masses within a few per cent of each other, whose sums round to the same side again and again."""
+    wl = inputs.make_prefill("level", seed=85, B=1, T=4000, H=4, W=4, cube=(1, 4, 4), n_text=300, Hq=1, Hkv=1, D=64, top_p=top_p,
+                             offset_std=0.01)
+    _equal(wl, wl.k * 0.125)
