@@ -23,8 +23,8 @@
 //     product) and a mass by e = ln 2 times that plus 2^-22 (ex2.approx).  Masses off by e, of whatever signs, move a share q by at most
 //     2 q (1 - q) e; a sum in which no term passes through more than a additions is off by a 2^-24.  With q the smaller of p and
 //     1 - p:  eps = q Z (2 (1 - q) e + (additions of Z, of the base and of the list + 2) 2^-24).
-//   - a last selected cube and a first rejected one, or the edge of the list, that lie less than 2 rho + 4 |s| 2^-24 apart and
-//     are not copies of one cube.
+//   - a last selected cube and a first rejected one, listed or not, that lie less than 2 rho + 4 |s| 2^-24 apart and are not
+//     copies of one cube.  (For the unlisted ones the edge of the first bucket stands, and what finer buckets leave out.)
 // That is one row in 10^4 to 10^3 on the benchmark inputs, and no more with p nearer to 1 (sums up to p Z and an eps in
 // proportion to Z left 0.7 / 2.1 / 5.5 % undecided at p = 0.99 / 0.999 / 0.9999, 65536 tokens).  With them go the rows the score
 // kernel marked, and rows with more equal scores at the boundary than the list holds.
@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
         z = group_sum(z);
         const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * rule.share);
         float base = 0.f;                                                  // mass before the bucket
-        float to_edge = 0.f;                                               // u less this: where the list ends on the rejected side
+        float to_edge = 0.f;                                               // u + this = 0: the edge of the first bucket on the rejected side
+        float beyond = -INFINITY;                                          // my largest rejected score of that bucket that is not listed
         int adds = 2 * kAdds + 2;
         uint32_t before[kMasks], inside[kMasks];                           // per lane: bit e = its e-th score
 #pragma unroll
@@ -365,18 +366,21 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
 #pragma unroll
                 for (int k = 0; k < kMasks; ++k) inside[k] &= ~before[k];
             } else {
+                int n_add = 0;
                 for (int k = 0; k < kMasks; ++k) {
                     uint32_t bits = active ? inside[k] : 0u;
                     while (bits) {
                         const int e = __ffs(bits) - 1;
                         bits &= bits - 1u;
-                        const float d = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)] - top;
+                        const float x = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)], d = x - top;
                         const float u = fmaf(d, a_mul, a_add);
-                        if (u < lo_u) { before[k] |= 1u << e; inside[k] &= ~(1u << e); add += mass(d); }
+                        if (u < lo_u) { before[k] |= 1u << e; inside[k] &= ~(1u << e); add += mass(d); ++n_add; }
                         else if (!(u < hi_u)) inside[k] &= ~(1u << e);
+                        else continue;
+                        if (tail ? u < lo_u : !(u < lo_u)) beyond = fmaxf(beyond, x);
                     }
                 }
-                __syncwarp();
+                adds += __reduce_max_sync(kFull, n_add) + 6;               // (the lane's, its group's and the base's)
             }
 #pragma unroll
             for (int k = 0; k < kMasks; ++k) n_cand += __popc(inside[k]);
@@ -389,8 +393,7 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             }
             if (active) {
                 base += add;
-                to_edge = a_add - (tail ? lo_u : hi_u);
-                adds += level > 0 ? kK + 1 : 0;
+                if (level == 0) to_edge = a_add - (tail ? lo_u : hi_u);
             }
             if (n_cand <= kSelectCand) active = false;
             if (active && level + 1 == kMaxHistLevels) { give_up = true; active = false; }
@@ -490,8 +493,13 @@ __global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kern
             next = fmaxf(next, __shfl_xor_sync(kFull, next, o));
         }
         const float gap = fmaf(4.f * kUlp, fabsf(last), 2.f * err);
-        // an unlisted cube lies beyond the edge (u is off by a small part of the guard)
-        unsure = unsure || (n_list < n && fabsf(fmaf(last - top, a_mul, to_edge)) <= fmaf(gap, fabsf(a_mul), 0.5f * kGuard));
+        // an unlisted cube lies beyond the edge (u is off by a small part of the guard) or has been looked at
+        unsure = unsure || (n_list < n && fabsf(fmaf(last - top, tail ? per_unit : -per_unit, to_edge)) <= fmaf(gap, per_unit, 0.5f * kGuard));
+        if (__any_sync(kFull, beyond > -INFINITY)) {
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) beyond = fmaxf(beyond, __shfl_xor_sync(kFull, beyond, o));
+            unsure = unsure || last - beyond <= gap;
+        }
         bool tied = last < INFINITY && last - next <= gap;                 // (a row without a listed cube that is selected is unsure)
         if (__any_sync(kFull, tied)) {
             // The boundary runs through cubes whose order these scores cannot tell.  If they are copies of one cube (frames
