@@ -118,7 +118,6 @@ Geom make_geom(const adaspark_attn* h, int n_text, int frame_begin = 0, int fram
     g.n_tiles_cap = h->S_cap / kTileRows;
     g.div_nW.init(g.nW);
     g.div_nH.init(g.nH);
-    g.div_n_tiles.init(g.n_tiles);
     g.n_kv_blocks_cap = h->S_cap / kBlockTok;
     g.Hq = h->cfg.n_q_heads; g.Hkv = h->cfg.n_kv_heads; g.G = g.Hq / g.Hkv; g.D = h->cfg.head_dim;
     g.div_Hq.init(g.Hq);

@@ -46,7 +46,7 @@ struct Geom {
     int C, N;            // tokens per cube (a power of two), cubes
     int c_shift;         // log2(C)
     int cw_shift, ch_shift;   // log2(cw), log2(ch): C is a power of two, so every window side is one
-    FastDiv div_nW, div_nH, div_n_tiles, div_Hq;
+    FastDiv div_nW, div_nH, div_Hq;
     int S_v, n_text, S;  // video slots N*C of the partition, text tokens so far (prefix included), slots present after this call
     int S_tok;           // video tokens T*H*W (= S_v unless the grid is ragged)
     int n_prefix;        // text tokens of the sequence that precede the video
