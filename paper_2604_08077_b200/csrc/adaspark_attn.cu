@@ -65,7 +65,9 @@ constexpr uint64_t kGatherDefaultBudget = 24ull << 30;
 constexpr uint64_t kGatherEntriesPerRow = 128;
 constexpr size_t kGatherWindowBytes = 40u << 20;
 // Scores of the query tiles of one launch (fp32, all columns; about half of it is touched over a causal sequence):
-// in whole waves of one tile per SM, as many as fit this budget.  They lie where the query-gather path keeps its lists and
+// in whole waves of one tile per SM, as many as fit this budget.  Fewer, longer launches beat a buffer that stays in the L2:
+// 40 / 80 / 160 / 320 / 640 MB give 0.50 / 0.42 / 0.39 / 0.36 / 0.36 ms of selection stage at 16384 tokens and 9.3 / 5.8 / 5.4 /
+// 4.8 / 4.6 ms at 65536 (28 heads, 64-token cubes).  They lie where the query-gather path keeps its lists and
 // partial results: the selection is over when those are begun.  A workspace that holds fewer tiles' scores is taken as it
 // is, down to kScoreItemsMin tiles (less than the 9472 N_ld bytes that the fp64 kernel's score rows once took).
 constexpr size_t kScoreBytes = 640u << 20;
@@ -455,7 +457,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         }
         int32_t* fallback_rows = (int32_t*)(ws + h->fw_fallback_off);
         const bool all = g.top_k <= 0 && !(g.top_p < 1.0);
-        const bool small = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 3 * kScoreWave / 2;   // the selection kernel fits the chip at once
+        const bool small = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 3 * kScoreWave / 2;   // the selection kernel's 444 CTAs fit the chip at once (in the shapes for up to 1024 candidates)
         auto launch_exact = [&](const int32_t* rows, const uint32_t* n_list, long long n_ids) {
             if (D == 128)
                 launch_kernel(small, select_exact_kernel<128>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
@@ -519,7 +521,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         else ADASPARK_LAUNCH_SELECT(GG, KK, RES, kTail);                                                               \
     } while (0)
                 // Candidate counts fall with the items (late tiles come first): runs of items of one kernel shape, a run
-                // of less than eight tiles per SM joins its neighbour (another launch would cost what it saves).
+                // of less than eight tiles per SM joins its neighbour.  A launch at every change of shape instead: 0.359 for
+                // 0.353 ms at 16384 tokens, but 4.38 for 4.48 at 65536; none but one a buffer: 0.368 and 4.49.
                 for (int first = 0, next; first < n_here; first = next) {
                     const int shape = select_shape(tile_max_candidates(g, g.n_tiles - 1 - (item0 + first) / n_hb));
                     int largest = shape;
