@@ -29,13 +29,14 @@
 // proportion to Z left 0.7 / 2.1 / 5.5 % undecided at p = 0.99 / 0.999 / 0.9999, 65536 tokens).  With them go the rows the score
 // kernel marked, and rows with more equal scores at the boundary than the list holds.
 //
-// What bounds it: instruction issue at few candidates (about 12 instructions per cube and lane and 800 per pass of 32 / G
-// rows, issue slots 60 to 65 % used), the stream of scores from memory at many (4 bytes per pair).  Sharing a warp among
+// What bounds it: instruction issue at few candidates (about 20 instructions per score of a lane in the two sweeps and 900
+// per pass of 32 / G rows beside them; 1390 per pass with 128 to 256 candidates, issue slots 63 % used, 1000 with fewer, 80 %),
+// the stream of scores from memory at many (4 bytes per pair).  Sharing a warp among
 // 32 / G rows spreads the second figure over several rows; the per-cube work is spread over the pipes (the bits come
 // from funnel shifts of signs, the mass before the bucket from a saturating multiply, the exponential from the MUFU unit,
 // the rest from packed fp32 pairs), because the integer / comparison pipe issues at half the rate of the fp32 pipe.
 // Measured, scoring and selection together, 28 heads, against one kernel that recomputed the scores in every pass: 0.78 ->
-// 0.345 ms at 16384 tokens and 256 cubes, 13.6 -> 4.4 at 65536 and 1024, 59.5 -> 24.3 at 131072 and 2048.
+// 0.354 ms at 16384 tokens and 256 cubes, 13.6 -> 4.4 at 65536 and 1024, 59.5 -> 25.3 at 131072 and 2048, half static.
 #pragma once
 #include <cmath>
 #include <cstring>
