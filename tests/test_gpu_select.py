@@ -107,13 +107,17 @@ def test_a_bias_that_all_keys_share(shared):
 
 @pytest.mark.parametrize("first", [0.0, 8.0])
 @pytest.mark.parametrize("outlier", [0.0, 30.0])
-def test_first_cube_and_one_other_far_from_the_rest(first, outlier):
+@pytest.mark.parametrize("level", [False, True])
+def test_first_cube_and_one_other_far_from_the_rest(first, outlier, level):
     """Scores are taken relative to cube 0, in the fixed point of the head's largest element: a first cube and one in the
-    middle that are far larger than all others cost resolution, not correctness."""
-    wl = inputs.make_prefill("far", seed=83, B=1, T=40, H=8, W=8, cube=(1, 4, 4), n_text=31, Hq=4, Hkv=2, D=64, top_p=0.9,
+    middle that are far larger than all others cost resolution, not correctness.  With queries whose elements are all of one
+    size (level) a row's shift is the largest there is, 12."""
+    wl = inputs.make_prefill("far", seed=83, B=1, T=40, H=8, W=8, cube=(1, 4, 4), n_text=31, Hq=4, Hkv=2, D=128, top_p=0.9,
                              offset_std=1.0)
+    if level:
+        wl.q = (torch.sign(wl.q.float()) * 1.984375).to(torch.bfloat16)
     k = wl.k.float()
-    frames = k[:, :wl.S_v].view(1, 40, 2, 4, 2, 4, 2, 64)
+    frames = k[:, :wl.S_v].view(1, 40, 2, 4, 2, 4, 2, 128)
     frames[:, 0, 0, :, 0] += first
     frames[:, 17, 1, :, 0] -= outlier
     _equal(wl, k.to(torch.bfloat16))
