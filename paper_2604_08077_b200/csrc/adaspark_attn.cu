@@ -56,6 +56,8 @@ struct adaspark_attn {
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr size_t kNextPairTileOffset = 128;   // in the 256 bytes of the workspace header (cleared per call), behind the public fields
+static_assert(sizeof(adaspark_attn_workspace_header_t) <= kNextPairTileOffset, "the counter lies behind the header's fields");
 constexpr int kExactCtas = 592;   // CTAs of the fp64 selection kernel: four per SM
 // query-gather path: pairs of query tiles take it when their rows' (row, key block) entries are at most this
 // many per key block of the pair's union (measured break-even on a B200, see the attention profile), and the
@@ -253,10 +255,10 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     if ((long long)batch * S_cap * c.n_q_heads * c.head_dim >= (1ll << 40) || S_cap >= (1ll << 30))
         return fail(h, ADASPARK_ERR_UNSUPPORTED, "partition: problem too large");
 #ifdef ADASPARK_WITH_TCGEN05
-    // the attention kernel keeps one bit per 64-key block of a sequence in shared memory
-    if (S_cap / kBlockTok > 32ll * kMaxBlockWords)
+    // the attention kernel keeps the numbers of a pair tile's key blocks in shared memory, 16 bits each
+    if (S_cap / kBlockTok > kMaxKeyBlocks)
         return fail(h, ADASPARK_ERR_UNSUPPORTED, "partition: %lld cache rows per sequence > %d", S_cap,
-                    32 * kMaxBlockWords * kBlockTok);
+                    kMaxKeyBlocks * kBlockTok);
 #endif
     h->B = batch; h->T = frames; h->H = grid_h; h->W = grid_w; h->n_text_max = n_text_max;
     h->N = (int)N; h->S_v = (int)S_v; h->S_cap = (int)S_cap;
@@ -275,7 +277,7 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // buffers of the query-gather path
     size_t off = 0;
     h->fw_status_off = off; off = align_up(off + 256);
-    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 3);   // mean-key exponents, largest |k|^2, largest |mean key|
+    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 4);   // mean-key exponents, largest |k|^2, largest |mean key|, largest |v|
     h->fw_valid_off = off; off = align_up(off + (size_t)(S_cap / kBlockTok) * 2 * 4);   // which slots of a block hold a token
     const size_t n_cols = (size_t)(S_v + kBlockTok - 1) / kBlockTok;                     // key blocks that hold video
     // query-gather path: the rows are cut into windows whose slice of Q (all heads) is about a third of the L2
@@ -428,11 +430,19 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         const int blk_end = last_call ? g.n_kv_blocks_cap : (g.S + kBlockTok - 1) / kBlockTok;
         dim3 grid(blk_end - blk_begin, g.Hkv, g.B);
         uint32_t* slot_valid = (!cache_only && g.ragged) ? (uint32_t*)((char*)workspace + h->fw_valid_off) : nullptr;
-        // largest |k|^2 per (batch, kv head): only a call that brings the sequence from its first frame sees every key
-        uint32_t* key_norm2 = (!cache_only && frame_begin == 0) ? (uint32_t*)((char*)workspace + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
-        if (D == 128) relayout_pool_kernel<128><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
-        else relayout_pool_kernel<64><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
+        // largest |k|^2 and |v| per (batch, kv head)
+        uint32_t* key_norm2 = !cache_only ? (uint32_t*)((char*)workspace + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
+        uint32_t* value_max = !cache_only ? key_norm2 + 2 * g.B * g.Hkv : nullptr;
+        if (D == 128) relayout_pool_kernel<128><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2, value_max);
+        else relayout_pool_kernel<64><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2, value_max);
         if (!launch_ok(h, "relayout_pool_kernel")) return ADASPARK_ERR_CUDA;
+        if (!cache_only && g.pos_begin > 0 && h->prefill_kernel != 0) {     // the keys and values of earlier calls
+            const int ctas = g.pos_begin * (D / 8) / 1024;              // four 16-byte pieces of K and V a thread, at least
+            const dim3 ngrid(ctas < 1024 ? (ctas < 1 ? 1 : ctas) : 1024, g.Hkv, g.B);
+            if (D == 128) launch_kernel(true, seen_norms_kernel<128>, ngrid, dim3(256), 0, st, g, g.pos_begin, (const __nv_bfloat16*)kc, (const __nv_bfloat16*)vc, key_norm2, value_max);
+            else launch_kernel(true, seen_norms_kernel<64>, ngrid, dim3(256), 0, st, g, g.pos_begin, (const __nv_bfloat16*)kc, (const __nv_bfloat16*)vc, key_norm2, value_max);
+            if (!launch_ok(h, "seen_norms_kernel")) return ADASPARK_ERR_CUDA;
+        }
         const int cube_begin = g.pos_begin >> g.c_shift;
         if (g.C > kBlockTok && g.N_live > cube_begin) {
             launch_kernel(true, pool_large_cubes_kernel, dim3(g.N_live - cube_begin, g.Hkv, g.B), dim3(D), 0, st, g, kc, cube_keys);
@@ -573,9 +583,12 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         const uint32_t qbox[5] = {64u, bx, by, bt, 1u};
         if (!encode_bf16_5d(&tmQ, qb + (size_t)g.n_prefix * g.Hq * D, qdims, qstr, qbox) ||
             !encode_bf16_2d(&tmK, kc, (uint64_t)g.B * g.Hkv * g.S_cap, D, 64, 64) ||
-            !encode_bf16_2d(&tmV, vc, (uint64_t)g.B * g.Hkv * g.n_kv_blocks_cap * D, 64, 64, D))
+            !encode_bf16_2d(&tmV, vc, (uint64_t)g.B * g.Hkv * g.n_kv_blocks_cap * D, 64, 64, D / 2))
             return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
         dim3 grid(((g.S + kPairRows - 1) / kPairRows - g.pos_begin / kPairRows) * g.Hq * g.B);
+        uint32_t* next_pair_tile = (uint32_t*)(ws + h->fw_status_off + kNextPairTileOffset);
+        // a cluster of two CTAs per pair of SMs, persistent
+        const int attn_grid = 2 * ((int)grid.x < h->sm_count / 2 ? (int)grid.x : h->sm_count / 2);
         const uint32_t* slot_valid_c = (const uint32_t*)(ws + h->fw_valid_off);
         // query-gather path for pairs of query tiles with sparse selections (off for p >= 1: nothing is skipped)
         const bool all_sel = g.top_k <= 0 && !(g.top_p < 1.0);
@@ -624,19 +637,20 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             if (!launch_ok(h, "gather_items_kernel")) return ADASPARK_ERR_CUDA;
         }
         const uint32_t* pair_mode_c = gather ? gw.pair_mode : nullptr;
-        const uint32_t* key_norm2_c = frame_begin == 0 ? (const uint32_t*)(ws + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
+        const uint32_t* key_norm2_c = (const uint32_t*)(ws + h->fw_headmax_off) + g.B * g.Hkv;
+        const uint32_t* value_max_c = key_norm2_c + 2 * g.B * g.Hkv;
         mark(h, 5, st);
         if (D == 128) {
             size_t smem = sizeof(TcAttnSmem<128>) + 1024;
             if (!set_smem(h, attn_prefill_tc_kernel<128>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
-            launch_kernel(true, attn_prefill_tc_kernel<128>, dim3(grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
-                                                                        gw.n_pairs_cap, gw.ml_local, key_norm2_c, (__nv_bfloat16*)out,
+            launch_kernel(true, attn_prefill_tc_kernel<128>, dim3(attn_grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
+                                                                        gw.n_pairs_cap, gw.ml_local, key_norm2_c, value_max_c, (__nv_bfloat16*)out, next_pair_tile,
                                                                         (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);
         } else {
             size_t smem = sizeof(TcAttnSmem<64>) + 1024;
             if (!set_smem(h, attn_prefill_tc_kernel<64>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
-            launch_kernel(true, attn_prefill_tc_kernel<64>, dim3(grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
-                                                                       gw.n_pairs_cap, gw.ml_local, key_norm2_c, (__nv_bfloat16*)out,
+            launch_kernel(true, attn_prefill_tc_kernel<64>, dim3(attn_grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
+                                                                       gw.n_pairs_cap, gw.ml_local, key_norm2_c, value_max_c, (__nv_bfloat16*)out, next_pair_tile,
                                                                        (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);
         }
         if (!launch_ok(h, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
@@ -644,14 +658,15 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         if (gather) {
             launch_kernel(true, gather_fill_kernel, dim3(grid), dim3(256), 0, st, g, gw, tile_mask);
             if (!launch_ok(h, "gather_fill_kernel")) return ADASPARK_ERR_CUDA;
-            CUtensorMap tmKg;      // one key block per load: box of 64 d x 64 keys (tmK's) serves as it is
-            tmKg = tmK;
+            CUtensorMap tmVg;      // whole V^T blocks (K's box, one block, serves as it is)
+            if (!encode_bf16_2d(&tmVg, vc, (uint64_t)g.B * g.Hkv * g.n_kv_blocks_cap * D, 64, 64, D))
+                return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
             const int ggrid = h->sm_count;                      // persistent: one CTA per SM
             const long long n_rows = (long long)g.B * g.Hq * (g.S - g.pos_begin);    // at most: the rows of all pairs
             if (D == 128) {
                 const size_t smem = sizeof(GatherSmem<128>) + 1024;
                 if (!set_smem(h, attn_gather_kernel<128>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                launch_kernel(true, attn_gather_kernel<128>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmKg, tmV, qb, slot_valid_c,
+                launch_kernel(true, attn_gather_kernel<128>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmK, tmVg, qb, slot_valid_c,
                                                                             (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
                 if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
                 const long long ctas = (n_rows + 15) / 16;
@@ -659,7 +674,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             } else {
                 const size_t smem = sizeof(GatherSmem<64>) + 1024;
                 if (!set_smem(h, attn_gather_kernel<64>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                launch_kernel(true, attn_gather_kernel<64>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmKg, tmV, qb, slot_valid_c,
+                launch_kernel(true, attn_gather_kernel<64>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmK, tmVg, qb, slot_valid_c,
                                                                            (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
                 if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
                 const long long ctas = (n_rows + 31) / 32;

@@ -1,0 +1,58 @@
+"""The prefill attention kernel where its forms meet: softmax references fixed in advance (near and far) and running, in one
+call and in chunks, and block lists of more blocks than are kept twice; against the CPU oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2604_08077_b200 import inputs
+
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+
+def scaled(wl, scale_q, scale_v):
+    times = lambda t, s: (t.float() * s).to(torch.bfloat16)  # noqa: E731
+    return dataclasses.replace(wl, q=times(wl.q, scale_q)), times(wl.v, scale_v)
+
+
+# The bound of a row's scores is 27 to 42 (log2 units) at scale 1: below 88 at 2, on both sides of it at 2.4, above at 4; values
+# of 2^40 move the limit to 77, values of 2^110 out of reach.
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("scale_q", [2.0, 2.4, 4.0])
+@pytest.mark.parametrize("scale_v", [1.0, 2.0 ** 40, 2.0 ** 110])
+def test_softmax_references(D, scale_q, scale_v):
+    """Every row, in one call and in three chunks (whose later calls take the norms of earlier keys from the caches).  The output is
+    linear in V and the scales are powers of two: it is compared at scale 1."""
+    base = inputs.small_prefill(seed=51, T=24, H=8, W=8, n_text=29, D=D)
+    wl, v = scaled(base, scale_q, scale_v)
+    eng = pu.make_engine(wl)
+    q, k, v = wl.q.cuda(), wl.k.cuda(), v.cuda()
+    out, bitmap, count = eng.forward(q, k, v, wl.n_text, want_selection=True)
+    torch.cuda.synchronize()
+    assert eng.header().status == 0
+    pu.compare_rows(wl, oracle.all_rows(oracle.shape_of(wl)), out.float() / scale_v, bitmap, count, label=f"{scale_q} {scale_v}")
+    outs = []
+    for fb, fc, nt in [(0, 8, -1), (8, 12, -1), (20, 4, wl.n_text)]:
+        lo, hi = fb * 64, (fb + fc) * 64 + max(nt, 0)
+        outs.append(eng.forward_chunk(q[:, lo:hi].contiguous(), k[:, lo:hi].contiguous(), v[:, lo:hi].contiguous(), fb, fc, nt)[0])
+        torch.cuda.synchronize()
+        assert eng.header().status == 0
+    pu.compare_rows(wl, oracle.all_rows(oracle.shape_of(wl)), torch.cat(outs, 1).float() / scale_v, bitmap, count,
+                    label=f"chunks {scale_q} {scale_v}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_long_block_list(D):
+    """163840 tokens are 2560 key blocks (2304 fit a list that is kept twice): sampled rows of the union path, the last tiles whole."""
+    wl = inputs.make_prefill("long", seed=52, B=1, T=640, H=16, W=16, cube=(4, 16, 16), n_text=37, Hq=1, Hkv=1, D=D, top_p=0.9,
+                             offset_std=0.5)
+    eng, out, bitmap, count = pu.run_forward(wl, gather=0.0)
+    assert eng.header().status == 0
+    assert eng.header().max_tile_kv_blocks > 2304
+    n_tiles = (wl.S + 127) // 128
+    rows = pu.sample_rows(wl, 60, seed=3, whole_tiles=[(0, 0, n_tiles - 1)])
+    pu.compare_rows(wl, rows, out, bitmap, count, label="long list")
