@@ -483,6 +483,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
         bool ok = true;
         int g0 = 0;                                               // steps of the pair tiles before this one
         uint32_t s_ph = 0;                                        // phase of the warpgroup's score tile
+        // The rows of an epilogue leave shared memory while this warpgroup goes on; it says so after the steps of its next pair tile
+        // (waiting for it at once held the next step up: 128 copies of a row each; ragged grid 743 -> 737 us).
+        bool out_pending = false;
+        auto release_out = [&]() {
+            if (out_pending) {
+                asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&sm.out_free);
+                out_pending = false;
+            }
+        };
         for (int k = 0;; ++k) {
             const int slot = plan_slot(k);
             if (!(ok = tc::mbar_wait(&sm.plan_full[slot], plan_phase(k), abort_flag))) break;
@@ -718,6 +729,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&sm.plan_empty[slot]);
             // ---- the sums of the three warpgroups meet in the one that took the last step; the others go on to the next pair tile
+            release_out();
             const int ps = k & 1, p_ph = (k >> 1) & 1;
             if (!last_wg) {
                 if (!(ok = tc::mbar_wait(&sm.part_free[ps], p_ph ^ 1, abort_flag))) break;
@@ -773,12 +785,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(smem_u32(srow)), "n"(2 * D) : "memory");
                 }
                 asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-                asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");   // the row has left shared memory
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&sm.out_free);
+                out_pending = true;
             }
             g0 += n_steps;
         }
+        release_out();
     }
     // ---------------------------------------------------------------- teardown
     __syncwarp();

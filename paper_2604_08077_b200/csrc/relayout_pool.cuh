@@ -36,6 +36,19 @@ __device__ __forceinline__ uint32_t abs_max_bf16x2(uint32_t m, const uint4& x) {
 // ... of both halves as float bits
 __device__ __forceinline__ uint32_t larger_half_bits(uint32_t m) { return max(m & 0xffff0000u, m << 16); }
 
+// Largest |k|^2 and |v| of a CTA of 256 threads joined with the head's: one atomic each (one per warp, all of them to a few
+// addresses, cost the re-layout of 16384 tokens 8 of 32 us).  Holds a barrier.
+__device__ __forceinline__ void block_norms(float k2, uint32_t v_max, uint32_t (&part)[2][8], uint32_t* key_norm2_bits, uint32_t* value_max_bits) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(k2)), v = __reduce_max_sync(0xffffffffu, larger_half_bits(v_max));
+    if (lane == 0) { part[0][warp] = m; part[1][warp] = v; }
+    __syncthreads();
+    if (warp == 0 && lane < 16) {
+        const uint32_t x = __reduce_max_sync(lane < 8 ? 0xffu : 0xff00u, part[lane >> 3][lane & 7]);
+        if ((lane & 7) == 0 && x) atomicMax(lane == 0 ? key_norm2_bits : value_max_bits, x);
+    }
+}
+
 // Largest |k|^2 and |v| of the cache rows [0, n_rows) that earlier calls wrote (n_rows: a multiple of 64; V^T blocks hold
 // the same rows).  Reads them once: 84 MB for 40960 rows of 4 heads.  grid (CTAs, Hkv, B), 256 threads.
 template <int D>
@@ -44,6 +57,7 @@ __global__ void __launch_bounds__(256) seen_norms_kernel(Geom g, int n_rows, con
     launch_dependents();
     wait_for_previous_kernel();
     constexpr int kChunks = D / 8;                                // 16-byte chunks per row, neighbouring lanes
+    __shared__ uint32_t part[2][8];
     const int bh = blockIdx.z * g.Hkv + blockIdx.y;
     const uint4* k = reinterpret_cast<const uint4*>(k_cube + (size_t)bh * g.S_cap * D);
     const uint4* v = reinterpret_cast<const uint4*>(v_cube + (size_t)bh * g.S_cap * D);
@@ -65,10 +79,7 @@ __global__ void __launch_bounds__(256) seen_norms_kernel(Geom g, int n_rows, con
         for (int o = kChunks / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         row_max = fmaxf(row_max, n2);
     }
-    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(row_max));
-    v_max = __reduce_max_sync(0xffffffffu, larger_half_bits(v_max));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(key_norm2_bits + bh, m);
-    if ((threadIdx.x & 31) == 0 && v_max) atomicMax(value_max_bits + bh, v_max);
+    block_norms(row_max, v_max, part, key_norm2_bits + bh, value_max_bits + bh);
 }
 
 template <int D>
@@ -90,6 +101,7 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
     const int tid = threadIdx.x;
     float row_max = 0.f;
     uint32_t v_max = 0u;
+    __shared__ uint32_t part[2][8];
 
     for (int idx = tid; idx < kBlockTok * kChunks; idx += 256) {
         int row = idx / kChunks, c = idx - row * kChunks;
@@ -120,13 +132,8 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
         uint32_t* vdst = reinterpret_cast<uint32_t*>(&Vs[row][c * 8]);
         vdst[0] = vv4.x; vdst[1] = vv4.y; vdst[2] = vv4.z; vdst[3] = vv4.w;
     }
-    if (key_norm2_bits != nullptr) {
-        const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(row_max));
-        v_max = __reduce_max_sync(0xffffffffu, larger_half_bits(v_max));
-        if ((tid & 31) == 0 && m) atomicMax(key_norm2_bits + b * g.Hkv + gk, m);
-        if ((tid & 31) == 0 && v_max) atomicMax(value_max_bits + b * g.Hkv + gk, v_max);
-    }
-    __syncthreads();
+    if (key_norm2_bits != nullptr) block_norms(row_max, v_max, part, key_norm2_bits + b * g.Hkv + gk, value_max_bits + b * g.Hkv + gk);
+    else __syncthreads();
 
     // Which of the block's 64 slots hold a token (two words per block; read by the attention kernels of a
     // ragged grid, whose boundary cubes have empty slots)
