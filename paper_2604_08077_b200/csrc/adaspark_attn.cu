@@ -34,7 +34,7 @@ struct adaspark_attn {
     adaspark_attn_layout_t layout;
     // workspace carving (byte offsets)
     size_t fw_status_off, fw_headmax_off, fw_valid_off, fw_gcol_off, fw_mask_off, fw_union_off, fw_fallback_off,
-        fw_kplanes_off, fw_keyhash_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
+        fw_kplanes_off, fw_keyhash_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gref_off, fw_glocal_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
         fw_gpartml_off, fw_min, fw_total;      // fw_min: the smallest workspace a forward takes, fw_total: the one it is best given
     int score_items;            // query tiles per launch of the score / selection pair, at most
     // query-gather path of the prefill: capacity in (row, key block) entries, decision threshold, byte budget
@@ -199,10 +199,11 @@ int select_shape(int n) { return n <= 64 ? 0 : n <= 128 ? 1 : n <= 256 ? 2 : n <
 // estimate forces the path and is not judged.)
 bool gather_can_pay(const Geom& g, float pairs_per_block) {
     if (pairs_per_block > (float)kGatherBreakEven) return true;
+    const float least = gather_entry_cost(g.C) / (float)(g.C > kBlockTok ? g.C / kBlockTok : 1);    // an entry per column of the union
     long long blocks = 0;
     for (int pair = g.pos_begin / kPairRows; pair < (g.S + kPairRows - 1) / kPairRows; ++pair) {
         blocks += (long long)g.Hq * g.B * pair_first_local_blk(g, pair * kPairRows);
-        if (blocks * (kGatherBreakEven - 1) >= kGatherMinGain) return true;
+        if ((float)blocks * ((float)kGatherBreakEven - least) >= (float)kGatherMinGain) return true;
     }
     return false;
 }
@@ -279,7 +280,7 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     h->fw_status_off = off; off = align_up(off + 256);
     h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 4);   // mean-key exponents, largest |k|^2, largest |mean key|, largest |v|
     h->fw_valid_off = off; off = align_up(off + (size_t)(S_cap / kBlockTok) * 2 * 4);   // which slots of a block hold a token
-    const size_t n_cols = (size_t)(S_v + kBlockTok - 1) / kBlockTok;                     // key blocks that hold video
+    const size_t n_cols = gather_columns((size_t)S_v, (size_t)N, h->C);                  // key blocks that hold video (large cubes: cubes)
     // query-gather path: the rows are cut into windows whose slice of Q (all heads) is about a third of the L2
     {
         const size_t q_bytes = (size_t)batch * Hq * S_cap * D * 2;
@@ -311,11 +312,13 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // per row (m, l) of the local range | per key block offsets + work items | entries | partial outputs | partial (m, l)
     {
         const size_t rows_cap = (size_t)batch * Hq * S_cap, n_pairs_cap = ((size_t)S_cap + 255) / 256;
-        const uint64_t per_entry = 2ull * D + 16ull + 8ull;      // partial output + (m, l) + entry
+        const uint64_t part_bytes = (h->C > kBlockTok ? 4ull : 2ull) * D;    // partial output: fp32 of whole cubes, else bf16
+        const uint64_t per_entry = part_bytes + 16ull + 8ull;    // + (m, l) + entry
         uint64_t cap = h->gather_budget / per_entry;
         // a pair qualifies with at most threshold x (blocks of its union) entries for its 256 rows, and over a causal
         // sequence a pair's union averages half the video's key blocks: threshold x n_cols / 512 entries per row
-        double per_row = std::ceil((double)h->gather_pairs_per_block * (double)n_cols / 512.0);
+        const double n_blocks = (double)((S_v + kBlockTok - 1) / kBlockTok);
+        double per_row = std::ceil((double)h->gather_pairs_per_block * n_blocks / 512.0 / (double)gather_entry_cost(h->C));
         if (!(per_row < (double)kGatherEntriesPerRow)) per_row = (double)kGatherEntriesPerRow;
         if ((double)cap > (double)rows_cap * per_row) cap = (uint64_t)((double)rows_cap * per_row);
         if (cap > 0xfffffff0ull) cap = 0xfffffff0ull;
@@ -323,9 +326,11 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
         h->fw_gpair_off = off; off = align_up(off + (size_t)batch * Hq * n_pairs_cap * 5 * 4);
         h->fw_grow_off = off; off = align_up(off + (cap ? rows_cap * 2 * 4 : 0));
         h->fw_gml_off = off; off = align_up(off + (cap ? rows_cap * 8 : 0));
+        h->fw_glocal_off = off; off = align_up(off + (cap && h->C > kBlockTok ? rows_cap * D * 4 : 0));
+        h->fw_gref_off = off; off = align_up(off + (cap && h->C > kBlockTok ? rows_cap * 4 : 0));
         h->fw_gitems_off = off; off = align_up(off + (cap ? align_up((n_lists * n_cols * (kGatherClasses + 2) + 2) * 4) + (n_lists * n_cols + cap / 128 + 1) * 16 : 0));
         h->fw_gentries_off = off; off = align_up(off + (size_t)cap * 8);
-        h->fw_gparto_off = off; off = align_up(off + (size_t)cap * D * 2);
+        h->fw_gparto_off = off; off = align_up(off + (size_t)cap * part_bytes);
         h->fw_gpartml_off = off; off = align_up(off + (size_t)cap * 8);
     }
     h->fw_min = off > scores_end_min ? off : scores_end_min;
@@ -438,7 +443,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         if (!launch_ok(h, "relayout_pool_kernel")) return ADASPARK_ERR_CUDA;
         if (!cache_only && g.pos_begin > 0 && h->prefill_kernel != 0) {     // the keys and values of earlier calls
             const int ctas = g.pos_begin * (D / 8) / 1024;              // four 16-byte pieces of K and V a thread, at least
-            const dim3 ngrid(ctas < 1024 ? (ctas < 1 ? 1 : ctas) : 1024, g.Hkv, g.B);
+            const dim3 ngrid(ctas < 256 ? (ctas < 1 ? 1 : ctas) : 256, g.Hkv, g.B);
             if (D == 128) launch_kernel(true, seen_norms_kernel<128>, ngrid, dim3(256), 0, st, g, g.pos_begin, (const __nv_bfloat16*)kc, (const __nv_bfloat16*)vc, key_norm2, value_max);
             else launch_kernel(true, seen_norms_kernel<64>, ngrid, dim3(256), 0, st, g, g.pos_begin, (const __nv_bfloat16*)kc, (const __nv_bfloat16*)vc, key_norm2, value_max);
             if (!launch_ok(h, "seen_norms_kernel")) return ADASPARK_ERR_CUDA;
@@ -597,7 +602,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         GatherWs gw;
         std::memset(&gw, 0, sizeof(gw));
         if (gather) {
-            const size_t n_cols = (size_t)(g.S_v + kBlockTok - 1) / kBlockTok;
+            const size_t n_cols = gather_columns((size_t)g.S_v, (size_t)g.N, g.C);
             const size_t n_lists = (size_t)h->gather_windows * g.B * g.Hkv, n_col_all = n_lists * n_cols;
             const int n_pairs_win = (g.S + kPairRows - 1) / kPairRows - g.pos_begin / kPairRows;
             const size_t rows_cap = (size_t)g.B * g.Hq * g.S_cap, n_pairs_cap = ((size_t)g.S_cap + 255) / 256;
@@ -618,9 +623,10 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             gw.items = (uint4*)(ws + h->fw_gitems_off + align_up((n_col_all * (kGatherClasses + 2) + 2) * 4));
             gw.entries = (uint32_t*)(ws + h->fw_gentries_off);
             gw.row_slots = gw.entries + h->gather_cap;
-            gw.part_o = (__nv_bfloat16*)(ws + h->fw_gparto_off);
+            gw.part_o = ws + h->fw_gparto_off;
             gw.part_ml = (float2*)(ws + h->fw_gpartml_off);
             gw.ml_local = (float2*)(ws + h->fw_gml_off);
+            gw.local_o = (float*)(ws + h->fw_glocal_off);
             gw.cap_entries = h->gather_cap;
             gw.n_cols = (int)n_cols;
             gw.n_lists = (int)n_lists;
@@ -628,6 +634,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             gw.pairs_per_window = (n_pairs_win + h->gather_windows - 1) / h->gather_windows;
             gw.n_pairs_cap = (int)n_pairs_cap;
             gw.pairs_per_block = h->gather_pairs_per_block;
+            gw.entry_cost = gather_entry_cost(g.C);
+            gw.item_rows = gather_item_rows(g.C);
             launch_kernel(true, gather_count_kernel, dim3(grid), dim3(256), 0, st, g, gw, tile_mask, tile_union);
             if (!launch_ok(h, "gather_count_kernel")) return ADASPARK_ERR_CUDA;
             launch_kernel(true, gather_scan_kernel, dim3(1), dim3(1024), 0, st, g, gw);
@@ -637,51 +645,78 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             if (!launch_ok(h, "gather_items_kernel")) return ADASPARK_ERR_CUDA;
         }
         const uint32_t* pair_mode_c = gather ? gw.pair_mode : nullptr;
+        GatherTiles local_tiles;                   // of pairs whose cubes are gathered whole the local range stays in fp32 for the merge
+        std::memset(&local_tiles, 0, sizeof(local_tiles));
+        if (gather && g.C > kBlockTok) local_tiles.part_o = gw.local_o;
+        float* row_ref = gather && g.C > kBlockTok ? (float*)(ws + h->fw_gref_off) : nullptr;   // softmax references of the rows of gathered pairs
         const uint32_t* key_norm2_c = (const uint32_t*)(ws + h->fw_headmax_off) + g.B * g.Hkv;
         const uint32_t* value_max_c = key_norm2_c + 2 * g.B * g.Hkv;
         mark(h, 5, st);
-        if (D == 128) {
-            size_t smem = sizeof(TcAttnSmem<128>) + 1024;
-            if (!set_smem(h, attn_prefill_tc_kernel<128>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
-            launch_kernel(true, attn_prefill_tc_kernel<128>, dim3(attn_grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
-                                                                        gw.n_pairs_cap, gw.ml_local, key_norm2_c, value_max_c, (__nv_bfloat16*)out, next_pair_tile,
-                                                                        (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);
+#define ADASPARK_LAUNCH_ATTN(DD)                                                                                              \
+    do {                                                                                                                    \
+        const size_t smem = sizeof(TcAttnSmem<DD>) + 1024;                                                                  \
+        if (!set_smem(h, attn_prefill_tc_kernel<DD>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;              \
+        launch_kernel(true, attn_prefill_tc_kernel<DD>, dim3(attn_grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV,   \
+                      tile_mask, tile_union, slot_valid_c, pair_mode_c, gw.n_pairs_cap, gw.ml_local, key_norm2_c, value_max_c, \
+                      (__nv_bfloat16*)out, next_pair_tile, (unsigned long long*)&hdr->executed_kv_blocks,                    \
+                      &hdr->max_tile_kv_blocks, &hdr->status);                                                              \
+    } while (0)
+#define ADASPARK_LAUNCH_CUBES(DD, GATHERED, GRID, TILES, COUNTER)                                                             \
+    do {                                                                                                                    \
+        const size_t smem = sizeof(CubesSmem<DD, GATHERED>) + 1024;                                                          \
+        if (!set_smem(h, attn_cubes_tc_kernel<DD, GATHERED>, smem, "attn_cubes_tc_kernel")) return ADASPARK_ERR_CUDA;        \
+        launch_kernel(true, attn_cubes_tc_kernel<DD, GATHERED>, dim3(GRID), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, \
+                      tile_mask, tile_union, slot_valid_c, pair_mode_c, gw.n_pairs_cap, gw.ml_local, TILES, row_ref,         \
+                      key_norm2_c, value_max_c, (__nv_bfloat16*)out, COUNTER,                                               \
+                      (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);                \
+    } while (0)
+        if (gather && g.C > kBlockTok) {
+            if (D == 128) ADASPARK_LAUNCH_CUBES(128, false, attn_grid, local_tiles, next_pair_tile);
+            else ADASPARK_LAUNCH_CUBES(64, false, attn_grid, local_tiles, next_pair_tile);
         } else {
-            size_t smem = sizeof(TcAttnSmem<64>) + 1024;
-            if (!set_smem(h, attn_prefill_tc_kernel<64>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
-            launch_kernel(true, attn_prefill_tc_kernel<64>, dim3(attn_grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, tile_mask, tile_union, slot_valid_c, pair_mode_c,
-                                                                       gw.n_pairs_cap, gw.ml_local, key_norm2_c, value_max_c, (__nv_bfloat16*)out, next_pair_tile,
-                                                                       (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);
+            if (D == 128) ADASPARK_LAUNCH_ATTN(128); else ADASPARK_LAUNCH_ATTN(64);
         }
         if (!launch_ok(h, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;
         mark(h, 6, st);
         if (gather) {
             launch_kernel(true, gather_fill_kernel, dim3(grid), dim3(256), 0, st, g, gw, tile_mask);
             if (!launch_ok(h, "gather_fill_kernel")) return ADASPARK_ERR_CUDA;
-            CUtensorMap tmVg;      // whole V^T blocks (K's box, one block, serves as it is)
-            if (!encode_bf16_2d(&tmVg, vc, (uint64_t)g.B * g.Hkv * g.n_kv_blocks_cap * D, 64, 64, D))
-                return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
-            const int ggrid = h->sm_count;                      // persistent: one CTA per SM
             const long long n_rows = (long long)g.B * g.Hq * (g.S - g.pos_begin);    // at most: the rows of all pairs
-            if (D == 128) {
-                const size_t smem = sizeof(GatherSmem<128>) + 1024;
-                if (!set_smem(h, attn_gather_kernel<128>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                launch_kernel(true, attn_gather_kernel<128>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmK, tmVg, qb, slot_valid_c,
-                                                                            (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
-                if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                const long long ctas = (n_rows + 15) / 16;
-                launch_kernel(false, gather_merge_kernel<128>, dim3((unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count)), dim3(256), 0, st, g, gw, (__nv_bfloat16*)out);
+            if (g.C > kBlockTok) {
+                GatherTiles gt;
+                gt.items = gw.items; gt.ctrl = gw.ctrl; gt.entries = gw.entries; gt.part_o = (float*)gw.part_o; gt.part_ml = gw.part_ml; gt.n_cols = gw.n_cols;
+                const int ggrid = 2 * (h->sm_count / 2);
+                if (D == 128) ADASPARK_LAUNCH_CUBES(128, true, ggrid, gt, next_pair_tile + 1);
+                else ADASPARK_LAUNCH_CUBES(64, true, ggrid, gt, next_pair_tile + 1);
+                if (!launch_ok(h, "attn_cubes_tc_kernel")) return ADASPARK_ERR_CUDA;
             } else {
-                const size_t smem = sizeof(GatherSmem<64>) + 1024;
-                if (!set_smem(h, attn_gather_kernel<64>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                launch_kernel(true, attn_gather_kernel<64>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmK, tmVg, qb, slot_valid_c,
-                                                                           (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
-                if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
-                const long long ctas = (n_rows + 31) / 32;
-                launch_kernel(false, gather_merge_kernel<64>, dim3((unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count)), dim3(256), 0, st, g, gw, (__nv_bfloat16*)out);
+                CUtensorMap tmVg;      // whole V^T blocks (K's box, one block, serves as it is)
+                if (!encode_bf16_2d(&tmVg, vc, (uint64_t)g.B * g.Hkv * g.n_kv_blocks_cap * D, 64, 64, D))
+                    return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
+                const int ggrid = h->sm_count;                      // persistent: one CTA per SM
+                if (D == 128) {
+                    const size_t smem = sizeof(GatherSmem<128>) + 1024;
+                    if (!set_smem(h, attn_gather_kernel<128>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
+                    launch_kernel(true, attn_gather_kernel<128>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmK, tmVg, qb, slot_valid_c,
+                                                                                (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
+                    if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
+                } else {
+                    const size_t smem = sizeof(GatherSmem<64>) + 1024;
+                    if (!set_smem(h, attn_gather_kernel<64>, smem, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
+                    launch_kernel(true, attn_gather_kernel<64>, dim3(ggrid), dim3(kGatherThreads), smem, st, g, gw, tmK, tmVg, qb, slot_valid_c,
+                                                                               (unsigned long long*)&hdr->executed_kv_blocks, &hdr->status);
+                    if (!launch_ok(h, "attn_gather_kernel")) return ADASPARK_ERR_CUDA;
+                }
             }
+            const long long ctas = (n_rows + 2048 / D - 1) / (2048 / D);      // rows of a CTA: 2048 / D
+            const dim3 mgrid((unsigned)(ctas < 8ll * h->sm_count ? ctas : 8ll * h->sm_count));
+            auto* merge = D == 128 ? (g.C > kBlockTok ? gather_merge_kernel<128, true> : gather_merge_kernel<128, false>)
+                                   : (g.C > kBlockTok ? gather_merge_kernel<64, true> : gather_merge_kernel<64, false>);
+            launch_kernel(false, merge, mgrid, dim3(256), 0, st, g, gw, (__nv_bfloat16*)out);
             if (!launch_ok(h, "gather_merge_kernel")) return ADASPARK_ERR_CUDA;
         }
+#undef ADASPARK_LAUNCH_ATTN
+#undef ADASPARK_LAUNCH_CUBES
     } else
 #endif
     {

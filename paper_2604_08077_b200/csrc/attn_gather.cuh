@@ -22,16 +22,17 @@
 //   gather_count_kernel   per pair: row counts, P, U, the decision, entries per key block list (the warp's
 //                         32 x 32 mask bits are transposed so that lane j holds the rows that selected cube j)
 //   gather_scan_kernel    one CTA: which pairs are kept, prefix sums over pairs and key block lists
-//   gather_items_kernel   work items of up to 128 entries of one list
+//   gather_items_kernel   work items of up to 128 (cubes above 64 tokens: 256) entries of one list
 //   (attn_prefill_tc_kernel, which reads the decisions)
 //   gather_fill_kernel    per pair: row -> its slots, entries into the lists of their key blocks
-//   attn_gather_kernel    per item: gathered Q rows x one key block -> partial results, in entry order
+//   attn_gather_kernel    per item: gathered Q rows x one key block -> partial results, in entry order (cubes above 64
+//                         tokens: attn_cubes_tc_kernel<D, true>, gathered Q rows x the key blocks of one cube)
 //   gather_merge_kernel   per row of the gathered pairs: merge into `out`
 // The order of a list's entries depends on the order of atomics, but an entry's arithmetic does not depend
 // on its neighbours in the item, and a row merges its partials in ascending block order: results are
 // deterministic.
 #pragma once
-#include "attn_prefill_tc.cuh"
+#include "attn_cubes_tc.cuh"
 
 namespace adaspark {
 
@@ -50,11 +51,21 @@ constexpr int kGatherClasses = 4;       // a qualifying pair falls into a class 
 // launches, the scan) eat the gain.
 constexpr long long kGatherBreakEven = 44;
 constexpr long long kGatherMinGain = 300000;
-constexpr uint32_t kEntryPosMask = 0x1fffffu;   // 21 bits of token index (a sequence holds at most 2^21 rows)
+// Cubes of 128 tokens and more are gathered whole: an entry is a (row, cube) pair, an item holds up to 256 rows and
+// attn_cubes_tc_kernel<D, true> takes it, one partial result for all key blocks of the cube, in fp32 like the local
+// range's.  An entry of a 256-token cube costs 0.35 ns (its Q row, 4 D bytes written and read, the steps between items; not the
+// tensor core) where its four key blocks cost 0.62.  Cost of an entry for the decision, in entries of one 64-key block; with the
+// default threshold up to 15 entries per union block (16 of 128-token cubes, 14 of 512) are gathered, break-even lies at 14 to
+// 18.  16 heads, 24576 tokens, union path / gathered: 256-token cubes, p 0.7 1.97 / 1.76 ms, p 0.5 1.98 / 1.18, 512, p 0.7
+// 1.97 / 1.46, 128, p 0.7 2.10 / 3.10 (stays on the union path); 28 heads, 65536 tokens, 256, p 0.7 25.5 / 17.3.
+inline float gather_entry_cost(int cube_tokens) { return cube_tokens <= kBlockTok ? 1.f : 1.7f + 0.06f * (float)(cube_tokens / kBlockTok); }
+__host__ __device__ constexpr int gather_item_rows(int cube_tokens) { return cube_tokens > kBlockTok ? 256 : kGatherItemRows; }
+// key block columns (cubes above 64 tokens) that have entry lists
+inline size_t gather_columns(size_t s_video, size_t n_cubes, int cube_tokens) { return cube_tokens > kBlockTok ? n_cubes : (s_video + kBlockTok - 1) / kBlockTok; }
 
 // Pointers into the forward workspace and sizes (all filled by the host).
 struct GatherWs {
-    uint32_t* ctrl;        // [0] entries, [1] items, [2] pairs on this path (0 entries: the path is off)
+    uint32_t* ctrl;        // [0] (row, key block) pairs of the entries, [1] items, [2] pairs on this path (0 entries: the path is off)
     uint32_t* pair_mode;   // [B*Hq*n_pairs_cap] 0: union path; c + 1: this path, ratio class c
     uint32_t* pair_cnt;    // entries of the pair's rows (0 when the pair stays on the tile kernel)
     uint32_t* pair_off;    // exclusive prefix sum of pair_cnt
@@ -68,13 +79,14 @@ struct GatherWs {
     uint32_t* col_roff;    // [kGatherClasses][...] first entry of the set's share of the block's list
     uint32_t* col_off;     // [lists * n_cols + 1] first entry of the block's list (exclusive prefix sum)
     uint32_t* col_item;    // [lists * n_cols + 1] first work item of the list
-    uint4* items;          // (key block column, first entry, entries (<= 128), 0)
+    uint4* items;          // (key block column, first entry, entries (<= item_rows), 0)
     uint32_t* entries;     // per key block, its entries: row of the call's tensors | head in group << 21 | cube bits << 25
     uint32_t* row_slots;   // per row (from row_ptr on), the indices of its entries in ascending block order
-    __nv_bfloat16* part_o; // [cap_entries][D] normalised partial output of every entry (in entry order: an item
-                           // of the attention kernel writes one contiguous piece)
+    void* part_o;          // [cap_entries][D] normalised partial output of every entry, bf16, of whole cubes fp32 (in entry order:
+                           // an item of the attention kernel writes one contiguous piece)
     float2* part_ml;       // [cap_entries] (reference exponent in log2 units, sum)
     float2* ml_local;      // [B*Hq*S_cap] the same for the local range, written by the tile kernel
+    float* local_o;        // [B*Hq*S_cap][D] normalised output of the local range, of whole cubes only (else it lies in `out`)
     uint32_t cap_entries;
     int n_cols;            // key blocks that hold video slots: ceil(S_v / 64)
     int n_lists;           // entry lists per key block column set: windows x B x Hkv (each of n_cols lists)
@@ -84,6 +96,8 @@ struct GatherWs {
                            // slice of Q that stays in L2, and a row's partial results lie close together.
     int n_pairs_cap;       // pairs of query tiles per (b, head): ceil(S_cap / 256)
     float pairs_per_block; // decision threshold (entries per union block)
+    float entry_cost;      // gather_entry_cost
+    int item_rows;         // gather_item_rows
 };
 
 // bit of the first cube of every 64-key block in which `word` has a selected cube (cubes of 16 / 32 tokens;
@@ -133,15 +147,14 @@ __device__ __forceinline__ PairItem pair_item(const Geom& g, int bid) {
     return it;
 }
 
-// entries of the lane's row before the pair's local range, in key blocks
+// entries of the lane's row before the pair's local range
 __device__ __forceinline__ uint32_t row_entries(const Geom& g, const PairItem& it, const uint32_t* my) {
-    const int bshift = max(g.c_shift - 6, 0);
     uint32_t cnt = 0;
 #pragma unroll 4
     for (int w = 0; w < it.n_w; ++w) {
         uint32_t word = *(my + (size_t)w * kTileRows);
         if (w == it.n_w - 1) word &= it.last_keep;
-        cnt += (uint32_t)__popc(fold_to_blocks(word, g.c_shift)) << bshift;
+        cnt += (uint32_t)__popc(fold_to_blocks(word, g.c_shift));
     }
     return cnt;
 }
@@ -180,7 +193,8 @@ __global__ void __launch_bounds__(256) gather_count_kernel(Geom g, GatherWs ws, 
         for (int i = 0; i < 8; ++i) { P += red[0][i]; U += red[1][i]; }
         uint32_t mode = 0u;
         const float lim = ws.pairs_per_block * (float)U;
-        if (P > 0 && (float)P <= lim) mode = (float)P <= 0.125f * lim ? 1u : ((float)P <= 0.25f * lim ? 2u : ((float)P <= 0.5f * lim ? 3u : 4u));
+        const float cost = (float)P * ws.entry_cost;
+        if (P > 0 && cost <= lim) mode = cost <= 0.125f * lim ? 1u : (cost <= 0.25f * lim ? 2u : (cost <= 0.5f * lim ? 3u : 4u));
         const size_t slot = bh * ws.n_pairs_cap + it.pair;
         ws.pair_mode[slot] = mode;
         ws.pair_cnt[slot] = mode ? P : 0u;
@@ -206,11 +220,7 @@ __global__ void __launch_bounds__(256) gather_count_kernel(Geom g, GatherWs ws, 
             const uint32_t n = (uint32_t)__popc(transpose_32x32(fold_to_blocks(wd[k], g.c_shift), lane));
             if (n) {
                 const int cube = (w0 + k) * 32 + lane;
-                if (g.c_shift >= 6) {
-                    for (int i = 0; i < (1 << bshift); ++i) atomicAdd(col_cnt + ((size_t)cube << bshift) + i, n);
-                } else {
-                    atomicAdd(col_cnt + (cube >> (6 - g.c_shift)), n);
-                }
+                atomicAdd(col_cnt + (g.c_shift >= 6 ? cube : cube >> (6 - g.c_shift)), n);
             }
         }
     }
@@ -273,7 +283,7 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
             if (mode) {
                 v = ws.pair_cnt[slot];
                 unit = (int)(mode - 1) * kGatherMaxWindows + pr / ws.pairs_per_window;
-                gain = (int)(kGatherBreakEven * (long long)ws.pair_u[slot] - (long long)v);   // v <= 256 rows x 32768 blocks
+                gain = (int)(kGatherBreakEven * (long long)ws.pair_u[slot] - (long long)((float)v * ws.entry_cost));   // v <= 256 rows x 32768 blocks
             }
         }
         // one pair of 64-bit (compare-and-swap) atomics per unit and warp: a warp's pairs share a few units
@@ -337,7 +347,8 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
         return;
     }
     if (tid == 0) {
-        ws.ctrl[0] = (uint32_t)carry;
+        const unsigned long long blocks = carry * (unsigned long long)max(g.C / kBlockTok, 1);    // (row, key block) pairs
+        ws.ctrl[0] = (uint32_t)min(blocks, 0xffffffffull);
         ws.ctrl[2] = n_on;
     }
     // ---- key blocks: offsets of their entry lists (and of every counter set's share) and of their work items.
@@ -365,7 +376,7 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
         for (int r = 0; r < kGatherClasses; ++r) v += part[r];
         if (base + lane >= c1) v = 0u;
         my_e += v;
-        my_i += (v + kGatherItemRows - 1) / kGatherItemRows;
+        my_i += (v + ws.item_rows - 1) / ws.item_rows;
     }
     my_e = __reduce_add_sync(0xffffffffu, my_e);
     my_i = __reduce_add_sync(0xffffffffu, my_i);
@@ -383,7 +394,7 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
         uint32_t v = 0;
 #pragma unroll
         for (int r = 0; r < kGatherClasses; ++r) v += part[r];
-        const uint32_t n_it = (v + kGatherItemRows - 1) / kGatherItemRows;
+        const uint32_t n_it = (v + ws.item_rows - 1) / ws.item_rows;
         uint32_t ve = v, vi = n_it;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -420,8 +431,8 @@ __global__ void __launch_bounds__(256) gather_items_kernel(Geom g, GatherWs ws) 
     const int lane = threadIdx.x & 31;
     for (int col = blockIdx.x * 8 + (threadIdx.x >> 5); col < n_cols_all; col += gridDim.x * 8) {
         const uint32_t first = ws.col_off[col], n = ws.col_off[col + 1] - first, ib = ws.col_item[col];
-        for (uint32_t c = lane; c * kGatherItemRows < n; c += 32)
-            ws.items[ib + c] = make_uint4((uint32_t)col, first + c * kGatherItemRows, min(n - c * kGatherItemRows, (uint32_t)kGatherItemRows), 0u);
+        const uint32_t rows = (uint32_t)ws.item_rows;
+        for (uint32_t c = lane; c * rows < n; c += 32) ws.items[ib + c] = make_uint4((uint32_t)col, first + c * rows, min(n - c * rows, rows), 0u);
     }
 }
 
@@ -436,7 +447,6 @@ __global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, c
     const uint32_t mode = ws.pair_mode[slot];
     if (ws.ctrl[0] == 0u || mode == 0u) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bshift = max(g.c_shift - 6, 0);
     const int tile = it.pair * 2 + (warp >> 2), r = (warp & 3) * 32 + lane, pos = it.pair_pos0 + tid;
     const bool tile_ok = tile < g.n_tiles;
     // first partial of every row: prefix sum of the row counts inside the pair
@@ -466,7 +476,6 @@ __global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, c
     // return value of an atomic takes about a microsecond: one round per selected cube was the whole run time);
     // then every row walks its own cubes, fetching start and row set from the lane that owns the cube.
     const int group = g.c_shift >= 6 ? 1 : (kBlockTok >> g.c_shift);    // cubes per key block (small cubes)
-    const int nblk = 1 << bshift;                                       // key blocks per cube (large cubes)
     for (int w0 = 0; w0 < it.n_w; w0 += 4) {
         uint32_t wd[4], fw[4], tw[4];
 #pragma unroll
@@ -481,16 +490,16 @@ __global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, c
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             slot0[k] = ptr;
-            ptr += (uint32_t)(__popc(fw[k]) * nblk);
+            ptr += (uint32_t)__popc(fw[k]);
         }
-        for (int i = 0; i < nblk; ++i) {
+        {
             uint32_t st[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 st[k] = 0u;
                 if (tw[k]) {
                     const int cube = (w0 + k) * 32 + lane;
-                    const size_t col = colbase + (g.c_shift >= 6 ? ((size_t)cube << bshift) + i : (size_t)(cube >> (6 - g.c_shift)));
+                    const size_t col = colbase + (size_t)(g.c_shift >= 6 ? cube : cube >> (6 - g.c_shift));
                     st[k] = ws.col_roff[col] + atomicAdd(ws.col_cur + col, (uint32_t)__popc(tw[k]));
                 }
             }
@@ -504,7 +513,7 @@ __global__ void __launch_bounds__(256) gather_fill_kernel(Geom g, GatherWs ws, c
                     if (t) {
                         const uint32_t e = start + (uint32_t)__popc(m & lt_mask);
                         ws.entries[e] = ent_x | (((wd[k] >> beta) & ((1u << group) - 1u)) << 25);
-                        ws.row_slots[slot0[k] + (uint32_t)(j * nblk + i)] = e;
+                        ws.row_slots[slot0[k] + (uint32_t)j] = e;
                         t &= t - 1;
                     }
                 }
@@ -708,7 +717,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
             // 32 rows (contiguous in the partial buffer: entry order) as whole 128-byte lines, four rows per
             // instruction.
             unsigned char* stage = sm.out_stage[warp];
-            unsigned char* gdst = reinterpret_cast<unsigned char*>(ws.part_o + (size_t)(d_cur.y + (row & ~31)) * D);
+            unsigned char* gdst = reinterpret_cast<unsigned char*>(static_cast<__nv_bfloat16*>(ws.part_o) + (size_t)(d_cur.y + (row & ~31)) * D);
             const int n_warp_rows = min(32, (int)d_cur.z - (row & ~31));          // rows of this warp that hold an entry
 #pragma unroll
             for (int hf = 0; hf < D / 64; ++hf) {
@@ -879,7 +888,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
 // ------------------------------------------------------------------------------------------------ merge
 // D/8 threads per row, 16 bytes (8 elements) of the row each.  The partials are folded in one pass with a
 // running reference exponent (their loads do not depend on it, so several are in flight per thread).
-template <int D>
+template <int D, bool kWholeCubes>
 __global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, __nv_bfloat16* out) {
     launch_dependents();
     wait_for_previous_kernel();
@@ -897,14 +906,25 @@ __global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, 
         const uint32_t cnt = *(ws.row_cnt + row);              // 0: a pair on the union path, or a slot without token
         const uint32_t ptr = *(ws.row_ptr + row);
         const float2 loc = *(ws.ml_local + row);
-        if (cnt == 0u) continue;
+        if (kWholeCubes ? !slot_live(g, pos) : cnt == 0u) continue;    // (whole cubes: the local range is not in `out` yet)
         const int b = bh / g.Hq, h = bh - b * g.Hq;
         uint4* dst = reinterpret_cast<uint4*>(out + (io_row(g, b, pos) * g.Hq + h) * D) + sub;
-        const uint4 own = *dst;
-        const uint4* src = reinterpret_cast<const uint4*>(ws.part_o) + sub;
+        const uint4 own = kWholeCubes ? make_uint4(0u, 0u, 0u, 0u) : *dst;
+        constexpr int kPieces = kWholeCubes ? 2 : 1;               // 16-byte pieces of a partial row per thread: 8 fp32 or bf16
+        const uint4* src = reinterpret_cast<const uint4*>(ws.part_o) + kPieces * sub;
         float acc[8];
         float M = loc.x, W = loc.y;                                // the local range always has a visible key
-        {
+        if constexpr (kWholeCubes) {
+            const float4* lo = reinterpret_cast<const float4*>(ws.local_o + row * D) + 2 * sub;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float4 x = __ldcs(lo + k);
+                acc[4 * k] = W * x.x;
+                acc[4 * k + 1] = W * x.y;
+                acc[4 * k + 2] = W * x.z;
+                acc[4 * k + 3] = W * x.w;
+            }
+        } else {
             const uint32_t u[4] = {own.x, own.y, own.z, own.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -916,31 +936,46 @@ __global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, 
             // four partials at a time: indices, then (m, l) and data of all four, then the arithmetic
             uint32_t e[4];
             float2 ml[4];
-            uint4 v[4];
+            uint4 v[4][kPieces];
 #pragma unroll
             for (int k = 0; k < 4; ++k) e[k] = i0 + k < cnt ? *(ws.row_slots + ptr + i0 + k) : 0xffffffffu;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 ml[k] = make_float2(0.f, 0.f);
-                v[k] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int p = 0; p < kPieces; ++p) v[k][p] = make_uint4(0u, 0u, 0u, 0u);
                 if (e[k] != 0xffffffffu) {
                     ml[k] = __ldcs(ws.part_ml + e[k]);
-                    v[k] = __ldcs(src + (size_t)e[k] * kLanes);
+#pragma unroll
+                    for (int p = 0; p < kPieces; ++p) v[k][p] = __ldcs(src + (size_t)e[k] * (kLanes * kPieces) + p);
                 }
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if (ml[k].y > 0.f) {                               // a partial without a visible key has sum 0
-                    const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+                    float x[8];
+                    if constexpr (kWholeCubes) {
+#pragma unroll
+                        for (int p = 0; p < 2; ++p) {
+                            x[4 * p] = __uint_as_float(v[k][p].x);
+                            x[4 * p + 1] = __uint_as_float(v[k][p].y);
+                            x[4 * p + 2] = __uint_as_float(v[k][p].z);
+                            x[4 * p + 3] = __uint_as_float(v[k][p].w);
+                        }
+                    } else {
+                        const uint32_t u[4] = {v[k][0].x, v[k][0].y, v[k][0].z, v[k][0].w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            x[2 * q] = __uint_as_float(u[q] << 16);
+                            x[2 * q + 1] = __uint_as_float(u[q] & 0xffff0000u);
+                        }
+                    }
                     const float Mn = fmaxf(M, ml[k].x);
                     const float so = exp2f(M - Mn), w = ml[k].y * exp2f(ml[k].x - Mn);
                     M = Mn;
                     W = fmaf(W, so, w);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        acc[2 * q] = fmaf(w, __uint_as_float(u[q] << 16), acc[2 * q] * so);
-                        acc[2 * q + 1] = fmaf(w, __uint_as_float(u[q] & 0xffff0000u), acc[2 * q + 1] * so);
-                    }
+                    for (int q = 0; q < 8; ++q) acc[q] = fmaf(w, x[q], acc[q] * so);
                 }
             }
         }

@@ -1,5 +1,6 @@
 """The prefill attention kernel where its forms meet: softmax references fixed in advance (near and far) and running, in one
-call and in chunks, and block lists of more blocks than are kept twice; against the CPU oracle."""
+call and in chunks, block lists of more blocks than are kept twice, and whole cubes of more than 64 tokens gathered; against the
+CPU oracle."""
 import dataclasses
 
 import numpy as np
@@ -56,3 +57,35 @@ def test_long_block_list(D):
     n_tiles = (wl.S + 127) // 128
     rows = pu.sample_rows(wl, 60, seed=3, whole_tiles=[(0, 0, n_tiles - 1)])
     pu.compare_rows(wl, rows, out, bitmap, count, label="long list")
+
+
+# 128, 256 and 512 tokens, whole and at the ragged faces of a grid, lists of a few rows and of many; Top-K of one cube
+@pytest.mark.parametrize("cube, T, H, W, D, top_k", [((2, 8, 8), 16, 8, 8, 128, 0), ((4, 8, 8), 16, 16, 8, 64, 0), ((8, 8, 8), 32, 8, 16, 128, 1),
+                                                     ((2, 8, 8), 9, 14, 11, 128, 0), ((4, 8, 8), 10, 12, 12, 64, 2)])
+def test_gathered_cubes(cube, T, H, W, D, top_k):
+    wl = inputs.small_prefill(seed=53, T=T, H=H, W=W, cube=cube, n_text=21, Hq=6, Hkv=2, D=D, top_p=0.8, offset_std=1.5)
+    wl.top_k = top_k
+    eng, out, bitmap, count = pu.run_forward(wl, prefill_kernel=1, gather=pu.FORCE_GATHER)
+    hdr = eng.header()
+    assert hdr.status == 0 and hdr.gather_entries > 0
+    rep = pu.compare_rows(wl, oracle.all_rows(oracle.shape_of(wl)), out, bitmap, count, label=str(cube))
+    assert rep["rows"] == wl.B * wl.Hq * wl.S
+    again = eng.forward(wl.q.cuda(), wl.k.cuda(), wl.v.cuda(), wl.n_text)[0]
+    torch.cuda.synchronize()
+    assert torch.equal(out, again)
+
+
+@pytest.mark.parametrize("cube, D", [((2, 8, 8), 64), ((2, 8, 8), 128), ((4, 8, 8), 128), ((8, 8, 8), 64)])
+def test_many_gathered_items(cube, D):
+    """Thousands of items of one, two and four steps: the warpgroups run several items apart."""
+    wl = inputs.make_prefill("items", seed=54, B=1, T=64, H=16, W=16, cube=cube, n_text=100, Hq=8, Hkv=2, D=D, top_p=0.7, offset_std=1.5)
+    eng, out, bitmap, count = pu.run_forward(wl, prefill_kernel=1, gather=pu.FORCE_GATHER)
+    hdr = eng.header()
+    assert hdr.status == 0 and hdr.gather_items > 1000
+    n_tiles = (wl.S + 127) // 128
+    rows = pu.sample_rows(wl, 400, seed=4, whole_tiles=[(0, 3, n_tiles - 2)])
+    pu.compare_rows(wl, rows, out, bitmap, count, label=str(cube))
+    for _ in range(5):
+        again = eng.forward(wl.q.cuda(), wl.k.cuda(), wl.v.cuda(), wl.n_text)[0]
+        torch.cuda.synchronize()
+        assert eng.header().status == 0 and torch.equal(out, again)
