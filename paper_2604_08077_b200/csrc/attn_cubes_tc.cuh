@@ -435,23 +435,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
             bool ended = false;
             int ks = -1, s_left = 0, sbuf = 0, kst = 0, kph = 0, ahead = 0;
             int n_steps0 = 0, n_steps1 = 0, n_steps2 = 0;         // steps of pair tiles ks, ks - 1, ks - 2
-            // S of the next step, if there is one.  The next pair tile is begun only when its plan is there, unless nothing
-            // else is left to do: a plan may wait for the steps that this thread has still to issue.
+            // S of the next step, if there is one.  While products are left to issue (must = false) the next pair tile is begun only
+            // when its plan and both CTAs' Q tiles are there, and is not waited for: its plan, in either CTA, may wait for steps
+            // whose rows wait for these products (see the header of attn_prefill_tc.cuh).
             auto next_scores = [&](bool must) -> bool {
                 if (s_left == 0) {
                     if (ended) return false;
-                    const int slot = plan_slot(ks + 1);
-                    if (!tc::mbar_try_wait(&sm.plan_full[slot], plan_phase(ks + 1))) {
-                        if (!must || !(ok = tc::mbar_wait(&sm.plan_full[slot], plan_phase(ks + 1), abort_flag))) return false;
-                    }
+                    const int kn = ks + 1, slot = plan_slot(kn);
+                    auto there = [&](uint64_t* bar, uint32_t phase) -> bool { return must ? (ok = tc::mbar_wait(bar, phase, abort_flag)) : tc::mbar_test(bar, phase); };
+                    if (!there(&sm.plan_full[slot], plan_phase(kn))) return false;
                     if ((ended = sm.plan_item[slot] < 0)) return false;
-                    ++ks;
+                    if (!there(&sm.q_full[q_slot(kn)], q_phase(kn)) || !there(&sm.q_peer[q_slot(kn)], q_phase(kn))) return false;
+                    ks = kn;
                     n_steps2 = n_steps1;
                     n_steps1 = n_steps0;
                     s_left = n_steps0 = (sm.plan_blocks[slot] + 1) / 2;
                     tc::mbar_arrive(&sm.plan_empty[slot]);
-                    if (!(ok = tc::mbar_wait(&sm.q_full[q_slot(ks)], q_phase(ks), abort_flag))) return false;
-                    if (!(ok = tc::mbar_wait(&sm.q_peer[q_slot(ks)], q_phase(ks), abort_flag))) return false;
                 }
                 if (!(ok = tc::mbar_wait(&sm.k_full[kst], kph, abort_flag))) return false;
                 tc::tc_fence_after_sync();

@@ -15,6 +15,17 @@
 // range (own cubes / text prefix).  Each softmax thread masks its own row: one selection bit per
 // (row, cube) for blocks before the local range, the exact per-key rule inside it.
 //
+// Who waits for whom, so that nobody waits in a circle.  The issuer never waits for a pair tile that it has not begun while a
+// product of an earlier one is still to be issued.  For the plan of pair tile k, in either CTA, waits for the softmax warps of
+// k - 2 to have finished (k - 1, where long block lists leave one slot), and their rows, where no reference is fixed in
+// advance, wait with the rescaling in step g for the product of step g - 1 to have completed.  Were the issuer to wait for k with
+// products of k - 1 outstanding, CTA 1 could wait for those products and the issuer for CTA 1 (its Q of k is loaded behind its plan
+// of k).  With every product up to k - 1 issued all softmax warps get to the end of k - 1: scores have been issued ahead of
+// the products, K / V^T loads wait for scores and products only, an epilogue for the last product, the sums of its own pair tile and the
+// output rows of the one before; so plan, Q and first scores of k follow.  Inside a begun pair tile the issuer waits for K, V^T
+// (loaded behind plans that both CTAs have: CTA 1 reports its Q behind its plan), for weights (the softmax of scores issued before, in
+// the order of the steps) and for the epilogue before the first product.
+//
 // TMEM (512 columns): three tiles of 128 columns for S (fp32) -- P (bf16 pairs) overwrites the first 64 -- and D columns
 // for O.  What bounds a step is the chain S -> softmax -> P -> O, S of one such tile, 3100 to 3800 cycles.  With two tiles (and two
 // O, 256 rows of one CTA) it took 3180 cycles for both, 2048 of them tensor core; three tiles leave two steps in the softmax while
@@ -413,23 +424,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
             bool ended = false;
             int ks = -1, s_left = 0, sbuf = 0, kst = 0, kph = 0, ahead = 0;
             int n_steps0 = 0, n_steps1 = 0, n_steps2 = 0;         // steps of pair tiles ks, ks - 1, ks - 2
-            // S of the next step, if there is one.  The next pair tile is begun only when its plan is there, unless nothing
-            // else is left to do: a plan may wait for the steps that this thread has still to issue.
+            // S of the next step, if there is one.  While products are left to issue (must = false) the next pair tile is begun only
+            // when its plan and both CTAs' Q tiles are there, and is not waited for: its plan, in either CTA, may wait for steps
+            // whose rows wait for these products (see the file's header).
             auto next_scores = [&](bool must) -> bool {
                 if (s_left == 0) {
                     if (ended) return false;
-                    const int slot = plan_slot(ks + 1);
-                    if (!tc::mbar_try_wait(&sm.plan_full[slot], plan_phase(ks + 1))) {
-                        if (!must || !(ok = tc::mbar_wait(&sm.plan_full[slot], plan_phase(ks + 1), abort_flag))) return false;
-                    }
+                    const int kn = ks + 1, slot = plan_slot(kn);
+                    auto there = [&](uint64_t* bar, uint32_t phase) -> bool { return must ? (ok = tc::mbar_wait(bar, phase, abort_flag)) : tc::mbar_test(bar, phase); };
+                    if (!there(&sm.plan_full[slot], plan_phase(kn))) return false;
                     if ((ended = sm.plan_item[slot] < 0)) return false;
-                    ++ks;
+                    if (!there(&sm.q_full[kn & 1], (kn >> 1) & 1) || !there(&sm.q_peer[kn & 1], (kn >> 1) & 1)) return false;
+                    ks = kn;
                     n_steps2 = n_steps1;
                     n_steps1 = n_steps0;
                     s_left = n_steps0 = (sm.plan_blocks[slot] + 1) / 2;
                     tc::mbar_arrive(&sm.plan_empty[slot]);
-                    if (!(ok = tc::mbar_wait(&sm.q_full[ks & 1], (ks >> 1) & 1, abort_flag))) return false;
-                    if (!(ok = tc::mbar_wait(&sm.q_peer[ks & 1], (ks >> 1) & 1, abort_flag))) return false;
                 }
                 if (!(ok = tc::mbar_wait(&sm.k_full[kst], kph, abort_flag))) return false;
                 tc::tc_fence_after_sync();

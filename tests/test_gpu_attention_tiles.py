@@ -59,6 +59,24 @@ def test_long_block_list(D):
     pu.compare_rows(wl, rows, out, bitmap, count, label="long list")
 
 
+# Queries four times as large: bounds of the scores above 88, every row on the running maximum, whose rescaling waits for products while
+# a list that is kept once lets no plan run ahead.  Union tiles, and gathered pairs, whose tiles are two or three steps long.
+@pytest.mark.parametrize("cube, D, top_p, gather", [((4, 4, 4), 128, 0.9, 0.0), ((4, 8, 8), 64, 0.7, 0.0), ((4, 4, 4), 64, 0.9, pu.FORCE_GATHER),
+                                                    ((4, 8, 8), 128, 0.9, pu.FORCE_GATHER)])
+def test_long_block_list_running_maximum(cube, D, top_p, gather):
+    base = inputs.make_prefill("long", seed=55, B=1, T=640, H=16, W=16, cube=cube, n_text=37, Hq=2, Hkv=1, D=D, top_p=top_p, offset_std=1.0)
+    wl, _ = scaled(base, 4.0, 1.0)
+    eng, out, bitmap, count = pu.run_forward(wl, prefill_kernel=1, gather=gather, gather_budget=4 << 30)
+    hdr = eng.header()
+    assert hdr.status == 0 and (hdr.gather_pair_tiles > 1000) == (gather > 0.0)
+    n_tiles = (wl.S + 127) // 128
+    rows = pu.sample_rows(wl, 60, seed=5, whole_tiles=[(0, 1, n_tiles - 1), (0, 0, n_tiles // 2)])
+    pu.compare_rows(wl, rows, out, bitmap, count, label="long list, running maximum")
+    again = eng.forward(wl.q.cuda(), wl.k.cuda(), wl.v.cuda(), wl.n_text)[0]
+    torch.cuda.synchronize()
+    assert eng.header().status == 0 and torch.equal(out, again)
+
+
 # 128, 256 and 512 tokens, whole and at the ragged faces of a grid, lists of a few rows and of many; Top-K of one cube
 @pytest.mark.parametrize("cube, T, H, W, D, top_k", [((2, 8, 8), 16, 8, 8, 128, 0), ((4, 8, 8), 16, 16, 8, 64, 0), ((8, 8, 8), 32, 8, 16, 128, 1),
                                                      ((2, 8, 8), 9, 14, 11, 128, 0), ((4, 8, 8), 10, 12, 12, 64, 2)])
