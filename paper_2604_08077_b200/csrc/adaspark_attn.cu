@@ -278,7 +278,7 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // buffers of the query-gather path
     size_t off = 0;
     h->fw_status_off = off; off = align_up(off + 256);
-    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 4);   // mean-key exponents, largest |k|^2, largest |mean key|, largest |v|
+    h->fw_headmax_off = off; off = align_up(off + (size_t)batch * Hkv * 4 * 3);   // mean-key exponents, largest |k|^2, largest |mean key|
     h->fw_valid_off = off; off = align_up(off + (size_t)(S_cap / kBlockTok) * 2 * 4);   // which slots of a block hold a token
     const size_t n_cols = gather_columns((size_t)S_v, (size_t)N, h->C);                  // key blocks that hold video (large cubes: cubes)
     // query-gather path: the rows are cut into windows whose slice of Q (all heads) is about a third of the L2
@@ -435,19 +435,11 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         const int blk_end = last_call ? g.n_kv_blocks_cap : (g.S + kBlockTok - 1) / kBlockTok;
         dim3 grid(blk_end - blk_begin, g.Hkv, g.B);
         uint32_t* slot_valid = (!cache_only && g.ragged) ? (uint32_t*)((char*)workspace + h->fw_valid_off) : nullptr;
-        // largest |k|^2 and |v| per (batch, kv head)
-        uint32_t* key_norm2 = !cache_only ? (uint32_t*)((char*)workspace + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
-        uint32_t* value_max = !cache_only ? key_norm2 + 2 * g.B * g.Hkv : nullptr;
-        if (D == 128) relayout_pool_kernel<128><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2, value_max);
-        else relayout_pool_kernel<64><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2, value_max);
+        // largest |k|^2 per (batch, kv head): only a call that brings the sequence from its first frame sees every key
+        uint32_t* key_norm2 = (!cache_only && frame_begin == 0) ? (uint32_t*)((char*)workspace + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
+        if (D == 128) relayout_pool_kernel<128><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
+        else relayout_pool_kernel<64><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
         if (!launch_ok(h, "relayout_pool_kernel")) return ADASPARK_ERR_CUDA;
-        if (!cache_only && g.pos_begin > 0 && h->prefill_kernel != 0) {     // the keys and values of earlier calls
-            const int ctas = g.pos_begin * (D / 8) / 1024;              // four 16-byte pieces of K and V a thread, at least
-            const dim3 ngrid(ctas < 256 ? (ctas < 1 ? 1 : ctas) : 256, g.Hkv, g.B);
-            if (D == 128) launch_kernel(true, seen_norms_kernel<128>, ngrid, dim3(256), 0, st, g, g.pos_begin, (const __nv_bfloat16*)kc, (const __nv_bfloat16*)vc, key_norm2, value_max);
-            else launch_kernel(true, seen_norms_kernel<64>, ngrid, dim3(256), 0, st, g, g.pos_begin, (const __nv_bfloat16*)kc, (const __nv_bfloat16*)vc, key_norm2, value_max);
-            if (!launch_ok(h, "seen_norms_kernel")) return ADASPARK_ERR_CUDA;
-        }
         const int cube_begin = g.pos_begin >> g.c_shift;
         if (g.C > kBlockTok && g.N_live > cube_begin) {
             launch_kernel(true, pool_large_cubes_kernel, dim3(g.N_live - cube_begin, g.Hkv, g.B), dim3(D), 0, st, g, kc, cube_keys);
@@ -649,15 +641,14 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         std::memset(&local_tiles, 0, sizeof(local_tiles));
         if (gather && g.C > kBlockTok) local_tiles.part_o = gw.local_o;
         float* row_ref = gather && g.C > kBlockTok ? (float*)(ws + h->fw_gref_off) : nullptr;   // softmax references of the rows of gathered pairs
-        const uint32_t* key_norm2_c = (const uint32_t*)(ws + h->fw_headmax_off) + g.B * g.Hkv;
-        const uint32_t* value_max_c = key_norm2_c + 2 * g.B * g.Hkv;
+        const uint32_t* key_norm2_c = frame_begin == 0 ? (const uint32_t*)(ws + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
         mark(h, 5, st);
 #define ADASPARK_LAUNCH_ATTN(DD)                                                                                              \
     do {                                                                                                                    \
         const size_t smem = sizeof(TcAttnSmem<DD>) + 1024;                                                                  \
         if (!set_smem(h, attn_prefill_tc_kernel<DD>, smem, "attn_prefill_tc_kernel")) return ADASPARK_ERR_CUDA;              \
         launch_kernel(true, attn_prefill_tc_kernel<DD>, dim3(attn_grid), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV,   \
-                      tile_mask, tile_union, slot_valid_c, pair_mode_c, gw.n_pairs_cap, gw.ml_local, key_norm2_c, value_max_c, \
+                      tile_mask, tile_union, slot_valid_c, pair_mode_c, gw.n_pairs_cap, gw.ml_local, key_norm2_c, \
                       (__nv_bfloat16*)out, next_pair_tile, (unsigned long long*)&hdr->executed_kv_blocks,                    \
                       &hdr->max_tile_kv_blocks, &hdr->status);                                                              \
     } while (0)
@@ -667,7 +658,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         if (!set_smem(h, attn_cubes_tc_kernel<DD, GATHERED>, smem, "attn_cubes_tc_kernel")) return ADASPARK_ERR_CUDA;        \
         launch_kernel(true, attn_cubes_tc_kernel<DD, GATHERED>, dim3(GRID), dim3(kTcThreads), smem, st, g, tmQ, qb, tmK, tmV, \
                       tile_mask, tile_union, slot_valid_c, pair_mode_c, gw.n_pairs_cap, gw.ml_local, TILES, row_ref,         \
-                      key_norm2_c, value_max_c, (__nv_bfloat16*)out, COUNTER,                                               \
+                      key_norm2_c, (__nv_bfloat16*)out, COUNTER,                                               \
                       (unsigned long long*)&hdr->executed_kv_blocks, &hdr->max_tile_kv_blocks, &hdr->status);                \
     } while (0)
         if (gather && g.C > kBlockTok) {

@@ -57,7 +57,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
     Geom g, const __grid_constant__ CUtensorMap tmQ, const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap tmK,
     const __grid_constant__ CUtensorMap tmV, const uint32_t* tile_mask, const uint32_t* tile_union, const uint32_t* slot_valid,
     const uint32_t* pair_mode, int n_pairs_cap, float2* ml_local, const GatherTiles gt, float* row_ref, const uint32_t* key_norm2_bits,
-    const uint32_t* value_max_bits, __nv_bfloat16* out, uint32_t* next_pair_tile, unsigned long long* executed_blocks, uint32_t* max_tile_blocks, int32_t* status) {
+    __nv_bfloat16* out, uint32_t* next_pair_tile, unsigned long long* executed_blocks, uint32_t* max_tile_blocks, int32_t* status) {
     extern __shared__ unsigned char tc_smem_raw[];
     using Smem = CubesSmem<D, kGathered>;
     Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -169,12 +169,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                 return true;
             }
             // Bound of a row's scores: |s| <= |q| |k| for every key; the largest key norm of the head comes from the re-layout
-            // kernel.
+            // kernel (none when not every attended key went through this call's re-layout).
             const int qs = q_slot(k);
             const unsigned char* qt = reinterpret_cast<const unsigned char*>(&sm.q[qs][0][0][0]);
             {
                 if (!tc::mbar_wait(&sm.q_full[qs], q_phase(k), abort_flag)) return false;
-                const float k2 = __uint_as_float(key_norm2_bits[bkv]), v_max = __uint_as_float(value_max_bits[bkv]);
+                const float k2 = key_norm2_bits != nullptr ? __uint_as_float(key_norm2_bits[bkv]) : INFINITY;
 #pragma unroll 1
                 for (int row = lane; row < 128; row += 32) {
                     unsigned long long qq[2] = {0ull, 0ull};
@@ -190,8 +190,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                     }
                     float qa, qb;
                     unpack_f32x2(add_f32x2(qq[0], qq[1]), qa, qb);
-                    const float q2 = qa + qb;
-                    sm.fixed[k & 3][row] = fixed_reference(sqrtf(q2 * k2) * g.scale_log2 * 1.01f + 0.01f, v_max);   // 1 % for the rounding of the norms and of s
+                    sm.fixed[k & 3][row] = fixed_reference(qa + qb, k2, g.scale_log2);
                 }
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&sm.bound_full[k & 3]);

@@ -51,16 +51,16 @@ constexpr int kPairRows = 256;
 constexpr int kScoreBufs = 3;         // score / weight tiles in TMEM
 static_assert(kScoreBufs == kSoftmaxGroups, "a warpgroup owns a tile");
 constexpr int kRefSlots = 4;          // a warpgroup is at most three steps behind the others: slots of the running reference
-// Reference of a row's softmax fixed in advance, from the bound B of its scores (log2 units; every score lies in [-B, B]).
-// Up to B = 48 it is B itself: every weight 2^(s - B) is at least 2^-96, nothing underflows, and 30 binades remain
-// above the smallest normal fp32 for the products with V.  Beyond, it is 96 - B, so that the smallest weight stays at
-// 2^-96 and the largest is 2^(2B - 96): the sums of at most 2^21 weights or products with |v| <= v_max stay below
-// 2^120 for B up to 97.5 - log2(v_max) / 2, and 88 is taken at most.
-constexpr float kFixedRefMax = 48.f, kFixedRefFar = 88.f;
-__host__ __device__ inline float fixed_reference(float bound, float v_max) {     // infinite: not in advance
-    if (bound <= kFixedRefMax) return bound;
-    if (bound <= kFixedRefFar && 2.f * bound + log2f(fmaxf(v_max, 1.f)) <= 195.f) return 2.f * kFixedRefMax - bound;
-    return INFINITY;
+// Reference of a row's softmax fixed in advance: the bound B of its scores (log2 units; every score lies in [-B, B]), up to this B.
+// Every weight 2^(s - B) is at least 2^-2B = 2^-96: nothing underflows, and 30 binades remain above the smallest normal fp32 for
+// the products with V.  Not beyond: the largest weights of a row, 1 or a power of two near it on the running maximum, are any numbers with
+// a fixed reference and lose up to 2^-9 each in bf16.  References up to B = 88 (96 - B) and in later chunks gained 7 % on a chunk, but
+// their error against 64 bits was up to 5 % larger (sharp queries, p 0.95: 0.00226 -> 0.00234; a chunk 0.00232 -> 0.00235).
+constexpr float kFixedRefMax = 48.f;
+// |q|^2, largest |k|^2 of the head: infinite, not in advance
+__device__ __forceinline__ float fixed_reference(float q2, float k2, float scale_log2) {
+    const float bound = sqrtf(q2 * k2) * scale_log2 * 1.01f + 0.01f;     // 1 % for the rounding of the norms and of s
+    return bound <= kFixedRefMax ? bound : INFINITY;
 }
 constexpr int kFmaExpEvery = 2;       // of every 4 kFmaExpEvery exponentials one is a cubic on the FMA pipe (one in four: no faster, four times the error)
 constexpr int kMaxKeyBlocks = 32768;  // key blocks per sequence (2M positions): a number and a flag fit 16 bits
@@ -106,7 +106,7 @@ template <int D>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_prefill_tc_kernel(
     Geom g, const __grid_constant__ CUtensorMap tmQ, const __nv_bfloat16* __restrict__ q, const __grid_constant__ CUtensorMap tmK,
     const __grid_constant__ CUtensorMap tmV, const uint32_t* tile_mask, const uint32_t* tile_union, const uint32_t* slot_valid,
-    const uint32_t* pair_mode, int n_pairs_cap, float2* ml_local, const uint32_t* key_norm2_bits, const uint32_t* value_max_bits, __nv_bfloat16* out,
+    const uint32_t* pair_mode, int n_pairs_cap, float2* ml_local, const uint32_t* key_norm2_bits, __nv_bfloat16* out,
     uint32_t* next_pair_tile, unsigned long long* executed_blocks, uint32_t* max_tile_blocks, int32_t* status) {
     extern __shared__ unsigned char tc_smem_raw[];
     TcAttnSmem<D>& sm = *reinterpret_cast<TcAttnSmem<D>*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -329,10 +329,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
             blocks_sum += (unsigned long long)(2 * n_needed);
             blocks_max = max(blocks_max, (uint32_t)n_needed);
             // Bound of a row's scores: |s| <= |q| |k| for every key; the largest key norm of the head comes from the re-layout
-            // kernel.
+            // kernel (none when not every attended key went through this call's re-layout).
             {
                 if (!(ok = tc::mbar_wait(&sm.q_full[qs], (k >> 1) & 1, abort_flag))) break;
-                const float k2 = __uint_as_float(key_norm2_bits[it.b * g.Hkv + it.gk]), v_max = __uint_as_float(value_max_bits[it.b * g.Hkv + it.gk]);
+                const float k2 = key_norm2_bits != nullptr ? __uint_as_float(key_norm2_bits[it.b * g.Hkv + it.gk]) : INFINITY;
 #pragma unroll 1
                 for (int row = lane; row < 128; row += 32) {
                     unsigned long long qq[2] = {0ull, 0ull};
@@ -348,8 +348,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                     }
                     float qa, qb;
                     unpack_f32x2(add_f32x2(qq[0], qq[1]), qa, qb);
-                    const float q2 = qa + qb;
-                    sm.fixed[k & 3][row] = fixed_reference(sqrtf(q2 * k2) * g.scale_log2 * 1.01f + 0.01f, v_max);     // 1 % for the rounding of the norms and of s
+                    sm.fixed[k & 3][row] = fixed_reference(qa + qb, k2, g.scale_log2);
                 }
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&sm.bound_full[k & 3]);

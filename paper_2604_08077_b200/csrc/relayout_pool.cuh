@@ -8,10 +8,9 @@
 //   cube_keys [B,Hkv,N,D] fp32    mean over the C keys of each cube inside the block (C <= 64);
 //                                 cubes larger than a block are pooled by pool_large_cubes_kernel.
 // Positions >= S are zero-filled so that later tensor-core reads never meet non-finite data.
-// The kernel also leaves the largest |k|^2 and the largest |v| element of every (batch, kv head) among the rows it wrote
-// (float bits, atomic maximum): with |q| the first bounds every score of a query row (Cauchy-Schwarz), which lets the
-// attention kernel fix a row's softmax reference in advance, with the second as far as the products with V allow.
-// seen_norms_kernel adds those of the rows that earlier calls of a chunked prefill wrote.
+// The kernel also leaves the largest |k|^2 of every (batch, kv head) among the rows it wrote (float bits,
+// atomic maximum): with |q| it bounds every score of a query row (Cauchy-Schwarz), which lets the attention
+// kernel fix a row's softmax reference in advance.
 #pragma once
 #include "common.cuh"
 
@@ -26,60 +25,17 @@ __device__ __forceinline__ int cube_tokens_held(const Geom& g, int cube) {
     return min(g.ct, g.T - cb * g.ct) * min(g.ch, g.H - cy * g.ch) * min(g.cw, g.W - cx * g.cw);
 }
 
-// largest |x| of bf16 pairs, each half for itself (the bits of non-negative bf16 numbers order like integers)
-__device__ __forceinline__ uint32_t abs_max_bf16x2(uint32_t m, const uint4& x) {
-    m = __vmaxu2(m, x.x & 0x7fff7fffu);
-    m = __vmaxu2(m, x.y & 0x7fff7fffu);
-    m = __vmaxu2(m, x.z & 0x7fff7fffu);
-    return __vmaxu2(m, x.w & 0x7fff7fffu);
-}
-// ... of both halves as float bits
-__device__ __forceinline__ uint32_t larger_half_bits(uint32_t m) { return max(m & 0xffff0000u, m << 16); }
-
-// Largest |k|^2 and |v| of a CTA of 256 threads joined with the head's: one atomic each (one per warp, all of them to a few
-// addresses, cost the re-layout of 16384 tokens 8 of 32 us).  Holds a barrier.
-__device__ __forceinline__ void block_norms(float k2, uint32_t v_max, uint32_t (&part)[2][8], uint32_t* key_norm2_bits, uint32_t* value_max_bits) {
+// Largest |k|^2 of a CTA of 256 threads joined with the head's: one atomic (one per warp, all of them to a few addresses, cost the
+// re-layout of 16384 tokens 8 of 32 us when there were two of them).  Holds a barrier.
+__device__ __forceinline__ void block_norm(float k2, uint32_t (&part)[8], uint32_t* key_norm2_bits) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(k2)), v = __reduce_max_sync(0xffffffffu, larger_half_bits(v_max));
-    if (lane == 0) { part[0][warp] = m; part[1][warp] = v; }
+    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(k2));
+    if (lane == 0) part[warp] = m;
     __syncthreads();
-    if (warp == 0 && lane < 16) {
-        const uint32_t x = __reduce_max_sync(lane < 8 ? 0xffu : 0xff00u, part[lane >> 3][lane & 7]);
-        if ((lane & 7) == 0 && x) atomicMax(lane == 0 ? key_norm2_bits : value_max_bits, x);
+    if (warp == 0 && lane < 8) {
+        const uint32_t x = __reduce_max_sync(0xffu, part[lane]);
+        if (lane == 0 && x) atomicMax(key_norm2_bits, x);
     }
-}
-
-// Largest |k|^2 and |v| of the cache rows [0, n_rows) that earlier calls wrote (n_rows: a multiple of 64; V^T blocks hold
-// the same rows).  Reads them once: 84 MB for 40960 rows of 4 heads.  grid (CTAs, Hkv, B), 256 threads.
-template <int D>
-__global__ void __launch_bounds__(256) seen_norms_kernel(Geom g, int n_rows, const __nv_bfloat16* k_cube, const __nv_bfloat16* v_cube,
-                                                         uint32_t* key_norm2_bits, uint32_t* value_max_bits) {
-    launch_dependents();
-    wait_for_previous_kernel();
-    constexpr int kChunks = D / 8;                                // 16-byte chunks per row, neighbouring lanes
-    __shared__ uint32_t part[2][8];
-    const int bh = blockIdx.z * g.Hkv + blockIdx.y;
-    const uint4* k = reinterpret_cast<const uint4*>(k_cube + (size_t)bh * g.S_cap * D);
-    const uint4* v = reinterpret_cast<const uint4*>(v_cube + (size_t)bh * g.S_cap * D);
-    float row_max = 0.f;
-    uint32_t v_max = 0u;
-    const int n = n_rows * kChunks;                               // a multiple of 512: warps stay whole
-#pragma unroll 4
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
-        const uint4 kv4 = k[i];
-        v_max = abs_max_bf16x2(v_max, v[i]);
-        const uint32_t w[4] = {kv4.x, kv4.y, kv4.z, kv4.w};
-        float n2 = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float lo = __uint_as_float(w[e] << 16), hi = __uint_as_float(w[e] & 0xffff0000u);
-            n2 = fmaf(lo, lo, fmaf(hi, hi, n2));
-        }
-#pragma unroll
-        for (int o = kChunks / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-        row_max = fmaxf(row_max, n2);
-    }
-    block_norms(row_max, v_max, part, key_norm2_bits + bh, value_max_bits + bh);
 }
 
 template <int D>
@@ -89,7 +45,7 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
                                                             __nv_bfloat16* __restrict__ v_cube,
                                                             float* __restrict__ cube_keys,
                                                             uint32_t* __restrict__ slot_valid,
-                                                            uint32_t* __restrict__ key_norm2_bits, uint32_t* __restrict__ value_max_bits) {
+                                                            uint32_t* __restrict__ key_norm2_bits) {
     launch_dependents();
     constexpr int kChunks = D / 8;    // 16-byte chunks per row
     constexpr int kVPitch = D + 2;    // padded pitch (elements) of the V staging tile
@@ -100,8 +56,7 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
     const int pos0 = blk * kBlockTok;
     const int tid = threadIdx.x;
     float row_max = 0.f;
-    uint32_t v_max = 0u;
-    __shared__ uint32_t part[2][8];
+    __shared__ uint32_t part[8];
 
     for (int idx = tid; idx < kBlockTok * kChunks; idx += 256) {
         int row = idx / kChunks, c = idx - row * kChunks;
@@ -127,12 +82,11 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
 #pragma unroll
             for (int o = kChunks / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
             row_max = fmaxf(row_max, n2);
-            v_max = abs_max_bf16x2(v_max, vv4);
         }
         uint32_t* vdst = reinterpret_cast<uint32_t*>(&Vs[row][c * 8]);
         vdst[0] = vv4.x; vdst[1] = vv4.y; vdst[2] = vv4.z; vdst[3] = vv4.w;
     }
-    if (key_norm2_bits != nullptr) block_norms(row_max, v_max, part, key_norm2_bits + b * g.Hkv + gk, value_max_bits + b * g.Hkv + gk);
+    if (key_norm2_bits != nullptr) block_norm(row_max, part, key_norm2_bits + b * g.Hkv + gk);
     else __syncthreads();
 
     // Which of the block's 64 slots hold a token (two words per block; read by the attention kernels of a

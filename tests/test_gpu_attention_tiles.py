@@ -1,4 +1,4 @@
-"""The prefill attention kernel where its forms meet: softmax references fixed in advance (near and far) and running, in one
+"""The prefill attention kernel where its forms meet: softmax references fixed in advance and running, in one
 call and in chunks, block lists of more blocks than are kept twice, and whole cubes of more than 64 tokens gathered; against the
 CPU oracle."""
 import dataclasses
@@ -20,13 +20,13 @@ def scaled(wl, scale_q, scale_v):
     return dataclasses.replace(wl, q=times(wl.q, scale_q)), times(wl.v, scale_v)
 
 
-# The bound of a row's scores is 27 to 42 (log2 units) at scale 1: below 88 at 2, on both sides of it at 2.4, above at 4; values
-# of 2^40 move the limit to 77, values of 2^110 out of reach.
+# The bound of a row's scores is 27 to 42 (log2 units) at scale 1: on both sides of 48, up to which the reference is fixed in advance, at
+# 1.4, above at the others.
 @pytest.mark.parametrize("D", [64, 128])
-@pytest.mark.parametrize("scale_q", [2.0, 2.4, 4.0])
+@pytest.mark.parametrize("scale_q", [1.4, 2.0, 2.4, 4.0])
 @pytest.mark.parametrize("scale_v", [1.0, 2.0 ** 40, 2.0 ** 110])
 def test_softmax_references(D, scale_q, scale_v):
-    """Every row, in one call and in three chunks (whose later calls take the norms of earlier keys from the caches).  The output is
+    """Every row, in one call and in three chunks (whose later calls are on the running maximum).  The output is
     linear in V and the scales are powers of two: it is compared at scale 1."""
     base = inputs.small_prefill(seed=51, T=24, H=8, W=8, n_text=29, D=D)
     wl, v = scaled(base, scale_q, scale_v)
@@ -46,6 +46,31 @@ def test_softmax_references(D, scale_q, scale_v):
                     label=f"chunks {scale_q} {scale_v}")
 
 
+def rel_error(out, rows, ref):
+    got = out[rows[:, 0], rows[:, 2], rows[:, 1]].float().cpu().numpy()
+    return float(np.sqrt(((got - ref) ** 2).sum() / (ref ** 2).sum()))
+
+
+# The mma.sync path takes a row's maximum as it is, the tcgen05 path moves its reference when the maximum grows by 2^8: weights near 1, of
+# which few lose bits in bf16 where the row is peaked.  Error against fp64 over that of the mma.sync path: 1.11 to 1.13 on the running
+# maximum, 1.26 with references fixed at a bound of 54 to 84.
+@pytest.mark.parametrize("D", [64, 128])
+def test_peaked_rows_keep_their_precision(D):
+    wl, _ = scaled(inputs.small_prefill(seed=57, T=32, H=8, W=8, n_text=29, D=D, offset_std=1.5, top_p=0.95), 2.0, 1.0)
+    rows = np.asarray(oracle.all_rows(pu.oracle_shape(wl)))
+    ref = oracle.rows(pu.oracle_shape(wl), wl.q, wl.k, wl.v, rows)["out"]
+    base = rel_error(pu.run_forward(wl, prefill_kernel=0, gather=0.0)[1], rows, ref)
+    eng, one, _, _ = pu.run_forward(wl, prefill_kernel=1, gather=0.0)
+    q, k, v = wl.q.cuda(), wl.k.cuda(), wl.v.cuda()
+    outs = []
+    for fb, fc, nt in [(0, 4, -1), (4, 28, wl.n_text)]:
+        lo, hi = fb * 64, (fb + fc) * 64 + max(nt, 0)
+        outs.append(eng.forward_chunk(q[:, lo:hi].contiguous(), k[:, lo:hi].contiguous(), v[:, lo:hi].contiguous(), fb, fc, nt)[0])
+    torch.cuda.synchronize()
+    for out in (one, torch.cat(outs, 1)):
+        assert rel_error(out, rows, ref) < 1.18 * base
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_long_block_list(D):
     """163840 tokens are 2560 key blocks (2304 fit a list that is kept twice): sampled rows of the union path, the last tiles whole."""
@@ -59,7 +84,7 @@ def test_long_block_list(D):
     pu.compare_rows(wl, rows, out, bitmap, count, label="long list")
 
 
-# Queries four times as large: bounds of the scores above 88, every row on the running maximum, whose rescaling waits for products while
+# Queries four times as large: bounds of the scores above 48, every row on the running maximum, whose rescaling waits for products while
 # a list that is kept once lets no plan run ahead.  Union tiles, and gathered pairs, whose tiles are two or three steps long.
 @pytest.mark.parametrize("cube, D, top_p, gather", [((4, 4, 4), 128, 0.9, 0.0), ((4, 8, 8), 64, 0.7, 0.0), ((4, 4, 4), 64, 0.9, pu.FORCE_GATHER),
                                                     ((4, 8, 8), 128, 0.9, pu.FORCE_GATHER)])
