@@ -673,23 +673,41 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                 if (!(ok = tc::mbar_wait(&sm.s_full[wg], s_ph, abort_flag))) break;
                 s_ph ^= 1u;
                 tc::tc_fence_after_sync();
+                bool rescale = false;                                     // some row of the warp moves its reference: O is scaled by its factor
+                float factor = 1.f;
                 if (!fixed_ref) {
                     // ---- row maximum over the visible keys; the reference moves through the warpgroups step by step
                     float mx = -INFINITY;
-#pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
-                        uint32_t s[32];
-                        tc::tmem_ld_32x32(s_addr + c * 32, s);
-                        tc::tmem_wait_ld_for(s);
-                        if (by_cube) {
-                            float a0 = -INFINITY, a1 = -INFINITY;
+                    auto fold = [&](const uint32_t (&s)[32], int c) {
+                        float a0 = -INFINITY, a1 = -INFINITY;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                a0 = fmax3(a0, __uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1]));
-                                a1 = fmax3(a1, __uint_as_float(s[16 + 2 * i]), __uint_as_float(s[17 + 2 * i]));
-                            }
-                            mx = fmax3(mx, (groups >> (2 * c)) & 1u ? a0 : -INFINITY, (groups >> (2 * c)) & 2u ? a1 : -INFINITY);
-                        } else {
+                        for (int i = 0; i < 8; ++i) {
+                            a0 = fmax3(a0, __uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1]));
+                            a1 = fmax3(a1, __uint_as_float(s[16 + 2 * i]), __uint_as_float(s[17 + 2 * i]));
+                        }
+                        mx = fmax3(mx, (groups >> (2 * c)) & 1u ? a0 : -INFINITY, (groups >> (2 * c)) & 2u ? a1 : -INFINITY);
+                    };
+                    if (!kGathered && by_cube) {
+                        uint32_t s0[32], s1[32];                          // the next chunk is requested before the present one is looked at
+                        tc::tmem_ld_32x32(s_addr, s0);
+                        tc::tmem_wait_ld_for(s0);
+                        tc::tmem_ld_32x32(s_addr + 32, s1);
+                        fold(s0, 0);
+                        tc::tmem_wait_ld_for(s1);
+                        tc::tmem_ld_32x32(s_addr + 64, s0);
+                        fold(s1, 1);
+                        tc::tmem_wait_ld_for(s0);
+                        tc::tmem_ld_32x32(s_addr + 96, s1);
+                        fold(s0, 2);
+                        tc::tmem_wait_ld_for(s1);
+                        fold(s1, 3);
+                    } else {
+#pragma unroll 1
+                        for (int c = 0; c < 4; ++c) {
+                            uint32_t s[32];
+                            tc::tmem_ld_32x32(s_addr + c * 32, s);
+                            tc::tmem_wait_ld_for(s);
+                            if (by_cube) { fold(s, c); continue; }
                             const uint32_t am = c < 2 ? (c == 0 ? amask[0] : amask[1]) : (c == 2 ? amask[2] : amask[3]);
                             float a0 = -INFINITY, a1 = -INFINITY;
 #pragma unroll
@@ -710,21 +728,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                     sm.ref[rs][row] = m_new;
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&sm.ref_done[rs][quad]);
-                    if (j > 0 && __any_sync(0xffffffffu, need)) {
-                        // O holds the products of all steps up to the last one, and no later one starts before this step's weights
-                        if (!(ok = tc::mbar_wait(&sm.v_empty[(gs - 1) % n_stages], ((gs - 1) / n_stages) & 1, abort_flag))) break;
-                        tc::tc_fence_after_sync();
-                        const float factor = need ? fast_exp2(m_prev - mx_x) : 1.f;   // 0 when nothing was visible before
-#pragma unroll 1
-                        for (int c = 0; c < D / 32; ++c) {
-                            uint32_t o[32];
-                            tc::tmem_ld_32x32(lane_addr + kOCol + c * 32, o);
-                            tc::tmem_wait_ld_for(o);
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * factor);
-                            tc::tmem_st_32x32(lane_addr + kOCol + c * 32, o);
-                        }
-                    }
+                    rescale = j > 0 && __any_sync(0xffffffffu, need);
+                    if (need) factor = fast_exp2(m_prev - mx_x);          // 0 when nothing was visible before
                     // this warpgroup's sum is relative to the reference of its previous step
                     l_sum = m_ref == -INFINITY ? 0.f : l_sum * fast_exp2(m_ref - m_new);
                     m_ref = m_new;
@@ -793,6 +798,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                             pk[i] = pack_bf16x2(p0, p1);
                         }
                         tc::tmem_st_32x16(s_addr + c * 16, pk);
+                    }
+                }
+                if (rescale) {
+                    // O holds the products of all steps up to the last one, and no later one starts before this step's weights are
+                    // reported: it is scaled behind them, so that the last product may complete meanwhile
+                    if (!(ok = tc::mbar_wait(&sm.v_empty[(gs - 1) % n_stages], ((gs - 1) / n_stages) & 1, abort_flag))) break;
+                    tc::tc_fence_after_sync();
+#pragma unroll 1
+                    for (int c = 0; c < D / 32; c += 2) {
+                        uint32_t o0[32], o1[32];
+                        tc::tmem_ld_32x32(lane_addr + kOCol + c * 32, o0);
+                        tc::tmem_wait_ld_for(o0);
+                        tc::tmem_ld_32x32(lane_addr + kOCol + c * 32 + 32, o1);
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) o0[e] = __float_as_uint(__uint_as_float(o0[e]) * factor);
+                        tc::tmem_st_32x32(lane_addr + kOCol + c * 32, o0);
+                        tc::tmem_wait_ld_for(o1);
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) o1[e] = __float_as_uint(__uint_as_float(o1[e]) * factor);
+                        tc::tmem_st_32x32(lane_addr + kOCol + c * 32 + 32, o1);
                     }
                 }
                 tc::tmem_wait_st();
