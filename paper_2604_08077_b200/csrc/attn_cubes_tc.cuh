@@ -272,10 +272,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                 for (int idx = lane; idx < (128 - n_vid) * (D / 8); idx += 32) {
                     const int row = n_vid + idx / (D / 8), c = idx % (D / 8);
                     const int pos = tile_pos0 + row;
-                    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-                    if (pos < g.S) val = __ldg(reinterpret_cast<const uint4*>(q + (io_row(g, it.b, pos) * g.Hq + it.h) * D) + c);
-                    *reinterpret_cast<uint4*>(qt + (c >> 3) * (128 * 128) + sw128(row, c & 7)) = val;
+                    unsigned char* dst = qt + (c >> 3) * (128 * 128) + sw128(row, c & 7);
+                    if (pos < g.S) cp_async_16(dst, q + (io_row(g, it.b, pos) * g.Hq + it.h) * D + c * 8);
+                    else *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
                 }
+                // all copies under way at once
+                cp_async_commit();
+                cp_async_wait<0>();
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the copied rows are read by the tensor core
                 __syncwarp();
                 if (lane == 0) {
