@@ -312,10 +312,15 @@ adaspark_status_t adaspark_attn_set_prefill_kernel(adaspark_attn_t *handle, int3
  * key blocks in the pair's union -- and only if all qualifying pairs together save more than the fixed
  * cost of the path (about 50 us by the library's estimate, in which a union block costs as much as 44
  * entries).  pairs_per_block = 0 switches the path off (every pair takes the union path); a value above 44
- * forces it for every pair that meets the threshold, a huge value for every pair with a selected cube.  budget_bytes bounds the workspace
- * the path may use for its partial results (2*head_dim + 24 bytes per entry; _partition reserves
- * min(budget, pairs_per_block * video key blocks / 512 entries per query row -- what the pairs of a causal
- * sequence can produce on average --, 128 entries per query row));
+ * forces it for every pair that meets the threshold, a huge value for every pair with a selected cube.  Cubes of
+ * more than 64 tokens are gathered whole: an entry is a (row, cube) pair, items hold up to 256 rows, and the threshold
+ * and the estimate count an entry as 1.7 + 0.06 * cube_tokens / 64 of the entries above (what it was measured to cost).
+ * budget_bytes bounds the workspace the path may use for its entries and their partial results (2*head_dim + 24 bytes per
+ * (row, key block) entry; _partition reserves min(budget, pairs_per_block * video key blocks / 512 entries per query
+ * row -- what the pairs of a causal sequence can produce on average --, 128 entries per query row)).  With cubes of more
+ * than 64 tokens the same bytes hold entries of 4*head_dim + 16 bytes (partial results in fp32), 4 bytes per query row and, for
+ * as many pairs as that leaves room for (at most half of it), the results of their local range in fp32
+ * (1024*head_dim bytes per pair);
  * if the pairs that qualify in a call need more, only part of them is gathered in that call: the pairs fall
  * into four classes by entries per union block (up to 1/8, 1/4, 1/2 of the threshold, up to the threshold)
  * and into row windows; (class, window) units are kept while they fit, sparsest class first and inside a

@@ -37,6 +37,7 @@ struct adaspark_attn {
         fw_kplanes_off, fw_keyhash_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gref_off, fw_glocal_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
         fw_gpartml_off, fw_min, fw_total;      // fw_min: the smallest workspace a forward takes, fw_total: the one it is best given
     int score_items;            // query tiles per launch of the score / selection pair, at most
+    uint32_t gather_pairs;      // pairs of query tiles that may be gathered at once, at most (whole cubes: room for their local range)
     // query-gather path of the prefill: capacity in (row, key block) entries, decision threshold, byte budget
     uint32_t gather_cap;
     int gather_windows;
@@ -312,22 +313,40 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
     // per row (m, l) of the local range | per key block offsets + work items | entries | partial outputs | partial (m, l)
     {
         const size_t rows_cap = (size_t)batch * Hq * S_cap, n_pairs_cap = ((size_t)S_cap + 255) / 256;
-        const uint64_t part_bytes = (h->C > kBlockTok ? 4ull : 2ull) * D;    // partial output: fp32 of whole cubes, else bf16
-        const uint64_t per_entry = part_bytes + 16ull + 8ull;    // + (m, l) + entry
-        uint64_t cap = h->gather_budget / per_entry;
+        const bool whole = h->C > kBlockTok;                     // whole cubes are gathered
+        uint64_t cap = h->gather_budget / (2ull * D + 24ull);    // bf16 partial output + (m, l) + entry
         // a pair qualifies with at most threshold x (blocks of its union) entries for its 256 rows, and over a causal
         // sequence a pair's union averages half the video's key blocks: threshold x n_cols / 512 entries per row
         const double n_blocks = (double)((S_v + kBlockTok - 1) / kBlockTok);
-        double per_row = std::ceil((double)h->gather_pairs_per_block * n_blocks / 512.0 / (double)gather_entry_cost(h->C));
-        if (!(per_row < (double)kGatherEntriesPerRow)) per_row = (double)kGatherEntriesPerRow;
-        if ((double)cap > (double)rows_cap * per_row) cap = (uint64_t)((double)rows_cap * per_row);
+        auto entries_per_row = [&](double cost) -> double {
+            const double n = std::ceil((double)h->gather_pairs_per_block * n_blocks / 512.0 / cost);
+            return n < (double)kGatherEntriesPerRow ? n : (double)kGatherEntriesPerRow;
+        };
+        if ((double)cap > (double)rows_cap * entries_per_row(1.0)) cap = (uint64_t)((double)rows_cap * entries_per_row(1.0));
         if (cap > 0xfffffff0ull) cap = 0xfffffff0ull;
+        uint64_t pairs = (uint64_t)batch * Hq * n_pairs_cap;
+        if (whole) {
+            // Fp32 partial results, a softmax reference per row and the local range of the gathered pairs in fp32, in the bytes that
+            // entries of single key blocks would take.  As many pairs as would fill the entries with an eighth of the most that a
+            // pair has on average (the limit of the sparsest class, which is kept first): a fifth of the bytes from 25000 tokens on, half
+            // below 6500.
+            const uint64_t pool = cap * (2ull * D + 16ull), fixed = rows_cap * 4 + 4 * kAlign, entry = 4ull * D + 16ull, local = 256ull * 4 * D;
+            const uint64_t avail = pool > fixed ? pool - fixed : 0;
+            const double per_row = entries_per_row((double)gather_entry_cost(h->C));
+            const uint64_t least = local + 256ull * (uint64_t)std::ceil(per_row / 8) * entry;
+            if (pairs > avail / least) pairs = avail / least;
+            cap = (avail - pairs * local) / entry;
+            if ((double)cap > (double)rows_cap * per_row) cap = (uint64_t)((double)rows_cap * per_row);
+            if (pairs == 0) cap = 0;
+        }
+        const uint64_t part_bytes = (whole ? 4ull : 2ull) * D;   // partial output: fp32 of whole cubes, else bf16
+        h->gather_pairs = (uint32_t)(pairs < 0xffffffffull ? pairs : 0xffffffffull);
         h->gather_cap = (uint32_t)cap;
         h->fw_gpair_off = off; off = align_up(off + (size_t)batch * Hq * n_pairs_cap * 5 * 4);
         h->fw_grow_off = off; off = align_up(off + (cap ? rows_cap * 2 * 4 : 0));
         h->fw_gml_off = off; off = align_up(off + (cap ? rows_cap * 8 : 0));
-        h->fw_glocal_off = off; off = align_up(off + (cap && h->C > kBlockTok ? rows_cap * D * 4 : 0));
-        h->fw_gref_off = off; off = align_up(off + (cap && h->C > kBlockTok ? rows_cap * 4 : 0));
+        h->fw_glocal_off = off; off = align_up(off + (cap && whole ? (size_t)pairs * 256 * D * 4 : 0));
+        h->fw_gref_off = off; off = align_up(off + (cap && whole ? rows_cap * 4 : 0));
         h->fw_gitems_off = off; off = align_up(off + (cap ? align_up((n_lists * n_cols * (kGatherClasses + 2) + 2) * 4) + (n_lists * n_cols + cap / 128 + 1) * 16 : 0));
         h->fw_gentries_off = off; off = align_up(off + (size_t)cap * 8);
         h->fw_gparto_off = off; off = align_up(off + (size_t)cap * part_bytes);
@@ -620,6 +639,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             gw.ml_local = (float2*)(ws + h->fw_gml_off);
             gw.local_o = (float*)(ws + h->fw_glocal_off);
             gw.cap_entries = h->gather_cap;
+            gw.cap_pairs = h->gather_pairs;
             gw.n_cols = (int)n_cols;
             gw.n_lists = (int)n_lists;
             gw.n_windows = h->gather_windows;
@@ -639,7 +659,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         const uint32_t* pair_mode_c = gather ? gw.pair_mode : nullptr;
         GatherTiles local_tiles;                   // of pairs whose cubes are gathered whole the local range stays in fp32 for the merge
         std::memset(&local_tiles, 0, sizeof(local_tiles));
-        if (gather && g.C > kBlockTok) local_tiles.part_o = gw.local_o;
+        if (gather && g.C > kBlockTok) { local_tiles.part_o = gw.local_o; local_tiles.pair_place = gw.pair_u; }
         float* row_ref = gather && g.C > kBlockTok ? (float*)(ws + h->fw_gref_off) : nullptr;   // softmax references of the rows of gathered pairs
         const uint32_t* key_norm2_c = frame_begin == 0 ? (const uint32_t*)(ws + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
         mark(h, 5, st);
@@ -675,7 +695,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             const long long n_rows = (long long)g.B * g.Hq * (g.S - g.pos_begin);    // at most: the rows of all pairs
             if (g.C > kBlockTok) {
                 GatherTiles gt;
-                gt.items = gw.items; gt.ctrl = gw.ctrl; gt.entries = gw.entries; gt.part_o = (float*)gw.part_o; gt.part_ml = gw.part_ml; gt.n_cols = gw.n_cols;
+                gt.items = gw.items; gt.ctrl = gw.ctrl; gt.entries = gw.entries; gt.part_o = (float*)gw.part_o; gt.part_ml = gw.part_ml; gt.n_cols = gw.n_cols; gt.pair_place = nullptr;
                 const int ggrid = 2 * (h->sm_count / 2);
                 if (D == 128) ADASPARK_LAUNCH_CUBES(128, true, ggrid, gt, next_pair_tile + 1);
                 else ADASPARK_LAUNCH_CUBES(64, true, ggrid, gt, next_pair_tile + 1);

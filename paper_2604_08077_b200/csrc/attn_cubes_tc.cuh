@@ -46,7 +46,8 @@ struct GatherTiles {
     const uint4* items;          // (column, first entry, entries, 0)
     const uint32_t* ctrl;        // [0] 0: none, [1] items
     const uint32_t* entries;     // token of the call's tensors | head in group << 21
-    float* part_o;               // [entries][D]; (not gathered: the local range of the rows of gathered pairs, [B*Hq*S_cap][D])
+    float* part_o;               // [entries][D]; (not gathered: the local range of the rows of gathered pairs, [place][256][D])
+    const uint32_t* pair_place;  // (not gathered) of a gathered pair, in the order of that buffer
     float2* part_ml;
     int n_cols;                  // columns (cubes) of a list set
 };
@@ -906,14 +907,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
                     }
                     if (lane == 0) tc::mbar_arrive(&sm.out_free[k & 3]);
                 };
-                const bool gathered = !kGathered && pair_mode != nullptr && pair_mode[(size_t)(it.b * g.Hq + it.h) * n_pairs_cap + it.pair] != 0u;
+                const size_t pair_slot = (size_t)(it.b * g.Hq + it.h) * n_pairs_cap + it.pair;
+                const bool gathered = !kGathered && pair_mode != nullptr && pair_mode[pair_slot] != 0u;
                 if constexpr (kGathered) {
                     const int r0 = rank * 128 + quad * 32, n_rows = min(max((int)rows.z - r0, 0), 32);
                     if (lane < n_rows) __stcs(gt.part_ml + rows.y + r0 + lane, make_float2(m_ref, l_fin));
                     store_partials(gt.part_o + (size_t)(rows.y + r0) * D, n_rows);
                 } else if (gathered) {               // the local range of rows whose cubes are gathered whole
-                    const size_t at = (size_t)(it.b * g.Hq + it.h) * g.S_cap + (tile_pos0 + quad * 32);
-                    if (slot_live(g, pr)) ml_local[at + lane] = make_float2(m_ref, l_fin);
+                    if (slot_live(g, pr)) ml_local[(size_t)(it.b * g.Hq + it.h) * g.S_cap + pr] = make_float2(m_ref, l_fin);
+                    const size_t at = (size_t)gt.pair_place[pair_slot] * kPairRows + rank * 128 + quad * 32;
                     store_partials(gt.part_o + at * D, min(max(g.S_cap - (tile_pos0 + quad * 32), 0), 32));
                 } else {
 #pragma unroll 1

@@ -69,7 +69,7 @@ struct GatherWs {
     uint32_t* pair_mode;   // [B*Hq*n_pairs_cap] 0: union path; c + 1: this path, ratio class c
     uint32_t* pair_cnt;    // entries of the pair's rows (0 when the pair stays on the tile kernel)
     uint32_t* pair_off;    // exclusive prefix sum of pair_cnt
-    uint32_t* pair_u;      // key blocks in the pair's union (before its local range)
+    uint32_t* pair_u;      // key blocks in the pair's union (before its local range); from the scan on a kept pair's place in pair_list
     uint32_t* pair_list;   // the pairs on this path, compacted (ctrl[2] of them)
     uint32_t* row_cnt;     // [B*Hq*S_cap] entries of a row
     uint32_t* row_ptr;     // index of the row's first slot in row_slots
@@ -86,8 +86,9 @@ struct GatherWs {
                            // an item of the attention kernel writes one contiguous piece)
     float2* part_ml;       // [cap_entries] (reference exponent in log2 units, sum)
     float2* ml_local;      // [B*Hq*S_cap] the same for the local range, written by the tile kernel
-    float* local_o;        // [B*Hq*S_cap][D] normalised output of the local range, of whole cubes only (else it lies in `out`)
-    uint32_t cap_entries;
+    float* local_o;        // [cap_pairs][256][D] normalised output of the local range, by place in pair_list, of whole cubes only (else
+                           // it lies in `out`)
+    uint32_t cap_entries, cap_pairs;
     int n_cols;            // key blocks that hold video slots: ceil(S_v / 64)
     int n_lists;           // entry lists per key block column set: windows x B x Hkv (each of n_cols lists)
     int n_windows;         // row windows (<= kGatherMaxWindows)
@@ -265,11 +266,13 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
     // ---- which (ratio class, row window) units fit the workspace, and whether they are worth the fixed cost
     __shared__ unsigned long long unit_entries[kGatherClasses][kGatherMaxWindows];
     __shared__ long long unit_gain[kGatherClasses][kGatherMaxWindows];
+    __shared__ uint32_t unit_pairs[kGatherClasses][kGatherMaxWindows];
     __shared__ uint32_t unit_keep[kGatherClasses];          // bit w: window w of the class takes the path
     __shared__ int any_keep_s;
     for (int i = tid; i < kGatherClasses * kGatherMaxWindows; i += 1024) {
         (&unit_entries[0][0])[i] = 0ull;
         (&unit_gain[0][0])[i] = 0ll;
+        (&unit_pairs[0][0])[i] = 0u;
     }
     __syncthreads();
     for (int idx0 = 0; idx0 < n_slots; idx0 += 1024) {
@@ -293,18 +296,21 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
         if (unit >= 0 && (tid & 31) == __ffs(peers) - 1) {
             atomicAdd(&unit_entries[0][0] + unit, (unsigned long long)sum_v);
             atomicAdd(reinterpret_cast<unsigned long long*>(&unit_gain[0][0] + unit), (unsigned long long)(long long)sum_gain);
+            atomicAdd(&unit_pairs[0][0] + unit, (uint32_t)__popc(peers));
         }
     }
     __syncthreads();
     if (tid == 0) {
         unsigned long long tot = 0ull;
         long long gain = 0ll;
+        uint32_t pairs = 0u;
         for (int c = 0; c < kGatherClasses; ++c) {
             uint32_t keep = 0u;
             for (int w = ws.n_windows - 1; w >= 0; --w) {
                 const unsigned long long e = unit_entries[c][w];
-                if (e == 0ull || tot + e > (unsigned long long)ws.cap_entries) continue;
+                if (e == 0ull || tot + e > (unsigned long long)ws.cap_entries || pairs + unit_pairs[c][w] > ws.cap_pairs) continue;
                 tot += e;
+                pairs += unit_pairs[c][w];
                 gain += unit_gain[c][w];
                 keep |= 1u << w;
             }
@@ -337,7 +343,10 @@ __global__ void __launch_bounds__(1024) gather_scan_kernel(Geom g, GatherWs ws) 
         const uint32_t ex = cta_exclusive_scan_1024(v, warp_sums, &total_s);
         if (idx < n_slots) ws.pair_off[slot] = (uint32_t)(carry + ex);
         const uint32_t exl = cta_exclusive_scan_1024(v != 0u ? 1u : 0u, warp_sums, &total_s2);
-        if (idx < n_slots && v != 0u) ws.pair_list[n_on + exl] = (uint32_t)slot;
+        if (idx < n_slots && v != 0u) {
+            ws.pair_list[n_on + exl] = (uint32_t)slot;
+            ws.pair_u[slot] = n_on + exl;
+        }
         n_on += total_s2;
         carry += total_s;
     }
@@ -915,7 +924,7 @@ __global__ void __launch_bounds__(256) gather_merge_kernel(Geom g, GatherWs ws, 
         float acc[8];
         float M = loc.x, W = loc.y;                                // the local range always has a visible key
         if constexpr (kWholeCubes) {
-            const float4* lo = reinterpret_cast<const float4*>(ws.local_o + row * D) + 2 * sub;
+            const float4* lo = reinterpret_cast<const float4*>(ws.local_o + (size_t)idx * D) + 2 * sub;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const float4 x = __ldcs(lo + k);

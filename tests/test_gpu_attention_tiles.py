@@ -118,6 +118,28 @@ def test_gathered_cubes(cube, T, H, W, D, top_k):
     assert torch.equal(out, again)
 
 
+@pytest.mark.parametrize("cube, D, shares", [((2, 8, 8), 128, (6, 3, 1)), ((4, 8, 8), 64, (6, 3, 1))])
+def test_gathered_cubes_in_small_budgets(cube, D, shares):
+    """A budget bounds entries and the local range of gathered pairs, whose places are counted: what fits is gathered, the rest takes the
+    union path."""
+    wl = inputs.make_prefill("budget", seed=56, B=2, T=64, H=16, W=16, cube=cube, n_text=61, Hq=8, Hkv=2, D=D, top_p=0.5, offset_std=2.5)
+    full, want, bitmap, _ = pu.run_forward(wl, prefill_kernel=1, gather=60.0)
+    pairs = full.header().gather_pair_tiles
+    assert pairs > 0.8 * wl.B * wl.Hq * (wl.S // 256)
+    entry = 4 * D + 16
+    got = []
+    for share in shares:                                   # tenths of what the gathered rows need
+        rows = pairs * 256
+        need = rows * 4 * D + full.header().gather_entries // (wl.C // 64) * entry
+        eng, out, bm, count = pu.run_forward(wl, prefill_kernel=1, gather=60.0, gather_budget=need * share // 10)
+        hdr = eng.header()
+        assert hdr.status == 0
+        got.append(hdr.gather_pair_tiles)
+        assert torch.equal(bm, bitmap) and eng.layout.forward_workspace_bytes < full.layout.forward_workspace_bytes
+        pu.compare_rows(wl, pu.sample_rows(wl, 300, seed=share, whole_tiles=[(1, 3, 100)]), out, bm, count, label=f"{share} tenths")
+    assert pairs > got[0] > got[-1] and got[0] > 0, (pairs, got)
+
+
 @pytest.mark.parametrize("cube, D", [((2, 8, 8), 64), ((2, 8, 8), 128), ((4, 8, 8), 128), ((8, 8, 8), 64)])
 def test_many_gathered_items(cube, D):
     """Thousands of items of one, two and four steps: the warpgroups run several items apart."""

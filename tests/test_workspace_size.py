@@ -1,4 +1,4 @@
-"""How large a forward workspace has to be.
+"""How large a forward workspace has to be at least: no larger than the library ever asked for.
 
 The scores of the tensor-core selection lie in the place of the query-gather buffers and give way when the caller's
 workspace is smaller than the library asks for: it is taken down to the size that held the fp64 kernel's score rows
@@ -23,6 +23,20 @@ SIZES = [
     ((16, 512, 16, 16, (4, 4, 4), 512, 28, 4, 128, 0.9, 0, 0), 15618092288),
     ((3, 8, 8, 8, (4, 4, 4), 5, 4, 4, 64, 0.9, 7, 0), 1082112),
 ]
+# cubes of more than 64 tokens, whose partial results and local range are fp32: the bytes that the entries of single key blocks take, so
+# that the budget bounds them too; and more heads than the words kept for each fill up to a multiple of 256 bytes
+LARGE = [
+    ((1, 64, 16, 16, (4, 8, 8), 128, 28, 4, 128, 0.7, 0, 100 << 20), 115393792),
+    ((1, 256, 16, 16, (4, 8, 8), 256, 28, 4, 128, 0.7, 0, 100 << 20), 202591232),
+    ((1, 512, 16, 16, (4, 8, 8), 0, 28, 4, 128, 0.7, 0, 100 << 20), 423151104),
+    ((1, 512, 16, 16, (4, 8, 8), 0, 28, 4, 128, 0.7, 0, 24 << 30), 25366270976),
+    ((1, 64, 16, 16, (2, 8, 8), 128, 16, 4, 64, 0.9, 0, 24 << 30), 585576192),
+    ((2, 30, 14, 14, (8, 8, 8), 98, 16, 2, 128, 0.7, 0, 1 << 30), 586249472),
+    ((1, 16, 8, 8, (16, 8, 8), 5, 4, 4, 64, 0.9, 3, 1 << 20), 930816),
+    ((1, 384, 8, 8, (4, 8, 8), 201, 16, 2, 128, 0.7, 0, 24 << 30), 2499828480),
+    ((5, 8, 8, 8, (4, 4, 4), 5, 4, 4, 64, 0.9, 0, 0), 1089792),
+    ((21, 8, 8, 8, (4, 4, 4), 5, 8, 1, 64, 0.9, 0, 0), 1884160),
+]
 
 
 def _handle(B, T, H, W, cube, n_text, Hq, Hkv, D, top_p, top_k, budget):
@@ -33,7 +47,7 @@ def _handle(B, T, H, W, cube, n_text, Hq, Hkv, D, top_p, top_k, budget):
 
 
 @pytest.mark.skipif(torch.cuda.is_available(), reason="looks at the order of the host's checks, with pointers that are none")
-@pytest.mark.parametrize("sizes,nbytes", SIZES)
+@pytest.mark.parametrize("sizes,nbytes", SIZES + LARGE)
 def test_a_workspace_without_room_for_the_scores_is_taken(sizes, nbytes):
     hd, _ = _handle(*sizes)
     fake = 0x1000
