@@ -96,9 +96,10 @@ typedef struct {
     uint32_t max_tile_kv_blocks;  /* prefill: largest number of 64-key blocks one 256-row pair of
                                      query tiles visited (load imbalance: compare with the mean
                                      executed_kv_blocks / 2 / number of pair tiles)           */
-    uint32_t gather_entries;      /* prefill: (query row, 64-key block) entries computed by the
+    uint32_t gather_entries;      /* prefill: (query row, 64-key block) pairs computed by the
                                      query-gather path (0: every pair took the union path)     */
-    uint32_t gather_items;        /* ... in this many items of up to 128 gathered rows          */
+    uint32_t gather_items;        /* ... in this many items of up to 128 gathered rows (cubes of
+                                     more than 64 tokens: up to 256 rows and a whole cube)      */
     uint32_t gather_pair_tiles;   /* ... for this many 256-row pairs of query tiles             */
     uint32_t reserved2;
 } adaspark_attn_workspace_header_t;

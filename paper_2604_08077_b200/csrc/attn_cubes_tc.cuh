@@ -9,7 +9,7 @@
 //                                   every entry.  Items are short (C / 128 steps), so what bounds it are the steps between items: 5500
 //                                   to 7000 cycles for one of two steps, 2100 of them tensor core
 // It is a source of its own because it costs the other kernel registers: both in one template ran 16384 tokens 1.5 %, ragged grids
-// 2 % slower (softmax warps of 144 registers, 70 spilled bytes for 20).  What a call of 256-token cubes gains by it: 24576 tokens,
+// 2 % slower (softmax warps of 144 registers, which spill either way).  What a call of 256-token cubes gains by it: 24576 tokens,
 // 16 heads, p 0.7 2.15 -> 1.78 ms; 65536, 28 heads 25.5 -> 17.1.
 #pragma once
 #include "attn_prefill_tc.cuh"

@@ -15,7 +15,7 @@
 //
 // Which pairs of query tiles take this path is decided on the device, per pair, from the counts the selection
 // left: entries of the pair's rows (P) against key blocks in the pair's union (U), gathered iff
-// P <= pairs_per_block * U -- provided the qualifying pairs fit the workspace (else part of them, see
+// P <= pairs_per_block * U (P times gather_entry_cost, where whole cubes are gathered) -- provided the qualifying pairs fit the workspace (else part of them, see
 // kGatherClasses) and together save more than the path costs (kGatherMinGain).  The query rows are cut into a
 // few row windows, and every (window, batch, kv head, key block) has its own entry list: the items of a window
 // gather from a slice of Q that stays in L2.  Kernels, in launch order:
@@ -77,7 +77,7 @@ struct GatherWs {
                            // pairs they come from; zero at the start of a forward
     uint32_t* col_cur;     // [kGatherClasses][...] fill cursors; zero at the start of a forward
     uint32_t* col_roff;    // [kGatherClasses][...] first entry of the set's share of the block's list
-    uint32_t* col_off;     // [lists * n_cols + 1] first entry of the block's list (exclusive prefix sum)
+    uint32_t* col_off;     // [lists * n_cols + 1] first entry of the column's list (exclusive prefix sum)
     uint32_t* col_item;    // [lists * n_cols + 1] first work item of the list
     uint4* items;          // (key block column, first entry, entries (<= item_rows), 0)
     uint32_t* entries;     // per key block, its entries: row of the call's tensors | head in group << 21 | cube bits << 25
@@ -89,7 +89,7 @@ struct GatherWs {
     float* local_o;        // [cap_pairs][256][D] normalised output of the local range, by place in pair_list, of whole cubes only (else
                            // it lies in `out`)
     uint32_t cap_entries, cap_pairs;
-    int n_cols;            // key blocks that hold video slots: ceil(S_v / 64)
+    int n_cols;            // columns of an entry list set: key blocks that hold video slots, ceil(S_v / 64); cubes above 64 tokens: cubes
     int n_lists;           // entry lists per key block column set: windows x B x Hkv (each of n_cols lists)
     int n_windows;         // row windows (<= kGatherMaxWindows)
     int pairs_per_window;  // The query rows are cut into windows of this many pairs of tiles and every (window,

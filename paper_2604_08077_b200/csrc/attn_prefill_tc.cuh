@@ -54,7 +54,7 @@ constexpr int kRefSlots = 4;          // a warpgroup is at most three steps behi
 // Reference of a row's softmax fixed in advance: the bound B of its scores (log2 units; every score lies in [-B, B]), up to this B.
 // Every weight 2^(s - B) is at least 2^-2B = 2^-96: nothing underflows, and 30 binades remain above the smallest normal fp32 for
 // the products with V.  Not beyond: the largest weights of a row, 1 or a power of two near it on the running maximum, are any numbers with
-// a fixed reference and lose up to 2^-9 each in bf16.  References up to B = 88 (96 - B) and in later chunks gained 7 % on a chunk, but
+// a fixed reference and lose up to 2^-9 each in bf16.  References up to B = 88 (96 - B) and in later chunks gained 8 % on a chunk, but
 // their error against 64 bits was up to 5 % larger (sharp queries, p 0.95: 0.00226 -> 0.00234; a chunk 0.00232 -> 0.00235).
 constexpr float kFixedRefMax = 48.f;
 // |q|^2, largest |k|^2 of the head: infinite, not in advance

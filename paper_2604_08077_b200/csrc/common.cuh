@@ -217,11 +217,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
 // 2^x on the FMA pipe, for part of a softmax row's exponentials when the MUFU unit (4 lanes per
 // scheduler: 8 cycles per warp instruction) is the busier pipe.  x = n + f with n = round(x), f in
 // [-0.5, 0.5]: a cubic for 2^f (minimax in relative error over that interval, 7.7e-5: far inside the
-// bf16 rounding of the probabilities it feeds), n added to the exponent field.  x is clamped at -125,
-// so a masked score (-inf) yields about 2^-125 = 2e-38 instead of 0: next to any visible key (weight
-// >= 2^-8 of the row's reference) that is nothing in an fp32 sum, and it is multiplied by 0 when the
-// row meets its first visible key.  (An exact zero costs one more instruction per element, which
-// measurably undoes the gain.)
+// bf16 rounding of the probabilities it feeds; with one in eight of them the error of the output against 64 bits is the same to
+// seven digits as with ex2 throughout), n added to the exponent field.  x is clamped at -125, so a masked score (-inf) yields
+// 2^-125 instead of 0 (an exact zero costs one more instruction per element, which measurably undoes the gain).  What that adds to a
+// row: with a reference fixed in advance a visible weight is at least 2^-96, and of at most 2^21 masked keys one in eight comes here:
+// 2^18 * 2^-125 = 2^-107, 2^-11 of even a lone visible key of the smallest weight there can be, against the 2^-9 of its rounding to
+// bf16.  On the running maximum the largest weight of a row is at least 1, and what was added before the first visible key is
+// multiplied by 0 there.
 __device__ __forceinline__ float fma_exp2(float x) {
     const float xc = fmaxf(x, -125.f);
     const float xr = xc + 12582912.f;                  // 1.5 * 2^23: the low mantissa bits now hold n

@@ -118,6 +118,35 @@ def test_gathered_cubes(cube, T, H, W, D, top_k):
     assert torch.equal(out, again)
 
 
+# Rows of whole gathered cubes on the running maximum (2, 4: every bound above 48), and at 1.4 rows with a reference fixed in advance beside
+# rows without one in a warp of an item; values that leave little room.
+@pytest.mark.parametrize("scale_q, scale_v", [(1.4, 1.0), (2.0, 2.0 ** 40), (4.0, 1.0), (4.0, 2.0 ** 110)])
+@pytest.mark.parametrize("cube, D", [((2, 8, 8), 64), ((4, 8, 8), 128), ((8, 8, 8), 128)])
+def test_gathered_cubes_softmax_references(cube, D, scale_q, scale_v):
+    base = inputs.small_prefill(seed=58, T=24, H=16, W=8, cube=cube, n_text=21, Hq=4, Hkv=2, D=D, top_p=0.8, offset_std=1.0)
+    wl, v = scaled(base, scale_q, scale_v)
+    eng = pu.make_engine(wl, prefill_kernel=1, gather=pu.FORCE_GATHER)
+    q, k, v = wl.q.cuda(), wl.k.cuda(), v.cuda()
+    out, bitmap, count = eng.forward(q, k, v, wl.n_text, want_selection=True)
+    torch.cuda.synchronize()
+    hdr = eng.header()
+    assert hdr.status == 0 and hdr.gather_entries > 0
+    rows = oracle.all_rows(oracle.shape_of(wl))
+    pu.compare_rows(wl, rows, out.float() / scale_v, bitmap, count, label=f"{cube} {scale_q} {scale_v}")
+    again = eng.forward(q, k, v, wl.n_text)[0]
+    torch.cuda.synchronize()
+    assert torch.equal(out, again)
+    outs, entries = [], 0                                  # later chunks: no row has a reference
+    for fb, fc, nt in [(0, 8, -1), (8, 16, wl.n_text)]:
+        lo, hi = fb * 128, (fb + fc) * 128 + max(nt, 0)
+        outs.append(eng.forward_chunk(q[:, lo:hi].contiguous(), k[:, lo:hi].contiguous(), v[:, lo:hi].contiguous(), fb, fc, nt)[0])
+        torch.cuda.synchronize()
+        assert eng.header().status == 0
+        entries += eng.header().gather_entries
+    assert entries > 0
+    pu.compare_rows(wl, rows, torch.cat(outs, 1).float() / scale_v, bitmap, count, label=f"chunks {cube} {scale_q} {scale_v}")
+
+
 @pytest.mark.parametrize("cube, D, shares", [((2, 8, 8), 128, (6, 3, 1)), ((4, 8, 8), 64, (6, 3, 1))])
 def test_gathered_cubes_in_small_budgets(cube, D, shares):
     """A budget bounds entries and the local range of gathered pairs, whose places are counted: what fits is gathered, the rest takes the
