@@ -187,9 +187,9 @@ bool set_smem(adaspark_attn* h, K kernel, size_t bytes, const char* what) {
 }
 
 #ifdef ADASPARK_WITH_TCGEN05
-// Kernel shape for up to n candidates a row: lanes per row x scores per lane = 8 x 8, 8 x 16, 8 x 32, 16 x 32, 32 x 32,
-// 32 x 64, 32 x 128.  A shape costs by the scores it has room for as much as by those it holds (registers, and with them
-// warps on an SM): 8 x 32 for 64 candidates took 0.29 instead of 0.23 ms (16384 tokens, 28 heads, 64 cubes).
+// Kernel shape for up to n candidates a row: rows per pass x scores = 16 x 64, 8 x 128, 8 x 256, 4 x 512, 2 x 1024, 1 x 2048,
+// 1 x 4096.  A shape costs by the scores it has room for as much as by those it holds (shared memory, and with it warps on an
+// SM): 8 x 256 where 8 x 128 would do took 86 instead of 48 us (16384 tokens, 28 heads, the tiles of up to 128 candidates).
 int select_shape(int n) { return n <= 64 ? 0 : n <= 128 ? 1 : n <= 256 ? 2 : n <= 512 ? 3 : n <= 1024 ? 4 : n <= 2048 ? 5 : 6; }
 
 // Could the query-gather path save what it costs, whatever the rows select?  Its estimate (gather_scan_kernel) for a
@@ -483,7 +483,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         }
         int32_t* fallback_rows = (int32_t*)(ws + h->fw_fallback_off);
         const bool all = g.top_k <= 0 && !(g.top_p < 1.0);
-        const bool small = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 3 * kScoreWave / 2;   // the selection kernel's 444 CTAs fit the chip at once (in the shapes for up to 1024 candidates)
+        const bool small = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 3 * kScoreWave / 2;   // a call whose selection is about one wave
         auto launch_exact = [&](const int32_t* rows, const uint32_t* n_list, long long n_ids) {
             if (D == 128)
                 launch_kernel(small, select_exact_kernel<128>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
@@ -530,21 +530,21 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
                 if (D == 128) ADASPARK_LAUNCH_SCORE(128); else ADASPARK_LAUNCH_SCORE(64);
 #undef ADASPARK_LAUNCH_SCORE
                 if (!launch_ok(h, "score_tc_kernel")) return ADASPARK_ERR_CUDA;
-#define ADASPARK_LAUNCH_SELECT(GG, KK, RES, RULE)                                                                     \
+#define ADASPARK_LAUNCH_SELECT(RR, CC, BB, RULE)                                                                       \
     do {                                                                                                               \
-        const size_t smem = select_smem_bytes(sizeof(SelectWarpSmem<GG, KK>), g.n_words);                              \
-        if (!set_smem(h, select_nucleus_kernel<GG, KK, RES, RULE>, smem, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA; \
-        launch_kernel(small, select_nucleus_kernel<GG, KK, RES, RULE>, dim3(2 * (next - first)), dim3(kSelectThreads), \
-                      smem, st, g, select_target(RULE, g.top_p, GG * KK, GG * KK <= 256 ? 22 : GG * KK <= 1024 ? 21 : GG * KK <= 2048 ? 20 : 19), \
-                      item0, first, (const float*)scores, (const float4*)row_range, (const float*)row_err, tile_mask,  \
+        const size_t smem = sizeof(SelectSmem<RR, CC, BB>);                                                            \
+        const int warp_rows = small ? (RR < 8 ? 8 : RR) : 32;      /* few tiles: as many warps as there can be */      \
+        launch_kernel(small, select_nucleus_kernel<RR, CC, BB, RULE>, dim3(kTileRows / warp_rows * (next - first)), dim3(32), \
+                      smem, st, g, select_target(RULE, g.top_p, CC, CC <= 256 ? 22 : CC <= 1024 ? 21 : CC <= 2048 ? 20 : 19), \
+                      item0, first, warp_rows, (const float*)scores, (const float4*)row_range, (const float*)row_err, tile_mask,  \
                       tile_union, (const unsigned long long*)key_hash, sel_bitmap, sel_count, fallback_rows,           \
                       &hdr->fallback_rows);                                                                            \
     } while (0)
-#define ADASPARK_LAUNCH_SELECT_K(GG, KK, RES)                                                                         \
+#define ADASPARK_LAUNCH_SELECT_K(RR, CC, BB)                                                                          \
     do {                                                                                                               \
-        if (by_count) ADASPARK_LAUNCH_SELECT(GG, KK, RES, kCount);                                                     \
-        else if (g.top_p < 0.5) ADASPARK_LAUNCH_SELECT(GG, KK, RES, kHead);                                            \
-        else ADASPARK_LAUNCH_SELECT(GG, KK, RES, kTail);                                                               \
+        if (by_count) ADASPARK_LAUNCH_SELECT(RR, CC, BB, kCount);                                                      \
+        else if (g.top_p < 0.5) ADASPARK_LAUNCH_SELECT(RR, CC, BB, kHead);                                             \
+        else ADASPARK_LAUNCH_SELECT(RR, CC, BB, kTail);                                                                \
     } while (0)
                 // Candidate counts fall with the items (late tiles come first): runs of items of one kernel shape, a run
                 // of less than eight tiles per SM joins its neighbour.  A launch at every change of shape instead: 0.359 for
@@ -559,13 +559,13 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
                     }
                     next = next < n_here ? next : n_here;
                     switch (largest) {
-                        case 0: ADASPARK_LAUNCH_SELECT_K(8, 8, 5); break;
-                        case 1: ADASPARK_LAUNCH_SELECT_K(8, 16, 4); break;
-                        case 2: ADASPARK_LAUNCH_SELECT_K(8, 32, 3); break;
-                        case 3: ADASPARK_LAUNCH_SELECT_K(16, 32, 3); break;
-                        case 4: ADASPARK_LAUNCH_SELECT_K(32, 32, 3); break;
-                        case 5: ADASPARK_LAUNCH_SELECT_K(32, 64, 2); break;
-                        default: ADASPARK_LAUNCH_SELECT_K(32, 128, 1);
+                        case 0: ADASPARK_LAUNCH_SELECT_K(16, 64, 64); break;
+                        case 1: ADASPARK_LAUNCH_SELECT_K(8, 128, 128); break;
+                        case 2: ADASPARK_LAUNCH_SELECT_K(8, 256, 128); break;
+                        case 3: ADASPARK_LAUNCH_SELECT_K(4, 512, 256); break;
+                        case 4: ADASPARK_LAUNCH_SELECT_K(2, 1024, 512); break;
+                        case 5: ADASPARK_LAUNCH_SELECT_K(1, 2048, 512); break;
+                        default: ADASPARK_LAUNCH_SELECT_K(1, 4096, 512);
                     }
                     if (!launch_ok(h, "select_nucleus_kernel")) return ADASPARK_ERR_CUDA;
                 }

@@ -1,9 +1,9 @@
-// K3b: nucleus selection (Eq. 2) from the scores of score_tc.cuh, G lanes of a warp per query row.
+// K3b: nucleus selection (Eq. 2) from the scores of score_tc.cuh, R query rows at a time per warp.
 //
 // Scores s_j are in log2 units; the order is descending score, then ascending cube index, the mass of a cube is
-// 2^(s_j - max).  A row's scores stay in registers (kK per lane) and are swept twice:
+// 2^(s_j - max).  A row's scores lie in shared memory and are swept twice by its 32 / R lanes:
 //   sweep 1  masses are added to the row's total Z and, quantised, to a histogram over the distance from the maximum
-//            in shared memory (16 G buckets from the largest score to the smallest): the bucket in which the cumulative
+//            in shared memory (from the largest score to the smallest): the bucket in which the cumulative
 //            mass crosses p Z is found from it
 //   sweep 2  cubes before that bucket are selected (one bit each, collected from the sign of a subtraction) and their
 //            exact mass is summed; the few cubes inside it (widened by kGuard at both ends) are listed, and each
@@ -29,14 +29,19 @@
 // proportion to Z left 0.7 / 2.1 / 5.5 % undecided at p = 0.99 / 0.999 / 0.9999, 65536 tokens).  With them go the rows the score
 // kernel marked, and rows with more equal scores at the boundary than the list holds.
 //
-// What bounds it: instruction issue at few candidates (about 20 instructions per score of a lane in the two sweeps and 900
-// per pass of 32 / G rows beside them; 1390 per pass with 128 to 256 candidates, issue slots 63 % used, 1000 with fewer, 80 %),
-// the stream of scores from memory at many (4 bytes per pair).  Sharing a warp among
-// 32 / G rows spreads the second figure over several rows; the per-cube work is spread over the pipes (the bits come
-// from funnel shifts of signs, the mass before the bucket from a saturating multiply, the exponential from the MUFU unit,
-// the rest from packed fp32 pairs), because the integer / comparison pipe issues at half the rate of the fp32 pipe.
-// Measured, scoring and selection together, 28 heads, against one kernel that recomputed the scores in every pass: 0.78 ->
-// 0.354 ms at 16384 tokens and 256 cubes, 13.6 -> 4.4 at 65536 and 1024, 59.5 -> 25.3 at 131072 and 2048, half static.
+// What bounds it: latency and instruction issue (12 to 22 warps on an SM, as many as the scores of their rows leave room for): about
+// 13 instructions per score of a lane in the two sweeps and 700 to 1200 per pass of R rows beside them.  Lane = row + R x (which
+// of the row's lanes): the histogram [bucket][row] is met by neighbouring lanes in different banks, the bits of 8 columns are a
+// byte of the mask words without an exchange, and what is done per row (boundary, list, order of the list) is done for R rows at
+// once.  (With the lanes side by side on 1 to 4 rows per pass and the scores in registers, 1000 to 1400 instructions a pass, shuffles
+// for every row sum and nibbles transposed between lanes: selection kernels alone, us, before / now: 64 candidates 105 / 53, 128 to
+// 256 120 / 86 (28 heads, 16384 tokens), 1024 1683 / 1263 (65536 tokens), 2048 13470 / 8950 (131072, half static).)  The per-cube work
+// is spread over the pipes: the bits come from funnel shifts of signs, the mass before the bucket from a saturating multiply, the
+// exponential from the MUFU unit, the rest from packed fp32 pairs, because the integer / comparison pipe issues at half the
+// rate of the fp32 pipe.
+// Rows per pass: twice as many (half as many warps on the SM) 72 / 121 / 1442 / 13973 us for the figures above; CTAs of 4 warps that
+// share 8 or 16 rows and meet at barriers 136 / 124 / 1494 / 12280; scores read from global memory in both sweeps instead of staged
+// 76 / 137 / 1822.  Buckets: half as many 1240 at 1024 candidates but 2910 for 2600 with static frames, whose scores lie in clumps.
 #pragma once
 #include <cmath>
 #include <cstring>
@@ -45,14 +50,11 @@
 
 namespace adaspark {
 
-constexpr int kSelectThreads = 256;
-constexpr int kSelectRows = 8;           // consecutive rows of a warp: its mask words fill 32-byte sectors
-constexpr int kSelectWarps = kSelectThreads / 32;
 constexpr int kSelectCand = 32;          // cubes of the crossing bucket a row may list
 constexpr int kMaxHistLevels = 8;        // histograms of a row before it is handed to the fp64 kernel
 constexpr float kUlp = 5.9604645e-8f;    // 2^-24: the largest relative error of a rounding
 constexpr float kGuard = 1e-3f;          // of a bucket
-constexpr int kSumSteps = 8;             // steps of a lane (2 additions each) whose masses are summed before they join the rest
+constexpr int kSumIters = 4;             // chunks of a thread (4 additions each) whose masses are summed before they join the rest
 enum SelectRule { kHead, kTail, kCount };                 // Top-p from the front and from the other end, Top-K
 
 // What a row is decided by (the same for all rows of a launch).
@@ -84,478 +86,489 @@ inline SelectTarget select_target(SelectRule rule, double top_p, int capacity, i
     return t;
 }
 
-// Lanes per row grow with the candidate count, and the buckets with the lanes: a bucket holds at most about 5 of 256
-// cubes (G = 8), 512 (16) or 1024 (32) with normally distributed scores.
-// Shared memory of one warp; its mask words [n_words][8 rows] follow those of all warps.
-template <int G, int kK>
-struct SelectWarpSmem {
-    float rows[32 / G][G * kK];                           // scores of the rows of a pass
-    float4 range[32 / G][2];                              // partial ranges of the rows of a pass
-    uint32_t hist[512];                                   // [bucket][row of the warp]
-    float4 cand[32 / G][kSelectCand];                     // score, mass, cube
-    float err[2][32 / G];                                 // row_err of this pass and of the next
-    int32_t count[32 / G];
+// Shared memory of a warp on R rows of up to kCols scores (a bucket holds some 5 of them, with normally distributed scores).  The padding of a row keeps the 16-byte loads of 8 neighbouring
+// lanes (8 rows, or with fewer rows several chunks of each, see `swap`) in 8 different bank groups.
+template <int R, int kCols, int kBuckets>
+struct SelectSmem {
+    static constexpr int kOut = R < 8 ? 8 : R;            // rows whose mask words leave together: whole 32-byte sectors
+    float rows[R][kCols + (R == 4 || R == 2 ? 8 : 4)];
+    union {
+        uint32_t hist[kBuckets][R];
+        float4 cand[kSelectCand][R];                      // score, mass, cube; once the histogram has been read
+    };
+    uint32_t words[kCols / 32][kOut];
 };
-__host__ __device__ inline size_t select_smem_bytes(size_t warp_bytes, int n_words) {
-    return kSelectWarps * (warp_bytes + (size_t)n_words * kSelectRows * 4);
-}
 
 __device__ __forceinline__ float sat_fma(float a, float b, float c) {     // min(max(a b + c, 0), 1)
     return __saturatef(fmaf(a, b, c));
 }
 
-// One warp per 8 rows of a tile, warps work on their own: 2 CTAs per item, items [first, ..) of those that the scores were
-// computed for.  scores / row_range / row_err: what score_tc_kernel left for the items [item0, ..).
+// One warp per CTA and `warp_rows` rows (8, 16 or 32, at least R): 128 / warp_rows CTAs per item, items [first, ..) of those that
+// the scores were computed for.  scores / row_range / row_err: what score_tc_kernel left for the items [item0, ..).
 // tile_mask as mask_index() describes; tile_union (cleared) receives the OR of each word over the tile's rows;
 // fallback_rows[0 .. *fallback_count) receives ((b*Hq+h)*n_tiles_cap + tile)*128 + r of the rows left to the fp64
-// kernel.  G * kK >= the largest candidate count of these items.
-template <int G, int kK, int kResident, SelectRule kRule>
-__global__ void __launch_bounds__(kSelectThreads, kResident) select_nucleus_kernel(
-    Geom g, SelectTarget rule, int item0, int first, const float* scores, const float4* row_range, const float* row_err, uint32_t* tile_mask, uint32_t* tile_union,
-    const unsigned long long* key_hash, uint32_t* sel_bitmap, int32_t* sel_count, int32_t* fallback_rows, uint32_t* fallback_count) {
+// kernel.  kCols >= the largest candidate count of these items.
+template <int R, int kCols, int kBuckets, SelectRule kRule>
+__global__ void __launch_bounds__(32) select_nucleus_kernel(
+    Geom g, SelectTarget rule, int item0, int first, int warp_rows, const float* scores, const float4* row_range, const float* row_err, uint32_t* tile_mask,
+    uint32_t* tile_union, const unsigned long long* key_hash, uint32_t* sel_bitmap, int32_t* sel_count, int32_t* fallback_rows, uint32_t* fallback_count) {
     extern __shared__ __align__(16) unsigned char select_raw[];
-    constexpr int R = 32 / G, kBuckets = 16 * G, kSteps = kK / 4;          // rows per warp; steps of 4 columns per lane
-    constexpr int kMasks = (kK + 31) / 32;                                 // bit words per lane
+    constexpr int U = 32 / R;                                              // lanes of a row
+    constexpr int kIter = kCols / (8 * U), kMasks = (kIter + 3) / 4;       // chunks of 8 columns per lane; bit words
     constexpr bool kByCount = kRule == kCount, tail = kRule == kTail;
-    constexpr int kBlocks = (kSteps + kSumSteps - 1) / kSumSteps;
-    constexpr int kAdds = kK / 2 / kBlocks + kBlocks + (G == 8 ? 3 : G == 16 ? 4 : 5);    // a mass passes through, in a row's sum
+    constexpr int kLaneSteps = R == 32 ? 0 : R == 16 ? 1 : R == 8 ? 2 : R == 4 ? 3 : R == 2 ? 4 : 5;     // additions that join the lanes of a row
+    constexpr int kBlocks = (kIter + kSumIters - 1) / kSumIters;
+    constexpr int kAdds = (kIter < kSumIters ? 4 * kIter : 4 * kSumIters) + kBlocks + 2 + kLaneSteps;    // a mass passes through, in a row's sum (at least 8 + those of the lanes)
     constexpr uint32_t kFull = 0xffffffffu;
+    constexpr uint32_t kRowLanes = R == 32 ? 1u : R == 16 ? 0x10001u : R == 8 ? 0x01010101u : R == 4 ? 0x11111111u : R == 2 ? 0x55555555u : kFull;   // of row 0
     constexpr float kMagic = 8388608.f;                                    // 2^23: low mantissa bits = the integer part
     constexpr uint32_t kMagicBits = 0x4B000000u;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int s = lane & (G - 1), row_w = lane / G;                        // lane inside the row's group, row of the warp
-    const int item = first + (blockIdx.x >> 1), row0 = ((blockIdx.x & 1) * kSelectWarps + warp) * kSelectRows;   // first row of the warp
+    static_assert(kIter * 8 * U == kCols && kCols % 64 == 0 && kIter >= 2, "shape");
+    using Smem = SelectSmem<R, kCols, kBuckets>;
+    constexpr int kOut = Smem::kOut;
+    const int lane = threadIdx.x, row = lane % R, u = lane / R;            // row of the pass, which of its lanes
+    const int per_item = kTileRows / warp_rows;
+    const int item = first + blockIdx.x / per_item, row_begin = (blockIdx.x % per_item) * warp_rows;
     const ScoreItem w = score_item(g, item0 + item);
     const size_t gt_cap = (size_t)(w.b * g.Hq + w.h) * g.n_tiles_cap + w.tile;
     const int n_words_live = min(2 * w.n_ct, g.n_words);                   // words that can hold a candidate
-    SelectWarpSmem<G, kK>& sm = reinterpret_cast<SelectWarpSmem<G, kK>*>(select_raw)[warp];
-    uint32_t* words = reinterpret_cast<uint32_t*>(select_raw + kSelectWarps * sizeof(SelectWarpSmem<G, kK>)) + (size_t)warp * g.n_words * kSelectRows;
-    uint32_t* hist = sm.hist;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = lane; i < n_words_live * kSelectRows; i += 32) words[i] = 0u;
-    __syncwarp();
+    Smem& sm = *reinterpret_cast<Smem*>(select_raw);
+    uint32_t* hist = &sm.hist[0][0];
+    auto clear_hist = [&]() {
+#pragma unroll 8
+        for (int i = lane; i < kBuckets * R / 4; i += 32) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    };
+    clear_hist();
     launch_dependents();
     wait_for_previous_kernel();
 
     constexpr float a_add0 = tail ? (float)(kBuckets - 1) : 0.f;
-    auto group_sum = [&](float x) -> float {
+    // Scores and range of a pass, requested as soon as those of the pass before are no longer read.  All rows of the pass are
+    // copied up to the largest candidate count among them (what a row does not have is not looked at).
+    float4 ra, rb;
+    float err_next;
+    auto request = [&](int r0) -> int {
+        const int pos = w.tile * kTileRows + r0 + row;
+        const int n = slot_live(g, pos) ? n_candidates(g, pos) : 0;
+        const int n4 = (__reduce_max_sync(kFull, n) + 3) >> 2;
+        constexpr int kLanes = kCols / 4 < 32 ? kCols / 4 : 32, kRowsAtOnce = 32 / kLanes;
+        const size_t srow0 = (size_t)item * kTileRows + r0;
+        const float* src = scores + (srow0 + lane / kLanes) * g.N_ld;
+        float* dst = sm.rows[lane / kLanes];
+#pragma unroll 1
+        for (int c = lane % kLanes; c < n4; c += kLanes) {
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-        return x;
-    };
-    auto group_any = [&](bool p) -> bool {
-        const uint32_t m = __ballot_sync(kFull, p);
-        return ((G == 32 ? m : (m >> (row_w * G)) & ((1u << (G & 31)) - 1u))) != 0u;
-    };
-    // The scores of a pass come through shared memory, requested while the pass before is still being decided (a warp
-    // that loaded them when it needed them spent half of its time waiting, with 32 warps on the SM).
-    auto candidates = [&](int pass) -> int {
-        const int pos = w.tile * kTileRows + row0 + pass * R + row_w;
-        return slot_live(g, pos) ? n_candidates(g, pos) : 0;
-    };
-    auto request = [&](int pass, int n) {
-        const size_t srow = (size_t)item * kTileRows + row0 + pass * R + row_w;
-        const float* src = scores + srow * g.N_ld + 4 * s;
-        float* dst = &sm.rows[row_w][4 * s];
-#pragma unroll
-        for (int c = 0; c < kSteps; ++c)
-            if (c * 4 * G + 4 * s < n) cp_async_16(dst + c * 4 * G, src + c * 4 * G);
-        if (s < 2 && n > 0) cp_async_16(&sm.range[row_w][s], row_range + 2 * srow + s);
-        if (s == 2 && n > 0) cp_async_4(&sm.err[pass & 1][row_w], row_err + srow);
+            for (int r = 0; r < R; r += kRowsAtOnce) cp_async_16(dst + r * (sizeof(sm.rows[0]) / 4) + 4 * c, src + (size_t)r * g.N_ld + 4 * c);
+        }
         cp_async_commit();
+        ra = row_range[2 * (srow0 + row)];
+        rb = row_range[2 * (srow0 + row) + 1];
+        err_next = row_err[srow0 + row];
+        return n;
     };
-    int n_next = candidates(0);
-    request(0, n_next);
+    int n_next = request(row_begin);
 #pragma unroll 1
-    for (int pass = 0; pass < kSelectRows / R; ++pass) {
-        const int rl = pass * R + row_w, r = row0 + rl;
+    for (int r0 = row_begin; r0 < row_begin + warp_rows; r0 += R) {
+        const int ro = r0 % kOut + row;                                    // the row's place among those that leave together
         const int n = n_next;
-        const int n_most = __reduce_max_sync(kFull, n), n_least = __reduce_min_sync(kFull, n);
-        cp_async_wait<0>();
-        __syncwarp();
-        n_next = pass + 1 < kSelectRows / R ? candidates(pass + 1) : 0;
-        if (n_most == 0) {
-            request(pass + 1, n_next);
-            continue;
-        }
-        // ---- the row's scores (column 4 G c + 4 s + i in v[4 c + i]), largest and smallest
-        const float* row_scores = sm.rows[row_w];
-        float v[kK];
-#pragma unroll
-        for (int c = 0; c < kSteps; ++c) {
-            float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if (c * 4 * G < n_most) {
-                const int col = c * 4 * G + 4 * s;
-                if (col < n) x = *reinterpret_cast<const float4*>(row_scores + col);
-                if ((c + 1) * 4 * G > n_least) {                           // the end of a row's candidates
-                    if (col + 1 >= n) x.y = -INFINITY;
-                    if (col + 2 >= n) x.z = -INFINITY;
-                    if (col + 3 >= n) x.w = -INFINITY;
-                }
-            }
-            v[4 * c] = x.x; v[4 * c + 1] = x.y; v[4 * c + 2] = x.z; v[4 * c + 3] = x.w;
-        }
-        float top = 0.f, low = 0.f;
-        if (n > 0) {
-            const float4 ra = sm.range[row_w][0], rb = sm.range[row_w][1];
-            top = fmaxf(fmaxf(ra.x, ra.z), fmaxf(rb.x, rb.z));
-            low = fminf(fminf(ra.y, ra.w), fminf(rb.y, rb.w));
-        }
+        float top = fmaxf(fmaxf(ra.x, ra.z), fmaxf(rb.x, rb.z)), low = fminf(fminf(ra.y, ra.w), fminf(rb.y, rb.w));
+        const float err = n > 0 ? err_next : 0.f;
         bool give_up = n > 0 && !(top > -INFINITY && low > -INFINITY);     // marked by the score kernel
-        if (give_up) {
-            top = low = 0.f;
+        const bool act = n > 0 && !give_up;
+        if (!act) top = low = 0.f;
+        cp_async_wait<0>();
+        if (R >= 8 || r0 % kOut == 0)
+            for (int i = lane; i < n_words_live * (kOut / 4); i += 32) reinterpret_cast<uint4*>(&sm.words[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+        n_next = 0;
+        if (__any_sync(kFull, n > 0)) {
+            const float* my_row = sm.rows[row];
+            auto mass = [&](float d) -> float { return kByCount ? 1.f : fast_exp2(d); };   // of a score at d = s - max
+            const int own = act ? max((n / 8 - u + U - 1) / U, 0) : 0;     // my whole chunks: columns 8 (U i + u) .. +7
+            const bool part = act && (n & 7) != 0 && u == (n / 8) % U;     // and the row's last columns
+            // With fewer than 8 rows a load of 8 lanes meets several chunks of a row: half of the lanes read the second
+            // 16 bytes of theirs first (column e of a lane's chunk is then column e ^ 4).
+            const int swap = R == 4 || R == 2 ? (u & 1) * 4 : R == 1 ? (u & 4) : 0;
+            const float* mine = my_row + 8 * u;
+            auto load_chunk = [&](int i, unsigned long long (&x2)[4]) {
+                const float4 x0 = *reinterpret_cast<const float4*>(mine + i * (8 * U) + swap), x1 = *reinterpret_cast<const float4*>(mine + i * (8 * U) + (swap ^ 4));
+                x2[0] = pack_f32x2(x0.x, x0.y);
+                x2[1] = pack_f32x2(x0.z, x0.w);
+                x2[2] = pack_f32x2(x1.x, x1.y);
+                x2[3] = pack_f32x2(x1.z, x1.w);
+            };
+            // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, or from the other end, bucket = round(u): the
+            // buckets span the row
+            const float per_unit = fminf((float)(kBuckets - 1) / (top - low), 1e18f);
+            float a_mul = tail ? per_unit : -per_unit, a_add = a_add0;     // u = d * a_mul + a_add
+            uint32_t* my_hist = hist + row;
+            const uint32_t hist_addr = smem_u32(my_hist) - kMagicBits * (4u * R);   // plus 4 R times the bits of 2^23 + bucket
+            auto add_to_bucket = [&](uint32_t bucket_bits, uint32_t q) {
+                asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(hist_addr + bucket_bits * (4u * R)), "r"(q) : "memory");
+            };
+            auto row_sum = [&](float x) -> float {
 #pragma unroll
-            for (int e = 0; e < kK; ++e) v[e] = -INFINITY;
-        }
-        const int n_whole = __any_sync(kFull, give_up) ? 0 : n_least;      // columns below are scores in every row of the warp
-        // mass of a score at d = s - max
-        auto mass = [&](float d) -> float { return kByCount ? (d > -INFINITY ? 1.f : 0.f) : fast_exp2(d); };
-
-        // ---- sweep 1: Z and the histogram over u = (max - s) * per_unit, or from the other end, bucket = round(u): the
-        // buckets span the row
-        const float per_unit = fminf((float)(kBuckets - 1) / (top - low), 1e18f);
-        float a_mul = tail ? per_unit : -per_unit, a_add = a_add0;         // u = d * a_mul + a_add
-        float z = 0.f;
-        uint32_t* my_hist = hist + row_w;
-        const uint32_t hist_addr = smem_u32(my_hist) - kMagicBits * (4u * R);   // plus 4 R times the bits of 2^23 + bucket
-        auto add_to_bucket = [&](uint32_t bucket_bits, uint32_t q) {
-            asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(hist_addr + bucket_bits * (4u * R)), "r"(q) : "memory");
-        };
-        {
-            unsigned long long z2 = 0ull, zs2 = 0ull;                      // of all steps, of the last few
+                for (int o = 16; o >= R; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+                return x;
+            };
             const unsigned long long neg_top2 = pack_f32x2(-top, -top), a_mul2 = pack_f32x2(a_mul, a_mul);
-            const unsigned long long magic2 = pack_f32x2(kMagic + a_add0, kMagic + a_add0), q_unit2 = pack_f32x2(rule.q_unit, rule.q_unit);
-#pragma unroll
-            for (int c = 0; c < kSteps; ++c) {
-                if ((c + 1) * 4 * G <= n_whole) {
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        const unsigned long long d2 = add_f32x2(pack_f32x2(v[4 * c + i], v[4 * c + i + 1]), neg_top2);
-                        float d0, d1, b0, b1;
-                        unpack_f32x2(d2, d0, d1);
-                        v[4 * c + i] = d0;
-                        v[4 * c + i + 1] = d1;
-                        unpack_f32x2(fma_f32x2(d2, a_mul2, magic2), b0, b1);
-                        if (kByCount) {
-                            z += 2.f;
-                            add_to_bucket(__float_as_uint(b0), 1u);
-                            add_to_bucket(__float_as_uint(b1), 1u);
-                        } else {
-                            const unsigned long long m2 = pack_f32x2(mass(d0), mass(d1));
-                            zs2 = add_f32x2(zs2, m2);
-                            float q0, q1;
-                            unpack_f32x2(mul_f32x2(m2, q_unit2), q0, q1);
-                            add_to_bucket(__float_as_uint(b0), __float_as_uint(q0));
-                            add_to_bucket(__float_as_uint(b1), __float_as_uint(q1));
-                        }
-                    }
-                } else if (c * 4 * G < n_most) {                           // some columns hold no candidate (-inf: no mass)
-#pragma unroll
-                    for (int i = 0; i < 4; i += 2) {
-                        float m[2];
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            const float d = v[4 * c + i + k] - top;
-                            v[4 * c + i + k] = d;
-                            m[k] = mass(d);
-                            const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), tail ? 1.f : 0.f);
-                            add_to_bucket(__float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)), __float_as_uint(m[k] * rule.q_unit));
-                        }
-                        zs2 = add_f32x2(zs2, pack_f32x2(m[0], m[1]));
-                    }
-                }
-                if (c % kSumSteps == kSumSteps - 1 || c == kSteps - 1) {
-                    z2 = c < kSumSteps ? zs2 : add_f32x2(z2, zs2);
-                    zs2 = 0ull;
-                }
-            }
-            float z0, z1;
-            unpack_f32x2(z2, z0, z1);
-            z += z0 + z1;
-        }
-        z = group_sum(z);
-        const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * rule.share);
-        float base = 0.f;                                                  // mass before the bucket
-        float to_edge = 0.f;                                               // u + this = 0: the edge of the first bucket on the rejected side
-        float beyond = -INFINITY;                                          // my largest rejected score of that bucket that is not listed
-        int adds = 2 * kAdds + 2;
-        uint32_t before[kMasks], inside[kMasks];                           // per lane: bit e = its e-th score
-#pragma unroll
-        for (int k = 0; k < kMasks; ++k) { before[k] = 0u; inside[k] = 0u; }
-        bool unsure = false;
-        bool active = n > 0 && !give_up;                                   // the row still narrows its interval
-        int n_cand = 0;
+            float z = 0.f;
+            {
+                unsigned long long z2 = 0ull;
+                const unsigned long long magic2 = pack_f32x2(kMagic + a_add0, kMagic + a_add0), q_unit2 = pack_f32x2(rule.q_unit, rule.q_unit);
 #pragma unroll 1
-        for (int level = 0;; ++level) {
-            __syncwarp();
-            // ---- the bucket in which the cumulative (quantised) mass crosses the target: first the lane whose 16
-            // buckets hold it, then the bucket (read in an order of its own by each lane: no bank is met twice)
-            uint32_t sum = 0u;
+                for (int i0 = 0; i0 < own; i0 += kSumIters) {
+                    unsigned long long zs2 = 0ull;                         // of the last few chunks
 #pragma unroll
-            for (int u = 0; u < 16; ++u) sum += my_hist[(s * 16 + (u ^ (s & 15))) * R];
-            uint32_t incl = sum;
+                    for (int q = 0; q < kSumIters; ++q) {
+                        if (q >= kIter || i0 + q >= own) break;
+                        unsigned long long x2[4];
+                        load_chunk(i0 + q, x2);
 #pragma unroll
-            for (int o = 1; o < G; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(kFull, incl, o, G);
-                if (s >= o) incl += t;
-            }
-            const uint32_t thr = max((uint32_t)fmaxf((target - base) * rule.unit, 0.f), 1u);
-            uint32_t over = __ballot_sync(kFull, incl >= thr);
-            if (G < 32) over = (over >> (row_w * G)) & ((1u << (G & 31)) - 1u);
-            const int own = over ? __ffs(over) - 1 : G - 1;
-            const uint32_t cum = __shfl_sync(kFull, incl - sum, own, G);
-            constexpr int kPer = 16 / (G < 16 ? G : 16);                   // buckets per lane in the second step
-            uint32_t part[kPer], psum = 0u;
-#pragma unroll
-            for (int u = 0; u < kPer; ++u) {
-                part[u] = s * kPer < 16 ? my_hist[(own * 16 + (s & 15) * kPer + u) * R] : 0u;
-                psum += part[u];
-            }
-            uint32_t pincl = psum;
-#pragma unroll
-            for (int o = 1; o < (G < 16 ? G : 16); o <<= 1) {
-                const uint32_t t = __shfl_up_sync(kFull, pincl, o, G);
-                if (s >= o) pincl += t;
-            }
-            over = __ballot_sync(kFull, s * kPer < 16 && cum + pincl >= thr);
-            if (G < 32) over = (over >> (row_w * G)) & ((1u << (G & 31)) - 1u);
-            const int own2 = over ? __ffs(over) - 1 : (G < 16 ? G : 16) - 1;
-            int cb = s * kPer;
-            if (kPer == 2 && cum + (pincl - psum) + part[0] < thr) ++cb;
-            cb = __shfl_sync(kFull, cb, own2, G) + own * 16;
-            __syncwarp();
-#pragma unroll
-            for (int u = 0; u < 4; ++u) reinterpret_cast<uint4*>(hist)[lane + 32 * u] = make_uint4(0u, 0u, 0u, 0u);
-            // ---- sweep 2: before / inside the bucket [cb - 1/2, cb + 1/2], widened by the guard
-            const float lo_u = (float)cb - (0.5f + kGuard);
-            const float hi_u = (float)cb + (0.5f + kGuard);
-            float add = 0.f;
-            n_cand = 0;
-            if (level == 0) {
-                const unsigned long long a_mul2 = pack_f32x2(a_mul, a_mul), lo2 = pack_f32x2(a_add0 - lo_u, a_add0 - lo_u);
-                const unsigned long long width2 = pack_f32x2(lo_u - hi_u, lo_u - hi_u);
-                unsigned long long add2 = 0ull, adds2 = 0ull;              // of all steps, of the last few
-#pragma unroll
-                for (int c = kSteps - 1; c >= 0; --c) {
-                    if (c * 4 * G < n_most) {
-#pragma unroll
-                        for (int i = 2; i >= 0; i -= 2) {
-                            const float d0 = v[4 * c + i], d1 = v[4 * c + i + 1];
-                            const int k = (4 * c + i) >> 5;
-                            const unsigned long long u2 = fma_f32x2(pack_f32x2(d0, d1), a_mul2, lo2);
-                            float ua0, ua1, ub0, ub1;
-                            unpack_f32x2(u2, ua0, ua1);
-                            unpack_f32x2(add_f32x2(u2, width2), ub0, ub1);
-                            before[k] = __funnelshift_l(__float_as_uint(ua1), before[k], 1);
-                            before[k] = __funnelshift_l(__float_as_uint(ua0), before[k], 1);
-                            inside[k] = __funnelshift_l(__float_as_uint(ub1), inside[k], 1);
-                            inside[k] = __funnelshift_l(__float_as_uint(ub0), inside[k], 1);
-                            // the mass of what lies before: times 2^100 and clamped, the distance is 1 before and 0 else
-                            adds2 = fma_f32x2(pack_f32x2(mass(d0), mass(d1)),
-                                              pack_f32x2(__saturatef(ua0 * -1.2676506e30f), __saturatef(ua1 * -1.2676506e30f)), adds2);
+                        for (int k = 0; k < 4; ++k) {
+                            const unsigned long long d2 = add_f32x2(x2[k], neg_top2);
+                            float d0, d1, b0, b1;
+                            unpack_f32x2(d2, d0, d1);
+                            unpack_f32x2(fma_f32x2(d2, a_mul2, magic2), b0, b1);
+                            if (kByCount) {
+                                z += 2.f;
+                                add_to_bucket(__float_as_uint(b0), 1u);
+                                add_to_bucket(__float_as_uint(b1), 1u);
+                            } else {
+                                const unsigned long long m2 = pack_f32x2(mass(d0), mass(d1));
+                                zs2 = add_f32x2(zs2, m2);
+                                float q0, q1;
+                                unpack_f32x2(mul_f32x2(m2, q_unit2), q0, q1);
+                                add_to_bucket(__float_as_uint(b0), __float_as_uint(q0));
+                                add_to_bucket(__float_as_uint(b1), __float_as_uint(q1));
+                            }
                         }
                     }
-                    if (c % kSumSteps == 0) {
-                        add2 = c + kSumSteps >= kSteps ? adds2 : add_f32x2(add2, adds2);
-                        adds2 = 0ull;
+                    z2 = add_f32x2(z2, zs2);
+                }
+                float z0, z1, zp = 0.f;
+                if (part) {
+#pragma unroll 1
+                    for (int j = n & ~7; j < n; ++j) {
+                        const float d = my_row[j] - top, m = mass(d);
+                        zp += m;
+                        add_to_bucket(__float_as_uint(fmaf(d, a_mul, kMagic + a_add0)), kByCount ? 1u : __float_as_uint(m * rule.q_unit));
                     }
                 }
-                float add0, add1;
-                unpack_f32x2(add2, add0, add1);
-                add = add0 + add1;
+                unpack_f32x2(z2, z0, z1);
+                z += z0 + z1;
+                z += zp;
+            }
+            __syncwarp();
+            z = row_sum(z);
+            const float target = kByCount ? fminf(z, (float)g.top_k) : (float)((double)z * rule.share);
+            float base = 0.f;                                              // mass before the bucket
+            uint32_t inside[kMasks];                                       // bit 8 i + e: column e of my i-th chunk
 #pragma unroll
-                for (int k = 0; k < kMasks; ++k) inside[k] &= ~before[k];
-            } else {
-                int n_add = 0;
+            for (int k = 0; k < kMasks; ++k) inside[k] = 0u;
+            auto column = [&](int k, int e) -> int { return ((4 * k + (e >> 3)) * U + u) * 8 + ((e & 7) ^ swap); };
+            auto of_row = [&](uint32_t ballot) -> uint32_t { return (ballot >> row) & kRowLanes; };
+            // The bucket in which the cumulative (quantised) mass crosses the target.  A lane sums the buckets of its part of the
+            // row (in an order of its own: no bank is met twice), the one that finds the target in it looks where.
+            auto find_bucket = [&]() -> int {
+                constexpr int kSeg = kBuckets / U, kGroup = R <= 2 ? 16 : 8, kGroups = kSeg / kGroup;
+                uint32_t group[kGroups], sum = 0u;
+                const uint32_t* seg = my_hist + u * (kSeg * R);
+#pragma unroll
+                for (int i = 0; i < kGroups; ++i) {
+                    group[i] = 0u;
+#pragma unroll
+                    for (int k = 0; k < kGroup; ++k) group[i] += seg[(i * kGroup + (k ^ (u & (kGroup - 1)))) * R];
+                    sum += group[i];
+                }
+                uint32_t incl = sum;
+#pragma unroll
+                for (int o = R; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const uint32_t thr = max((uint32_t)fmaxf((target - base) * rule.unit, 0.f), 1u);
+                const uint32_t over = of_row(__ballot_sync(kFull, incl >= thr));
+                const int finder = over ? __ffs(over) - 1 + row : 32 - R + row;
+                int at = kBuckets - 1;
+                if (lane == finder && over) {
+                    uint32_t cum = incl - sum;
+                    at = 0;
+#pragma unroll
+                    for (int i = 0; i < kGroups - 1; ++i)
+                        if (at == i * kGroup && cum + group[i] < thr) { cum += group[i]; at += kGroup; }
+                    uint32_t h[kGroup];
+#pragma unroll
+                    for (int k = 0; k < kGroup; ++k) h[k] = seg[(at + k) * R];
+                    int step = 0;
+#pragma unroll
+                    for (int k = 0; k < kGroup - 1; ++k) {
+                        cum += h[k];
+                        if (step == k && cum < thr) ++step;
+                    }
+                    at += step + u * kSeg;
+                }
+                __syncwarp();
+                return __shfl_sync(kFull, at, finder);
+            };
+            // ---- sweep 2: before / inside the bucket [cb - 1/2, cb + 1/2], widened by the guard; what is before, or else what
+            // is neither before nor inside, goes to the row's mask words
+            int cb = find_bucket();
+            float lo_u = (float)cb - (0.5f + kGuard), hi_u = (float)cb + (0.5f + kGuard);
+            const float to_edge = a_add0 - (tail ? lo_u : hi_u);           // u + this = 0: the edge of the first bucket on the rejected side
+            uint8_t* my_words = reinterpret_cast<uint8_t*>(&sm.words[0][ro]);
+            auto word_byte = [&](int chunk) -> uint8_t* { return my_words + (chunk >> 2) * (4 * kOut) + (chunk & 3); };
+            {
+                const unsigned long long lo2 = pack_f32x2(a_add0 - lo_u, a_add0 - lo_u), width2 = pack_f32x2(lo_u - hi_u, lo_u - hi_u);
+                unsigned long long add2 = 0ull;
+#pragma unroll
                 for (int k = 0; k < kMasks; ++k) {
-                    uint32_t bits = active ? inside[k] : 0u;
-                    while (bits) {
-                        const int e = __ffs(bits) - 1;
-                        bits &= bits - 1u;
-                        const float x = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)], d = x - top;
-                        const float u = fmaf(d, a_mul, a_add);
-                        if (u < lo_u) { before[k] |= 1u << e; inside[k] &= ~(1u << e); add += mass(d); ++n_add; }
-                        else if (!(u < hi_u)) inside[k] &= ~(1u << e);
-                        else continue;
-                        if (tail ? u < lo_u : !(u < lo_u)) beyond = fmaxf(beyond, x);
+                    unsigned long long adds2 = 0ull;                       // of the last few chunks
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int i = 4 * k + q;
+                        if (i >= kIter) continue;
+                        if (i < own) {
+                            unsigned long long x2[4];
+                            load_chunk(i, x2);
+                            uint32_t bits = 0u, in = 0u;
+#pragma unroll
+                            for (int p = 3; p >= 0; --p) {
+                                const unsigned long long d2 = add_f32x2(x2[p], neg_top2), u2 = fma_f32x2(d2, a_mul2, lo2);
+                                float d0, d1, ua0, ua1, ub0, ub1;
+                                unpack_f32x2(d2, d0, d1);
+                                unpack_f32x2(u2, ua0, ua1);
+                                unpack_f32x2(add_f32x2(u2, width2), ub0, ub1);
+                                bits = __funnelshift_l(__float_as_uint(ua1), bits, 1);
+                                bits = __funnelshift_l(__float_as_uint(ua0), bits, 1);
+                                in = __funnelshift_l(__float_as_uint(ub1), in, 1);
+                                in = __funnelshift_l(__float_as_uint(ub0), in, 1);
+                                // the mass of what lies before: times 2^100 and clamped, the distance is 1 before and 0 else
+                                adds2 = fma_f32x2(pack_f32x2(mass(d0), mass(d1)),
+                                                  pack_f32x2(__saturatef(ua0 * -1.2676506e30f), __saturatef(ua1 * -1.2676506e30f)), adds2);
+                            }
+                            inside[k] |= (in & ~bits) << (8 * q);
+                            bits = tail ? ~(bits | in) & 0xffu : bits;
+                            if (R < 8) bits = (bits >> swap) | (bits << swap);
+                            *word_byte(i * U + u) = (uint8_t)bits;
+                        }
                     }
+                    add2 = add_f32x2(add2, adds2);
                 }
-                adds += __reduce_max_sync(kFull, n_add) + 6;               // (the lane's, its group's and the base's)
-            }
+                float add0, add1, addp = 0.f;
+                if (part) {
+                    uint32_t bits = 0u, in = 0u;                           // by column
+#pragma unroll 1
+                    for (int j = n & ~7; j < n; ++j) {
+                        const float d = my_row[j] - top, uj = fmaf(d, a_mul, a_add0 - lo_u);
+                        const uint32_t bit = 1u << (j & 7);
+                        if (uj < 0.f) { bits |= bit; addp += mass(d); }
+                        else if (uj + (lo_u - hi_u) < 0.f) in |= bit;
+                    }
+                    *word_byte(n >> 3) = (uint8_t)(tail ? ~(bits | in) & ((1u << (n & 7)) - 1u) : bits);
+                    if (R < 8) in = ((in >> swap) | (in << swap)) & 0xffu;
 #pragma unroll
-            for (int k = 0; k < kMasks; ++k) n_cand += __popc(inside[k]);
-            add = group_sum(add);
-            if (G == 32) {
-                n_cand = __reduce_add_sync(kFull, n_cand);
-            } else {
+                    for (int k = 0; k < kMasks; ++k)
+                        if (k == own >> 2) inside[k] |= in << (8 * (own & 3));
+                }
+                unpack_f32x2(add2, add0, add1);
+                float add = add0 + add1;
+                add += addp;
+                base = row_sum(add);
+            }
+            // my place in the row's list, and how long it is
+            int slot, n_cand;
+            auto count_inside = [&]() {
+                int mine_in = 0;
 #pragma unroll
-                for (int o = G / 2; o > 0; o >>= 1) n_cand += __shfl_xor_sync(kFull, n_cand, o);
+                for (int k = 0; k < kMasks; ++k) mine_in += __popc(inside[k]);
+                int incl = mine_in;
+#pragma unroll
+                for (int o = R; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                slot = incl - mine_in;
+                n_cand = __shfl_sync(kFull, incl, 32 - R + row);
+            };
+            count_inside();
+            int adds = 2 * kAdds + 2;
+            float beyond = -INFINITY;                                      // my largest rejected score of that bucket that is not listed
+            bool active = act && n_cand > kSelectCand;
+            if (__any_sync(kFull, active)) {
+                // ---- rare: split the bucket of the rows that hold too many cubes in it
+                constexpr float fine = (float)(kBuckets - 1) / (1.f + 2.f * kGuard);
+#pragma unroll 1
+                for (int level = 1;; ++level) {
+                    if (active) {
+                        a_add = (a_add - lo_u) * fine;
+                        a_mul = a_mul * fine;
+                        if (level == kMaxHistLevels || !(fabsf(a_mul) < 1e30f)) { give_up = true; active = false; }
+                    }
+                    if (!__any_sync(kFull, active)) break;
+                    clear_hist();
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < kMasks; ++k) {
+                        uint32_t bits = active ? inside[k] : 0u;
+                        while (bits) {
+                            const float d = my_row[column(k, __ffs(bits) - 1)] - top;
+                            bits &= bits - 1u;
+                            const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), a_add * (1.f / (kBuckets - 1)));
+                            add_to_bucket(__float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)), kByCount ? 1u : __float_as_uint(mass(d) * rule.q_unit));
+                        }
+                    }
+                    __syncwarp();
+                    cb = find_bucket();
+                    float add = 0.f;
+                    int n_add = 0;
+                    if (active) {
+                        lo_u = (float)cb - (0.5f + kGuard);
+                        hi_u = (float)cb + (0.5f + kGuard);
+#pragma unroll
+                        for (int k = 0; k < kMasks; ++k) {
+                            uint32_t bits = inside[k];
+                            while (bits) {
+                                const int e = __ffs(bits) - 1, j = column(k, e);
+                                bits &= bits - 1u;
+                                const float x = my_row[j], d = x - top, uj = fmaf(d, a_mul, a_add);
+                                const bool bef = uj < lo_u;
+                                if (!bef && uj < hi_u) continue;
+                                inside[k] &= ~(1u << e);
+                                if (bef) { add += mass(d); ++n_add; }
+                                if (bef == tail) beyond = fmaxf(beyond, x);                // rejected, or else selected
+                                else atomicOr(&sm.words[j >> 5][ro], 1u << (j & 31));
+                            }
+                        }
+                    }
+                    adds += __reduce_max_sync(kFull, n_add) + 6;           // (the lane's, its row's and the base's)
+                    base += row_sum(add);
+                    count_inside();
+                    if (n_cand <= kSelectCand) active = false;
+                }
+#pragma unroll
+                for (int o = 16; o >= R; o >>= 1) beyond = fmaxf(beyond, __shfl_xor_sync(kFull, beyond, o));
             }
-            if (active) {
-                base += add;
-                if (level == 0) to_edge = a_add - (tail ? lo_u : hi_u);
-            }
-            if (n_cand <= kSelectCand) active = false;
-            if (active && level + 1 == kMaxHistLevels) { give_up = true; active = false; }
-            if (!__any_sync(kFull, active)) break;
-            // ---- rare: split the bucket of the rows that hold too many cubes in it
-            constexpr float fine = (float)(kBuckets - 1) / (1.f + 2.f * kGuard);
-            if (active) {
-                a_add = (a_add - lo_u) * fine;
-                a_mul = a_mul * fine;
-                if (!(fabsf(a_mul) < 1e30f)) { give_up = true; active = false; }
-            }
+            // ---- list the cubes inside the bucket
+            const bool decide = act && !give_up;
+            const int n_list = decide ? n_cand : 0;
+            const int n_list_most = __reduce_max_sync(kFull, n_list);
+            __syncwarp();
+            for (int i = n_list + u; i < n_list_most; i += U) sm.cand[i][row] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+#pragma unroll
             for (int k = 0; k < kMasks; ++k) {
-                uint32_t bits = active ? inside[k] : 0u;
+                uint32_t bits = decide ? inside[k] : 0u;
                 while (bits) {
-                    const int e = __ffs(bits) - 1;
+                    const int j = column(k, __ffs(bits) - 1);
                     bits &= bits - 1u;
-                    const float d = row_scores[((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3)] - top;
-                    const float u01 = sat_fma(d, a_mul * (1.f / (kBuckets - 1)), a_add * (1.f / (kBuckets - 1)));
-                    const uint32_t b = __float_as_uint(fmaf(u01, (float)(kBuckets - 1), kMagic)) - kMagicBits;
-                    atomicAdd(&my_hist[b * R], __float_as_uint(mass(d) * rule.q_unit));
+                    const float x = my_row[j];
+                    sm.cand[slot++][row] = make_float4(x, mass(x - top), __int_as_float(j), 0.f);
                 }
             }
             __syncwarp();
-        }
-        // ---- list the cubes inside the bucket
-        const bool decide = n > 0 && !give_up;
-        const int n_list = decide ? n_cand : 0;
-        const int n_list_most = __reduce_max_sync(kFull, n_list);
-        if (s == 0) sm.count[row_w] = 0;
-        for (int i = n_list + s; i < n_list_most; i += G) sm.cand[row_w][i] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < kMasks; ++k) {
-            uint32_t bits = decide ? inside[k] : 0u;
-            int slot = bits ? atomicAdd(&sm.count[row_w], __popc(bits)) : 0;
-            while (bits) {
-                const int e = __ffs(bits) - 1;
-                bits &= bits - 1u;
-                const int j = ((k * 32 + e) >> 2) * 4 * G + 4 * s + (e & 3);
-                const float x = row_scores[j];
-                sm.cand[row_w][slot++] = make_float4(x, mass(x - top), __int_as_float(j), 0.f);
-            }
-        }
-        __syncwarp();
-        request(pass + 1, n_next);                                         // the rows' scores are no longer read
-        // ---- the words of what lies before the bucket, or else of what is neither before nor inside it: lane s holds nibble
-        // s & 7 of words (s >> 3) + c G / 8
-#pragma unroll
-        for (int k = 0; k < kMasks; ++k) {
-            uint32_t t = tail ? before[k] | inside[k] : before[k];         // nibble c: columns of step 8 k + c
-            // transpose the 8 x 8 nibbles of 8 neighbouring lanes: lane c then holds word c
-            uint32_t o = __shfl_xor_sync(kFull, t, 4);
-            t = (s & 4) ? ((t & 0xffff0000u) | (o >> 16)) : ((t & 0x0000ffffu) | (o << 16));
-            o = __shfl_xor_sync(kFull, t, 2);
-            t = (s & 2) ? ((t & 0xff00ff00u) | ((o >> 8) & 0x00ff00ffu)) : ((t & 0x00ff00ffu) | ((o << 8) & 0xff00ff00u));
-            o = __shfl_xor_sync(kFull, t, 1);
-            t = (s & 1) ? ((t & 0xf0f0f0f0u) | ((o >> 4) & 0x0f0f0f0fu)) : ((t & 0x0f0f0f0fu) | ((o << 4) & 0xf0f0f0f0u));
-            const int wd = (8 * k + (s & 7)) * (G / 8) + (s >> 3);
-            if (tail) {
-                t = ~t & __funnelshift_lc(0xffffffffu, 0u, max(n - wd * 32, 0));   // of the row's candidates in the word
-            }
-            if (wd < n_words_live && decide) words[wd * kSelectRows + rl] = t;
-        }
-        __syncwarp();
-        // ---- each listed cube: the mass before it and with it
-        const float err = n > 0 ? sm.err[pass & 1][row_w] : 0.f;
-        const float mass_err = fmaf(0.6931472f, fmaf(2.f * kUlp, (top - low) + fmaxf(top, -low), err), 4.f * kUlp);
-        const float eps = kByCount ? 0.f : z * fmaf(rule.eps_mass, mass_err, rule.eps_add * (float)(adds + n_list));
-        float last = INFINITY, next = -INFINITY;                           // lowest selected, highest rejected score of my cubes
-        bool reached = false;
-        for (int i0 = 0; i0 < n_list_most; i0 += G) {
-            const int i = i0 + s;
-            const bool mine = i < n_list;
-            const float4 me = sm.cand[row_w][min(i, n_list_most - 1)];
-            const int ji = __float_as_int(me.z);
-            float acc = base;                                              // and the listed cubes before mine
-            for (int k = 0; k < n_list_most; ++k) {
-                const float4 ck = sm.cand[row_w][k];
-                const bool earlier = tail ? ck.x < me.x || (ck.x == me.x && __float_as_int(ck.z) > ji)
-                                          : ck.x > me.x || (ck.x == me.x && __float_as_int(ck.z) < ji);
-                if (earlier) acc += ck.y;
-            }
-            if (mine) {
-                if (tail ? acc + me.y > target : acc < target) {
-                    atomicOr(&words[(ji >> 5) * kSelectRows + rl], 1u << (ji & 31));
-                    last = fminf(last, me.x);
-                } else {
-                    next = fmaxf(next, me.x);
+            if (r0 + R < row_begin + warp_rows) n_next = request(r0 + R);  // the rows' scores are no longer read
+            // ---- each listed cube: the mass before it and with it
+            const float mass_err = fmaf(0.6931472f, fmaf(2.f * kUlp, (top - low) + fmaxf(top, -low), err), 4.f * kUlp);
+            const float eps = kByCount ? 0.f : z * fmaf(rule.eps_mass, mass_err, rule.eps_add * (float)(adds + n_list));
+            float last = INFINITY, next = -INFINITY;                       // lowest selected, highest rejected score of my cubes
+            bool reached = false, unsure = false;
+            for (int i0 = 0; i0 < n_list_most; i0 += U) {
+                const int i = i0 + u;
+                const float4 me = sm.cand[min(i, n_list_most - 1)][row];
+                const int ji = __float_as_int(me.z);
+                float acc = base;                                          // and the listed cubes before mine
+#pragma unroll 4
+                for (int k = 0; k < n_list_most; ++k) {
+                    const float4 ck = sm.cand[k][row];
+                    const bool earlier = tail ? ck.x < me.x || (ck.x == me.x && __float_as_int(ck.z) > ji)
+                                              : ck.x > me.x || (ck.x == me.x && __float_as_int(ck.z) < ji);
+                    if (earlier) acc += ck.y;
                 }
-                reached = reached || (tail ? acc + me.y > target : acc + me.y >= target);
-                if (!kByCount) unsure = unsure || fabsf(acc - target) <= eps || fabsf(acc + me.y - target) <= eps;
-            }
-        }
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) {
-            last = fminf(last, __shfl_xor_sync(kFull, last, o));
-            next = fmaxf(next, __shfl_xor_sync(kFull, next, o));
-        }
-        const float gap = fmaf(4.f * kUlp, fabsf(last), 2.f * err);
-        // an unlisted cube lies beyond the edge (u is off by a small part of the guard) or has been looked at
-        unsure = unsure || (n_list < n && fabsf(fmaf(last - top, tail ? per_unit : -per_unit, to_edge)) <= fmaf(gap, per_unit, 0.5f * kGuard));
-        if (__any_sync(kFull, beyond > -INFINITY)) {
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) beyond = fmaxf(beyond, __shfl_xor_sync(kFull, beyond, o));
-            unsure = unsure || last - beyond <= gap;
-        }
-        bool tied = last < INFINITY && last - next <= gap;                 // (a row without a listed cube that is selected is unsure)
-        if (__any_sync(kFull, tied)) {
-            // The boundary runs through cubes whose order these scores cannot tell.  If they are copies of one cube (frames
-            // that repeat: the mean keys are equal bit by bit) their scores are equal in fp64 too and the index orders them.
-            // (All such rows went to the fp64 kernel: every frame twice, 65536 tokens, 57.8 instead of 4.3 ms of selection.)
-            const unsigned long long* hash = key_hash + (size_t)(w.b * g.Hkv + w.gk) * g.N_ld;
-            unsigned long long h_min = ~0ull, h_max = 0ull;
-            for (int i = s; i < n_list; i += G) {
-                const float4 me = sm.cand[row_w][i];
-                if (last - me.x <= gap && me.x - next <= gap) {
-                    const unsigned long long hj = hash[__float_as_int(me.z)];
-                    h_min = min(h_min, hj);
-                    h_max = max(h_max, hj);
+                if (i < n_list) {
+                    if (tail ? acc + me.y > target : acc < target) {
+                        atomicOr(&sm.words[ji >> 5][ro], 1u << (ji & 31));
+                        last = fminf(last, me.x);
+                    } else {
+                        next = fmaxf(next, me.x);
+                    }
+                    reached = reached || (tail ? acc + me.y > target : acc + me.y >= target);
+                    if (!kByCount) unsure = unsure || fabsf(acc - target) <= eps || fabsf(acc + me.y - target) <= eps;
                 }
             }
 #pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                h_min = min(h_min, __shfl_xor_sync(kFull, h_min, o));
-                h_max = max(h_max, __shfl_xor_sync(kFull, h_max, o));
+            for (int o = 16; o >= R; o >>= 1) {
+                last = fminf(last, __shfl_xor_sync(kFull, last, o));
+                next = fmaxf(next, __shfl_xor_sync(kFull, next, o));
             }
-            tied = tied && h_min != h_max;
-        }
-        unsure = unsure || tied || !(last < INFINITY);
-        const bool any_unsure = group_any(unsure), any_reached = group_any(reached);   // both by all lanes
-        unsure = any_unsure || !any_reached || !(tail ? base <= target : base < target);
-        if (n > 0 && (give_up || unsure)) {
-            for (int wd = s; wd < n_words_live; wd += G) words[wd * kSelectRows + rl] = 0u;
-            if (s == 0) fallback_rows[atomicAdd(fallback_count, 1u)] = (int32_t)(gt_cap * kTileRows + r);
+            const float gap = fmaf(4.f * kUlp, fabsf(last), 2.f * err);
+            // an unlisted cube lies beyond the edge (u is off by a small part of the guard) or has been looked at
+            unsure = unsure || (n_list < n && fabsf(fmaf(last - top, tail ? per_unit : -per_unit, to_edge)) <= fmaf(gap, per_unit, 0.5f * kGuard));
+            unsure = unsure || (beyond > -INFINITY && last - beyond <= gap);
+            bool tied = last < INFINITY && last - next <= gap;             // (a row without a listed cube that is selected is unsure)
+            if (__any_sync(kFull, tied)) {
+                // The boundary runs through cubes whose order these scores cannot tell.  If they are copies of one cube (frames
+                // that repeat: the mean keys are equal bit by bit) their scores are equal in fp64 too and the index orders them.
+                // (All such rows went to the fp64 kernel: every frame twice, 65536 tokens, 57.8 instead of 4.3 ms of selection.)
+                const unsigned long long* hash = key_hash + (size_t)(w.b * g.Hkv + w.gk) * g.N_ld;
+                unsigned long long h_min = ~0ull, h_max = 0ull;
+                for (int i = u; i < n_list; i += U) {
+                    const float4 me = sm.cand[i][row];
+                    if (last - me.x <= gap && me.x - next <= gap) {
+                        const unsigned long long hj = hash[__float_as_int(me.z)];
+                        h_min = min(h_min, hj);
+                        h_max = max(h_max, hj);
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o >= R; o >>= 1) {
+                    h_min = min(h_min, __shfl_xor_sync(kFull, h_min, o));
+                    h_max = max(h_max, __shfl_xor_sync(kFull, h_max, o));
+                }
+                tied = tied && h_min != h_max;
+            }
+            unsure = unsure || tied || !(last < INFINITY);
+            const uint32_t any_unsure = of_row(__ballot_sync(kFull, unsure)), any_reached = of_row(__ballot_sync(kFull, reached));   // both by all lanes
+            unsure = any_unsure != 0u || any_reached == 0u || !(tail ? base <= target : base < target);
+            if (n > 0 && (give_up || unsure)) {
+                for (int wd = u; wd < n_words_live; wd += U) sm.words[wd][ro] = 0u;
+                if (u == 0) fallback_rows[atomicAdd(fallback_count, 1u)] = (int32_t)(gt_cap * kTileRows + r0 + row);
+            }
+            __syncwarp();
+            clear_hist();
+        } else if (r0 + R < row_begin + warp_rows) {
+            n_next = request(r0 + R);
         }
         __syncwarp();
-    }
-    // ---- mask words (32-byte sectors of 8 rows), union words, the caller's copies
-    for (int i0 = 0; i0 < g.n_words * 2; i0 += 32) {
-        const int wd = (i0 + lane) >> 1, c4 = lane & 1;
-        const uint4 val = wd < n_words_live ? *reinterpret_cast<const uint4*>(&words[wd * kSelectRows + c4 * 4]) : make_uint4(0u, 0u, 0u, 0u);
-        if (wd < g.n_words)
-            *reinterpret_cast<uint4*>(tile_mask + (gt_cap * g.n_words + wd) * kTileRows + row0 + c4 * 4) = val;
-        uint32_t u = (val.x | val.y) | (val.z | val.w);                    // OR over the two lanes of the word
-        u |= __shfl_xor_sync(kFull, u, 1);
-        if (c4 == 0 && u) atomicOr(tile_union + gt_cap * g.n_words + wd, u);
-    }
-    if (sel_bitmap != nullptr || sel_count != nullptr) {
-        for (int rl = 0; rl < kSelectRows; ++rl) {
-            const int pos = w.tile * kTileRows + row0 + rl;
-            if (!slot_live(g, pos)) continue;
-            const size_t raster_row = (size_t)(w.b * g.Hq + w.h) * g.S_io + (pos_to_io(g, pos) - g.pos_begin);
-            int cnt = 0;
-            for (int wd = lane; wd < g.n_words; wd += 32) {
-                const uint32_t word = wd < n_words_live ? words[wd * kSelectRows + rl] : 0u;
-                cnt += __popc(word);
-                if (sel_bitmap) sel_bitmap[raster_row * g.n_words + wd] = word;
-            }
-            cnt = __reduce_add_sync(kFull, cnt);
-            if (sel_count && lane == 0) sel_count[raster_row] = cnt;
+        // ---- mask words (whole 32-byte sectors), union words, the caller's copies
+        if (R < 8 && (r0 + R) % kOut != 0) continue;
+        const int out0 = r0 / kOut * kOut;
+        constexpr int kParts = kOut / 4;                                   // 16-byte parts of a word's rows
+        for (int i0 = 0; i0 < g.n_words * kParts; i0 += 32) {
+            const int wd = (i0 + lane) / kParts, c4 = lane % kParts;
+            const uint4 val = wd < n_words_live ? *reinterpret_cast<const uint4*>(&sm.words[wd][c4 * 4]) : make_uint4(0u, 0u, 0u, 0u);
+            if (wd < g.n_words)
+                *reinterpret_cast<uint4*>(tile_mask + (gt_cap * g.n_words + wd) * kTileRows + out0 + c4 * 4) = val;
+            uint32_t un = (val.x | val.y) | (val.z | val.w);               // OR over the lanes of the word
+#pragma unroll
+            for (int o = kParts / 2; o > 0; o >>= 1) un |= __shfl_xor_sync(kFull, un, o);
+            if (c4 == 0 && un) atomicOr(tile_union + gt_cap * g.n_words + wd, un);
         }
+        if (sel_bitmap != nullptr || sel_count != nullptr) {
+            for (int r = 0; r < kOut; ++r) {
+                const int pos = w.tile * kTileRows + out0 + r;
+                if (!slot_live(g, pos)) continue;
+                const size_t raster_row = (size_t)(w.b * g.Hq + w.h) * g.S_io + (pos_to_io(g, pos) - g.pos_begin);
+                int cnt = 0;
+                for (int wd = lane; wd < g.n_words; wd += 32) {
+                    const uint32_t word = wd < n_words_live ? sm.words[wd][r] : 0u;
+                    cnt += __popc(word);
+                    if (sel_bitmap) sel_bitmap[raster_row * g.n_words + wd] = word;
+                }
+                cnt = __reduce_add_sync(kFull, cnt);
+                if (sel_count && lane == 0) sel_count[raster_row] = cnt;
+            }
+        }
+        __syncwarp();
     }
 }
 

@@ -140,3 +140,15 @@ def test_many_masses_that_are_nearly_equal(top_p):
     wl = inputs.make_prefill("level", seed=85, B=1, T=4000, H=4, W=4, cube=(1, 4, 4), n_text=300, Hq=1, Hkv=1, D=64, top_p=top_p,
                              offset_std=0.01)
     _equal(wl, wl.k * 0.125)
+
+
+@pytest.mark.parametrize("n_cubes", [7, 9, 16, 57, 63, 119, 127, 249, 505, 1017])
+@pytest.mark.parametrize("top_p", [0.2, 0.7, 0.99999])
+def test_last_columns_of_a_row(n_cubes, top_p):
+    """Candidate counts one off the 8 columns that a lane takes at a time, at the end of every kernel shape, with a text prefix
+    and a text that end inside the rows of a pass (rows without candidates beside rows with all of them) and cubes at the
+    faces that hold no more than a few rows.  No more rows than elsewhere are left to the fp64 kernel, also where two lanes
+    sum all buckets of a row."""
+    wl = inputs.make_prefill("chunks", seed=86, B=1, T=n_cubes, H=4, W=3, cube=(1, 4, 4), n_text=139, n_prefix=13, Hq=3, Hkv=1,
+                             D=128 if n_cubes % 2 else 64, top_p=top_p, offset_std=1.5)
+    assert _equal(wl).fallback_rows < 0.005 * wl.S * wl.Hq + 2
