@@ -845,10 +845,10 @@ adaspark_status_t adaspark_attn_decode(adaspark_attn_t* h, const void* q_new, co
         size_t smem = decode_select_smem_bytes(g.N_ld, g.G, g.n_words);
         if (D == 128) {
             if (!set_smem(h, decode_select_plan_kernel<128>, smem, "decode_select_plan_kernel")) return ADASPARK_ERR_CUDA;
-            decode_select_plan_kernel<128><<<dim3(kPlanCtas, g.Hkv, g.B), kPlanWarps * 32, smem, st>>>(g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, (uint32_t*)hdr);
+            launch_kernel(true, decode_select_plan_kernel<128>, dim3(kPlanCtas, g.Hkv, g.B), dim3(kPlanWarps * 32), smem, st, g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, (uint32_t*)hdr);
         } else {
             if (!set_smem(h, decode_select_plan_kernel<64>, smem, "decode_select_plan_kernel")) return ADASPARK_ERR_CUDA;
-            decode_select_plan_kernel<64><<<dim3(kPlanCtas, g.Hkv, g.B), kPlanWarps * 32, smem, st>>>(g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, (uint32_t*)hdr);
+            launch_kernel(true, decode_select_plan_kernel<64>, dim3(kPlanCtas, g.Hkv, g.B), dim3(kPlanWarps * 32), smem, st, g, qn, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, kc, vc, cube_keys, text_len, dec_bitmap, sel_bitmap, items, n_items, (uint32_t*)hdr);
         }
         if (!launch_ok(h, "decode_select_plan_kernel")) return ADASPARK_ERR_CUDA;
     }

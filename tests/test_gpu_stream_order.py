@@ -1,0 +1,34 @@
+"""Calls whose inputs are made by the kernel right before them in the stream, on one workspace.  The first kernel of a call is
+launched to overlap what comes before it, so it has to wait itself before it reads an input or writes the workspace."""
+from __future__ import annotations
+
+import pytest
+import torch
+
+from paper_2604_08077_b200 import inputs
+
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B", [1, 9])
+def test_decode_inputs_made_right_before(B):
+    wl = inputs.small_decode(seed=91, B=B, T=64, H=8, W=8, cube=(1, 4, 4), n_text=40, Hq=8, Hkv=2, D=128)
+    eng = pu.make_engine(wl, n_text_max=wl.n_text + 1)
+    eng.forward(None, wl.k.cuda(), wl.v.cuda(), wl.n_text)
+    steps = [(wl.q_new.cuda() * s, wl.k_new.cuda() * s, wl.v_new.cuda() * s) for s in (1.0, -0.5, 2.0)]
+    tl = torch.full((B,), wl.n_text, dtype=torch.int32, device="cuda")
+    want = []
+    for q, k, v in steps:
+        want.append(eng.decode(q, k, v, tl)[0].clone())
+        torch.cuda.synchronize()
+    q, k, v = (torch.empty_like(x) for x in steps[0])
+    big, t = torch.empty(1 << 26, device="cuda"), torch.empty_like(tl)
+    for _ in range(30):
+        for (a, b, c), w in zip(steps, want):
+            big.fill_(1.0)                                        # keeps the GPU busy while the host goes on
+            q.copy_(a), k.copy_(b), v.copy_(c), t.copy_(tl)
+            out, _ = eng.decode(q, k, v, t)
+            t.fill_(-5), q.zero_()
+            assert torch.equal(out, w)
