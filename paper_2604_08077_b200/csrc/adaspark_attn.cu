@@ -445,7 +445,12 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
     auto* vc = (__nv_bfloat16*)v_cube;
 
     // header and head exponents start at zero
-    if (!cache_only) cudaMemsetAsync((char*)workspace + h->fw_status_off, 0, h->fw_mask_off - h->fw_status_off, st);
+    if (!cache_only) {
+        const uint32_t n16 = (uint32_t)((h->fw_mask_off - h->fw_status_off) / 16);       // (offsets are multiples of 256)
+        const uint32_t ctas = (n16 + 1023) / 1024;
+        launch_kernel(true, clear_workspace_kernel, dim3(ctas < 592u ? ctas : 592u), dim3(256), 0, st, (uint4*)((char*)workspace + h->fw_status_off), n16);
+        if (!launch_ok(h, "clear_workspace_kernel")) return ADASPARK_ERR_CUDA;
+    }
     mark(h, 0, st);
     // K1: re-layout + pooling
     {
@@ -456,8 +461,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         uint32_t* slot_valid = (!cache_only && g.ragged) ? (uint32_t*)((char*)workspace + h->fw_valid_off) : nullptr;
         // largest |k|^2 per (batch, kv head): only a call that brings the sequence from its first frame sees every key
         uint32_t* key_norm2 = (!cache_only && frame_begin == 0) ? (uint32_t*)((char*)workspace + h->fw_headmax_off) + g.B * g.Hkv : nullptr;
-        if (D == 128) relayout_pool_kernel<128><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
-        else relayout_pool_kernel<64><<<grid, 256, 0, st>>>(g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
+        if (D == 128) launch_kernel(!cache_only, relayout_pool_kernel<128>, grid, dim3(256), 0, st, g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
+        else launch_kernel(!cache_only, relayout_pool_kernel<64>, grid, dim3(256), 0, st, g, kb, vb, kc, vc, cube_keys, slot_valid, key_norm2);
         if (!launch_ok(h, "relayout_pool_kernel")) return ADASPARK_ERR_CUDA;
         const int cube_begin = g.pos_begin >> g.c_shift;
         if (g.C > kBlockTok && g.N_live > cube_begin) {

@@ -38,6 +38,14 @@ __device__ __forceinline__ void block_norm(float k2, uint32_t (&part)[8], uint32
     }
 }
 
+// Zeroes the start of the workspace (n 16-byte pieces).  The first kernel of a call, launched to overlap whatever comes before it in
+// the stream; the next one is let in only when that is finished.  (A memset in its place: 39.3 instead of 37.1 us for 544 tokens, 221.5 / 219.8 for 8256, dense.)
+__global__ void __launch_bounds__(256) clear_workspace_kernel(uint4* dst, uint32_t n) {
+    wait_for_previous_kernel();
+    launch_dependents();
+    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 template <int D>
 __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_bfloat16* __restrict__ k,
                                                             const __nv_bfloat16* __restrict__ v,
@@ -47,6 +55,7 @@ __global__ void __launch_bounds__(256) relayout_pool_kernel(Geom g, const __nv_b
                                                             uint32_t* __restrict__ slot_valid,
                                                             uint32_t* __restrict__ key_norm2_bits) {
     launch_dependents();
+    wait_for_previous_kernel();
     constexpr int kChunks = D / 8;    // 16-byte chunks per row
     constexpr int kVPitch = D + 2;    // padded pitch (elements) of the V staging tile
     __shared__ __align__(16) __nv_bfloat16 Ks[kBlockTok][D];

@@ -32,3 +32,28 @@ def test_decode_inputs_made_right_before(B):
             out, _ = eng.decode(q, k, v, t)
             t.fill_(-5), q.zero_()
             assert torch.equal(out, w)
+
+
+@pytest.mark.parametrize("C", [(1, 4, 4), (2, 8, 8)])
+def test_prefill_inputs_made_right_before(C):
+    """The header and counters of the workspace are cleared on the stream, after the call before: outputs, counters and status
+    of a call do not depend on what follows at once."""
+    wl = inputs.make_prefill("order", seed=92, B=2, T=16, H=8, W=8, cube=C, n_text=21, Hq=8, Hkv=2, D=128, top_p=0.8, offset_std=1.5)
+    eng = pu.make_engine(wl)
+    steps = [(wl.q.cuda() * s, wl.k.cuda() * s, wl.v.cuda() * s) for s in (1.0, -0.5)]
+    want = []
+    for q, k, v in steps:
+        out = eng.forward(q, k, v, wl.n_text)[0].clone()
+        torch.cuda.synchronize()
+        want.append((out, eng.header().executed_kv_blocks))
+    q, k, v = (torch.empty_like(x) for x in steps[0])
+    big = torch.empty(1 << 26, device="cuda")
+    for _ in range(20):
+        for (a, b, c), w in zip(steps, want):
+            big.fill_(1.0)                                        # keeps the GPU busy while the host goes on
+            q.copy_(a), k.copy_(b), v.copy_(c)
+            out = eng.forward(q, k, v, wl.n_text)[0]
+            q.zero_(), k.zero_(), v.zero_()
+            assert torch.equal(out, w[0])
+            hdr = eng.header()
+            assert hdr.status == 0 and hdr.executed_kv_blocks == w[1]
