@@ -59,6 +59,9 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr size_t kNextPairTileOffset = 128;   // in the 256 bytes of the workspace header (cleared per call), behind the public fields
 static_assert(sizeof(adaspark_attn_workspace_header_t) <= kNextPairTileOffset, "the counter lies behind the header's fields");
+// Warps of two waves of the selection kernel (15 an SM): a launch with fewer gives each fewer than 32 rows.  28 heads: 65.1 -> 63.0 us
+// at 1024 tokens, 127 -> 120.5 with 16-token cubes (one wave: 122), 3072 tokens 170.5 -> 167.9.
+constexpr int kSelectWave = 4440;
 constexpr int kExactCtas = 592;   // CTAs of the fp64 selection kernel: four per SM
 // query-gather path: pairs of query tiles take it when their rows' (row, key block) entries are at most this
 // many per key block of the pair's union (measured break-even on a B200, see the attention profile), and the
@@ -157,8 +160,7 @@ bool launch_ok(adaspark_attn* h, const char* what) {
 // be put on the SMs while that one still runs.  That hides the launch and the set-up, but the CTAs that wait take their
 // places SM by SM as these become free: a grid of several waves ends up unevenly spread, and a kernel that lives off its
 // L1 gets what the previous one's shared memory left.  Measured against plain launches: 544 tokens 55.5 -> 45.8 us; but
-// 65536 tokens with every launch overlapped 4.39 -> 4.66 ms in the selection stage (the selection kernel) and 4.42 -> 4.69
-// ms in the attention stage of sparse selections (the merge kernel).
+// 4.42 -> 4.69 ms in the attention stage of sparse selections (the merge kernel, 65536 tokens).
 template <typename... KArgs, typename... Args>
 void launch_kernel(bool overlap, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg;
@@ -488,13 +490,16 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         }
         int32_t* fallback_rows = (int32_t*)(ws + h->fw_fallback_off);
         const bool all = g.top_k <= 0 && !(g.top_p < 1.0);
-        const bool small = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 3 * kScoreWave / 2;   // a call whose selection is about one wave
+        // Up to 2368 query tiles the selection kernels' launches overlap: 1024 tokens, 28 heads, 65.1 -> 58.7 us, 2048 109 -> 101, 4096
+        // 219 -> 213, 16 of 16-token cubes 127 -> 110; beyond that the launches no longer show and the early start costs what it
+        // gains (16384 tokens, 3612 tiles, 1931 / 1938, 65536 7274 / 7259).
+        const bool overlap_select = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 16 * kScoreWave;
         auto launch_exact = [&](const int32_t* rows, const uint32_t* n_list, long long n_ids) {
             if (D == 128)
-                launch_kernel(small, select_exact_kernel<128>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
+                launch_kernel(overlap_select, select_exact_kernel<128>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
                                                                                    tile_mask, tile_union, sel_bitmap, sel_count);
             else
-                launch_kernel(small, select_exact_kernel<64>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
+                launch_kernel(overlap_select, select_exact_kernel<64>, dim3(kExactCtas), dim3(kExactWarps * 32), g.N_ld * 8, st, g, qb, cube_keys, rows, n_list, n_ids,
                                                                                   tile_mask, tile_union, sel_bitmap, sel_count);
             return launch_ok(h, "select_exact_kernel");
         };
@@ -538,8 +543,9 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
 #define ADASPARK_LAUNCH_SELECT(RR, CC, BB, RULE)                                                                       \
     do {                                                                                                               \
         const size_t smem = sizeof(SelectSmem<RR, CC, BB>);                                                            \
-        const int warp_rows = small ? (RR < 8 ? 8 : RR) : 32;      /* few tiles: as many warps as there can be */      \
-        launch_kernel(small, select_nucleus_kernel<RR, CC, BB, RULE>, dim3(kTileRows / warp_rows * (next - first)), dim3(32), \
+        int warp_rows = 32;                                                                                            \
+        while (warp_rows > 8 && warp_rows > RR && kTileRows / warp_rows * (next - first) < kSelectWave) warp_rows /= 2; \
+        launch_kernel(overlap_select, select_nucleus_kernel<RR, CC, BB, RULE>, dim3(kTileRows / warp_rows * (next - first)), dim3(32), \
                       smem, st, g, select_target(RULE, g.top_p, CC, CC <= 256 ? 22 : CC <= 1024 ? 21 : CC <= 2048 ? 20 : 19), \
                       item0, first, warp_rows, (const float*)scores, (const float4*)row_range, (const float*)row_err, tile_mask,  \
                       tile_union, (const unsigned long long*)key_hash, sel_bitmap, sel_count, fallback_rows,           \
