@@ -98,7 +98,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1) attn_
     auto q_phase = [&](int k) -> uint32_t { return (uint32_t)((kGathered ? k / 3 : k >> 1) & 1); };
 
     // ---------------------------------------------------------------- set-up
-    launch_dependents();
+    if (!kGathered) launch_dependents();                        // (the merge: its CTAs start when this grid ends, see its launch)
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(&sm.part_full[i], (kSoftmaxGroups - 1) * 4);

@@ -567,7 +567,6 @@ __global__ void __launch_bounds__(kGatherThreads, 1) attn_gather_kernel(
     Geom g, GatherWs ws, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
     const __nv_bfloat16* __restrict__ q, const uint32_t* slot_valid, unsigned long long* executed_blocks, int32_t* status) {
     extern __shared__ unsigned char gather_smem_raw[];
-    launch_dependents();
     wait_for_previous_kernel();
     GatherSmem<D>& sm = *reinterpret_cast<GatherSmem<D>*>((reinterpret_cast<uintptr_t>(gather_smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int kPanels = D / 64, kQKSteps = D / 16;
