@@ -71,9 +71,11 @@ constexpr uint64_t kGatherDefaultBudget = 24ull << 30;
 constexpr uint64_t kGatherEntriesPerRow = 128;
 constexpr size_t kGatherWindowBytes = 40u << 20;
 // Scores of the query tiles of one launch (fp32, all columns; about half of it is touched over a causal sequence):
-// in whole waves of one tile per SM, as many as fit this budget.  Fewer, longer launches beat a buffer that stays in the L2:
+// the workspace is sized for whole waves of one tile per SM, as many as fit this budget, and a call uses whatever room there is.  Fewer,
+// longer launches beat a buffer that stays in the L2:
 // 40 / 80 / 160 / 320 / 640 MB give 0.50 / 0.42 / 0.39 / 0.36 / 0.36 ms of selection stage at 16384 tokens and 9.3 / 5.8 / 5.4 /
-// 4.8 / 4.6 ms at 65536 (28 heads, 64-token cubes).  They lie where the query-gather path keeps its lists and
+// 4.8 / 4.6 ms at 65536 (28 heads, 64-token cubes); whole calls with 640 MB / 1.5 / 4 GB / all the room beside the query-gather buffers: 65536
+// tokens sharp 7.46 / 7.43 / 7.31 / 7.29 ms, 131072 120.7 / 120.8 / 119.1 / 116.9.  They lie where the query-gather path keeps its lists and
 // partial results: the selection is over when those are begun.  A workspace that holds fewer tiles' scores is taken as it
 // is, down to kScoreItemsMin tiles (less than the 9472 N_ld bytes that the fp64 kernel's score rows once took).
 constexpr size_t kScoreBytes = 640u << 20;
@@ -512,7 +514,10 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             float* head_norm = (float*)(head_max + 2 * g.B * g.Hkv);
             unsigned char* kplanes = (unsigned char*)(ws + h->fw_kplanes_off);
             const size_t room = (workspace_bytes - h->fw_scores_off) / score_item_bytes(g.N_ld);
-            const int score_items = room < (size_t)h->score_items ? (int)room : h->score_items;
+            const int n_hb = g.B * g.Hq, n_items = n_hb * (g.n_tiles - g.tile_begin);
+            // as many query tiles per launch as there is room for, in whole waves
+            const size_t waves = room / kScoreWave;
+            const int score_items = (int)(room >= (size_t)n_items ? (size_t)n_items : waves > 0 ? waves * kScoreWave : room);
             auto* row_range = (float2*)(ws + h->fw_scores_off);
             float* row_err = (float*)(row_range + (size_t)score_items * kTileRows * kRangeParts);
             float* scores = row_err + (size_t)score_items * kTileRows;
@@ -524,7 +529,6 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             if (!encode_u8_2d(&tmKs, kplanes, (uint64_t)4 * n_rows + 128, kDigitRowBytes, kDigitRowBytes, kScoreTcCols) ||
                 !encode_f32_2d(&tmS, scores, (uint64_t)score_items * kTileRows, g.N_ld, 32))
                 return fail(h, ADASPARK_ERR_CUDA, "%s: cuTensorMapEncodeTiled failed", who);
-            const int n_hb = g.B * g.Hq, n_items = n_hb * (g.n_tiles - g.tile_begin);
             const bool by_count = g.top_k > 0;
             for (int item0 = 0; item0 < n_items; item0 += score_items) {
                 const int n_here = n_items - item0 < score_items ? n_items - item0 : score_items;
