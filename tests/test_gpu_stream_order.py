@@ -57,3 +57,31 @@ def test_prefill_inputs_made_right_before(C):
             assert torch.equal(out, w[0])
             hdr = eng.header()
             assert hdr.status == 0 and hdr.executed_kv_blocks == w[1]
+
+
+def test_captured_behind_copies_and_memsets():
+    """In a graph the node before a call's first kernel may be a copy or a memset instead of a kernel."""
+    wl = inputs.make_prefill("graph", seed=93, B=1, T=8, H=8, W=8, cube=(1, 4, 4), n_text=21, Hq=8, Hkv=2, D=128, top_p=0.8, offset_std=1.5)
+    eng = pu.make_engine(wl, n_text_max=wl.n_text + 1)
+    src = [x.cuda() for x in (wl.q, wl.k, wl.v)]
+    q, k, v = (torch.empty_like(x) for x in src)
+    new = [torch.randn(1, 1, h, 128, device="cuda").to(torch.bfloat16) for h in (8, 2, 2)]
+    tl = torch.full((1,), wl.n_text, dtype=torch.int32, device="cuda")
+    want = eng.forward(*src, wl.n_text)[0].clone()
+    want_new = eng.decode(*new, tl)[0].clone()
+    out, out_new, q_new = torch.empty_like(want), torch.empty_like(want_new), torch.empty_like(new[0])
+    torch.cuda.synchronize()
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        for a, b in zip((q, k, v), src):
+            a.copy_(b)
+        eng.forward(q, k, v, wl.n_text, out=out)
+        q_new.copy_(new[0])
+        eng.decode(q_new, new[1], new[2], tl, out=out_new)
+        q.zero_()
+        out_new.add_(0.0)
+        eng.forward(*src, wl.n_text, out=out)
+    for _ in range(10):
+        out.zero_(), out_new.zero_()
+        graph.replay()
+        assert torch.equal(out, want) and torch.equal(out_new, want_new)
