@@ -529,6 +529,7 @@ __global__ void __launch_bounds__(32) select_nucleus_kernel(
             unsure = unsure || tied || !(last < INFINITY);
             const uint32_t any_unsure = of_row(__ballot_sync(kFull, unsure)), any_reached = of_row(__ballot_sync(kFull, reached));   // both by all lanes
             unsure = any_unsure != 0u || any_reached == 0u || !(tail ? base <= target : base < target);
+            __syncwarp();                                                  // bits of the row's other lanes have arrived: none follows the zeros
             if (n > 0 && (give_up || unsure)) {
                 for (int wd = u; wd < n_words_live; wd += U) sm.words[wd][ro] = 0u;
                 if (u == 0) fallback_rows[atomicAdd(fallback_count, 1u)] = (int32_t)(gt_cap * kTileRows + r0 + row);

@@ -152,3 +152,33 @@ def test_last_columns_of_a_row(n_cubes, top_p):
     wl = inputs.make_prefill("chunks", seed=86, B=1, T=n_cubes, H=4, W=3, cube=(1, 4, 4), n_text=139, n_prefix=13, Hq=3, Hkv=1,
                              D=128 if n_cubes % 2 else 64, top_p=top_p, offset_std=1.5)
     assert _equal(wl).fallback_rows < 0.005 * wl.S * wl.Hq + 2
+
+
+@pytest.mark.parametrize("D,heads", [(128, 4), (64, 3)])
+def test_rows_left_to_the_fp64_kernel_leave_nothing_in_the_union(D, heads):
+    """Cubes whose scores differ by less than the fixed point can tell, ordered against their index: the kernel sets bits for such a
+    row, finds that it cannot decide it and takes them back before the words enter the tile's union.  All rows of a head share one
+    query, so that a tile selects few cubes; a bit too many would be a block visited more than with the fp64 kernel's selection
+    (cubes are single key blocks here)."""
+    wl = inputs.make_prefill("union", seed=87, B=1, T=160, H=8, W=8, cube=(4, 4, 4), n_text=33, Hq=heads, Hkv=1, D=D, top_p=0.8, offset_std=1.5)
+    k = wl.k.clone()
+    frames = k[:, :wl.S_v].view(1, 40, 4, 64, 1, D)
+    frames.copy_(frames[:, ::8].repeat_interleave(8, 1))
+    frames[..., 5] = torch.arange(40).view(1, 40, 1, 1, 1).to(torch.bfloat16) / 16
+    q = (wl.q[:, :1] * 2).expand_as(wl.q).clone()
+    q[..., 5] = 2.0 ** -22
+    got = []
+    for kernel in (1, 2):
+        eng = binding.AdaSAttn(cube=wl.cube, n_q_heads=wl.Hq, n_kv_heads=wl.Hkv, head_dim=wl.D, top_p=wl.top_p)
+        binding.adaspark_attn_set_prefill_kernel(eng.handle, kernel)
+        eng.set_gather(0.0, 0)
+        eng.partition(wl.B, wl.T, wl.H, wl.W, wl.n_text)
+        out, bitmap, count = eng.forward(q.cuda(), k.cuda(), wl.v.cuda(), wl.n_text, want_selection=True)
+        torch.cuda.synchronize()
+        got.append((out, bitmap, count, eng.header()))
+    assert all(torch.equal(a, b) for a, b in zip(got[0][:3], got[1][:3]))
+    mine, want = got[0][3], got[1][3]
+    assert mine.status == want.status == 0 and mine.fallback_rows > 0.1 * wl.S * wl.Hq
+    assert mine.executed_kv_blocks == want.executed_kv_blocks and mine.max_tile_kv_blocks == want.max_tile_kv_blocks
+    tiles = (wl.S + 127) // 128
+    assert mine.executed_kv_blocks < 0.7 * wl.Hq * tiles * (tiles + 1)       # of the blocks of dense causal attention
