@@ -121,8 +121,10 @@ adaspark_status_t adaspark_attn_create(const adaspark_attn_config_t *config,
  * ERR_UNSUPPORTED if N > 4096 or the cache would hold more than 2097152 rows per sequence
  * (s_video + n_text_max + 1).
  * The forward workspace holds the selection masks, the digit planes of the mean keys and, one after the other in
- * the same place, the cube scores of as many query tiles as one launch covers (at most 640 MB; none with top_p >= 1)
- * and the buffers of the query-gather path.  Q is read where the caller left it.  A program that only decodes
+ * the same place, the cube scores of as many query tiles as one launch covers (none with top_p >= 1) and the buffers of
+ * the query-gather path.  It is sized for 640 MB of scores (or those of the whole call, if less) or for the query-gather buffers,
+ * whichever is more, and a launch covers the tiles that there is room for: a smaller budget of adaspark_attn_set_gather can mean
+ * more launches in long calls (1 to 3 % of a call of 65536 tokens and more).  Q is read where the caller left it.  A program that only decodes
  * and builds caches (_forward with q = NULL takes no workspace) needs decode_workspace_bytes alone. */
 adaspark_status_t adaspark_attn_partition(adaspark_attn_t *handle, int32_t batch, int32_t frames,
                                           int32_t grid_h, int32_t grid_w, int32_t n_text_max,
@@ -142,8 +144,8 @@ adaspark_status_t adaspark_attn_get_layout(const adaspark_attn_t *handle,
  *   sel_bitmap   out, nullable: uint32 [B, Hq, S, bitmap_words], bit j of a row (raster token
  *                     order) is set iff cube j is in the row's nucleus S_i.
  *   sel_count    out, nullable: int32 [B, Hq, S] = |S_i|.
- *   workspace    device scratch, 256-byte aligned, of forward_workspace_bytes; also taken with room for the scores of
- *                fewer query tiles (down to 8), which are then computed in more launches.
+ *   workspace    device scratch, 256-byte aligned, of forward_workspace_bytes (of a larger one no more is used); also taken
+ *                with room for the scores of fewer query tiles (down to 8), which are then computed in more launches.
  * Enqueues its kernels on `cuda_stream` and returns; no host synchronisation, no other stream, no
  * allocation.  The Q tiles of the attention kernel are TMA boxes of `q` itself (the tensor map is built
  * on the host per call): `q` needs 16-byte alignment and must stay valid until the call's work is done.

@@ -36,7 +36,6 @@ struct adaspark_attn {
     size_t fw_status_off, fw_headmax_off, fw_valid_off, fw_gcol_off, fw_mask_off, fw_union_off, fw_fallback_off,
         fw_kplanes_off, fw_keyhash_off, fw_scores_off, fw_gpair_off, fw_grow_off, fw_gml_off, fw_gref_off, fw_glocal_off, fw_gitems_off, fw_gentries_off, fw_gparto_off,
         fw_gpartml_off, fw_min, fw_total;      // fw_min: the smallest workspace a forward takes, fw_total: the one it is best given
-    int score_items;            // query tiles per launch of the score / selection pair, at most
     uint32_t gather_pairs;      // pairs of query tiles that may be gathered at once, at most (whole cubes: room for their local range)
     // query-gather path of the prefill: capacity in (row, key block) entries, decision threshold, byte budget
     uint32_t gather_cap;
@@ -71,8 +70,9 @@ constexpr uint64_t kGatherDefaultBudget = 24ull << 30;
 constexpr uint64_t kGatherEntriesPerRow = 128;
 constexpr size_t kGatherWindowBytes = 40u << 20;
 // Scores of the query tiles of one launch (fp32, all columns; about half of it is touched over a causal sequence):
-// the workspace is sized for whole waves of one tile per SM, as many as fit this budget, and a call uses whatever room there is.  Fewer,
-// longer launches beat a buffer that stays in the L2:
+// the workspace is sized for whole waves of one tile per SM, as many as fit this budget.  A call uses the room that there is: where the
+// query-gather buffers make the workspace larger (by its budget and the number of tokens), fewer launches do.  Fewer, longer launches
+// beat a buffer that stays in the L2:
 // 40 / 80 / 160 / 320 / 640 MB give 0.50 / 0.42 / 0.39 / 0.36 / 0.36 ms of selection stage at 16384 tokens and 9.3 / 5.8 / 5.4 /
 // 4.8 / 4.6 ms at 65536 (28 heads, 64-token cubes); whole calls with 640 MB / 1.5 / 4 GB / all the room beside the query-gather buffers: 65536
 // tokens sharp 7.46 / 7.43 / 7.31 / 7.29 ms, 131072 120.7 / 120.8 / 119.1 / 116.9.  They lie where the query-gather path keeps its lists and
@@ -308,8 +308,7 @@ adaspark_status_t adaspark_attn_partition(adaspark_attn_t* h, int32_t batch, int
         const size_t n_items = (size_t)batch * Hq * n_tiles_cap;
         size_t waves = kScoreBytes / ((size_t)kTileRows * N_ld * 4 * kScoreWave);
         if (waves < 1) waves = 1;
-        h->score_items = (int)(waves * kScoreWave < n_items ? waves * kScoreWave : n_items);
-        scores_end += (size_t)h->score_items * score_item_bytes(N_ld);
+        scores_end += (waves * kScoreWave < n_items ? waves * kScoreWave : n_items) * score_item_bytes(N_ld);
         scores_end_min += (n_items < kScoreItemsMin ? n_items : kScoreItemsMin) * score_item_bytes(N_ld);
     }
     // query-gather path, in the place of the scores: per pair (mode, entries, offset) | per row (entries, first partial) |
@@ -513,7 +512,8 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
             uint32_t* head_max = (uint32_t*)(ws + h->fw_headmax_off);
             float* head_norm = (float*)(head_max + 2 * g.B * g.Hkv);
             unsigned char* kplanes = (unsigned char*)(ws + h->fw_kplanes_off);
-            const size_t room = (workspace_bytes - h->fw_scores_off) / score_item_bytes(g.N_ld);
+            // nothing behind the size that the library asks for is touched, however large the buffer is
+            const size_t room = ((workspace_bytes < h->fw_total ? workspace_bytes : h->fw_total) - h->fw_scores_off) / score_item_bytes(g.N_ld);
             const int n_hb = g.B * g.Hq, n_items = n_hb * (g.n_tiles - g.tile_begin);
             // as many query tiles per launch as there is room for, in whole waves
             const size_t waves = room / kScoreWave;

@@ -99,3 +99,26 @@ def test_scores_of_few_tiles_at_a_time_give_the_same(kw, top_k):
             assert bool((eng.workspace[eng.ws_bytes:] == 77).all())
     assert all(torch.equal(a, b) for a, b in zip(got[0][:3], got[1][:3]))
     assert got[1][3] > got[0][3]                           # in several launches
+
+
+@pytest.mark.gpu
+def test_nothing_is_written_behind_the_size_the_library_asks_for():
+    """A workspace at the start of a larger buffer, whose whole size the call is told: what lies behind forward_workspace_bytes stays as it
+    was, also where the scores of one more launch would fit there (4096 cubes, 513 query tiles; the size asked for holds those of 296)."""
+    wl = inputs.make_prefill("behind", seed=302, B=1, T=4096, H=4, W=4, cube=(1, 4, 4), n_text=40, Hq=1, Hkv=1, D=64, top_p=0.9,
+                             offset_std=1.5)
+    eng = binding.AdaSAttn(cube=wl.cube, n_q_heads=1, n_kv_heads=1, head_dim=64, top_p=wl.top_p)
+    eng.set_gather(0.0, 0)
+    eng.partition(wl.B, wl.T, wl.H, wl.W, wl.n_text)
+    asked = eng.layout.forward_workspace_bytes
+    got = []
+    for more in (0, 600 << 20):
+        eng.ws_bytes = asked + more
+        eng.workspace = torch.full((eng.ws_bytes + (1 << 20),), 77, dtype=torch.uint8, device="cuda")
+        out, bitmap, _ = eng.forward(wl.q.cuda(), wl.k.cuda(), wl.v.cuda(), wl.n_text, want_selection=True)
+        torch.cuda.synchronize()
+        assert eng.header().status == 0
+        touched = int((eng.workspace[asked:] != 77).sum())
+        assert touched == 0
+        got.append((out, bitmap))
+    assert all(torch.equal(a, b) for a, b in zip(*got))
