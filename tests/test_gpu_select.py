@@ -1,9 +1,11 @@
 """Selection from the tensor-core scores: bit by bit the selection of the fp64 kernel.
 
 Rows whose boundary is nearer than fp32 can tell are handed to the fp64 kernel, all others are decided from fp32
-scores, so no bit may differ.  The candidate counts are those at which the kernel changes its shape (lanes per row,
-scores per lane, mask words) and their neighbours."""
+scores, so no bit may differ.  The candidate counts are those at which the kernel changes its shape (rows per pass,
+scores per row, buckets) and their neighbours."""
 from __future__ import annotations
+
+import math
 
 import pytest
 import torch
@@ -145,13 +147,35 @@ def test_many_masses_that_are_nearly_equal(top_p):
 @pytest.mark.parametrize("n_cubes", [7, 9, 16, 57, 63, 119, 127, 249, 505, 1017])
 @pytest.mark.parametrize("top_p", [0.2, 0.7, 0.99999])
 def test_last_columns_of_a_row(n_cubes, top_p):
-    """Candidate counts one off the 8 columns that a lane takes at a time, at the end of every kernel shape, with a text prefix
+    """Candidate counts one off the 8 columns that a lane takes at a time, at the end of the kernel shapes for up to 1024, with a text prefix
     and a text that end inside the rows of a pass (rows without candidates beside rows with all of them) and cubes at the
     faces that hold no more than a few rows.  No more rows than elsewhere are left to the fp64 kernel, also where two lanes
     sum all buckets of a row."""
     wl = inputs.make_prefill("chunks", seed=86, B=1, T=n_cubes, H=4, W=3, cube=(1, 4, 4), n_text=139, n_prefix=13, Hq=3, Hkv=1,
                              D=128 if n_cubes % 2 else 64, top_p=top_p, offset_std=1.5)
     assert _equal(wl).fallback_rows < 0.005 * wl.S * wl.Hq + 2
+
+
+@pytest.mark.parametrize("n_cubes", [2041, 4089])
+@pytest.mark.parametrize("top_p", [0.2, 0.7, 0.99999])
+def test_last_columns_of_the_largest_shapes(n_cubes, top_p):
+    """The same for the shapes of one row a pass, where more rows are too near to call: the boundary cube holds less of the mass.  A row is
+    handed over if the target lies within eps of the sum up to that cube or before it: eps <= 1e-5 q Z, q = min(p, 1 - p) (at most 88
+    additions of 2^-24 and, with scores of up to 24 in log2 units, 2 (1 - q) times 2.4e-6), so a share of 2 eps / its mass, measured on the text
+    rows, whose candidates are all cubes (the other rows have fewer, and larger masses).  Besides: 1e-3 of the rows whose last selected score
+    is at the edge of a bucket, and those where it is within 4e-6 of the next one."""
+    wl = inputs.make_prefill("chunks", seed=88, B=1, T=n_cubes, H=4, W=3, cube=(1, 4, 4), n_text=139, n_prefix=13, Hq=3, Hkv=1,
+                             D=128 if n_cubes == 2041 else 64, top_p=top_p, offset_std=1.5)
+    keys = wl.k[0, wl.n_prefix:wl.n_prefix + wl.S_v, 0].cuda().double().view(n_cubes, 12, wl.D).mean(1)
+    scores = (wl.q[0, -wl.n_text:].cuda().double().flatten(0, 1) @ keys.T * wl.D ** -0.5).sort(descending=True).values
+    probs = scores.softmax(1)
+    last = ((probs.cumsum(1) < top_p).sum(1, keepdim=True)).clamp(max=n_cubes - 2)
+    near = 2e-5 * min(top_p, 1 - top_p) / probs.gather(1, last)
+    gap = (scores.gather(1, last) - scores.gather(1, last + 1)) / math.log(2.0)
+    share = float(near.clamp(max=1.0).mean() + (gap < 4e-6).double().mean()) + 1e-3
+    hdr = _equal(wl)
+    print(f"{n_cubes} cubes, p {top_p}: {hdr.fallback_rows} rows of {wl.S * wl.Hq}, {share * wl.S * wl.Hq:.0f} allowed")
+    assert share < 0.1 and hdr.fallback_rows < share * wl.S * wl.Hq + 2
 
 
 @pytest.mark.parametrize("D,heads", [(128, 4), (64, 3)])
