@@ -92,7 +92,8 @@ typedef struct {
     uint64_t decode_kv_blocks;    /* decode: 64-key blocks gathered, summed over (b, kv head) */
     uint32_t fallback_rows;       /* prefill: query rows whose selection the tensor-core kernel
                                      left to the fp64 selection kernel: their boundary is nearer
-                                     than fp32 can tell (about one row in 10^4 to 10^3)       */
+                                     than fp32 can tell (about one row in 10^4 to 10^3, with
+                                     4096 cubes one in 10^2)                                  */
     uint32_t max_tile_kv_blocks;  /* prefill: largest number of 64-key blocks one 256-row pair of
                                      query tiles visited (load imbalance: compare with the mean
                                      executed_kv_blocks / 2 / number of pair tiles)           */

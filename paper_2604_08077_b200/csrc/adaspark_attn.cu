@@ -58,8 +58,9 @@ namespace {
 constexpr size_t kAlign = 256;
 constexpr size_t kNextPairTileOffset = 128;   // in the 256 bytes of the workspace header (cleared per call), behind the public fields
 static_assert(sizeof(adaspark_attn_workspace_header_t) <= kNextPairTileOffset, "the counter lies behind the header's fields");
-// Warps of two waves of the selection kernel (15 an SM): a launch with fewer gives each fewer than 32 rows.  28 heads: 65.1 -> 63.0 us
-// at 1024 tokens, 127 -> 120.5 with 16-token cubes (one wave: 122), 3072 tokens 170.5 -> 167.9.
+// A selection launch of fewer warps than this gives each fewer than 32 rows.  A measured line (two waves of 15 warps an SM; the shapes hold
+// 9 to 24), taken with 28 heads of 128 and up to 256 candidates: 65.1 -> 63.0 us at 1024 tokens, 127 -> 120.5 with 16-token cubes (a line at
+// half of it: 122), 3072 tokens 170.5 -> 167.9.
 constexpr int kSelectWave = 4440;
 constexpr int kExactCtas = 592;   // CTAs of the fp64 selection kernel: four per SM
 // query-gather path: pairs of query tiles take it when their rows' (row, key block) entries are at most this
@@ -490,7 +491,7 @@ adaspark_status_t forward_impl(adaspark_attn_t* h, const char* who, const void* 
         }
         int32_t* fallback_rows = (int32_t*)(ws + h->fw_fallback_off);
         const bool all = g.top_k <= 0 && !(g.top_p < 1.0);
-        // Up to 2368 query tiles the selection kernels' launches overlap: 1024 tokens, 28 heads, 65.1 -> 58.7 us, 2048 109 -> 101, 4096
+        // Up to 2368 query tiles the selection kernels' launches overlap (measured with 28 heads of 128): 1024 tokens, 28 heads, 65.1 -> 58.7 us, 2048 109 -> 101, 4096
         // 219 -> 213, 16 of 16-token cubes 127 -> 110; beyond that the launches no longer show and the early start costs what it
         // gains (16384 tokens, 3612 tiles, 1931 / 1938, 65536 7274 / 7259).
         const bool overlap_select = (long long)g.B * g.Hq * (g.n_tiles - g.tile_begin) <= 16 * kScoreWave;

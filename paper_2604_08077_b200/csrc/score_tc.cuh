@@ -19,9 +19,9 @@
 // W_j = V_j >> sh an int32: sh is the row's own shift, the smallest for which |q| max|k_j - k_0| (Cauchy-Schwarz over the
 // head) proves that no score overflows (on the benchmark inputs sh = 8: one unit of W is 1e-8 in the
 // scaled logit, below the 2e-8 that the dropped levels leave), and the largest and smallest score of every row.  The
-// selection kernel (select_nucleus.cuh) reads them from an L2-sized scratch buffer and decides every row whose
-// boundary is clearer than fp32 can be wrong; a launch covers as many query tiles as the buffer holds, and the two
-// kernels alternate over the call.
+// selection kernel (select_nucleus.cuh) reads them from the workspace and decides every row whose boundary is clearer than
+// fp32 can be wrong.  A launch covers as many query tiles as the workspace has room for, mostly those of the whole call; where it has
+// less, the two kernels alternate over the call.
 //
 // Rows whose exponents are so large that the fixed-point error could reach the margin (f > kMaxScorePerUnit) are
 // marked (NaN scores) and go to the fp64 kernel of select_exact.cuh.

@@ -25,17 +25,20 @@
 //     1 - p:  eps = q Z (2 (1 - q) e + (additions of Z, of the base and of the list + 2) 2^-24).
 //   - a last selected cube and a first rejected one, listed or not, that lie less than 2 rho + 4 |s| 2^-24 apart and are not
 //     copies of one cube.  (For the unlisted ones the edge of the first bucket stands, and what finer buckets leave out.)
-// That is one row in 10^4 to 10^3 on the benchmark inputs, and no more with p nearer to 1 (sums up to p Z and an eps in
+// That is one row in 10^4 to 10^3 on the benchmark inputs (the more cubes, the smaller the masses at the boundary: 0.8 % with 4096 cubes),
+// and no more with p nearer to 1 (sums up to p Z and an eps in
 // proportion to Z left 0.7 / 2.1 / 5.5 % undecided at p = 0.99 / 0.999 / 0.9999, 65536 tokens).  With them go the rows the score
 // kernel marked, and rows with more equal scores at the boundary than the list holds.
 //
-// What bounds it: latency and instruction issue (12 to 22 warps on an SM, as many as the scores of their rows leave room for): about
-// 13 instructions per score of a lane in the two sweeps and 700 to 1200 per pass of R rows beside them.  Lane = row + R x (which
+// What bounds it: latency and instruction issue.  An SM holds 16 or 17 warps (24 in the shape for 128 candidates, 9 in that for 4096), as many
+// as the scores of their rows leave room for, and issues in 58 to 70 % of the cycles (42 % with 9 warps): 18 to 20 instructions per score of
+// a lane in the two sweeps and 820 to 1100 per pass of R rows beside them (ncu; 77 a row for 64 candidates, 843 for 730).  Lane = row + R x (which
 // of the row's lanes): the histogram [bucket][row] is met by neighbouring lanes in different banks, the bits of 8 columns are a
 // byte of the mask words without an exchange, and what is done per row (boundary, list, order of the list) is done for R rows at
 // once.  (With the lanes side by side on 1 to 4 rows per pass and the scores in registers, 1000 to 1400 instructions a pass, shuffles
 // for every row sum and nibbles transposed between lanes: selection kernels alone, us, before / now: 64 candidates 105 / 53, 128 to
-// 256 120 / 86 (28 heads, 16384 tokens), 1024 1683 / 1263 (65536 tokens), 2048 13470 / 8950 (131072, half static).)  The per-cube work
+// 256 120 / 86 (28 heads, 16384 tokens), 1024 1683 / 1263 (65536 tokens), 2048 13470 / 8950 (131072, half static); with scores and
+// fp64 rows, 4096 cubes of 65536 tokens 23.1 / 16.3 ms.)  The per-cube work
 // is spread over the pipes: the bits come from funnel shifts of signs, the mass before the bucket from a saturating multiply, the
 // exponential from the MUFU unit, the rest from packed fp32 pairs, because the integer / comparison pipe issues at half the
 // rate of the fp32 pipe.
@@ -86,7 +89,8 @@ inline SelectTarget select_target(SelectRule rule, double top_p, int capacity, i
     return t;
 }
 
-// Shared memory of a warp on R rows of up to kCols scores (a bucket holds some 5 of them, with normally distributed scores).  The padding of a row keeps the 16-byte loads of 8 neighbouring
+// Shared memory of a warp on R rows of up to kCols scores.  (Normally distributed, the fullest bucket holds some 2 of 64 and 128 scores, 5 of 256
+// to 1024, 11 of 2048 and 23 of 4096: the list's 32 places are near in the largest shape, which therefore splits buckets more often.)  The padding of a row keeps the 16-byte loads of 8 neighbouring
 // lanes (8 rows, or with fewer rows several chunks of each, see `swap`) in 8 different bank groups.
 template <int R, int kCols, int kBuckets>
 struct SelectSmem {
