@@ -188,6 +188,13 @@ __device__ __forceinline__ ScoreItem score_item(const Geom& g, int it) {
     return w;
 }
 
+// Ranges of a row of the items it, it + step, .. whose scores have not been computed (a wait has expired; the call's status says so).  The
+// selection kernel goes by a range without bounds of its own, and the workspace holds anything: with a lower end of -inf it leaves the
+// row to the fp64 kernel, which needs no scores, whatever the row's other parts are.
+__host__ __device__ inline void abandon_ranges(float2* row_range, int it, int n_items, int step, int row, int part) {
+    for (; it < n_items; it += step) row_range[kRangeParts * ((size_t)it * kTileRows + row) + part] = make_float2(-INFINITY, -INFINITY);
+}
+
 // Scores of the items [item0, item0 + n_items): row r of item item0 + i goes to row 128 * i + r of the scratch
 // matrix that tmS describes (fp32 [rows][N_ld]; columns beyond the tile's last candidate are not written), the
 // largest and smallest score of its candidates to row_range[4 * (128 * i + r) + part], part = which 16 of every 64
@@ -375,8 +382,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
         unsigned char* stage = reinterpret_cast<unsigned char*>(&sm.stage[warp][0][0]) + lane * 64;
         const int swz = (lane >> 1) & 3;                              // 64-byte swizzle: chunk ^ (row / 2) % 4
         bool ok = true;
-        int c = 0, n_done = 0;
-        for (int it = blockIdx.x; ok && it < n_items; it += gridDim.x) {
+        int c = 0, n_done = 0, it = blockIdx.x;
+        for (; it < n_items; it += gridDim.x) {
             const ScoreItem w = score_item(g, item0 + it);
             if (w.n_ct == 0) continue;
             const int qb = n_done & 1;
@@ -390,7 +397,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
             if (lane == 0) tc::mbar_arrive(&sm.qd_free[qb]);
             const uint32_t m1 = 1u << (16 - sh), m0 = m1 << 8;
             float top = -INFINITY, low = INFINITY;
-            for (int ct = 0; ok && ct < w.n_ct; ++ct, ++c) {
+            for (int ct = 0; ct < w.n_ct; ++ct, ++c) {
                 const int s = c & 1;
                 if (!(ok = tc::mbar_wait(&sm.acc_full[s], (c >> 1) & 1, abort_flag))) break;
                 tc::tc_fence_after_sync();
@@ -442,9 +449,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1) score_tc_kernel(
                     if (lane == 0) tc::mbar_arrive(&sm.acc_free[s]);
                 }
             }
+            if (!ok) break;
             row_range[kRangeParts * ((size_t)it * kTileRows + quarter * 32 + lane) + part] = make_float2(top, low);
             ++n_done;
         }
+        if (!ok) abandon_ranges(row_range, it, n_items, gridDim.x, quarter * 32 + lane, part);
         if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");   // every box is in global memory
     } else if (warp == kClearWarp) {
         for (int it = blockIdx.x; it < n_items; it += gridDim.x) {

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(32) select_nucleus_kernel(
         const int n = n_next;
         float top = fmaxf(fmaxf(ra.x, ra.z), fmaxf(rb.x, rb.z)), low = fminf(fminf(ra.y, ra.w), fminf(rb.y, rb.w));
         const float err = n > 0 ? err_next : 0.f;
-        bool give_up = n > 0 && !(top > -INFINITY && low > -INFINITY);     // marked by the score kernel
+        bool give_up = n > 0 && !(top > -INFINITY && low > -INFINITY);     // marked by the score kernel, or its scores are missing
         const bool act = n > 0 && !give_up;
         if (!act) top = low = 0.f;
         cp_async_wait<0>();
