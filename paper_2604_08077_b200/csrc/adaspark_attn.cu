@@ -80,7 +80,7 @@ constexpr size_t kGatherWindowBytes = 40u << 20;
 // partial results: the selection is over when those are begun.  A workspace that holds fewer tiles' scores is taken as it
 // is, down to kScoreItemsMin tiles (less than the 9472 N_ld bytes that the fp64 kernel's score rows once took).
 constexpr size_t kScoreBytes = 640u << 20;
-constexpr int kScoreWave = 148;
+constexpr int kScoreWave = 148;       // SMs of a B200 (the workspace is sized without a device)
 constexpr int kScoreItemsMin = 8;
 size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 // one query tile's scores, score ranges and error bounds (a multiple of kAlign)
